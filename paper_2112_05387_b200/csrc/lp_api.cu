@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "../../include/lp.h"
+#include "conv_f32.cuh"
 #include "conv_simt.cuh"
 #include "conv_tc.cuh"
 #include "conv_tc2.cuh"
@@ -163,7 +164,7 @@ struct Device {
   int sm_count = 148;
   EncodeTiledFn encode = nullptr;
   // kernel attributes are per device: set on the first launch of each kernel family on that device
-  bool conv_attr = false, wgrad_attr = false, wgrad_halo_attr = false, conv2_attr = false;
+  bool conv_attr = false, wgrad_attr = false, wgrad_halo_attr = false, conv2_attr = false, f32_attr = false;
   int max_pairs = 0;   // CTA pairs of conv_tc2_kernel that can be resident at once (0: not usable)
   int init() {
     if (ready) return LP_OK;
@@ -876,6 +877,127 @@ static int fewch_cpt(int cout, int dtype) {
   return 0;
 }
 
+// ---------------------------------------------------------------------------------------------
+// fp32 convolutions (conv_f32.cuh)
+// ---------------------------------------------------------------------------------------------
+static bool f32_tile_ok(const ConvDef& c) {
+  return c.cin % 4 == 0 && c.cout % 4 == 0 && (c.R == 1 || c.R == 3) && c.pad == c.R / 2 && (c.stride == 1 || c.stride == 2) &&
+         (reinterpret_cast<uintptr_t>(c.w) & 15) == 0;   // 16-byte copies of the weights (always, in a valid network's blob)
+}
+static const size_t kF32MaxSmem = 100 * 1024;
+static int f32_set_attributes() {
+  bool& done = cur_dev().f32_attr;
+  if (done) return LP_OK;
+  LP_CUDA_OK(cudaFuncSetAttribute(conv_f32_tile_kernel<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32MaxSmem));
+  LP_CUDA_OK(cudaFuncSetAttribute(conv_f32_tile_kernel<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32MaxSmem));
+  LP_CUDA_OK(cudaFuncSetAttribute(conv_f32_tile_kernel<8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32MaxSmem));
+  LP_CUDA_OK(cudaFuncSetAttribute(conv_f32_tile_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32MaxSmem));
+  done = true;
+  return LP_OK;
+}
+// Launch over the classes and taps already in `p` (everything else is derived here); N images.
+static int launch_conv_f32(lp_handle* h, ConvF32Params& p, int N, bool dgrad, cudaStream_t st) {
+  int rc = f32_set_attributes();
+  if (rc != LP_OK) return rc;
+  int reach_h = 0, reach_w = 0, max_taps = 1;
+  for (int i = 0; i < p.ncls; ++i) {
+    int h0 = 0, h1 = 0, w0 = 0, w1 = 0;
+    for (int t = 0; t < p.cls_ntaps[i]; ++t) {
+      const int dh = p.tap_dh[p.cls_tap0[i] + t], dw = p.tap_dw[p.cls_tap0[i] + t];
+      if (t == 0) { h0 = h1 = dh; w0 = w1 = dw; }
+      h0 = std::min(h0, dh); h1 = std::max(h1, dh); w0 = std::min(w0, dw); w1 = std::max(w1, dw);
+    }
+    p.cls_dh0[i] = h0; p.cls_dw0[i] = w0;
+    reach_h = std::max(reach_h, h1 - h0); reach_w = std::max(reach_w, w1 - w0);
+    max_taps = std::max(max_taps, p.cls_ntaps[i]);
+  }
+  p.PH = 7 * p.in_step + reach_h + 1;
+  p.PW = 7 * p.in_step + reach_w + 1;
+  p.row_pitch = p.PW * 16;
+  while (p.row_pitch % 32 != 4) p.row_pitch += 4;
+  p.w_pitch = max_taps * 16 + 4;
+  p.w_off = p.PH * p.row_pitch;
+  p.stage_floats = p.w_off + 16 * p.w_pitch;
+  p.tiles_w = (p.OWl + 7) / 8;
+  p.tiles_h = (p.OHl + 7) / 8;
+  const dim3 grid((unsigned)(p.tiles_w * p.tiles_h * N), (unsigned)((p.Cout + 15) / 16), (unsigned)p.ncls);
+  // eight warps a block where there are at most two blocks per SM, four (twice the blocks resident) otherwise
+  const long long blocks = (long long)grid.x * grid.y * grid.z;
+  const int ks = blocks <= 2LL * cur_dev().sm_count ? 8 : 4;
+  const size_t smem = std::max((size_t)2 * p.stage_floats * 4, (size_t)ks * 64 * 20 * 4);
+  if (smem > kF32MaxSmem) return LP_ERR_UNSUPPORTED;
+  if (ks == 8 && dgrad) LP_CUDA_OK(launch_pdl(conv_f32_tile_kernel<8, true>, grid, dim3(256), smem, st, p));
+  else if (ks == 8) LP_CUDA_OK(launch_pdl(conv_f32_tile_kernel<8, false>, grid, dim3(256), smem, st, p));
+  else if (dgrad) LP_CUDA_OK(launch_pdl(conv_f32_tile_kernel<4, true>, grid, dim3(128), smem, st, p));
+  else LP_CUDA_OK(launch_pdl(conv_f32_tile_kernel<4, false>, grid, dim3(128), smem, st, p));
+  if (h) h->launches++;
+  return LP_OK;
+}
+static int conv_forward_f32(lp_handle* h, const ConvDef& c, int N, const float* x, float* y, const float* addend, double* stats,
+                            cudaStream_t st) {
+  ConvF32Params p;
+  memset(&p, 0, sizeof(p));
+  p.act = x; p.w = c.w; p.addend = addend; p.out = y; p.stats = stats;
+  p.aH = c.H; p.aW = c.W; p.aC = c.cin;
+  p.OHl = p.out_H = c.OH; p.OWl = p.out_W = c.OW; p.Cout = c.cout;
+  p.in_step = c.stride; p.os = 1; p.wtaps = c.R * c.R; p.ncls = 1;
+  p.cls_ntaps[0] = c.R * c.R;
+  for (int t = 0; t < c.R * c.R; ++t) { p.tap_dh[t] = t / c.R - c.pad; p.tap_dw[t] = t % c.R - c.pad; p.tap_w[t] = t; }
+  return launch_conv_f32(h, p, N, false, st);
+}
+static int conv_dgrad_f32(lp_handle* h, const ConvDef& c, int N, const float* dy, float* dx, const float* addend, cudaStream_t st) {
+  ConvF32Params p;
+  memset(&p, 0, sizeof(p));
+  p.act = dy; p.w = c.w; p.addend = addend; p.out = dx;
+  p.aH = c.OH; p.aW = c.OW; p.aC = c.cout;
+  p.out_H = c.H; p.out_W = c.W; p.Cout = c.cin;
+  p.in_step = 1; p.os = c.stride; p.wtaps = c.R * c.R;
+  p.OHl = (c.H + c.stride - 1) / c.stride; p.OWl = (c.W + c.stride - 1) / c.stride;
+  p.ncls = c.stride * c.stride;
+  int n = 0;
+  for (int cls = 0; cls < p.ncls; ++cls) {   // one class per parity of the input pixel (an empty one writes addend or zero)
+    const int ph = cls / c.stride, pw = cls % c.stride;
+    p.cls_oh[cls] = ph; p.cls_ow[cls] = pw; p.cls_tap0[cls] = n;
+    for (int r = 0; r < c.R; ++r) {
+      if ((ph + c.pad - r) % c.stride) continue;
+      for (int q = 0; q < c.R; ++q) {
+        if ((pw + c.pad - q) % c.stride) continue;
+        p.tap_dh[n] = (ph + c.pad - r) / c.stride; p.tap_dw[n] = (pw + c.pad - q) / c.stride; p.tap_w[n] = r * c.R + q;
+        ++n;
+      }
+    }
+    p.cls_ntaps[cls] = n - p.cls_tap0[cls];
+  }
+  return launch_conv_f32(h, p, N, true, st);
+}
+static int conv_wgrad_f32(lp_handle* h, const ConvDef& c, int N, const float* x, const float* dy, float* dw, cudaStream_t st) {
+  WgradF32Params p;
+  memset(&p, 0, sizeof(p));
+  p.x = x; p.dy = dy; p.dw = dw;
+  p.H = c.H; p.W = c.W; p.Cin = c.cin; p.OH = c.OH; p.OW = c.OW; p.Cout = c.cout; p.pad = c.pad;
+  p.tiles_w = (c.OW + 7) / 8; p.tiles_h = (c.OH + 7) / 8;
+  p.tiles = p.tiles_w * p.tiles_h * N;
+  p.co_tiles = (c.cout + 15) / 16;
+  p.vec_red = (reinterpret_cast<uintptr_t>(dw) & 15) == 0 ? 1 : 0;
+  const int combos = (c.cin + 15) / 16 * p.co_tiles;
+  // pixel splits: about two blocks per SM over all (input, output) channel tiles, at least one tile each
+  const int splits = std::max(1, std::min(p.tiles, 2 * cur_dev().sm_count / combos));
+  const dim3 grid((unsigned)splits, (unsigned)combos);
+  if (c.R == 3 && c.stride == 1)
+    LP_CUDA_OK(launch_pdl(wgrad_f32_tile_kernel<3, 1>, grid, dim3(WgradF32Cfg<3, 1>::kThreads), WgradF32Cfg<3, 1>::kSmem, st, p));
+  else if (c.R == 3)
+    LP_CUDA_OK(launch_pdl(wgrad_f32_tile_kernel<3, 2>, grid, dim3(WgradF32Cfg<3, 2>::kThreads), WgradF32Cfg<3, 2>::kSmem, st, p));
+  else if (c.stride == 1)
+    LP_CUDA_OK(launch_pdl(wgrad_f32_tile_kernel<1, 1>, grid, dim3(WgradF32Cfg<1, 1>::kThreads), WgradF32Cfg<1, 1>::kSmem, st, p));
+  else
+    LP_CUDA_OK(launch_pdl(wgrad_f32_tile_kernel<1, 2>, grid, dim3(WgradF32Cfg<1, 2>::kThreads), WgradF32Cfg<1, 2>::kSmem, st, p));
+  if (h) h->launches++;
+  return LP_OK;
+}
+static_assert(WgradF32Cfg<3, 1>::kSmem <= 48 * 1024 && WgradF32Cfg<3, 2>::kSmem <= 48 * 1024 &&
+              WgradF32Cfg<1, 1>::kSmem <= 48 * 1024 && WgradF32Cfg<1, 2>::kSmem <= 48 * 1024,
+              "the fp32 weight gradients stay within the shared memory that needs no attribute");
+
 // y = conv(x, w) [+ addend]; optional per-channel statistics of y
 static int conv_forward(lp_handle* h, int dtype, int impl, const ConvDef& c, int N, const void* x, void* y,
                         const void* addend, double* stats, bool* stats_done, int* dev_err, cudaStream_t st,
@@ -931,6 +1053,10 @@ static int conv_forward(lp_handle* h, int dtype, int impl, const ConvDef& c, int
     return launch_conv_tc(h, s, dev_err, st);
   }
   if (c.cout % 4) return LP_ERR_UNSUPPORTED;
+  if (dtype == LP_F32 && f32_tile_ok(c)) {
+    if (stats_done) *stats_done = stats != nullptr;
+    return conv_forward_f32(h, c, N, (const float*)x, (float*)y, (const float*)addend, stats, st);
+  }
   ConvGeom g{N, c.H, c.W, c.cin, c.OH, c.OW, c.cout, c.R, c.R, c.stride, c.pad};
   const size_t few_smem = (size_t)c.R * c.R * c.cin * c.cout * 4;
   const int few_cpt = fewch_cpt(c.cout, dtype);
@@ -1055,6 +1181,8 @@ static int conv_dgrad(lp_handle* h, int dtype, int impl, const ConvDef& c, int N
     return LP_OK;
   }
   if (c.cin % 4) return LP_ERR_UNSUPPORTED;
+  if (dtype == LP_F32 && f32_tile_ok(c))
+    return conv_dgrad_f32(h, c, N, (const float*)dy, (float*)dx, (const float*)addend, st);
   ConvGeom g{N, c.H, c.W, c.cin, c.OH, c.OW, c.cout, c.R, c.R, c.stride, c.pad};
   const long long work = (long long)N * c.H * c.W * (c.cin / 4);
   const int grid = grid_for(work, 128, cur_dev().sm_count, 16);
@@ -1101,6 +1229,7 @@ static int conv_wgrad(lp_handle* h, int dtype, int impl, const ConvDef& c, int N
     if (h) h->launches++;
     return rc;
   }
+  if (dtype == LP_F32 && f32_tile_ok(c)) return conv_wgrad_f32(h, c, N, (const float*)x, (const float*)dy, dw, st);
   ConvGeom g{N, c.H, c.W, c.cin, c.OH, c.OW, c.cout, c.R, c.R, c.stride, c.pad};
   const int n_out = c.cout * c.R * c.R * c.cin;
   const long long npix = (long long)N * c.OH * c.OW;
@@ -1252,6 +1381,7 @@ struct Planner {
   }
 
   bool conv_fuses_stats(const ConvDef& c) const {
+    if (dtype == LP_F32) return f32_tile_ok(c);
     return dtype == LP_BF16 && impl != LP_CONV_IMPL_SIMT && !(net.d.conv_impl & 16) && (tc_fwd_ok(c) || c.s2d) && c.wf;
   }
   Tensor emit_conv(Plan& P, std::vector<Op>& ops, const Tensor& in, int conv, const Tensor* addend, int stats_bn) {
@@ -1466,7 +1596,7 @@ struct Planner {
         if (final_block && !last) {
           // The module output is this convolution's accumulator plus the shortcut: on request its
           // epilogue also takes the residual against x_{k+1}, the loss sums and the terminal adjoint.
-          const bool fuse = (net.d.conv_impl & LP_CONV_LOSS_IN_EPILOGUE) && conv_fuses_stats(P.convs[r.c2]);
+          const bool fuse = dtype == LP_BF16 && (net.d.conv_impl & LP_CONV_LOSS_IN_EPILOGUE) && conv_fuses_stats(P.convs[r.c2]);
           if (fuse) F.back().fuse_loss = 1;
           Op op;
           op.fuse_loss = fuse ? 1 : 0;

@@ -181,3 +181,26 @@ def test_output_on_a_16_byte_boundary_takes_the_narrow_epilogue(op_name):
     np.testing.assert_array_equal(results[0], results[1])
     ref = O.conv_fwd(x, w, stride, pad) if op_name == "fwd" else O.conv_dgrad(dy, w, stride, pad, x.shape)
     assert rel_err(results[0], ref.reshape(-1)) < 6e-3
+
+
+# fp32 tile kernels: 8x8 pixel tiles, chunks of 16 channels: one partial tile and chunk, several with remainders in every
+# direction, both warp counts (few and many blocks), a filter that leaves parity classes of dx empty
+F32_CASES = [(1, 3, 5, 4, 4, 3, 1, 1), (2, 9, 17, 20, 36, 3, 1, 1), (3, 11, 9, 36, 20, 3, 2, 1), (2, 16, 8, 64, 48, 3, 2, 1),
+             (2, 7, 10, 12, 8, 1, 2, 0), (2, 13, 8, 40, 12, 1, 1, 0), (24, 32, 32, 16, 16, 3, 1, 1)]
+
+
+@pytest.mark.parametrize("case", F32_CASES)
+def test_fp32_tile_kernels_match_oracle(case):
+    """Relative error of a K-term fp32 sum in any order: sqrt(K) x 2^-24 in the mean over the outputs, K at most 24576
+    (weight gradient of the last case): 1e-5."""
+    import paper_2112_05387_b200 as lp
+    N, H, W, Cin, Cout, R, stride, pad = case
+    x, w, dy = make_case(*case, "f32")
+    st, y, stats = run_conv(lp.LP_CONV_FWD, "f32", 0, *case, x, w, want_stats=True)
+    assert st == 0 and rel_err(y, O.conv_fwd(x, w, stride, pad)) < 1e-5
+    np.testing.assert_allclose(stats[Cout:], (y ** 2).reshape(-1, Cout).sum(0), rtol=1e-5)
+    np.testing.assert_allclose(stats[:Cout], y.reshape(-1, Cout).sum(0), rtol=1e-5, atol=1e-5 * np.abs(y).sum() / Cout)
+    st, dx, _ = run_conv(lp.LP_CONV_DGRAD, "f32", 0, *case, dy, w)
+    assert st == 0 and rel_err(dx, O.conv_dgrad(dy, w, stride, pad, x.shape)) < 1e-5
+    st, dw, _ = run_conv(lp.LP_CONV_WGRAD, "f32", 0, *case, x, dy)
+    assert st == 0 and rel_err(dw, O.conv_wgrad(x, dy, w.shape, stride, pad)) < 1e-5
