@@ -669,6 +669,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       tile_first_pixel(p, pm, pw, phh, pn);
       pw += row_w; phh += row_h; pn += row_n;
       if (row >= rows_used || pw >= p.OWl || phh >= p.OHl || pn >= p.Nimg || grp) return;
+      if (phh * p.os + p.cls_oo_h[pcls] >= p.out_H || pw * p.os + p.cls_oo_w[pcls] >= p.out_W) return;
       const long long pb =
           (((long long)pn * p.out_H + (phh * p.os + p.cls_oo_h[pcls])) * p.out_W + (pw * p.os + p.cls_oo_w[pcls])) * p.out_C +
           pnt * p.n_tile_cols;
@@ -717,7 +718,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int ow = w0 + row_w;
         const int oh = h0 + row_h;
         const int n = n0 + row_n;
-        const bool valid = row < rows_used && ow < p.OWl && oh < p.OHl && n < p.Nimg;
+        // (the odd parity classes of an odd-sized stride-2 input gradient end before the logical grid does)
+        const bool valid = row < rows_used && ow < p.OWl && oh < p.OHl && n < p.Nimg &&
+                           oh * p.os + p.cls_oo_h[cls] < p.out_H && ow * p.os + p.cls_oo_w[cls] < p.out_W;
         const long long obase =
             (((long long)n * p.out_H + (oh * p.os + p.cls_oo_h[cls])) * p.out_W + (ow * p.os + p.cls_oo_w[cls])) * p.out_C;
         // one thread waits (bounded) and all epilogue threads agree on the outcome, so that the

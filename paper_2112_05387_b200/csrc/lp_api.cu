@@ -814,11 +814,9 @@ static int launch_conv_tc(lp_handle* h, const TcGemmSpec& s, int* dev_err, cudaS
 static bool tc_fwd_ok(const ConvDef& c) {
   return c.cin % 8 == 0 && c.cout % 8 == 0 && (c.R == 1 || c.R == 3) && (c.stride == 1 || c.stride == 2);
 }
-static bool tc_dgrad_ok(const ConvDef& c) {
-  return tc_fwd_ok(c) && (c.stride == 1 || (c.H % 2 == 0 && c.W % 2 == 0));
-}
-// A stride-2 input gradient runs as one launch per parity class of the input pixels; a class that no
-// filter tap reaches (1x1 filters) is not written by any epilogue.
+static bool tc_dgrad_ok(const ConvDef& c) { return tc_fwd_ok(c); }
+// A stride-2 input gradient runs over the parity classes of the input pixels; a class that no filter tap
+// reaches (1x1 filters) is not written by any epilogue.
 static bool dgrad_has_empty_class(const ConvDef& c) {
   for (int ph = 0; ph < c.stride; ++ph) {
     int cnt = 0;
@@ -1112,15 +1110,18 @@ static int conv_dgrad(lp_handle* h, int dtype, int impl, const ConvDef& c, int N
       if (!addend) LP_CUDA_OK(cudaMemsetAsync(dx, 0, (size_t)N * c.H * c.W * c.cin * 2, st));
     }
     ProfScope ps(h, st, 2.0 * N * c.OH * c.OW * (double)c.cout * c.R * c.R * c.cin);
-    if (st2 == 2 && !any_empty && c.H % 2 == 0 && c.W % 2 == 0 && c.R * c.R <= 16) {
+    if (st2 == 2 && !any_empty && c.R * c.R <= 16) {
       // every parity class has the same logical grid (H/2 x W/2) and only its taps and its offset into dx differ:
-      // one launch walks the four classes (tile classes of the kernel) instead of four quarter-size launches
+      // one launch walks the four classes (tile classes of the kernel) instead of four quarter-size launches.
+      // With an odd H or W the odd classes end one row or column earlier: the grid is rounded up and the epilogue
+      // masks what would lie outside (the two launches of a ResNet-50 step on 12 images of 176x176, 11x11 inputs, took
+      // 2.1 ms on the CUDA cores; the step 3.79 -> 1.81 ms)
       TcGemmSpec s;
       memset(&s, 0, sizeof(s));
       s.act = (const bf16*)dy; s.aN = N; s.aH = c.OH; s.aW = c.OW; s.aC = c.cout;
       s.wmat = c.wt; s.w_rows = c.cin; s.w_K = (long long)c.R * c.R * c.cout;
       s.in_step = 1;
-      s.OHl = c.H / 2; s.OWl = c.W / 2;
+      s.OHl = (c.H + 1) / 2; s.OWl = (c.W + 1) / 2;
       s.n_cls = 4;
       for (int cls = 0; cls < 4; ++cls) {
         const int ph = cls / 2, pw = cls % 2;

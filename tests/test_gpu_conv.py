@@ -204,3 +204,15 @@ def test_fp32_tile_kernels_match_oracle(case):
     assert st == 0 and rel_err(dx, O.conv_dgrad(dy, w, stride, pad, x.shape)) < 1e-5
     st, dw, _ = run_conv(lp.LP_CONV_WGRAD, "f32", 0, *case, x, dy)
     assert st == 0 and rel_err(dw, O.conv_wgrad(x, dy, w.shape, stride, pad)) < 1e-5
+
+
+@pytest.mark.parametrize("case", [(3, 11, 11, 64, 128, 3, 2, 1), (2, 7, 12, 32, 64, 3, 2, 1), (5, 16, 9, 160, 64, 3, 2, 1),
+                                  (2, 11, 9, 64, 128, 1, 2, 0)])
+def test_tensor_conv_dgrad_stride_2_of_odd_sizes_matches_oracle(case):
+    """Parity classes of unequal size (odd height, odd width, both); the bound of the even sizes."""
+    import paper_2112_05387_b200 as lp
+    N, H, W, Cin, Cout, R, stride, pad = case
+    x, w, dy = make_case(*case, "bf16")
+    st, dx, _ = run_conv(lp.LP_CONV_DGRAD, "bf16", lp.LP_CONV_IMPL_TENSOR, *case, dy, w)
+    assert st == 0, lp.lp_status_string(st)
+    assert rel_err(dx, O.conv_dgrad(dy, w, stride, pad, x.shape)) < 6e-3
