@@ -812,7 +812,28 @@ struct PackEntry {
   long long begin;       // first flat element index handled for this entry
   long long tile_begin;  // first 32x32 tile index of this entry (tiled kernel)
   long long tile64_begin;  // first 64x64 tile index of this entry (sgd_pack_tiled64_kernel)
+  // copies for the grouped form of a thin layer (conv_thin.cuh): g = 64 / C neighbouring pixels are one group of 64
+  // channels, rows (pixel of the output group, channel), columns = the K = 16 slices that hold a tap; the places that
+  // hold none are zero from the start and never written.  Null where there is no such form (or g = 1: wf and wt are it)
+  bf16* gf;
+  bf16* gt;
 };
+
+// Column of (kernel row r, pixel pi of the input group, channel c): per kernel row the four slices of the group itself,
+// then the near edge of its left (pi = -1) and of its right neighbour (pi = g).
+__host__ __device__ __forceinline__ int grouped_cols(int C) { return 3 * (64 + 2 * C); }
+__device__ __forceinline__ int grouped_col(int r, int pi, int c, int C) {
+  const int g = 64 / C;
+  return r * (64 + 2 * C) + (pi < 0 ? 64 : (pi >= g ? 64 + C : pi * C)) + c;
+}
+__device__ __forceinline__ void grouped_store(const PackEntry& e, int co, int t, int ci, bf16 v) {
+  const int C = e.cin, g = 64 / C, K = grouped_cols(C);
+  const int r = t / 3, o = t % 3 - 1;
+  for (int po = 0; po < g; ++po) {
+    e.gf[(po * C + co) * K + grouped_col(r, po + o, ci, C)] = v;
+    if (e.gt) e.gt[(po * C + ci) * K + grouped_col(r, po - o, co, C)] = v;
+  }
+}
 
 __global__ void pack_weights_kernel(const PackEntry* __restrict__ tab, int n_entries, long long total) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
@@ -862,6 +883,7 @@ __global__ void pack_weights_tiled_kernel(const PackEntry* __restrict__ tab, int
       const long long j = ((long long)co * e.taps + t) * e.cin + ci;
       v = e.w[j];
       e.wf[j] = __float2bfloat16_rn(v);
+      if (e.gf) grouped_store(e, co, t, ci, __float2bfloat16_rn(v));
     }
     tile[i][tx] = v;
   }
@@ -939,6 +961,10 @@ sgd_pack_tiled64_kernel(const PackEntry* __restrict__ tab, int n_entries, float*
       pk.x = *reinterpret_cast<const uint32_t*>(&lo2);
       pk.y = *reinterpret_cast<const uint32_t*>(&hi2);
       *reinterpret_cast<uint2*>(e.wf + j) = pk;
+      if (e.gf) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) grouped_store(e, co, t, ci + u, __float2bfloat16_rn(v[u]));
+      }
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) tile[row][cx + u] = v[u];

@@ -17,6 +17,7 @@
 #include "conv_tc.cuh"
 #include "conv_tc2.cuh"
 #include "kernels_elem.cuh"
+#include "conv_thin.cuh"
 #include "net.h"
 #include "wgrad_tc.cuh"
 
@@ -51,6 +52,11 @@ struct ConvDef {
   bool s2d = false;
   bf16* xs = nullptr;        // [N][H/2][W/2][16]
   float* dws = nullptr;      // [cout][16][16]
+  // 3x3 stride-1 layers of 16, 32 or 64 channels on grouped pixels (conv_thin.cuh): pixels per group (0: not such a
+  // layer), bf16 weights of the groups, and (g > 1) the weight gradient of the groups
+  int g = 0;
+  bf16 *gf = nullptr, *gt = nullptr;
+  float* dwg = nullptr;
 };
 struct BnDef {
   int C;
@@ -79,6 +85,11 @@ struct Op {
   // only the apply pass is left.
   int bwd_bn = -1, bwd_relu = 0, reduce_fused = 0;
   Tensor bwd_x;
+  // Thin layers produce their operand on the way in (conv_thin.cuh): pre = 1 relu(bn(in)), 2 bn(in) + pre_x,
+  // 3 batch-norm backward of in with the normalised tensor pre_x; pre_out is the produced tensor.  On the batch-norm
+  // backward: apply_fused = 1, only the reduction pass (if that) is left.
+  int pre = 0, pre_bn = -1, pre_relu = 0, apply_fused = 0;
+  Tensor pre_x, pre_out;
   uint8_t* arg = nullptr;  // max-pool argmax
 };
 
@@ -117,6 +128,11 @@ struct Plan {  // one module or one AuxNet
   void* stats_region = nullptr;
   size_t stats_bytes = 0;
   void* dx_fallback = nullptr;
+  // weight gradients of the grouped layers: one region, cleared before the first of them, folded back after the last
+  void* dwg_region = nullptr;
+  size_t dwg_bytes = 0;
+  std::vector<tc::FoldEntry> host_fold;
+  tc::FoldEntry* dev_fold = nullptr;
   bool interior = false;
   bool ran_fwd_bwd = false;
   // Weight gradients feed nothing but the update, so in the backward pass they leave the chain
@@ -164,7 +180,7 @@ struct Device {
   int sm_count = 148;
   EncodeTiledFn encode = nullptr;
   // kernel attributes are per device: set on the first launch of each kernel family on that device
-  bool conv_attr = false, wgrad_attr = false, wgrad_halo_attr = false, conv2_attr = false, f32_attr = false;
+  bool conv_attr = false, wgrad_attr = false, wgrad_halo_attr = false, conv2_attr = false, f32_attr = false, thin_attr = false;
   int max_pairs = 0;   // CTA pairs of conv_tc2_kernel that can be resident at once (0: not usable)
   int init() {
     if (ready) return LP_OK;
@@ -996,6 +1012,119 @@ static_assert(WgradF32Cfg<3, 1>::kSmem <= 48 * 1024 && WgradF32Cfg<3, 2>::kSmem 
               WgradF32Cfg<1, 1>::kSmem <= 48 * 1024 && WgradF32Cfg<1, 2>::kSmem <= 48 * 1024,
               "the fp32 weight gradients stay within the shared memory that needs no attribute");
 
+// ---------------------------------------------------------------------------------------------
+// thin layers on grouped pixels (conv_thin.cuh)
+// ---------------------------------------------------------------------------------------------
+// How the operand of a thin layer is produced (mode 1..3 of the kernel).
+struct ThinPre {
+  int mode; const void* in1; BnArgs bn; const float *dgamma, *dbeta; int relu; void* out;
+};
+static const size_t kThinMaxSmem = 160 * 1024;
+
+static int launch_conv_thin(lp_handle* h, const ConvDef& c, int N, bool bwd, const void* in, const ThinPre* pre, void* out,
+                            const void* addend, double* stats, const BnBwdFuse* red, int* dev_err, cudaStream_t st) {
+  tc::ConvThinParams p;
+  memset(&p, 0, sizeof(p));
+  const int C = c.cin, mode = pre ? pre->mode : 0;
+  if ((bwd ? (mode != 0 && mode != 3) : mode == 3) || (!bwd && (addend || red)) || !(bwd ? c.gt : c.gf)) return LP_ERR_UNSUPPORTED;
+  p.N = N; p.H = c.H; p.Wg = c.W / c.g; p.C = C;
+  // Tile: eight columns per row group of M, or -- one tile column of up to 14, where that leaves fewer rows of M empty than
+  // the last eight-column tile would -- runs of whole box rows.
+  const int tw8 = (p.Wg + 7) / 8;
+  if (p.Wg > 14 || (double)p.Wg / (8 * tw8) >= (double)p.Wg / (p.Wg + 2)) { p.BW = 8; p.P = p.S = 10; }
+  else { p.BW = p.Wg; p.P = p.Wg + 2; p.S = 8; }
+  const int tile_cols = p.S == 8 ? p.P : 8;
+  const int groups = 128 / tile_cols;                             // image rows per tile
+  if (p.H >= groups) {
+    p.BNI = 1;
+    const int th = (p.H + groups - 1) / groups;
+    p.BH = (p.H + th - 1) / th;
+  } else {
+    p.BH = p.H;
+    p.BNI = std::max(1, std::min(N, groups / p.H));
+    while (p.BNI > 1 && p.P * p.BNI * (p.BH + 2) > tc::kThinMaxBoxRows) --p.BNI;
+    const int tn = (N + p.BNI - 1) / p.BNI;
+    p.BNI = (N + tn - 1) / tn;
+  }
+  p.box_rows = p.P * p.BNI * (p.BH + 2);
+  p.tile_rows = tile_cols * p.BNI * p.BH;
+  if (p.box_rows > tc::kThinMaxBoxRows || p.tile_rows > 128) return LP_ERR_UNSUPPORTED;
+  p.tiles_w = (p.Wg + p.BW - 1) / p.BW;
+  p.tiles_h = (p.H + p.BH - 1) / p.BH;
+  p.tiles = p.tiles_w * p.tiles_h * ((N + p.BNI - 1) / p.BNI);
+  p.fd_w = tc::make_fastdiv(p.tiles_w); p.fd_h = tc::make_fastdiv(p.tiles_h);
+  p.fd_P = tc::make_fastdiv(p.P); p.fd_BNI = tc::make_fastdiv(p.BNI); p.fd_TP = tc::make_fastdiv(tile_cols);
+  // MMAs: K = 16 slices in the column order of the packed weights (grouped_col; g = 1: tap by tap)
+  int n = 0;
+  for (int r = 0; r < 3; ++r) {
+    const int dy = bwd ? 2 - r : r;
+    auto slice = [&](int dx, int j) { p.a_off[n++] = (uint16_t)((dy * p.BNI * p.P + dx) * 8 + 2 * j); };
+    if (c.g == 1) {
+      for (int s = 0; s < 3; ++s)
+        for (int j = 0; j < 4; ++j) slice(bwd ? 2 - s : s, j);
+    } else {
+      for (int j = 0; j < 4; ++j) slice(1, j);
+      for (int j = 4 - C / 16; j < 4; ++j) slice(0, j);
+      for (int j = 0; j < C / 16; ++j) slice(2, j);
+    }
+  }
+  p.n_mma = n;
+  p.n_wbox = (n + 3) / 4;
+  const size_t box_bytes = align_up((size_t)std::max(p.box_rows, 128) * 128, 1024), tile_bytes = 128 * 128;
+  p.a_offset = (uint32_t)(p.n_wbox * tc::kThinBoxBytesW);
+  p.b_offset = p.a_offset + (uint32_t)box_bytes;
+  p.b2_offset = p.b_offset + (addend ? (uint32_t)tile_bytes : 0u);
+  const size_t aux = (addend ? tile_bytes : 0) + (red ? tile_bytes : 0);
+  p.tail_offset = p.b_offset + (uint32_t)std::max(mode >= 2 ? box_bytes : (size_t)0, aux);
+  // the last row the MMAs of a tile touch may lie past the box (results of such rows are dropped): still inside the allocation
+  const size_t reach = (size_t)(15 * p.S + 7 + 2 * p.BNI * p.P + 2 + 1) * 128;
+  const size_t smem = std::max((size_t)p.tail_offset + sizeof(tc::ThinSmemTail), p.a_offset + reach) + 1024;
+  if (smem > kThinMaxSmem) return LP_ERR_UNSUPPORTED;
+  p.idesc = tc::instr_desc_bf16(128, 64, 0, 0);
+  p.desc_a = tc::smem_desc_hi(16, p.S * 128, 2);
+  p.desc_b = tc::smem_desc_hi(16, 1024, 2);
+  if (pre) {
+    p.bn = pre->bn; p.bn_dgamma = pre->dgamma; p.bn_dbeta = pre->dbeta; p.bn_relu = pre->relu; p.pre_out = (bf16*)pre->out;
+  }
+  p.has_addend = addend ? 1 : 0; p.stats = stats; p.err = dev_err;
+  if (red) {
+    p.has_red = 1; p.red_bn = red->bn; p.red_dgamma = red->dgamma; p.red_dbeta = red->dbeta; p.red_relu = red->relu;
+  }
+  CUtensorMap tmIn0, tmIn1, tmB, tmAdd, tmRed, tmOut;
+  memset(&tmIn1, 0, sizeof(tmIn1)); memset(&tmAdd, 0, sizeof(tmAdd)); memset(&tmRed, 0, sizeof(tmRed));
+  int rc = encode_act_map_halo(&tmIn0, in, N, p.H, p.Wg, 64, 64, p.P, p.BH, p.BNI, 128);
+  if (rc == LP_OK && mode >= 2) rc = encode_act_map_halo(&tmIn1, pre->in1, N, p.H, p.Wg, 64, 64, p.P, p.BH, p.BNI, 128);
+  if (rc == LP_OK && addend) rc = encode_act_map_halo(&tmAdd, addend, N, p.H, p.Wg, 64, 64, tile_cols, p.BH, p.BNI, 128, 0);
+  if (rc == LP_OK && red) rc = encode_act_map_halo(&tmRed, red->x, N, p.H, p.Wg, 64, 64, tile_cols, p.BH, p.BNI, 128, 0);
+  if (rc == LP_OK) rc = encode_act_map_halo(&tmOut, out, N, p.H, p.Wg, 64, 64, tile_cols, p.BH, p.BNI, 128, 0);
+  const int K = c.g == 1 ? 9 * 64 : grouped_cols(C);
+  if (rc == LP_OK) rc = encode_mat_map(&tmB, bwd ? c.gt : c.gf, K, 64, 64, 64, 128);
+  if (rc != LP_OK) return rc;
+  Device& D = cur_dev();
+  if (!D.thin_attr) {
+    LP_CUDA_OK(cudaFuncSetAttribute(tc::conv_thin_kernel<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kThinMaxSmem));
+    LP_CUDA_OK(cudaFuncSetAttribute(tc::conv_thin_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kThinMaxSmem));
+    LP_CUDA_OK(cudaFuncSetAttribute(tc::conv_thin_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kThinMaxSmem));
+    LP_CUDA_OK(cudaFuncSetAttribute(tc::conv_thin_kernel<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kThinMaxSmem));
+    LP_CUDA_OK(cudaFuncSetAttribute(tc::conv_thin_kernel<3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kThinMaxSmem));
+    D.thin_attr = true;
+  }
+  // One CTA per SM at most, several tiles each beyond that: a second CTA would find room, but the modules' other kernels
+  // need it more (256 tiles of ResNet-110's first stage: step 1.53 -> 1.46 ms).
+  const int per = std::max(1, (p.tiles + D.sm_count - 1) / D.sm_count);
+  const dim3 grid((p.tiles + per - 1) / per), block(tc::kThinThreads);
+  ProfScope ps(h, st, 2.0 * N * c.H * c.W * (double)C * 9 * C);
+  cudaError_t le;
+  if (mode == 1) le = launch_pdl(tc::conv_thin_kernel<1, false>, grid, block, smem, st, tmIn0, tmIn1, tmB, tmAdd, tmRed, tmOut, p);
+  else if (mode == 2) le = launch_pdl(tc::conv_thin_kernel<2, false>, grid, block, smem, st, tmIn0, tmIn1, tmB, tmAdd, tmRed, tmOut, p);
+  else if (mode == 3) le = launch_pdl(tc::conv_thin_kernel<3, true>, grid, block, smem, st, tmIn0, tmIn1, tmB, tmAdd, tmRed, tmOut, p);
+  else if (bwd) le = launch_pdl(tc::conv_thin_kernel<0, true>, grid, block, smem, st, tmIn0, tmIn1, tmB, tmAdd, tmRed, tmOut, p);
+  else le = launch_pdl(tc::conv_thin_kernel<0, false>, grid, block, smem, st, tmIn0, tmIn1, tmB, tmAdd, tmRed, tmOut, p);
+  LP_CUDA_OK(le);
+  if (h) h->launches++;
+  return LP_OK;
+}
+
 // y = conv(x, w) [+ addend]; optional per-channel statistics of y
 static int conv_forward(lp_handle* h, int dtype, int impl, const ConvDef& c, int N, const void* x, void* y,
                         const void* addend, double* stats, bool* stats_done, int* dev_err, cudaStream_t st,
@@ -1225,8 +1354,12 @@ static int conv_wgrad(lp_handle* h, int dtype, int impl, const ConvDef& c, int N
     // small layers of modules that run side by side share the SMs (see kSmallConvFlops)
     const bool shared_sm = h && h->concurrent && c.cin <= 64 && c.cout <= 64 &&
                            2.0 * N * c.OH * c.OW * (double)c.cout * c.R * c.R * c.cin < kSmallConvFlops;
-    int rc = launch_wgrad_tc(D.encode, D.sm_count, &D.wgrad_attr, &D.wgrad_halo_attr, (const bf16*)x, (const bf16*)dy, dw, N,
-                             c.H, c.W, c.cin, c.OH, c.OW, c.cout, c.R, c.stride, c.pad, dev_err, st, shared_sm);
+    // (thin layers: the gradient of the 64 x 64 group blocks, folded back after the pass -- rows of 128 bytes instead
+    // of 32 or 64, and a quarter or half of the pixels to sum over)
+    int rc = c.g > 1 ? launch_wgrad_tc(D.encode, D.sm_count, &D.wgrad_attr, &D.wgrad_halo_attr, (const bf16*)x, (const bf16*)dy,
+                                       c.dwg, N, c.H, c.W / c.g, 64, c.H, c.W / c.g, 64, 3, 1, 1, dev_err, st, shared_sm)
+                     : launch_wgrad_tc(D.encode, D.sm_count, &D.wgrad_attr, &D.wgrad_halo_attr, (const bf16*)x, (const bf16*)dy, dw, N,
+                                       c.H, c.W, c.cin, c.OH, c.OW, c.cout, c.R, c.stride, c.pad, dev_err, st, shared_sm);
     if (h) h->launches++;
     return rc;
   }
@@ -1312,6 +1445,13 @@ struct Planner {
       if (name == e.name) return &e;
     return nullptr;
   }
+  // Layers that take the thin kernel with its fusions (post-activation networks; none of the variant flags).
+  bool thin_ok(const ConvDef& c) const {
+    return dtype == LP_BF16 && net.d.block_kind != LP_PREACT && impl != LP_CONV_IMPL_SIMT &&
+           !(net.d.conv_impl & ~(15 | LP_CONV_WGRAD_IN_CHAIN | LP_CONV_BN_REDUCE_IN_EPILOGUE)) && c.R == 3 && c.stride == 1 && c.pad == 1 && c.cin == c.cout &&
+           (c.cin == 16 || c.cin == 32 || c.cin == 64) && c.W % (64 / c.cin) == 0 &&
+           2.0 * net.d.N * c.H * c.W * (double)c.cin * 9 * c.cin < kSmallConvFlops;
+  }
   int add_conv(Plan& P, const std::string& wname, int cin, int cout, int R, int stride, int pad, int H, int W,
                bool need_dgrad) {
     ConvDef c;
@@ -1326,6 +1466,16 @@ struct Planner {
       c.wf = (bf16*)A.alloc(n * 2);
       if (need_dgrad && tc_dgrad_ok(c)) c.wt = (bf16*)A.alloc(n * 2);
       PackEntry pe;
+      pe.gf = pe.gt = nullptr;
+      if (thin_ok(c)) {
+        c.g = 64 / cin;
+        c.gf = c.wf; c.gt = c.wt;
+        if (c.g > 1) {
+          const size_t gn = (size_t)64 * grouped_cols(cin);
+          pe.gf = c.gf = (bf16*)A.alloc(gn * 2);
+          if (c.wt) pe.gt = c.gt = (bf16*)A.alloc(gn * 2);
+        }
+      }
       pe.w = c.w; pe.wf = c.wf; pe.wt = c.wt; pe.cout = cout; pe.taps = R * R; pe.cin = cin;
       pe.begin = P.ps.pack_total;
       pe.tile_begin = P.ps.pack_tiles;
@@ -1364,6 +1514,15 @@ struct Planner {
     size_t off = 0;
     for (auto& b : P.bns) { b.stats = base + off; off += (size_t)2 * b.C; }
     P.loss_acc = (double*)A.alloc(2 * sizeof(double));
+    for (auto& c : P.convs) {
+      if (c.g <= 1) continue;
+      const size_t bytes = (size_t)64 * 9 * 64 * 4;      // (a multiple of the arena's alignment: the region is contiguous)
+      c.dwg = (float*)A.alloc(bytes);
+      if (!P.dwg_bytes) P.dwg_region = c.dwg;
+      P.dwg_bytes += bytes;
+      P.host_fold.push_back({c.dwg, c.gw, c.cin});
+    }
+    if (!P.host_fold.empty()) P.dev_fold = (tc::FoldEntry*)A.alloc(P.host_fold.size() * sizeof(tc::FoldEntry));
     if (!P.ps.host_pack.empty()) {
       P.ps.dev_pack = (PackEntry*)A.alloc(P.ps.host_pack.size() * sizeof(PackEntry));
       // complement of the packed entries in [0, n), cut into ranges of at most 16384 elements
@@ -1417,17 +1576,23 @@ struct Planner {
     return (net.d.conv_impl & LP_CONV_BN_REDUCE_IN_EPILOGUE) && dtype == LP_BF16 && impl != LP_CONV_IMPL_SIMT &&
            !(net.d.conv_impl & 32) && tc_dgrad_ok(c) && c.wt && !dgrad_has_empty_class(c);
   }
+  // The input gradient of a thin layer takes the reduction pass of the batch-norm backward that follows it; on tensors of
+  // up to 32768 elements, where the pass is a block or two, only on request as for every other convolution.
+  bool thin_fuses_bn_bwd(const ConvDef& c, const Tensor& dy) const {
+    return c.g > 0 && ((net.d.conv_impl & LP_CONV_BN_REDUCE_IN_EPILOGUE) || dy.elems() > 32768);
+  }
   Tensor emit_bn_bwd(Plan& P, std::vector<Op>& ops, const Tensor& dy, const Tensor& x, const Tensor* mask, int bn,
                      const Tensor* addend, const Tensor* out_override = nullptr) {
     Tensor out = out_override ? *out_override : new_tensor(x.n, x.h, x.w, x.c);
     Op op;
     op.type = OP_BN_BWD; op.in = dy; op.in2 = x; op.bn = bn; op.out = out;
-    // On request (LP_CONV_BN_REDUCE_IN_EPILOGUE): where the last kernel to write dy is a tensor-core input
-    // gradient, its epilogue takes this batch norm's reduction pass (one such consumer per convolution).
+    // Where the last kernel to write dy is the input gradient of a thin layer -- or, on request
+    // (LP_CONV_BN_REDUCE_IN_EPILOGUE), any tensor-core input gradient -- its epilogue takes this batch norm's
+    // reduction pass (one such consumer per convolution).
     for (int i = (int)ops.size() - 1; i >= 0; --i) {
       Op& w = ops[i];
       if (!(w.out.p == dy.p && w.out.ext == dy.ext) || !w.out.defined()) continue;
-      if (w.type == OP_CONV_DGRAD && w.bwd_bn < 0 && dgrad_fuses_bn_bwd(P.convs[w.conv])) {
+      if (w.type == OP_CONV_DGRAD && w.bwd_bn < 0 && (thin_fuses_bn_bwd(P.convs[w.conv], dy) || dgrad_fuses_bn_bwd(P.convs[w.conv]))) {
         w.bwd_bn = bn; w.bwd_x = x; w.bwd_relu = mask ? 1 : 0;
         op.reduce_fused = 1;
       }
@@ -1436,6 +1601,38 @@ struct Planner {
     if (mask) op.mask = *mask;
     if (addend) op.addend = *addend;
     ops.push_back(op);
+    return out;
+  }
+  // Convolution whose operand is relu(bn(y)) (shortcut == nullptr) or bn(y) + shortcut, which goes to `t`: produced by the
+  // convolution itself (thin layers), else by a kernel of its own.
+  Tensor emit_bn_conv(Plan& P, std::vector<Op>& ops, const Tensor& y, int bn, const Tensor* shortcut, Tensor& t, int conv,
+                      int stats_bn) {
+    if (!P.convs[conv].g) {
+      t = emit_bn_apply(ops, y, bn, nullptr, -1, shortcut, shortcut ? 0 : 1);
+      return emit_conv(P, ops, t, conv, nullptr, stats_bn);
+    }
+    t = new_tensor(y.n, y.h, y.w, y.c);
+    Tensor out = emit_conv(P, ops, y, conv, nullptr, stats_bn);
+    Op& op = ops.back();
+    op.pre = shortcut ? 2 : 1; op.pre_bn = bn; op.pre_out = t;
+    if (shortcut) op.pre_x = *shortcut;
+    return out;
+  }
+  // dy = backward of bn at (d, y), then the weight gradient (against x) and the input gradient of the convolution
+  // that wrote y; returns the input gradient.
+  Tensor emit_bn_bwd_conv(Plan& P, std::vector<Op>& ops, const Tensor& d, const Tensor& y, const Tensor* mask, int bn,
+                          const Tensor& x, int conv, const Tensor* addend, const Tensor* out_override) {
+    if (!P.convs[conv].g) {
+      Tensor dy = emit_bn_bwd(P, ops, d, y, mask, bn, nullptr);
+      emit_wgrad(ops, x, dy, conv);
+      return emit_dgrad(P, ops, dy, conv, addend, out_override);
+    }
+    Tensor dy = emit_bn_bwd(P, ops, d, y, mask, bn, nullptr);
+    ops.back().apply_fused = 1;
+    Tensor out = emit_dgrad(P, ops, d, conv, addend, out_override);
+    Op& op = ops.back();
+    op.pre = 3; op.pre_bn = bn; op.pre_relu = mask ? 1 : 0; op.pre_x = y; op.pre_out = dy;
+    emit_wgrad(ops, x, dy, conv);       // (dy exists once the input gradient has run)
     return out;
   }
   void emit_wgrad(std::vector<Op>& ops, const Tensor& x, const Tensor& dy, int conv) {
@@ -1560,15 +1757,22 @@ struct Planner {
       P.r = new_tensor(out_shape.n, out_shape.h, out_shape.w, out_shape.c);
       P.seed = new_tensor(out_shape.n, out_shape.h, out_shape.w, out_shape.c);
     }
+    // block i's first convolution is a thin layer and forms the sum that ends block i - 1
+    auto sum_pending = [&](size_t i) { return !bott && P.convs[recs[i].c1].g > 0 && !net.blocks[recs[i - 1].bi].proj; };
     for (size_t i = 0; i < recs.size(); ++i) {
       BlockRec& r = recs[i];
       const BlockDef& b = net.blocks[r.bi];
       const bool final_block = i + 1 == recs.size();
       r.x = cur;
       if (post) {
-        r.y1 = emit_conv(P, F, cur, r.c1, nullptr, r.bn1);
-        r.a1 = emit_bn_apply(F, r.y1, r.bn1, nullptr, -1, nullptr, 1);
-        r.y2 = emit_conv(P, F, r.a1, r.c2, nullptr, r.bn2);
+        if (i > 0 && sum_pending(i)) {   // the previous block's sum is formed on the way into this block's first convolution
+          const BlockRec& q = recs[i - 1];
+          r.y1 = emit_bn_conv(P, F, q.y2, q.bn2, &q.x, r.x, r.c1, r.bn1);
+          cur = r.x;
+        } else {
+          r.y1 = emit_conv(P, F, cur, r.c1, nullptr, r.bn1);
+        }
+        r.y2 = emit_bn_conv(P, F, r.y1, r.bn1, nullptr, r.a1, r.c2, r.bn2);
         if (bott) {
           r.a2 = emit_bn_apply(F, r.y2, r.bn2, nullptr, -1, nullptr, 1);
           r.y3 = emit_conv(P, F, r.a2, r.c3, nullptr, r.bn3);
@@ -1582,6 +1786,8 @@ struct Planner {
           if (b.proj) { op.in2 = r.ys; op.bn2 = r.bns; } else { op.addend = cur; }
           F.push_back(op);
           cur = P.out;
+        } else if (!final_block && sum_pending(i + 1)) {
+          cur = Tensor();
         } else {
           cur = b.proj ? emit_bn_apply(F, ylast, bnlast, &r.ys, r.bns, nullptr, 0)
                        : emit_bn_apply(F, ylast, bnlast, nullptr, -1, &cur, 0);
@@ -1644,26 +1850,24 @@ struct Planner {
       const bool first_of_module = i == 0 && k > 0;  // its input is x_k: dx goes to the caller
       const Tensor* dx_target = first_of_module ? &dx_ext : nullptr;
       if (post) {
-        Tensor dy2;
+        Tensor da1;
         if (bott) {
           Tensor dy3 = emit_bn_bwd(P, Bw, dcur, r.y3, nullptr, r.bn3, nullptr);
           emit_wgrad(Bw, r.a2, dy3, r.c3);
           Tensor da2 = emit_dgrad(P, Bw, dy3, r.c3, nullptr, nullptr);
-          dy2 = emit_bn_bwd(P, Bw, da2, r.y2, &r.a2, r.bn2, nullptr);
+          da1 = emit_bn_bwd_conv(P, Bw, da2, r.y2, &r.a2, r.bn2, r.a1, r.c2, nullptr, nullptr);
         } else {
-          dy2 = emit_bn_bwd(P, Bw, dcur, r.y2, nullptr, r.bn2, nullptr);
+          da1 = emit_bn_bwd_conv(P, Bw, dcur, r.y2, nullptr, r.bn2, r.a1, r.c2, nullptr, nullptr);
         }
-        emit_wgrad(Bw, r.a1, dy2, r.c2);
-        Tensor da1 = emit_dgrad(P, Bw, dy2, r.c2, nullptr, nullptr);
-        Tensor dy1 = emit_bn_bwd(P, Bw, da1, r.y1, &r.a1, r.bn1, nullptr);
-        emit_wgrad(Bw, r.x, dy1, r.c1);
         if (b.proj) {
+          Tensor dy1 = emit_bn_bwd(P, Bw, da1, r.y1, &r.a1, r.bn1, nullptr);
+          emit_wgrad(Bw, r.x, dy1, r.c1);
           Tensor dys = emit_bn_bwd(P, Bw, dcur, r.ys, nullptr, r.bns, nullptr);
           emit_wgrad(Bw, r.x, dys, r.cs);
           Tensor dx = emit_dgrad(P, Bw, dy1, r.c1, nullptr, dx_target);
           dcur = emit_dgrad(P, Bw, dys, r.cs, &dx, &dx);
         } else {
-          dcur = emit_dgrad(P, Bw, dy1, r.c1, &dcur, dx_target);
+          dcur = emit_bn_bwd_conv(P, Bw, da1, r.y1, &r.a1, r.bn1, r.x, r.c1, &dcur, dx_target);
         }
       } else {
         emit_wgrad(Bw, r.a1, dcur, r.c2);
@@ -1738,9 +1942,18 @@ struct Planner {
     std::vector<Tensor> ins, ys, acts;
     for (size_t i = 0; i < cv.size(); ++i) {
       ins.push_back(cur);
-      Tensor y = emit_conv(P, P.fwd, cur, ci[i], nullptr, bi[i]);
+      const bool pre = i > 0 && P.convs[ci[i]].g > 0;   // produces its own operand (see below)
+      Tensor act;
+      Tensor y = pre ? emit_bn_conv(P, P.fwd, ys[i - 1], bi[i - 1], nullptr, act, ci[i], bi[i])
+                     : emit_conv(P, P.fwd, cur, ci[i], nullptr, bi[i]);
+      if (pre) { acts[i - 1] = act; ins[i] = act; }
       ys.push_back(y);
       const bool final_conv = i + 1 == cv.size();
+      if (!final_conv && P.convs[ci[i + 1]].g > 0) {    // the next convolution normalises y on its way in
+        acts.push_back(Tensor());
+        cur = Tensor();
+        continue;
+      }
       Tensor out;
       Op op;
       op.type = OP_BN_APPLY; op.in = y; op.bn = bi[i]; op.relu = final_conv ? 0 : 1;
@@ -1762,10 +1975,13 @@ struct Planner {
     Tensor d = P.seed;
     for (int i = (int)cv.size() - 1; i >= 0; --i) {
       const bool relu_after = i + 1 < (int)cv.size();
-      Tensor dy = emit_bn_bwd(P, P.bwd, d, ys[i], relu_after ? &acts[i] : nullptr, bi[i], nullptr);
-      emit_wgrad(P.bwd, ins[i], dy, ci[i]);
-      if (i > 0) d = emit_dgrad(P, P.bwd, dy, ci[i], nullptr, nullptr);
-      else if (dx_out) emit_dgrad(P, P.bwd, dy, ci[i], nullptr, dx_out);
+      const Tensor* mask = relu_after ? &acts[i] : nullptr;
+      if (i > 0 || dx_out) {
+        d = emit_bn_bwd_conv(P, P.bwd, d, ys[i], mask, bi[i], ins[i], ci[i], nullptr, i > 0 ? nullptr : dx_out);
+      } else {
+        Tensor dy = emit_bn_bwd(P, P.bwd, d, ys[i], mask, bi[i], nullptr);
+        emit_wgrad(P.bwd, ins[i], dy, ci[i]);
+      }
     }
   }
 };
@@ -1803,6 +2019,15 @@ static int run_op_t(lp_handle* h, Plan& P, const Op& op, const RunCtx& c) {
       double* stats = op.stats_bn >= 0 ? P.bns[op.stats_bn].stats : nullptr;
       const void* addend = op.addend.defined() ? resolve(op.addend, c) : nullptr;
       bool done = false;
+      if (cv.g) {
+        ThinPre tp;
+        if (op.pre) {
+          const BnDef& b = P.bns[op.pre_bn];
+          tp = ThinPre{op.pre, op.pre == 2 ? resolve(op.pre_x, c) : nullptr, bn_args(b, eps), nullptr, nullptr, 1, resolve(op.pre_out, c)};
+        }
+        return launch_conv_thin(h, cv, op.in.n, false, resolve(op.in, c), op.pre ? &tp : nullptr, resolve(op.out, c), addend, stats,
+                                nullptr, h->dev_err, st);
+      }
       if (op.fuse_loss && !c.serial) {
         if (c.loss_wait) LP_CUDA_OK(cudaStreamWaitEvent(st, c.loss_wait, 0));   // x_{k+1} must exist
         LossFuse lf{c.xnext, c.kappa, P.r.p, P.seed.p, c.rho, P.loss_acc};
@@ -1821,6 +2046,15 @@ static int run_op_t(lp_handle* h, Plan& P, const Op& op, const RunCtx& c) {
         const BnDef& b = P.bns[op.bwd_bn];
         bf.x = resolve(op.bwd_x, c); bf.bn = bn_args(b, eps); bf.dgamma = b.dgamma; bf.dbeta = b.dbeta; bf.relu = op.bwd_relu;
         bfp = &bf;
+      }
+      if (cv.g) {
+        ThinPre tp;
+        if (op.pre) {
+          const BnDef& b = P.bns[op.pre_bn];
+          tp = ThinPre{3, resolve(op.pre_x, c), bn_args(b, eps), b.dgamma, b.dbeta, op.pre_relu, resolve(op.pre_out, c)};
+        }
+        return launch_conv_thin(h, cv, op.in.n, true, resolve(op.in, c), op.pre ? &tp : nullptr, resolve(op.out, c), addend, nullptr,
+                                bfp, h->dev_err, st);
       }
       return conv_dgrad(h, dtype, h->conv_impl, cv, op.in.n, resolve(op.in, c), resolve(op.out, c), addend, h->dev_err,
                         st, bfp);
@@ -1904,6 +2138,7 @@ static int run_op_t(lp_handle* h, Plan& P, const Op& op, const RunCtx& c) {
                               (const T*)resolve(op.in, c), (const T*)resolve(op.in2, c), mask, A, b.dgamma, b.dbeta, vecs, b.C));
         h->launches++;
       }
+      if (op.apply_fused) break;   // the input gradient that follows takes the rest
       const int grid_a = grid_for(vecs, threads * 4, cur_dev().sm_count, 2);
       LP_CUDA_OK(launch_pdl(bn_bwd_apply_kernel<T>, dim3(grid_a), dim3(threads), 0, st, (const T*)resolve(op.in, c),
                             (const T*)resolve(op.in2, c), mask, A, (const float*)b.dgamma, (const float*)b.dbeta, addend,
@@ -1999,11 +2234,11 @@ static double op_bytes(const lp_handle* h, const Plan& P, const Op& op) {
   switch (op.type) {
     case OP_CONV_FWD: {
       const ConvDef& c = P.convs[op.conv];
-      return sz(op.in) + sz(op.out) + sz(op.addend) + (double)c.cout * c.R * c.R * c.cin * e;
+      return sz(op.in) + sz(op.out) + sz(op.addend) + sz(op.pre_x) + sz(op.pre_out) + (double)c.cout * c.R * c.R * c.cin * e;
     }
     case OP_CONV_DGRAD: {
       const ConvDef& c = P.convs[op.conv];
-      return sz(op.in) + sz(op.out) + sz(op.addend) + (op.bwd_bn >= 0 ? sz(op.bwd_x) : 0.0) +
+      return sz(op.in) + sz(op.out) + sz(op.addend) + sz(op.pre_x) + sz(op.pre_out) + (op.bwd_bn >= 0 ? sz(op.bwd_x) : 0.0) +
              (double)c.cout * c.R * c.R * c.cin * e;
     }
     case OP_CONV_WGRAD: {
@@ -2015,7 +2250,8 @@ static double op_bytes(const lp_handle* h, const Plan& P, const Op& op) {
     case OP_OUT_LOSS:   // operands of the output, x_next, [kappa,] residual and terminal adjoint
       return op.fuse_loss ? 0.0 : sz(op.in) + sz(op.in2) + sz(op.addend) + 3.0 * sz(op.out);
     case OP_BN_BWD:     // reduction pass (dy, x; not where a convolution took it) and apply pass (dy, x, [addend] -> dx)
-      return (op.reduce_fused ? 1.0 : 2.0) * (sz(op.in) + sz(op.in2)) + sz(op.addend) + sz(op.out);
+      return ((op.reduce_fused ? 0.0 : 1.0) + (op.apply_fused ? 0.0 : 1.0)) * (sz(op.in) + sz(op.in2)) + sz(op.addend) +
+             (op.apply_fused ? 0.0 : sz(op.out));
     case OP_MAXPOOL_FWD: return sz(op.in) + sz(op.out) + (double)op.out.elems();
     case OP_MAXPOOL_BWD: return sz(op.in) + sz(op.out) + (double)op.in.elems();
     case OP_HEAD_FWD: return sz(op.in);
@@ -2028,20 +2264,29 @@ static int run_ops(lp_handle* h, Plan& P, const std::vector<Op>& ops, const RunC
   // (per-operation timing wants one stream: the time line and the convolution profile keep everything in order)
   const bool use_side = P.side && !h->tl.enabled && !h->prof.enabled;
   size_t nside = 0;
+  bool folds = false;
   int rc = LP_OK;
   for (const Op& op : ops) {
+    const bool grouped = op.type == OP_CONV_WGRAD && P.convs[op.conv].g > 1;
     if (use_side && op.type == OP_CONV_WGRAD && nside < P.side_ev.size()) {
       if (cudaEventRecord(P.side_ev[nside], c.st) != cudaSuccess ||
           cudaStreamWaitEvent(P.side, P.side_ev[nside], 0) != cudaSuccess) { rc = LP_ERR_CUDA; break; }
       ++nside;
       RunCtx c2 = c;
       c2.st = P.side;
+      if (grouped && !folds && (folds = true) && cudaMemsetAsync(P.dwg_region, 0, P.dwg_bytes, P.side) != cudaSuccess) { rc = LP_ERR_CUDA; break; }
       rc = h->dtype == LP_F32 ? run_op_t<float>(h, P, op, c2) : run_op_t<bf16>(h, P, op, c2);
     } else {
+      if (grouped && !folds && (folds = true) && cudaMemsetAsync(P.dwg_region, 0, P.dwg_bytes, c.st) != cudaSuccess) { rc = LP_ERR_CUDA; break; }
       TimelineScope ts(h, c.st, c.plan_id, (int)op.type, c.phase, h->tl.enabled ? op_bytes(h, P, op) : 0.0);
       rc = h->dtype == LP_F32 ? run_op_t<float>(h, P, op, c) : run_op_t<bf16>(h, P, op, c);
     }
     if (rc != LP_OK) break;
+  }
+  if (folds && rc == LP_OK) {   // the weight gradients of the grouped layers, after the last of them
+    tc::wgrad_fold_kernel<<<dim3((unsigned)P.host_fold.size(), 9), 256, 0, nside ? P.side : c.st>>>(P.dev_fold);
+    h->launches++;
+    if (cudaGetLastError() != cudaSuccess) rc = LP_ERR_CUDA;
   }
   // joined whatever happened: a stream left unjoined would invalidate a capture in progress
   if (nside && (cudaEventRecord(P.side_done, P.side) != cudaSuccess || cudaStreamWaitEvent(c.st, P.side_done, 0) != cudaSuccess))
@@ -2251,6 +2496,8 @@ int lp_create(const lp_net_desc* desc, void* dev_workspace, size_t bytes, lp_han
   plan_all(h->net, A, &h->modules, &h->auxs, &h->dev_err, &h->zero_labels);
   if (cudaMemset(dev_workspace, 0, need) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
   auto upload = [&](Plan& P) -> int {
+    if (!P.host_fold.empty())
+      LP_CUDA_OK(cudaMemcpy(P.dev_fold, P.host_fold.data(), P.host_fold.size() * sizeof(tc::FoldEntry), cudaMemcpyHostToDevice));
     if (P.ps.host_pack.empty()) return LP_OK;
     LP_CUDA_OK(cudaMemcpy(P.ps.dev_pack, P.ps.host_pack.data(), P.ps.host_pack.size() * sizeof(PackEntry),
                           cudaMemcpyHostToDevice));
@@ -2882,7 +3129,7 @@ int lp_conv2d(int op, int dtype, int impl, int N, int H, int W, int Cin, int Cou
       // pack on the fly: one-entry table placed after the two weight copies is not available on the
       // device, so build it in pinned-free fashion: the table lives in the scratch tail
       PackEntry pe;
-      pe.w = c.w; pe.wf = c.wf; pe.wt = c.wt; pe.cout = Cout; pe.taps = R * R; pe.cin = Cin; pe.begin = 0; pe.tile_begin = 0; pe.tile64_begin = 0;
+      pe.w = c.w; pe.wf = c.wf; pe.wt = c.wt; pe.cout = Cout; pe.taps = R * R; pe.cin = Cin; pe.begin = 0; pe.tile_begin = 0; pe.tile64_begin = 0; pe.gf = pe.gt = nullptr;
       PackEntry* dpe = (PackEntry*)(sp + 256 + 2 * align_up(n * 2, 256));
       LP_CUDA_OK(cudaMemcpyAsync(dpe, &pe, sizeof(pe), cudaMemcpyHostToDevice, st));
       LP_CUDA_OK(cudaStreamSynchronize(st));
@@ -2975,7 +3222,7 @@ int lp_conv2d_fwd_noalloc(int N, int H, int W, int Cin, int Cout, int R, int str
   c.wf = (bf16*)(sp + 256);
   c.wt = nullptr;
   PackEntry pe;
-  pe.w = c.w; pe.wf = c.wf; pe.wt = nullptr; pe.cout = Cout; pe.taps = R * R; pe.cin = Cin; pe.begin = 0; pe.tile_begin = 0; pe.tile64_begin = 0;
+  pe.w = c.w; pe.wf = c.wf; pe.wt = nullptr; pe.cout = Cout; pe.taps = R * R; pe.cin = Cin; pe.begin = 0; pe.tile_begin = 0; pe.tile64_begin = 0; pe.gf = pe.gt = nullptr;
   PackEntry* dpe = (PackEntry*)(sp + 256 + align_up(n * 2, 256));
   LP_CUDA_OK(cudaMemsetAsync(dev_err, 0, 4, st));  // the only word that must start at zero
   LP_CUDA_OK(cudaMemcpyAsync(dpe, &pe, sizeof(pe), cudaMemcpyHostToDevice, st));

@@ -288,6 +288,18 @@ def test_bf16_stem_7x7_stride_2_on_tensor_cores(impl):
     flat_module_parity(cfg, impl, 2e-2)
 
 
+# (channels, H, W, N): tiles of 8 columns with a ragged last row tile; one column of whole box rows (9 and 10 groups wide);
+# three column tiles of 17; several images per tile with a ragged last one; images of one and of two rows; one group wide
+@pytest.mark.parametrize("ch,H,W,N", [(16, 33, 32, 2), (16, 7, 36, 3), (32, 5, 20, 5), (64, 9, 17, 2), (64, 8, 8, 5),
+                                      (64, 2, 3, 9), (32, 1, 16, 20), (16, 12, 4, 7)])
+def test_thin_layers_with_their_batch_norms_taken_along(ch, H, W, N):
+    """3x3 stride-1 layers of 16, 32 and 64 channels on grouped pixels (operand produced from the batch norm before,
+    sums for the batch norm after), modules and AuxNets of two blocks, one step against the storage-model oracle."""
+    cfg = small_cfg("postbn", N=N, H=H, W=W, dtype="bf16", stage_channels=(ch, ch), stage_blocks=(2, 2), stage_stride=(1, 1),
+                    module_block_end=(2, 4), stem_channels=ch, classes=10, aux_width_div=1)
+    full_step_parity(cfg, steps=1)
+
+
 def test_resnet56_reduced_batch_bf16():
     full_step_parity(scaled("resnet56", N=16), steps=1)
 
