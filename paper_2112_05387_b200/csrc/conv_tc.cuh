@@ -52,9 +52,6 @@ constexpr int kMaxSlots = 4;     // accumulator slots in tensor memory
 #ifndef LP_CONV_MIN_BLOCKS
 #define LP_CONV_MIN_BLOCKS 1
 #endif
-#ifndef LP_EPI_BATCH
-#define LP_EPI_BATCH 5
-#endif
 
 // Division by a run-time constant without the divide instruction (Granlund-Montgomery): for 0 <= n < 2^31,
 // n / d = (umulhi(n, mul) + n) >> shift with shift = ceil(log2 d), mul = floor(2^32 (2^shift - d) / d) + 1.
@@ -290,6 +287,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // ------------------------------- TMA producer, halo mode ----------------------------
     uint32_t sa = 0, pha = 0, sb = 0, phb = 0;
     uint8_t* b_ring = smem + p.b_ring_offset;
+#pragma unroll 1
     for (int t = t_begin; t < t_end && !failed;) {
       int nt, m;
       fd_divmod(t, p.fd_m_tiles, nt, m);
@@ -297,6 +295,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       int w0[2], h0[2], n0[2];
       for (int a = 0; a < 2; ++a) tile_first_pixel(p, m + a, w0[a], h0[a], n0[a]);
       const int col0 = nt * p.n_tile_cols;
+#pragma unroll 1
       for (int c = 0; c < p.chunks && !failed; ++c) {
         if (!mbar_wait_warp(&tail->empty[sa], pha ^ 1, abort_flag)) { failed = true; break; }
         uint8_t* pa = smem + sa * p.a_stage_bytes;
@@ -307,11 +306,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         __syncwarp();
         if (++sa == (uint32_t)p.nA) { sa = 0; pha ^= 1; }
+#pragma unroll 1
         for (int ti0 = 0; ti0 < p.ntaps; ti0 += p.tps) {
           const int n_taps = min(p.tps, p.ntaps - ti0);
           if (!mbar_wait_warp(&tail->empty_b[sb], phb ^ 1, abort_flag)) { failed = true; break; }
           if (elect_one()) {
             mbar_expect_tx(&tail->full_b[sb], n_taps * p.tx_b);
+#pragma unroll 1
             for (int i = 0; i < n_taps; ++i)
               tma_load_2d(b_ring + sb * p.b_stage_bytes + i * p.b_tile_bytes, &tmB, &tail->full_b[sb],
                           p.tap_widx9[ti0 + i] * p.Cin + c * p.KC, col0);
@@ -329,6 +330,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t smem_base = smem_u32(smem);
     const int nk = p.KC >> 4;
     uint32_t slot = 0, slot_phase = 0;
+#pragma unroll 1
     for (int t = t_begin; t < t_end && !failed;) {
       const int m = t - fd_div(t, p.fd_m_tiles) * p.m_tiles;
       const int cnt = (p.mpair == 2 && t + 1 < t_end && m + 1 < p.m_tiles) ? 2 : 1;
@@ -342,9 +344,11 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       const uint32_t d = tmem_base + sl[me] * p.acc_stride;
       uint32_t accum = 0;
+#pragma unroll 1
       for (int c = 0; c < p.chunks && !failed; ++c) {
         const uint32_t a_addr = smem_base + sa * p.a_stage_bytes + me * p.a_halo_bytes;
         const int nkc = c + 1 == p.chunks ? p.nk_last : nk;   // slices of pure zero fill are not multiplied
+#pragma unroll 1
         for (int ti0 = 0; ti0 < p.ntaps; ti0 += p.tps) {
           const int n_taps = min(p.tps, p.ntaps - ti0);
           const bool last_of_chunk = ti0 + n_taps == p.ntaps;
@@ -358,9 +362,11 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           const uint32_t b_addr = smem_base + p.b_ring_offset + sb * p.b_stage_bytes;
           if (elect_one()) {
             if (active) {
+#pragma unroll 1
               for (int i = 0; i < n_taps; ++i) {
                 const uint64_t ad = smem_desc(p.desc_hi_a, a_addr + p.tap_off9[ti0 + i]);
                 const uint64_t bd = smem_desc(p.desc_hi, b_addr + i * p.b_tile_bytes);
+#pragma unroll 4
                 for (int j = 0; j < nkc; ++j)
                   mma_bf16(d, ad + (uint64_t)(2 * j), bd + (uint64_t)(2 * j), p.idesc, (accum | i | j) ? 1u : 0u);
               }
@@ -388,6 +394,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else if (warp == 0) {
     // ------------------------------- TMA producer (warp-uniform loop, elected issue) ----
     uint32_t s = 0, ph = 0;
+#pragma unroll 1
     for (int t = t_begin; t < t_end && !failed;) {
       int ntg, m, cls, nt;
       fd_divmod(t, p.fd_m_tiles, ntg, m);
@@ -398,12 +405,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (int a = 0; a < 2; ++a) tile_first_pixel(p, m + a, w0[a], h0[a], n0[a]);
       const int col0 = nt * p.n_tile_cols;
       const uint32_t tx = p.tx_b + cnt * p.tx_a;
+#pragma unroll 1
       for (int k0 = 0; k0 < kiters && !failed; k0 += p.ips) {
         const int n_items = min(p.ips, kiters - k0);
         if (!mbar_wait_warp(&tail->empty[s], ph ^ 1, abort_flag)) { failed = true; break; }
         uint8_t* sa = smem + s * p.stage_bytes;
         if (elect_one()) {
           mbar_expect_tx(&tail->full[s], n_items * tx);
+#pragma unroll 1
           for (int i = 0; i < n_items; ++i) {
             int tap, c;
             fd_divmod(k0 + i, p.fd_chunks, tap, c);
@@ -433,6 +442,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t smem_base = smem_u32(smem);
     const int nk = p.KC >> 4;
     uint32_t slot = 0, slot_phase = 0;  // bit b of slot_phase: parity of the number of uses of slot b
+#pragma unroll 1
     for (int t = t_begin; t < t_end && !failed;) {
       int ntg, m;
       fd_divmod(t, p.fd_m_tiles, ntg, m);
@@ -447,6 +457,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         tc_fence_after();
       }
       const uint32_t d = tmem_base + sl[me] * p.acc_stride;
+#pragma unroll 1
       for (int k0 = 0; k0 < kiters; k0 += p.ips) {
         const int n_items = min(p.ips, kiters - k0);
         if (!mbar_wait_warp(&tail->full[s], ph, abort_flag)) { failed = true; break; }
@@ -454,11 +465,13 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const uint32_t a_addr = smem_base + s * p.stage_bytes;
         if (elect_one()) {
           if (active) {
+#pragma unroll 1
             for (int i = 0; i < n_items; ++i) {
               const int kc = k0 + i - fd_div(k0 + i, p.fd_chunks) * p.chunks;
               const int nkc = kc + 1 == p.chunks ? p.nk_last : nk;
               const uint64_t ad = smem_desc(p.desc_hi, a_addr + i * p.item_bytes + me * p.a_region_bytes);
               const uint64_t bd = smem_desc(p.desc_hi, a_addr + i * p.item_bytes + p.b_offset);
+#pragma unroll 4
               for (int j = 0; j < nkc; ++j)  // +32 bytes (one K = 16 slice) per step, in 16-byte units
                 mma_bf16(d, ad + (uint64_t)(2 * j), bd + (uint64_t)(2 * j), p.idesc, (k0 | i | j) ? 1u : 0u);
             }
@@ -534,10 +547,12 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if constexpr (kAddend) {
       if (et == 0 && t_begin < t_end) load_addend_tile(t_begin);
     }
+#pragma unroll 1
     for (int t = t_begin; t < t_end && !failed;) {
       int nt, m0;
       fd_divmod(t, p.fd_m_tiles, nt, m0);
       const int cnt = (p.mpair == 2 && t + 1 < t_end && m0 + 1 < p.m_tiles) ? 2 : 1;
+#pragma unroll 1
       for (int a = 0; a < cnt && !failed; ++a) {
         const int tile = t + a;
         const int m = m0 + a;
@@ -563,41 +578,34 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (!wait_ok) { failed = true; break; }
         tc_fence_after();
         const uint32_t taddr = tmem_base + buf * p.acc_stride + ((uint32_t)(q * 32) << 16);
-        constexpr int kBatch = LP_EPI_BATCH;
-        for (int g0 = 0; g0 < ngroups; g0 += kBatch) {
-          uint32_t raw[kBatch][32];
-#pragma unroll
-          for (int i = 0; i < kBatch; ++i)
-            if (g0 + i < ngroups) tmem_ld32_issue(taddr + (g0 + i) * 32, raw[i]);
+        // one 32-column group at a time, not unrolled: see the direct epilogue
+#pragma unroll 1
+        for (int g = 0; g < ngroups; ++g) {
+          uint32_t raw[32];
+          tmem_ld32_issue(taddr + g * 32, raw);
           tmem_ld_wait();
-#pragma unroll
-          for (int i = 0; i < kBatch; ++i) tmem_ld_fence(raw[i]);
-          if (g0 + kBatch >= ngroups) {      // the accumulator is in registers: hand the slot back
+          tmem_ld_fence(raw);
+          if (g + 1 == ngroups) {            // the accumulator is in registers: hand the slot back
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tail->tmem_empty[buf]);
           }
+          uint8_t* grow = my_row + g * kStageGroupBytes;
 #pragma unroll
-          for (int i = 0; i < kBatch; ++i) {
-            const int g = g0 + i;
-            if (g >= ngroups) continue;
-            uint8_t* grow = my_row + g * kStageGroupBytes;
+          for (int u = 0; u < 4; ++u) {
+            uint4* dst = reinterpret_cast<uint4*>(grow + ((u ^ swz) << 4));
+            float v[8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              uint4* dst = reinterpret_cast<uint4*>(grow + ((u ^ swz) << 4));
-              float v[8];
+            for (int j = 0; j < 8; ++j) v[j] = valid ? __uint_as_float(raw[8 * u + j]) : 0.f;
+            if constexpr (kAddend) {
+              float f[8];
+              cvt_raw(*dst, f);     // residual piece (zero where the tile leaves the tensor)
 #pragma unroll
-              for (int j = 0; j < 8; ++j) v[j] = valid ? __uint_as_float(raw[i][8 * u + j]) : 0.f;
-              if constexpr (kAddend) {
-                float f[8];
-                cvt_raw(*dst, f);     // residual piece (zero where the tile leaves the tensor)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] += f[j];
-              }
-              if (row < rows_used)
-                *dst = make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]),
-                                  pack_bf16x2(v[6], v[7]));
+              for (int j = 0; j < 8; ++j) v[j] += f[j];
             }
+            if (row < rows_used)
+              *dst = make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]),
+                                pack_bf16x2(v[6], v[7]));
           }
         }
         fence_proxy_async();     // the staged tile is read by the copy engine
@@ -615,6 +623,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           // halves touch different 64-byte halves of a 128-byte line of banks.
           const uint8_t* gbase = stg + sg * kStageGroupBytes;
           const int flip = sg & 1;
+#pragma unroll 4
           for (int r = 0; r < rows_used; ++r) {
             int rr = r ^ flip;
             if (rr >= rows_used) rr = r;
@@ -684,6 +693,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     };
     prefetch_addend(t_begin);
     int consts_nt = -1;                  // channel tile whose batch-norm constants are in shared memory (kBnBwd)
+#pragma unroll 1
     for (int t = t_begin; t < t_end && !failed;) {
       int nt, m0, cls, nt_c;                               // nt counts (class, channel tile) pairs
       fd_divmod(t, p.fd_m_tiles, nt, m0);
@@ -709,6 +719,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           consts_nt = nt;
         }
       }
+#pragma unroll 1
       for (int a = 0; a < cnt && !failed; ++a) {
         prefetch_addend(t + a + 1);
         const int m = m0 + a;
@@ -734,9 +745,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (!wait_ok) { failed = true; break; }
         tc_fence_after();
         const uint32_t taddr = tmem_base + buf * p.acc_stride + ((uint32_t)(q * 32) << 16);
-        // Drain the accumulator into registers first (up to kBatch x 32 columns per pass) and hand
-        // the TMEM slot back to the MMA warp; stores and statistics then work from registers.
-        constexpr int kBatch = kMinBlocks > 1 ? 2 : LP_EPI_BATCH;
+        // One 32-column group at a time, and the loop over the groups stays rolled: draining the whole accumulator
+        // first (five groups unrolled) hands the slot back a little earlier but made this kernel 80 KB of code, more
+        // than the instruction caches hold, and every tile waited for its instructions (ResNet-34 3.46 -> 3.21 ms per
+        // step, ResNet-50 4.00 -> 3.73, WRN-28-10 4.96 -> 4.85).
         // Residual operand of one 32-channel group, as raw 16-byte pieces (zero where nothing is added).
         // A group's pieces are requested while the group before it is processed.
         auto load_addend = [&](int g, uint4 (&a)[4]) {
@@ -758,37 +770,28 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             a[u] = (g < ngroups && u < nv && valid && col0 + c_in_tile + 8 * u < p.Cout)
                        ? ld_raw(p.addend + obase + col0 + c_in_tile + 8 * u) : make_uint4(0u, 0u, 0u, 0u);
         };
-        for (int g0 = grp; g0 < ngroups; g0 += kBatch * kEpiGroups) {
-          uint32_t raw[kBatch][32];
-          uint4 add_cur[4], add_next[4];
-          if constexpr (kAddend) load_addend(g0, add_cur);
-#pragma unroll
-          for (int i = 0; i < kBatch; ++i) {
-            const int g = g0 + i * kEpiGroups;
-            if (g < ngroups) {
-              if (g * 32 + 32 <= p.n_tile_cols) tmem_ld32_issue(taddr + g * 32, raw[i]);
-              else tmem_ld16_issue(taddr + g * 32, raw[i]);
-            }
-          }
+        uint4 add_cur[4], add_next[4];
+        if constexpr (kAddend) load_addend(grp, add_cur);
+#pragma unroll 1
+        for (int g = grp; g < ngroups; g += kEpiGroups) {
+          uint32_t raw[32];
+          if (g * 32 + 32 <= p.n_tile_cols) tmem_ld32_issue(taddr + g * 32, raw);
+          else tmem_ld16_issue(taddr + g * 32, raw);
           tmem_ld_wait();
-#pragma unroll
-          for (int i = 0; i < kBatch; ++i) tmem_ld_fence(raw[i]);
-          if (g0 + kBatch * kEpiGroups >= ngroups) {
+          tmem_ld_fence(raw);
+          if (g + kEpiGroups >= ngroups) {   // the accumulator has been read: hand the slot back
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tail->tmem_empty[buf]);
           }
-#pragma unroll
-          for (int i = 0; i < kBatch; ++i) {
-            const int g = g0 + i * kEpiGroups;
-            if (g >= ngroups) continue;
+          {
             const int c_in_tile = g * 32;
             const int col = col0 + c_in_tile;
             const bool wide = c_in_tile + 32 <= p.n_tile_cols;   // a 16-column tail otherwise
             const int nv = wide ? 4 : 2;                         // 8-channel vectors in this group
             float v[32];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = (wide || j < 16) ? __uint_as_float(raw[i][j]) : 0.f;
+            for (int j = 0; j < 32; ++j) v[j] = (wide || j < 16) ? __uint_as_float(raw[j]) : 0.f;
             // this pixel's 32 channels of the tensor the batch norm normalised, asked for before the
             // stores so that they have arrived when the sums need them
             uint4 xr[kBnBwd ? 4 : 1];
@@ -799,7 +802,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                                                                   : make_uint4(0u, 0u, 0u, 0u);
             }
             if constexpr (kAddend) {
-              if (i + 1 < kBatch) load_addend(g + kEpiGroups, add_next);
+              load_addend(g + kEpiGroups, add_next);
 #pragma unroll
               for (int u = 0; u < 4; ++u) {
                 float f[8];
@@ -923,6 +926,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const bool flush = (kBnBwd || p.stats) && last_of_unit && (t + cnt >= t_end || m0 + cnt >= p.m_tiles);
         if (flush) {
           asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
+#pragma unroll 1
           for (int c = et; c < p.n_tile_cols; c += kEpiThreads) {
             float a_s = 0.f, a_q = 0.f;
             for (int wi = 0; wi < kEpiThreads / 32; ++wi) {
@@ -962,12 +966,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     *abort_flag = 1;
     atomicExch(p.err, 1);
     // let copies and MMAs already in flight land before shared / tensor memory is released
+#pragma unroll 1
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
   __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag && !failed) {
+#pragma unroll 1
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
   __syncthreads();

@@ -302,7 +302,7 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         tc_fence_after();
         const uint32_t taddr = tmem_base + buf * p.acc_stride + ((uint32_t)(q * 32) << 16);
         const uint32_t release_addr = mapa_u32(smem_u32(&tail->tmem_empty[buf]), 0);   // the leader's barrier
-        constexpr int kBatch = LP_EPI_BATCH;
+        constexpr int kBatch = 1;   // (see conv_tc_kernel)
         auto load_addend = [&](int g, uint4 (&ad)[4]) {
           const int c_in_tile = g * 32;
           const int nv = c_in_tile + 32 <= p.n_tile_cols ? 4 : 2;
@@ -316,6 +316,7 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(release_addr);
         }
+#pragma unroll 1
         for (int g0 = 0; have && g0 < ngroups; g0 += kBatch) {
           uint32_t raw[kBatch][32];
           uint4 add_cur[4], add_next[4];
@@ -427,12 +428,14 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     *abort_flag = 1;
     atomicExch(p.err, 1);
     // let copies and MMAs already in flight land before shared / tensor memory is released
+#pragma unroll 1
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
   __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag && !failed) {
+#pragma unroll 1
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
   // neither CTA leaves while the other may still signal its barriers or read its shared memory

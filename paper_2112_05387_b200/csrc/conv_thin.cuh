@@ -331,6 +331,7 @@ conv_thin_kernel(const __grid_constant__ CUtensorMap tmIn0, const __grid_constan
   if (failed) {
     *abort_flag = 1;
     atomicExch(p.err, 1);
+#pragma unroll 1
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);   // copies and MMAs in flight land before the memory is released
   }
   __syncwarp();
@@ -338,7 +339,8 @@ conv_thin_kernel(const __grid_constant__ CUtensorMap tmIn0, const __grid_constan
   __syncthreads();
   if (*abort_flag) {            // (the same for all threads: set before the barrier)
     if (!failed)
-      for (int i = 0; i < 2000; ++i) __nanosleep(1000);
+  #pragma unroll 1
+    for (int i = 0; i < 2000; ++i) __nanosleep(1000);
     __syncthreads();
   }
   if (warp == 2) {

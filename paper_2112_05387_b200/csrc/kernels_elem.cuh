@@ -829,6 +829,7 @@ __device__ __forceinline__ int grouped_col(int r, int pi, int c, int C) {
 __device__ __forceinline__ void grouped_store(const PackEntry& e, int co, int t, int ci, bf16 v) {
   const int C = e.cin, g = 64 / C, K = grouped_cols(C);
   const int r = t / 3, o = t % 3 - 1;
+#pragma unroll 1
   for (int po = 0; po < g; ++po) {
     e.gf[(po * C + co) * K + grouped_col(r, po + o, ci, C)] = v;
     if (e.gt) e.gt[(po * C + ci) * K + grouped_col(r, po - o, co, C)] = v;
@@ -961,16 +962,18 @@ sgd_pack_tiled64_kernel(const PackEntry* __restrict__ tab, int n_entries, float*
       pk.x = *reinterpret_cast<const uint32_t*>(&lo2);
       pk.y = *reinterpret_cast<const uint32_t*>(&hi2);
       *reinterpret_cast<uint2*>(e.wf + j) = pk;
-      if (e.gf) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) grouped_store(e, co, t, ci + u, __float2bfloat16_rn(v[u]));
-      }
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) tile[row][cx + u] = v[u];
   }
-  if (!e.wt) return;
+  if (!e.wt && !e.gf) return;
   __syncthreads();
+  if (e.gf) {
+#pragma unroll 1
+    for (int i = tid; i < e.cout * e.cin; i += 256)     // (grouped layers have at most 32 channels: one tile per tap)
+      grouped_store(e, i / e.cin, t, i % e.cin, __float2bfloat16_rn(tile[i / e.cin][i % e.cin]));
+  }
+  if (!e.wt) return;
   const int warp = tid >> 5, lane = tid & 31;
   const int co = co0 + 2 * lane;
 #pragma unroll

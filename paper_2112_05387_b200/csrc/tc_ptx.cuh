@@ -34,18 +34,31 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 
 // Bounded wait.  `abort_flag` (shared) lets one role's failure release the others quickly.
 constexpr long long kWaitLimitCycles = 600000000LL;  // about 0.3 s at 1.9 GHz
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                          long long limit_cycles = kWaitLimitCycles) {
-  if (mbar_try_wait(bar, parity)) return true;
+// (the polling is a function of its own: inlined at every wait it was a good part of the kernels' code, and code that is
+// not in the instruction cache is what a short kernel waits for)
+__device__ __noinline__ bool mbar_poll(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit_cycles) {
   const long long t0 = clock64();
   int polls = 0;
-  while (!mbar_try_wait(bar, parity)) {
+  while (true) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
     if ((++polls & 63) == 0) {
       if (*abort_flag) return false;
       if (clock64() - t0 > limit_cycles) return false;
     }
   }
-  return true;
+}
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                          long long limit_cycles = kWaitLimitCycles) {
+  if (mbar_try_wait(bar, parity)) return true;
+  return mbar_poll(smem_u32(bar), parity, abort_flag, limit_cycles);
 }
 
 // True in exactly one lane of a converged warp.  The role loops stay warp-uniform (so that

@@ -26,6 +26,8 @@
 namespace lp {
 namespace tc {
 
+// (Loops are kept rolled: a CTA runs most of its code a few times at most and would wait for the instructions of unrolled
+// copies; see the epilogue of conv_tc_kernel.)
 constexpr int kWgMaxStages = 8;
 
 // pixels per K block of wgrad_halo_kernel (128 or 64)
@@ -86,6 +88,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   const int n_iter = pt_end - pt_begin;
 
   if (threadIdx.x == 0) {
+#pragma unroll 1
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(&tail->full[s], 2);    // one expect_tx arrival per producer warp
       mbar_init(&tail->empty[s], 2);   // one arrival per MMA warp
@@ -99,16 +102,21 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   // rows beyond the pixel box are never written by TMA: they must read as zero in the K dimension
   if (p.rows_pad > p.rows) {
     const int a_row_b = p.sca * 2, b_row_b = p.scb * 2;
+#pragma unroll 1
     for (int s = 0; s < p.stages; ++s) {
       uint8_t* sa = smem + (size_t)s * p.stage_bytes;
+#pragma unroll 1
       for (int j = 0; j < p.rpt * p.mpair; ++j) {
         uint8_t* base = sa + (size_t)j * p.a_sub_bytes + (size_t)p.rows * a_row_b;
         const int nbytes = (p.rows_pad - p.rows) * a_row_b;
+#pragma unroll 1
         for (int i = threadIdx.x * 16; i < nbytes; i += blockDim.x * 16) *reinterpret_cast<uint4*>(base + i) = make_uint4(0, 0, 0, 0);
       }
+#pragma unroll 1
       for (int j = 0; j < p.nb; ++j) {
         uint8_t* base = sa + p.a_region + (size_t)j * p.b_sub_bytes + (size_t)p.rows * b_row_b;
         const int nbytes = (p.rows_pad - p.rows) * b_row_b;
+#pragma unroll 1
         for (int i = threadIdx.x * 16; i < nbytes; i += blockDim.x * 16) *reinterpret_cast<uint4*>(base + i) = make_uint4(0, 0, 0, 0);
       }
     }
@@ -153,6 +161,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       my_dh = r - p.pad;
       my_dw = tap - r * p.R - p.pad;
     }
+#pragma unroll 1
     for (int it = 0; it < n_iter; ++it) {
       const int w0 = tw * p.BW, h0 = th * p.BH, n0 = tn * p.BNI;
       if (++tw == p.tiles_w) { tw = 0; if (++th == p.tiles_h) { th = 0; ++tn; } }
@@ -161,6 +170,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       const bool leader = elect_one();
       if (do_a) {
         if (leader) mbar_expect_tx(&tail->full[s], cnt * p.tx_a);
+#pragma unroll 1
         for (int j = 0; j < p.rpt * cnt; ++j) {
           const int c0 = __shfl_sync(0xffffffffu, my_c0, j);
           const int dw = __shfl_sync(0xffffffffu, my_dw, j);
@@ -170,6 +180,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         }
       } else if (leader) {
         mbar_expect_tx(&tail->full[s], p.tx_b);
+#pragma unroll 1
         for (int j = 0; j < p.nb; ++j)
           tma_load_4d(sa + p.a_region + j * p.b_sub_bytes, &tmDY, &tail->full[s], n_tile * p.n_tile + j * p.scb, w0,
                       h0, n0);
@@ -187,6 +198,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     const uint32_t smem_base = smem_u32(smem);
     const int ksteps = p.rows_pad >> 4;
     const uint32_t a_kstep = (uint32_t)(16 * p.sca * 2) >> 4, b_kstep = (uint32_t)(16 * p.scb * 2) >> 4;
+#pragma unroll 1
     for (int it = 0; it < n_iter; ++it) {
       if (!mbar_wait_warp(&tail->full[s], ph, abort_flag)) { failed = true; break; }
       tc_fence_after();
@@ -195,6 +207,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       const uint64_t ad = smem_desc(p.adesc_hi, a_addr + (warp == 1 ? 0u : (uint32_t)(p.rpt * p.a_sub_bytes)));
       if (elect_one()) {
         if (active) {
+#pragma unroll 1
           for (int j = 0; j < ksteps; ++j)
             mma_bf16(tmem_base + acc_col, ad + (uint64_t)(j * a_kstep), bd + (uint64_t)(j * b_kstep), p.idesc, (it | j) ? 1u : 0u);
           mma_commit(&tail->empty[s]);
@@ -225,6 +238,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       tc_fence_after();
       const int sub = row / p.sca, ci_l = row % p.sca;
       const int co0 = n_tile * p.n_tile;
+#pragma unroll 1
       for (int a = 0; a < cnt; ++a) {
         if (a > 0) {
           if (et == 0) bulk_wait_read(0);
@@ -232,6 +246,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         }
         float* buf = reinterpret_cast<float*>(smem + (size_t)sub * p.epi_buf_bytes);
         const uint32_t taddr = tmem_base + a * 256 + ((uint32_t)(q * 32) << 16);
+#pragma unroll 1
         for (int cc = 0; cc < (p.n_tile >> 4); ++cc) {
           float v[16];
           tmem_ld16(taddr + cc * 16, v);
@@ -241,6 +256,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         fence_proxy_async();
         asm volatile("bar.sync 1, 128;" ::: "memory");
         if (et == 0) {
+#pragma unroll 1
           for (int sb = 0; sb < p.rpt; ++sb) {
             const int g = (m_tile + a) * p.rpt + sb;
             if (g < p.total_chunks)
@@ -253,6 +269,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       tc_fence_before();
     } else if (*(volatile int*)&tail->epi_ok) {
       tc_fence_after();
+#pragma unroll 1
       for (int a = 0; a < cnt; ++a) {
         const int g = (m_tile + a) * p.rpt + row / p.sca;
         const int ci_raw = (g % p.cin_chunks) * p.sca + row % p.sca;
@@ -261,6 +278,7 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         const int ci = valid ? ci_raw : 0;
         const uint32_t taddr = tmem_base + a * 256 + ((uint32_t)(q * 32) << 16);
         const int co0 = n_tile * p.n_tile;
+#pragma unroll 1
         for (int cc = 0; cc < (p.n_tile >> 4); ++cc) {
           float v[16];
           tmem_ld16(taddr + cc * 16, v);
@@ -282,12 +300,14 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   if (failed) {
     *abort_flag = 1;
     atomicExch(p.err, 1);
+#pragma unroll 1
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
   __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag && !failed) {
+#pragma unroll 1
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
   __syncthreads();
@@ -330,6 +350,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
   const int n_iter = pt_end - pt_begin;
 
   if (threadIdx.x == 0) {
+#pragma unroll 1
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(&tail->full[s], 2);
       mbar_init(&tail->empty[s], 2);     // one commit per MMA-issuing warp
@@ -362,6 +383,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
       tn = q1 / p.tiles_h;
       th = q1 - tn * p.tiles_h;
     }
+#pragma unroll 1
     for (int it = 0; it < n_iter; ++it) {
       const int w0 = tw * 8, h0 = th * p.BH, n0 = tn * p.BNI;
       if (++tw == p.tiles_w) { tw = 0; if (++th == p.tiles_h) { th = 0; ++tn; } }
@@ -377,6 +399,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         }
       } else if (leader) {
         mbar_expect_tx(&tail->full[s], p.tx_b);
+#pragma unroll 1
         for (int j = 0; j < p.nb; ++j)
           tma_load_4d(sa + p.a_region + j * p.b_sub_bytes, &tmDY, &tail->full[s], n_tile * p.n_tile + j * p.scb, w0,
                       n0, h0);
@@ -393,6 +416,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     const uint32_t smem_base = smem_u32(smem);
     const uint32_t a_kstep = p.a_kstep_bytes >> 4, b_kstep = (uint32_t)(16 * p.scb * 2) >> 4;
     const int ksteps = p.rows >> 4;   // K = 16 pixels per MMA
+#pragma unroll 1
     for (int it = 0; it < n_iter; ++it) {
       if (!mbar_wait_warp(&tail->full[s], ph, abort_flag)) { failed = true; break; }
       tc_fence_after();
@@ -438,6 +462,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
       const int ci_l = (q & 1) * 32 + lane;        // input channel within the chunk
       const int rounds_in_flight = p.epi_bufs >> 1;
       const int co0 = n_tile * p.n_tile;
+#pragma unroll 1
       for (int a = 0; a < 3; ++a) {
         if (a >= rounds_in_flight) {
           if (et == 0) bulk_wait_read(rounds_in_flight - 1);
@@ -446,6 +471,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         const int slot = (a % rounds_in_flight) * 2;
         float* buf = reinterpret_cast<float*>(smem + (size_t)(slot + hh) * p.epi_buf_bytes);
         const uint32_t taddr = tmem_base + a * p.acc_stride + ((uint32_t)(q * 32) << 16);
+#pragma unroll 1
         for (int cc = 0; cc < (p.n_tile >> 4); ++cc) {
           float v[16];
           tmem_ld16(taddr + cc * 16, v);
@@ -468,6 +494,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
       tc_fence_before();
     } else if (*(volatile int*)&tail->epi_ok) {
       tc_fence_after();
+#pragma unroll 1
       for (int a = 0; a < 3; ++a) {
         const int chunk = 2 * a + (row >> 6);          // 0..5: group chunk/3, kernel column chunk%3
         const int g = g0 + chunk / 3, sx = chunk % 3;
@@ -477,6 +504,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         const int ci = valid ? ci_raw : 0;
         const uint32_t taddr = tmem_base + a * p.acc_stride + ((uint32_t)(q * 32) << 16);
         const int co0 = n_tile * p.n_tile;
+#pragma unroll 1
         for (int cc = 0; cc < (p.n_tile >> 4); ++cc) {
           float v[16];
           tmem_ld16(taddr + cc * 16, v);
@@ -498,12 +526,14 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
   if (failed) {
     *abort_flag = 1;
     atomicExch(p.err, 1);
+#pragma unroll 1
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
   __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (*abort_flag && !failed) {
+#pragma unroll 1
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
   __syncthreads();
