@@ -127,7 +127,8 @@ struct ConvTcParams {
   uint32_t b_tile_bytes;         // weights of one tap inside a weight stage
   uint32_t tail_offset;          // barriers and scratch after the rings
   int tap_widx9[16];             // weight tap index of the taps in (dy, dx) order (nine for 3x3, sixteen for 4x4)
-  uint32_t tap_off9[16];         // byte offset of the tap's first row inside the box
+  int tap_k9[16];                // first column of the tap's weights: that index x C_in
+  uint32_t tap_off9[16];         // offset of the tap's first row inside the box, in units of 16 bytes
   int halo_dw0, halo_dh0;        // offset of the first tap: the box starts that many pixels from the tile (-1 for 3x3)
   uint64_t desc_hi_a;            // descriptor of the activation operand (row-group stride of the box)
   // local loss of an interior module, fused into the epilogue of the module's last convolution
@@ -242,9 +243,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   if (threadIdx.x < kMaxStages) {
     const int s = threadIdx.x;
     mbar_init(&tail->full[s], 1);
-    mbar_init(&tail->empty[s], 2);   // one arrival per MMA warp
+    mbar_init(&tail->empty[s], p.mpair);   // one arrival per MMA-issuing thread
     mbar_init(&tail->full_b[s], 1);
-    mbar_init(&tail->empty_b[s], 2);
+    mbar_init(&tail->empty_b[s], p.mpair);
     fence_barrier_init();
   } else if (threadIdx.x >= 32 && threadIdx.x < 32 + kMaxSlots) {
     const int b = threadIdx.x - 32;
@@ -284,212 +285,229 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   // All three roles walk the same sequence of units: a unit is one pixel tile, or two consecutive
   // ones of the same channel tile, and takes the next one or two accumulator slots of the ring.
   if (warp == 0 && p.halo) {
-    // ------------------------------- TMA producer, halo mode ----------------------------
-    uint32_t sa = 0, pha = 0, sb = 0, phb = 0;
-    uint8_t* b_ring = smem + p.b_ring_offset;
+    // ------------------------------- TMA producer, halo mode (one thread) ---------------
+    if (elect_one()) {
+      uint32_t sa = 0, pha = 0, sb = 0, phb = 0;
+      uint8_t* b_ring = smem + p.b_ring_offset;
 #pragma unroll 1
-    for (int t = t_begin; t < t_end && !failed;) {
-      int nt, m;
-      fd_divmod(t, p.fd_m_tiles, nt, m);
-      const int cnt = (p.mpair == 2 && t + 1 < t_end && m + 1 < p.m_tiles) ? 2 : 1;
-      int w0[2], h0[2], n0[2];
-      for (int a = 0; a < 2; ++a) tile_first_pixel(p, m + a, w0[a], h0[a], n0[a]);
-      const int col0 = nt * p.n_tile_cols;
+      for (int t = t_begin; t < t_end && !failed;) {
+        int nt, m;
+        fd_divmod(t, p.fd_m_tiles, nt, m);
+        const int cnt = (p.mpair == 2 && t + 1 < t_end && m + 1 < p.m_tiles) ? 2 : 1;
+        int w0, h0, n0, w1, h1, n1;
+        tile_first_pixel(p, m, w0, h0, n0);
+        tile_first_pixel(p, m + 1, w1, h1, n1);
+        const int col0 = nt * p.n_tile_cols;
 #pragma unroll 1
-      for (int c = 0; c < p.chunks && !failed; ++c) {
-        if (!mbar_wait_warp(&tail->empty[sa], pha ^ 1, abort_flag)) { failed = true; break; }
-        uint8_t* pa = smem + sa * p.a_stage_bytes;
-        if (elect_one()) {
+        for (int c = 0; c < p.chunks && !failed; ++c) {
+          if (!mbar_wait(&tail->empty[sa], pha ^ 1, abort_flag)) { failed = true; break; }
+          uint8_t* pa = smem + sa * p.a_stage_bytes;
           mbar_expect_tx(&tail->full[sa], cnt * p.tx_a);
-          tma_load_4d(pa, &tmA, &tail->full[sa], c * p.KC, w0[0] + p.halo_dw0, n0[0], h0[0] + p.halo_dh0);
-          if (cnt == 2) tma_load_4d(pa + p.a_halo_bytes, &tmA, &tail->full[sa], c * p.KC, w0[1] + p.halo_dw0, n0[1], h0[1] + p.halo_dh0);
-        }
-        __syncwarp();
-        if (++sa == (uint32_t)p.nA) { sa = 0; pha ^= 1; }
+          tma_load_4d(pa, &tmA, &tail->full[sa], c * p.KC, w0 + p.halo_dw0, n0, h0 + p.halo_dh0);
+          if (cnt == 2) tma_load_4d(pa + p.a_halo_bytes, &tmA, &tail->full[sa], c * p.KC, w1 + p.halo_dw0, n1, h1 + p.halo_dh0);
+          if (++sa == (uint32_t)p.nA) { sa = 0; pha ^= 1; }
 #pragma unroll 1
-        for (int ti0 = 0; ti0 < p.ntaps; ti0 += p.tps) {
-          const int n_taps = min(p.tps, p.ntaps - ti0);
-          if (!mbar_wait_warp(&tail->empty_b[sb], phb ^ 1, abort_flag)) { failed = true; break; }
-          if (elect_one()) {
-            mbar_expect_tx(&tail->full_b[sb], n_taps * p.tx_b);
+          for (int ti0 = 0; ti0 < p.ntaps; ti0 += p.tps) {
+            const int ti1 = min(ti0 + p.tps, p.ntaps);
+            if (!mbar_wait(&tail->empty_b[sb], phb ^ 1, abort_flag)) { failed = true; break; }
+            mbar_expect_tx(&tail->full_b[sb], (ti1 - ti0) * p.tx_b);
+            uint8_t* pb = b_ring + sb * p.b_stage_bytes;
 #pragma unroll 1
-            for (int i = 0; i < n_taps; ++i)
-              tma_load_2d(b_ring + sb * p.b_stage_bytes + i * p.b_tile_bytes, &tmB, &tail->full_b[sb],
-                          p.tap_widx9[ti0 + i] * p.Cin + c * p.KC, col0);
+            for (int i = ti0; i < ti1; ++i, pb += p.b_tile_bytes)
+              tma_load_2d(pb, &tmB, &tail->full_b[sb], p.tap_k9[i] + c * p.KC, col0);
+            if (++sb == (uint32_t)p.nB) { sb = 0; phb ^= 1; }
           }
-          __syncwarp();
-          if (++sb == (uint32_t)p.nB) { sb = 0; phb ^= 1; }
         }
+        t += cnt;
       }
-      t += cnt;
     }
+    __syncwarp();
+    failed = __any_sync(0xffffffffu, failed);
   } else if ((warp == 1 || warp == 2) && p.halo) {
     // ------------------------------- MMA issuers, halo mode -----------------------------
+    // One thread runs the whole loop.  What it does between the last MMA of a stage and the first of the next (poll,
+    // descriptors, commit) has to be shorter than the MMAs still queued, about four, or the tensor pipe runs dry: with a
+    // warp-uniform loop that elected a lane per stage a stage of four MMAs cost 800 to 850 cycles whatever their width
+    // (324 cycles of work at N = 160, 492 at N = 256).
     const int me = warp - 1;
-    uint32_t sa = 0, pha = 0, sb = 0, phb = 0;
-    const uint32_t smem_base = smem_u32(smem);
-    const int nk = p.KC >> 4;
-    uint32_t slot = 0, slot_phase = 0;
+    if (me < p.mpair && elect_one()) {
+      uint32_t sa = 0, pha = 0, sb = 0, phb = 0, slot = 0, slot_phase = 0;
+      const uint32_t base16 = smem_u32(smem) >> 4;
+      const uint32_t a_hi = (uint32_t)(p.desc_hi_a >> 32), b_hi = (uint32_t)(p.desc_hi >> 32);
+      const uint32_t a_stage16 = p.a_stage_bytes >> 4, b_stage16 = p.b_stage_bytes >> 4, b_tile16 = p.b_tile_bytes >> 4;
+      const uint32_t a_lo0 = (uint32_t)p.desc_hi_a + base16 + me * (p.a_halo_bytes >> 4);
+      const uint32_t b_lo0 = (uint32_t)p.desc_hi + base16 + (p.b_ring_offset >> 4);
+      const int nk = p.KC >> 4;
 #pragma unroll 1
-    for (int t = t_begin; t < t_end && !failed;) {
-      const int m = t - fd_div(t, p.fd_m_tiles) * p.m_tiles;
-      const int cnt = (p.mpair == 2 && t + 1 < t_end && m + 1 < p.m_tiles) ? 2 : 1;
-      uint32_t sl[2];
-      sl[0] = slot;
-      sl[1] = slot + 1 == (uint32_t)p.nslots ? 0 : slot + 1;
-      const bool active = me < cnt;
-      if (active) {
-        if (!mbar_wait_warp(&tail->tmem_empty[sl[me]], ((slot_phase >> sl[me]) & 1) ^ 1, abort_flag)) { failed = true; break; }
-        tc_fence_after();
-      }
-      const uint32_t d = tmem_base + sl[me] * p.acc_stride;
-      uint32_t accum = 0;
-#pragma unroll 1
-      for (int c = 0; c < p.chunks && !failed; ++c) {
-        const uint32_t a_addr = smem_base + sa * p.a_stage_bytes + me * p.a_halo_bytes;
-        const int nkc = c + 1 == p.chunks ? p.nk_last : nk;   // slices of pure zero fill are not multiplied
-#pragma unroll 1
-        for (int ti0 = 0; ti0 < p.ntaps; ti0 += p.tps) {
-          const int n_taps = min(p.tps, p.ntaps - ti0);
-          const bool last_of_chunk = ti0 + n_taps == p.ntaps;
-          // The box barrier is polled together with the first weight stage and released together
-          // with the last one: a separate trip (poll, election, commit) at every chunk boundary
-          // costs about 500 cycles in which the tensor pipe runs dry.
-          bool ok = ti0 ? true : mbar_wait(&tail->full[sa], pha, abort_flag);
-          ok = mbar_wait(&tail->full_b[sb], phb, abort_flag) && ok;
-          if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
+      for (int t = t_begin; t < t_end && !failed;) {
+        const int m = t - fd_div(t, p.fd_m_tiles) * p.m_tiles;
+        const int cnt = (p.mpair == 2 && t + 1 < t_end && m + 1 < p.m_tiles) ? 2 : 1;
+        const uint32_t slot1 = slot + 1 == (uint32_t)p.nslots ? 0 : slot + 1;
+        const uint32_t mine = me ? slot1 : slot;
+        const bool active = me < cnt;
+        if (active) {
+          if (!mbar_wait(&tail->tmem_empty[mine], ((slot_phase >> mine) & 1) ^ 1, abort_flag)) { failed = true; break; }
           tc_fence_after();
-          const uint32_t b_addr = smem_base + p.b_ring_offset + sb * p.b_stage_bytes;
-          if (elect_one()) {
-            if (active) {
+        }
+        const uint32_t d = tmem_base + mine * p.acc_stride;
+        uint32_t accum = 0;
 #pragma unroll 1
-              for (int i = 0; i < n_taps; ++i) {
-                const uint64_t ad = smem_desc(p.desc_hi_a, a_addr + p.tap_off9[ti0 + i]);
-                const uint64_t bd = smem_desc(p.desc_hi, b_addr + i * p.b_tile_bytes);
-#pragma unroll 4
-                for (int j = 0; j < nkc; ++j)
-                  mma_bf16(d, ad + (uint64_t)(2 * j), bd + (uint64_t)(2 * j), p.idesc, (accum | i | j) ? 1u : 0u);
+        for (int c = 0; c < p.chunks && !failed; ++c) {
+          const uint32_t a_lo = a_lo0 + sa * a_stage16;
+          const int nkc = c + 1 == p.chunks ? p.nk_last : nk;   // slices of pure zero fill are not multiplied
+#pragma unroll 1
+          for (int ti0 = 0; ti0 < p.ntaps; ti0 += p.tps) {
+            const int ti1 = min(ti0 + p.tps, p.ntaps);
+            if ((ti0 == 0 && !mbar_wait(&tail->full[sa], pha, abort_flag)) || !mbar_wait(&tail->full_b[sb], phb, abort_flag)) {
+              failed = true;
+              break;
+            }
+            tc_fence_after();
+            if (active) {
+              uint32_t b_lo = b_lo0 + sb * b_stage16;
+#pragma unroll 1
+              for (int i = ti0; i < ti1; ++i) {
+                const uint32_t at = a_lo + p.tap_off9[i];
+                mma_bf16_lh(d, at, a_hi, b_lo, b_hi, p.idesc, accum);
+                accum = 1;
+                if (nkc == 4) {
+                  mma_bf16_lh(d, at + 2, a_hi, b_lo + 2, b_hi, p.idesc, 1u);
+                  mma_bf16_lh(d, at + 4, a_hi, b_lo + 4, b_hi, p.idesc, 1u);
+                  mma_bf16_lh(d, at + 6, a_hi, b_lo + 6, b_hi, p.idesc, 1u);
+                } else {
+#pragma unroll 1
+                  for (int j = 1; j < nkc; ++j) mma_bf16_lh(d, at + 2 * j, a_hi, b_lo + 2 * j, b_hi, p.idesc, 1u);
+                }
+                b_lo += b_tile16;
               }
               mma_commit(&tail->empty_b[sb]);
-              if (last_of_chunk) mma_commit(&tail->empty[sa]);
+              if (ti1 == p.ntaps) mma_commit(&tail->empty[sa]);
             } else {
               mbar_arrive(&tail->empty_b[sb]);
-              if (last_of_chunk) mbar_arrive(&tail->empty[sa]);
+              if (ti1 == p.ntaps) mbar_arrive(&tail->empty[sa]);
             }
+            if (++sb == (uint32_t)p.nB) { sb = 0; phb ^= 1; }
           }
-          __syncwarp();
-          accum = 1;
-          if (++sb == (uint32_t)p.nB) { sb = 0; phb ^= 1; }
+          if (++sa == (uint32_t)p.nA) { sa = 0; pha ^= 1; }
         }
         if (failed) break;
-        if (++sa == (uint32_t)p.nA) { sa = 0; pha ^= 1; }
+        if (active) mma_commit(&tail->tmem_full[mine]);
+        slot_phase ^= 1u << slot;
+        if (cnt == 2) slot_phase ^= 1u << slot1;
+        slot = cnt == 2 ? (slot1 + 1 == (uint32_t)p.nslots ? 0 : slot1 + 1) : slot1;
+        t += cnt;
       }
-      if (failed) break;
-      if (active && elect_one()) mma_commit(&tail->tmem_full[sl[me]]);
-      __syncwarp();
-      for (int a = 0; a < cnt; ++a) slot_phase ^= 1u << sl[a];
-      slot = cnt == 2 ? (sl[1] + 1 == (uint32_t)p.nslots ? 0 : sl[1] + 1) : sl[1];
-      t += cnt;
     }
+    __syncwarp();
+    failed = __any_sync(0xffffffffu, failed);
   } else if (warp == 0) {
-    // ------------------------------- TMA producer (warp-uniform loop, elected issue) ----
-    uint32_t s = 0, ph = 0;
+    // ------------------------------- TMA producer (one thread) --------------------------
+    if (elect_one()) {
+      uint32_t s = 0, ph = 0;
 #pragma unroll 1
-    for (int t = t_begin; t < t_end && !failed;) {
-      int ntg, m, cls, nt;
-      fd_divmod(t, p.fd_m_tiles, ntg, m);
-      fd_divmod(ntg, p.fd_n_tiles, cls, nt);
-      const int kiters = p.cls_ntaps[cls] * p.chunks;
-      const int cnt = (p.mpair == 2 && t + 1 < t_end && m + 1 < p.m_tiles) ? 2 : 1;
-      int w0[2], h0[2], n0[2];
-      for (int a = 0; a < 2; ++a) tile_first_pixel(p, m + a, w0[a], h0[a], n0[a]);
-      const int col0 = nt * p.n_tile_cols;
-      const uint32_t tx = p.tx_b + cnt * p.tx_a;
+      for (int t = t_begin; t < t_end && !failed;) {
+        int ntg, m, cls, nt;
+        fd_divmod(t, p.fd_m_tiles, ntg, m);
+        fd_divmod(ntg, p.fd_n_tiles, cls, nt);
+        const int kiters = p.cls_ntaps[cls] * p.chunks;
+        const int cnt = (p.mpair == 2 && t + 1 < t_end && m + 1 < p.m_tiles) ? 2 : 1;
+        int w0, h0, n0, w1, h1, n1;
+        tile_first_pixel(p, m, w0, h0, n0);
+        tile_first_pixel(p, m + 1, w1, h1, n1);
+        w0 *= p.in_step; h0 *= p.in_step; w1 *= p.in_step; h1 *= p.in_step;
+        const int col0 = nt * p.n_tile_cols;
+        const uint32_t tx = p.tx_b + cnt * p.tx_a;
+        int tap = p.cls_tap0[cls], c = 0;
 #pragma unroll 1
-      for (int k0 = 0; k0 < kiters && !failed; k0 += p.ips) {
-        const int n_items = min(p.ips, kiters - k0);
-        if (!mbar_wait_warp(&tail->empty[s], ph ^ 1, abort_flag)) { failed = true; break; }
-        uint8_t* sa = smem + s * p.stage_bytes;
-        if (elect_one()) {
+        for (int k0 = 0; k0 < kiters; k0 += p.ips) {
+          const int n_items = min(p.ips, kiters - k0);
+          if (!mbar_wait(&tail->empty[s], ph ^ 1, abort_flag)) { failed = true; break; }
+          uint8_t* si = smem + s * p.stage_bytes;
           mbar_expect_tx(&tail->full[s], n_items * tx);
 #pragma unroll 1
-          for (int i = 0; i < n_items; ++i) {
-            int tap, c;
-            fd_divmod(k0 + i, p.fd_chunks, tap, c);
-            tap += p.cls_tap0[cls];
-            const int kb = p.tap_w[tap] * p.Cin;
-            uint8_t* si = sa + i * p.item_bytes;
-            tma_load_4d(si, &tmA, &tail->full[s], c * p.KC, w0[0] * p.in_step + p.tap_dw[tap],
-                        h0[0] * p.in_step + p.tap_dh[tap], n0[0]);
-            if (cnt == 2)
-              tma_load_4d(si + p.a_region_bytes, &tmA, &tail->full[s], c * p.KC, w0[1] * p.in_step + p.tap_dw[tap],
-                          h0[1] * p.in_step + p.tap_dh[tap], n0[1]);
-            tma_load_2d(si + p.b_offset, &tmB, &tail->full[s], kb + c * p.KC, col0);
+          for (int i = 0; i < n_items; ++i, si += p.item_bytes) {
+            const int ch = c * p.KC, dw = p.tap_dw[tap], dh = p.tap_dh[tap];
+            tma_load_4d(si, &tmA, &tail->full[s], ch, w0 + dw, h0 + dh, n0);
+            if (cnt == 2) tma_load_4d(si + p.a_region_bytes, &tmA, &tail->full[s], ch, w1 + dw, h1 + dh, n1);
+            tma_load_2d(si + p.b_offset, &tmB, &tail->full[s], p.tap_w[tap] * p.Cin + ch, col0);
+            if (++c == p.chunks) { c = 0; ++tap; }
           }
+          if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
         }
-        __syncwarp();
-        if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
+        t += cnt;
       }
-      t += cnt;
     }
+    __syncwarp();
+    failed = __any_sync(0xffffffffu, failed);
   } else if (warp == 1 || warp == 2) {
-    // ------------------------------- MMA issuers (warp-uniform loops, elected issue) ----
+    // ------------------------------- MMA issuers (one thread each) ----------------------
     // Warp 1 owns the first accumulator of every unit, warp 2 the second one of a pair.  Both
     // wait for every stage and both arrive on its "empty" barrier: with a commit after their
     // MMAs, or (warp 2 in a single-tile unit) with a plain arrive.
     const int me = warp - 1;
-    uint32_t s = 0, ph = 0;
-    const uint32_t smem_base = smem_u32(smem);
-    const int nk = p.KC >> 4;
-    uint32_t slot = 0, slot_phase = 0;  // bit b of slot_phase: parity of the number of uses of slot b
+    if (me < p.mpair && elect_one()) {
+      uint32_t s = 0, ph = 0, slot = 0, slot_phase = 0;  // bit b of slot_phase: parity of the number of uses of slot b
+      const uint32_t base16 = smem_u32(smem) >> 4;
+      const uint32_t hi = (uint32_t)(p.desc_hi >> 32);
+      const uint32_t stage16 = p.stage_bytes >> 4, item16 = p.item_bytes >> 4, b_off16 = p.b_offset >> 4;
+      const uint32_t a_lo0 = (uint32_t)p.desc_hi + base16, a_me16 = me * (p.a_region_bytes >> 4);
+      const int nk = p.KC >> 4;
 #pragma unroll 1
-    for (int t = t_begin; t < t_end && !failed;) {
-      int ntg, m;
-      fd_divmod(t, p.fd_m_tiles, ntg, m);
-      const int kiters = p.cls_ntaps[fd_div(ntg, p.fd_n_tiles)] * p.chunks;
-      const int cnt = (p.mpair == 2 && t + 1 < t_end && m + 1 < p.m_tiles) ? 2 : 1;
-      uint32_t sl[2];
-      sl[0] = slot;
-      sl[1] = slot + 1 == (uint32_t)p.nslots ? 0 : slot + 1;
-      const bool active = me < cnt;
-      if (active) {
-        if (!mbar_wait_warp(&tail->tmem_empty[sl[me]], ((slot_phase >> sl[me]) & 1) ^ 1, abort_flag)) { failed = true; break; }
-        tc_fence_after();
-      }
-      const uint32_t d = tmem_base + sl[me] * p.acc_stride;
+      for (int t = t_begin; t < t_end && !failed;) {
+        int ntg, m;
+        fd_divmod(t, p.fd_m_tiles, ntg, m);
+        const int kiters = p.cls_ntaps[fd_div(ntg, p.fd_n_tiles)] * p.chunks;
+        const int cnt = (p.mpair == 2 && t + 1 < t_end && m + 1 < p.m_tiles) ? 2 : 1;
+        const uint32_t slot1 = slot + 1 == (uint32_t)p.nslots ? 0 : slot + 1;
+        const uint32_t mine = me ? slot1 : slot;
+        const bool active = me < cnt;
+        if (active) {
+          if (!mbar_wait(&tail->tmem_empty[mine], ((slot_phase >> mine) & 1) ^ 1, abort_flag)) { failed = true; break; }
+          tc_fence_after();
+        }
+        const uint32_t d = tmem_base + mine * p.acc_stride;
+        uint32_t accum = 0;
+        int kc = 0;                        // K chunk of the item
 #pragma unroll 1
-      for (int k0 = 0; k0 < kiters; k0 += p.ips) {
-        const int n_items = min(p.ips, kiters - k0);
-        if (!mbar_wait_warp(&tail->full[s], ph, abort_flag)) { failed = true; break; }
-        tc_fence_after();
-        const uint32_t a_addr = smem_base + s * p.stage_bytes;
-        if (elect_one()) {
+        for (int k0 = 0; k0 < kiters; k0 += p.ips) {
+          const int n_items = min(p.ips, kiters - k0);
+          if (!mbar_wait(&tail->full[s], ph, abort_flag)) { failed = true; break; }
+          tc_fence_after();
           if (active) {
+            uint32_t item = a_lo0 + s * stage16;
 #pragma unroll 1
             for (int i = 0; i < n_items; ++i) {
-              const int kc = k0 + i - fd_div(k0 + i, p.fd_chunks) * p.chunks;
-              const int nkc = kc + 1 == p.chunks ? p.nk_last : nk;
-              const uint64_t ad = smem_desc(p.desc_hi, a_addr + i * p.item_bytes + me * p.a_region_bytes);
-              const uint64_t bd = smem_desc(p.desc_hi, a_addr + i * p.item_bytes + p.b_offset);
-#pragma unroll 4
-              for (int j = 0; j < nkc; ++j)  // +32 bytes (one K = 16 slice) per step, in 16-byte units
-                mma_bf16(d, ad + (uint64_t)(2 * j), bd + (uint64_t)(2 * j), p.idesc, (k0 | i | j) ? 1u : 0u);
+              const int nkc = ++kc == p.chunks ? p.nk_last : nk;
+              if (kc == p.chunks) kc = 0;
+              const uint32_t at = item + a_me16, bt = item + b_off16;
+              mma_bf16_lh(d, at, hi, bt, hi, p.idesc, accum);
+              accum = 1;
+              if (nkc == 4) {              // +32 bytes (one K = 16 slice) per step, in 16-byte units
+                mma_bf16_lh(d, at + 2, hi, bt + 2, hi, p.idesc, 1u);
+                mma_bf16_lh(d, at + 4, hi, bt + 4, hi, p.idesc, 1u);
+                mma_bf16_lh(d, at + 6, hi, bt + 6, hi, p.idesc, 1u);
+              } else {
+#pragma unroll 1
+                for (int j = 1; j < nkc; ++j) mma_bf16_lh(d, at + 2 * j, hi, bt + 2 * j, hi, p.idesc, 1u);
+              }
+              item += item16;
             }
             mma_commit(&tail->empty[s]);
           } else {
             mbar_arrive(&tail->empty[s]);
           }
+          if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
         }
-        __syncwarp();
-        if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
+        if (failed) break;
+        if (active) mma_commit(&tail->tmem_full[mine]);
+        slot_phase ^= 1u << slot;
+        if (cnt == 2) slot_phase ^= 1u << slot1;
+        slot = cnt == 2 ? (slot1 + 1 == (uint32_t)p.nslots ? 0 : slot1 + 1) : slot1;
+        t += cnt;
       }
-      if (failed) break;
-      if (active && elect_one()) mma_commit(&tail->tmem_full[sl[me]]);
-      __syncwarp();
-      for (int a = 0; a < cnt; ++a) slot_phase ^= 1u << sl[a];
-      slot = cnt == 2 ? (sl[1] + 1 == (uint32_t)p.nslots ? 0 : sl[1] + 1) : sl[1];
-      t += cnt;
     }
+    __syncwarp();
+    failed = __any_sync(0xffffffffu, failed);
   } else {
     if constexpr (kStaged) {
     // ------------------------------- epilogue, staged through shared memory -------------

@@ -679,8 +679,8 @@ static int launch_conv_tc(lp_handle* h, const TcGemmSpec& s, int* dev_err, cudaS
     p.a_halo_bytes = (uint32_t)align_up((size_t)halo_rows * row_bytes, 1024);
     for (int dy = 0; dy < halo_R; ++dy)
       for (int dx = 0; dx < halo_R; ++dx) {
-        p.tap_widx9[dy * halo_R + dx] = tapw[dy * halo_R + dx];
-        p.tap_off9[dy * halo_R + dx] = (uint32_t)((dy * halo_w * p.BNI + dx) * row_bytes);
+        p.tap_k9[dy * halo_R + dx] = tapw[dy * halo_R + dx] * s.aC;
+        p.tap_off9[dy * halo_R + dx] = (uint32_t)((dy * halo_w * p.BNI + dx) * row_bytes) >> 4;
       }
     // 8-row groups of the operand are one box row (halo_w pixels) apart
     p.desc_hi_a = tc::smem_desc_hi(16, halo_w * row_bytes, tc::swizzle_code_for_row_bytes(row_bytes));
@@ -2274,10 +2274,12 @@ static int run_ops(lp_handle* h, Plan& P, const std::vector<Op>& ops, const RunC
       ++nside;
       RunCtx c2 = c;
       c2.st = P.side;
-      if (grouped && !folds && (folds = true) && cudaMemsetAsync(P.dwg_region, 0, P.dwg_bytes, P.side) != cudaSuccess) { rc = LP_ERR_CUDA; break; }
+      if (grouped && !folds && cudaMemsetAsync(P.dwg_region, 0, P.dwg_bytes, P.side) != cudaSuccess) { rc = LP_ERR_CUDA; break; }
+      folds = folds || grouped;
       rc = h->dtype == LP_F32 ? run_op_t<float>(h, P, op, c2) : run_op_t<bf16>(h, P, op, c2);
     } else {
-      if (grouped && !folds && (folds = true) && cudaMemsetAsync(P.dwg_region, 0, P.dwg_bytes, c.st) != cudaSuccess) { rc = LP_ERR_CUDA; break; }
+      if (grouped && !folds && cudaMemsetAsync(P.dwg_region, 0, P.dwg_bytes, c.st) != cudaSuccess) { rc = LP_ERR_CUDA; break; }
+      folds = folds || grouped;
       TimelineScope ts(h, c.st, c.plan_id, (int)op.type, c.phase, h->tl.enabled ? op_bytes(h, P, op) : 0.0);
       rc = h->dtype == LP_F32 ? run_op_t<float>(h, P, op, c) : run_op_t<bf16>(h, P, op, c);
     }

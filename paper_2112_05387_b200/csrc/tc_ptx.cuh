@@ -36,29 +36,24 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 constexpr long long kWaitLimitCycles = 600000000LL;  // about 0.3 s at 1.9 GHz
 // (the polling is a function of its own: inlined at every wait it was a good part of the kernels' code, and code that is
 // not in the instruction cache is what a short kernel waits for)
-__device__ __noinline__ bool mbar_poll(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit_cycles) {
+__device__ __noinline__ bool mbar_poll(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit_cycles) {
+#pragma unroll 1
+  for (int i = 0; i < 16; ++i)
+    if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
   int polls = 0;
-  while (true) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
+  while (!mbar_try_wait(bar, parity)) {
     if ((++polls & 63) == 0) {
       if (*abort_flag) return false;
       if (clock64() - t0 > limit_cycles) return false;
     }
   }
+  return true;
 }
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                           long long limit_cycles = kWaitLimitCycles) {
   if (mbar_try_wait(bar, parity)) return true;
-  return mbar_poll(smem_u32(bar), parity, abort_flag, limit_cycles);
+  return mbar_poll(bar, parity, abort_flag, limit_cycles);
 }
 
 // True in exactly one lane of a converged warp.  The role loops stay warp-uniform (so that
@@ -141,6 +136,19 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
       ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// The same with the descriptors as register pairs: the loops that issue MMAs move operands by adding to the low words
+// (start address in units of 16 bytes) only.
+__device__ __forceinline__ void mma_bf16_lh(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                            uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 p, %6, 0;\n\t"
+      "mov.b64 a, {%1, %2};\n\t"
+      "mov.b64 b, {%3, %4};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 // Arrive on `bar` once all MMAs issued so far by this thread have completed.
