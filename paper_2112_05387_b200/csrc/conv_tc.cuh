@@ -300,7 +300,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int col0 = nt * p.n_tile_cols;
 #pragma unroll 1
         for (int c = 0; c < p.chunks && !failed; ++c) {
-          if (!mbar_wait(&tail->empty[sa], pha ^ 1, abort_flag)) { failed = true; break; }
+          if (!mbar_wait_hot(&tail->empty[sa], pha ^ 1, abort_flag)) { failed = true; break; }
           uint8_t* pa = smem + sa * p.a_stage_bytes;
           mbar_expect_tx(&tail->full[sa], cnt * p.tx_a);
           tma_load_4d(pa, &tmA, &tail->full[sa], c * p.KC, w0 + p.halo_dw0, n0, h0 + p.halo_dh0);
@@ -309,7 +309,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
           for (int ti0 = 0; ti0 < p.ntaps; ti0 += p.tps) {
             const int ti1 = min(ti0 + p.tps, p.ntaps);
-            if (!mbar_wait(&tail->empty_b[sb], phb ^ 1, abort_flag)) { failed = true; break; }
+            if (!mbar_wait_hot(&tail->empty_b[sb], phb ^ 1, abort_flag)) { failed = true; break; }
             mbar_expect_tx(&tail->full_b[sb], (ti1 - ti0) * p.tx_b);
             uint8_t* pb = b_ring + sb * p.b_stage_bytes;
 #pragma unroll 1
@@ -355,39 +355,64 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int c = 0; c < p.chunks && !failed; ++c) {
           const uint32_t a_lo = a_lo0 + sa * a_stage16;
           const int nkc = c + 1 == p.chunks ? p.nk_last : nk;   // slices of pure zero fill are not multiplied
+          if (!mbar_wait_hot(&tail->full[sa], pha, abort_flag)) { failed = true; break; }
+          if (active && nkc == 4 && p.tps == 1) {
+            // (stages of one tap in a loop of their own: as an inner loop of one trip they cost 160 cycles more each)
 #pragma unroll 1
-          for (int ti0 = 0; ti0 < p.ntaps; ti0 += p.tps) {
-            const int ti1 = min(ti0 + p.tps, p.ntaps);
-            if ((ti0 == 0 && !mbar_wait(&tail->full[sa], pha, abort_flag)) || !mbar_wait(&tail->full_b[sb], phb, abort_flag)) {
-              failed = true;
-              break;
+            for (int i = 0; i < p.ntaps; ++i) {
+              if (!mbar_wait_hot(&tail->full_b[sb], phb, abort_flag)) { failed = true; break; }
+              tc_fence_after();
+              const uint32_t at = a_lo + p.tap_off9[i], b_lo = b_lo0 + sb * b_stage16;
+              mma_bf16_lh(d, at, a_hi, b_lo, b_hi, p.idesc, accum);
+              accum = 1;
+              mma_bf16_lh(d, at + 2, a_hi, b_lo + 2, b_hi, p.idesc, 1u);
+              mma_bf16_lh(d, at + 4, a_hi, b_lo + 4, b_hi, p.idesc, 1u);
+              mma_bf16_lh(d, at + 6, a_hi, b_lo + 6, b_hi, p.idesc, 1u);
+              mma_commit(&tail->empty_b[sb]);
+              if (++sb == (uint32_t)p.nB) { sb = 0; phb ^= 1; }
             }
-            tc_fence_after();
-            if (active) {
-              uint32_t b_lo = b_lo0 + sb * b_stage16;
+          } else {
 #pragma unroll 1
-              for (int i = ti0; i < ti1; ++i) {
-                const uint32_t at = a_lo + p.tap_off9[i];
-                mma_bf16_lh(d, at, a_hi, b_lo, b_hi, p.idesc, accum);
-                accum = 1;
+            for (int ti0 = 0; ti0 < p.ntaps; ti0 += p.tps) {
+              const int ti1 = min(ti0 + p.tps, p.ntaps);
+              if (!mbar_wait_hot(&tail->full_b[sb], phb, abort_flag)) { failed = true; break; }
+              tc_fence_after();
+              if (active) {
+                uint32_t b_lo = b_lo0 + sb * b_stage16;
+                int i = ti0;
                 if (nkc == 4) {
-                  mma_bf16_lh(d, at + 2, a_hi, b_lo + 2, b_hi, p.idesc, 1u);
-                  mma_bf16_lh(d, at + 4, a_hi, b_lo + 4, b_hi, p.idesc, 1u);
-                  mma_bf16_lh(d, at + 6, a_hi, b_lo + 6, b_hi, p.idesc, 1u);
+#pragma unroll 1
+                  do {
+                    const uint32_t at = a_lo + p.tap_off9[i];
+                    mma_bf16_lh(d, at, a_hi, b_lo, b_hi, p.idesc, accum);
+                    accum = 1;
+                    mma_bf16_lh(d, at + 2, a_hi, b_lo + 2, b_hi, p.idesc, 1u);
+                    mma_bf16_lh(d, at + 4, a_hi, b_lo + 4, b_hi, p.idesc, 1u);
+                    mma_bf16_lh(d, at + 6, a_hi, b_lo + 6, b_hi, p.idesc, 1u);
+                    b_lo += b_tile16;
+                  } while (++i < ti1);
                 } else {
 #pragma unroll 1
-                  for (int j = 1; j < nkc; ++j) mma_bf16_lh(d, at + 2 * j, a_hi, b_lo + 2 * j, b_hi, p.idesc, 1u);
+                  do {
+                    const uint32_t at = a_lo + p.tap_off9[i];
+#pragma unroll 1
+                    for (int j = 0; j < nkc; ++j) {
+                      mma_bf16_lh(d, at + 2 * j, a_hi, b_lo + 2 * j, b_hi, p.idesc, accum);
+                      accum = 1;
+                    }
+                    b_lo += b_tile16;
+                  } while (++i < ti1);
                 }
-                b_lo += b_tile16;
+                mma_commit(&tail->empty_b[sb]);
+              } else {
+                mbar_arrive(&tail->empty_b[sb]);
               }
-              mma_commit(&tail->empty_b[sb]);
-              if (ti1 == p.ntaps) mma_commit(&tail->empty[sa]);
-            } else {
-              mbar_arrive(&tail->empty_b[sb]);
-              if (ti1 == p.ntaps) mbar_arrive(&tail->empty[sa]);
+              if (++sb == (uint32_t)p.nB) { sb = 0; phb ^= 1; }
             }
-            if (++sb == (uint32_t)p.nB) { sb = 0; phb ^= 1; }
           }
+          if (failed) break;
+          if (active) mma_commit(&tail->empty[sa]);
+          else mbar_arrive(&tail->empty[sa]);
           if (++sa == (uint32_t)p.nA) { sa = 0; pha ^= 1; }
         }
         if (failed) break;
@@ -421,7 +446,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
         for (int k0 = 0; k0 < kiters; k0 += p.ips) {
           const int n_items = min(p.ips, kiters - k0);
-          if (!mbar_wait(&tail->empty[s], ph ^ 1, abort_flag)) { failed = true; break; }
+          if (!mbar_wait_hot(&tail->empty[s], ph ^ 1, abort_flag)) { failed = true; break; }
           uint8_t* si = smem + s * p.stage_bytes;
           mbar_expect_tx(&tail->full[s], n_items * tx);
 #pragma unroll 1
@@ -467,30 +492,38 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         const uint32_t d = tmem_base + mine * p.acc_stride;
         uint32_t accum = 0;
+        const bool full4 = nk == 4 && p.nk_last == 4;
         int kc = 0;                        // K chunk of the item
 #pragma unroll 1
         for (int k0 = 0; k0 < kiters; k0 += p.ips) {
           const int n_items = min(p.ips, kiters - k0);
-          if (!mbar_wait(&tail->full[s], ph, abort_flag)) { failed = true; break; }
+          if (!mbar_wait_hot(&tail->full[s], ph, abort_flag)) { failed = true; break; }
           tc_fence_after();
           if (active) {
-            uint32_t item = a_lo0 + s * stage16;
+            uint32_t at = a_lo0 + s * stage16 + a_me16, bt = a_lo0 + s * stage16 + b_off16;
+            int i = 0;
+            if (full4) {                   // +32 bytes (one K = 16 slice) per step, in 16-byte units
 #pragma unroll 1
-            for (int i = 0; i < n_items; ++i) {
-              const int nkc = ++kc == p.chunks ? p.nk_last : nk;
-              if (kc == p.chunks) kc = 0;
-              const uint32_t at = item + a_me16, bt = item + b_off16;
-              mma_bf16_lh(d, at, hi, bt, hi, p.idesc, accum);
-              accum = 1;
-              if (nkc == 4) {              // +32 bytes (one K = 16 slice) per step, in 16-byte units
+              do {
+                mma_bf16_lh(d, at, hi, bt, hi, p.idesc, accum);
+                accum = 1;
                 mma_bf16_lh(d, at + 2, hi, bt + 2, hi, p.idesc, 1u);
                 mma_bf16_lh(d, at + 4, hi, bt + 4, hi, p.idesc, 1u);
                 mma_bf16_lh(d, at + 6, hi, bt + 6, hi, p.idesc, 1u);
-              } else {
+                at += item16; bt += item16;
+              } while (++i < n_items);
+            } else {
 #pragma unroll 1
-                for (int j = 1; j < nkc; ++j) mma_bf16_lh(d, at + 2 * j, hi, bt + 2 * j, hi, p.idesc, 1u);
-              }
-              item += item16;
+              do {
+                const int nkc = ++kc == p.chunks ? p.nk_last : nk;
+                if (kc == p.chunks) kc = 0;
+#pragma unroll 1
+                for (int j = 0; j < nkc; ++j) {
+                  mma_bf16_lh(d, at + 2 * j, hi, bt + 2 * j, hi, p.idesc, accum);
+                  accum = 1;
+                }
+                at += item16; bt += item16;
+              } while (++i < n_items);
             }
             mma_commit(&tail->empty[s]);
           } else {

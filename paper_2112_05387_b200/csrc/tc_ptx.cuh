@@ -56,6 +56,23 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return mbar_poll(bar, parity, abort_flag, limit_cycles);
 }
 
+// The same for one thread in a loop that issues MMAs: no call, because keeping the loop's values across one costs some
+// fifty cycles a trip.
+__device__ __forceinline__ bool mbar_wait_hot(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  uint32_t polls = 0;
+  long long t0 = 0;
+#pragma unroll 1
+  while (!mbar_try_wait(bar, parity)) {
+    if ((++polls & 1023) == 0) {
+      const long long t = clock64();
+      if (*abort_flag) return false;
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > kWaitLimitCycles) return false;
+    }
+  }
+  return true;
+}
+
 // True in exactly one lane of a converged warp.  The role loops stay warp-uniform (so that
 // addresses and descriptors live in uniform registers) and only the TMA / MMA issue is elected.
 __device__ __forceinline__ bool elect_one() {
