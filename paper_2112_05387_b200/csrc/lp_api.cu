@@ -1544,14 +1544,14 @@ struct Planner {
     if (!P.host_fold.empty()) P.dev_fold = (tc::FoldEntry*)A.alloc(P.host_fold.size() * sizeof(tc::FoldEntry));
     if (!P.ps.host_pack.empty()) {
       P.ps.dev_pack = (PackEntry*)A.alloc(P.ps.host_pack.size() * sizeof(PackEntry));
-      // complement of the packed entries in [0, n), cut into ranges of at most 16384 elements
+      // complement of the packed entries in [0, n), cut into ranges of at most 4096 elements
       std::vector<std::pair<long long, long long>> packed;
       for (const PackEntry& e : P.ps.host_pack)
         packed.push_back({(long long)(e.w - P.ps.p), (long long)(e.w - P.ps.p) + (long long)e.cout * e.taps * e.cin});
       std::sort(packed.begin(), packed.end());
       long long pos = 0;
       auto add = [&](long long a, long long b) {
-        for (long long q = a; q < b; q += 16384) P.ps.host_ranges.push_back({q, (int)std::min<long long>(16384, b - q)});
+        for (long long q = a; q < b; q += 4096) P.ps.host_ranges.push_back({q, (int)std::min<long long>(4096, b - q)});
       };
       for (const auto& pr : packed) { add(pos, pr.first); pos = pr.second; }
       add(pos, (long long)P.ps.n);
@@ -1756,15 +1756,17 @@ struct Planner {
       stem_y = emit_conv(P, F, x, stem_conv, nullptr, post ? stem_bn : first_bn1);
       cur = stem_y;
       if (post) {
-        stem_a = emit_bn_apply(F, stem_y, stem_bn, nullptr, -1, nullptr, 1);
-        cur = stem_a;
         if (net.stem_pool) {
+          stem_a = stem_y;   // (relu(bn(stem_y)) is not stored: the pool normalises on the way in)
           stem_pool_out = new_tensor(d.N, net.body_h, net.body_w, d.stem_channels);
           pool_arg = (uint8_t*)A.alloc((size_t)stem_pool_out.elems());
           Op op;
-          op.type = OP_MAXPOOL_FWD; op.in = stem_a; op.out = stem_pool_out; op.arg = pool_arg;
+          op.type = OP_MAXPOOL_FWD; op.in = stem_y; op.bn = stem_bn; op.out = stem_pool_out; op.arg = pool_arg;
           F.push_back(op);
           cur = stem_pool_out;
+        } else {
+          stem_a = emit_bn_apply(F, stem_y, stem_bn, nullptr, -1, nullptr, 1);
+          cur = stem_a;
         }
       }
     } else if (!post) {
@@ -2166,18 +2168,21 @@ static int run_op_t(lp_handle* h, Plan& P, const Op& op, const RunCtx& c) {
       break;
     }
     case OP_MAXPOOL_FWD: {
-      if (op.out.c % V) return LP_ERR_UNSUPPORTED;
+      const BnDef& b = P.bns[op.bn];
+      const int threads = threads_for_channels(b.C, dtype);
+      if (!threads || op.out.c % V) return LP_ERR_UNSUPPORTED;
       const long long total = op.out.elems() / V;
-      maxpool_fwd_kernel<T><<<grid_for(total, 256, cur_dev().sm_count, 16), 256, 0, st>>>(
-          (const T*)resolve(op.in, c), (T*)resolve(op.out, c), op.arg, op.in.n, op.in.h, op.in.w, op.in.c, op.out.h,
-          op.out.w);
+      LP_CUDA_OK(launch_pdl(bn_maxpool_fwd_kernel<T>, dim3(grid_for(total, threads, cur_dev().sm_count, 8)), dim3(threads), 0, st,
+                            (const T*)resolve(op.in, c), bn_args(b, eps), (T*)resolve(op.out, c), op.arg, op.in.n, op.in.h,
+                            op.in.w, op.in.c, op.out.h, op.out.w));
       h->launches++;
       break;
     }
     case OP_MAXPOOL_BWD: {
-      if (op.out.c % V) return LP_ERR_UNSUPPORTED;
-      const long long total = op.out.elems() / V;
-      maxpool_bwd_kernel<T><<<grid_for(total, 256, cur_dev().sm_count, 16), 256, 0, st>>>(
+      const int threads = threads_for_channels(op.out.c, dtype);
+      if (!threads || op.out.c % V) return LP_ERR_UNSUPPORTED;
+      const long long total = op.in.elems() / V;
+      maxpool_bwd_kernel<T><<<grid_for(total, threads, cur_dev().sm_count, 8), threads, 0, st>>>(
           (const T*)resolve(op.in, c), op.arg, (T*)resolve(op.out, c), op.out.n, op.out.h, op.out.w, op.out.c, op.in.h,
           op.in.w);
       h->launches++;
@@ -2186,7 +2191,7 @@ static int run_op_t(lp_handle* h, Plan& P, const Op& op, const RunCtx& c) {
     case OP_HEAD_FWD: {
       HeadDef& hd = P.head;
       const int32_t* labels = c.labels ? c.labels : h->zero_labels;  // logits-only runs use label 0
-      if (hd.classes <= 128 && (size_t)(hd.C + hd.classes) * 4 <= 40 * 1024) {
+      if (hd.classes <= 128 && (size_t)(hd.C + hd.classes) * 4 <= 36 * 1024) {
         head_fused_kernel<T><<<hd.N, 256, (size_t)(hd.C + hd.classes) * 4, st>>>(
             (const T*)resolve(op.in, c), hd.W, hd.b, labels, hd.pooled, hd.logits, hd.dlogits, P.loss_acc, hd.N, hd.HW, hd.C,
             hd.classes);
@@ -2197,9 +2202,9 @@ static int run_op_t(lp_handle* h, Plan& P, const Op& op, const RunCtx& c) {
         }
         break;
       }
-      avgpool_kernel<T><<<hd.N, 256, 0, st>>>((const T*)resolve(op.in, c), hd.pooled, hd.HW, hd.C);
+      avgpool_kernel<T><<<dim3(hd.N, (hd.C / V + 31) / 32), 256, 0, st>>>((const T*)resolve(op.in, c), hd.pooled, hd.HW, hd.C);
       h->launches++;
-      head_logits_kernel<<<dim3((hd.classes + 3) / 4, (hd.N + 7) / 8), 128, 0, st>>>(hd.pooled, hd.W, hd.b, hd.logits, hd.N,
+      head_logits_kernel<<<dim3((hd.classes + 15) / 16, (hd.N + 7) / 8), 128, 0, st>>>(hd.pooled, hd.W, hd.b, hd.logits, hd.N,
                                                                                      hd.C, hd.classes);
       head_fwd_kernel<<<hd.N, 128, (size_t)(hd.classes + 32) * 4, st>>>(labels, hd.logits, hd.dlogits, P.loss_acc, hd.N,
                                                                         hd.classes);
@@ -2212,11 +2217,11 @@ static int run_op_t(lp_handle* h, Plan& P, const Op& op, const RunCtx& c) {
     }
     case OP_HEAD_BWD: {
       HeadDef& hd = P.head;
-      const long long total = (long long)hd.classes * hd.C;
-      head_bwd_w_kernel<<<grid_for(total, 128, cur_dev().sm_count, 16), 128, 0, st>>>(hd.dlogits, hd.pooled, hd.dW, hd.db,
-                                                                                  hd.N, hd.C, hd.classes);
-      head_bwd_x_kernel<T><<<dim3(hd.N, (hd.C + 255) / 256), 256, 0, st>>>(hd.dlogits, hd.W, (T*)resolve(op.out, c), hd.HW,
-                                                                           hd.C, hd.classes);
+      head_bwd_x_kernel<T><<<dim3((hd.C + 31) / 32, (hd.N + 7) / 8), 256,
+                             (size_t)std::max(std::min(hd.classes, kHeadClassChunk) * 8, 8 * 8 * 32) * 4, st>>>(
+          hd.dlogits, hd.W, (T*)resolve(op.out, c), hd.N, hd.HW, hd.C, hd.classes);
+      const long long items = (long long)((hd.classes + 3) / 4) * (hd.C / 4);
+      head_bwd_w_kernel<<<(unsigned)((items + 31) / 32), 256, 0, st>>>(hd.dlogits, hd.pooled, hd.dW, hd.db, hd.N, hd.C, hd.classes);
       h->launches += 2;
       break;
     }
