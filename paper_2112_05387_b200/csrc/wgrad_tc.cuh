@@ -192,39 +192,55 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     // Two MMA-issuing warps (one thread cannot keep the tensor pipe full): warp 1 owns the first row tile of
     // the CTA, warp 7 the second one of a pair.  Both wait for every stage and both arrive on its "empty"
     // barrier: with a commit after their MMAs, or (warp 7 with a single row tile) with a plain arrive.
+    // One thread runs the loop (see the MMA issuers of conv_tc_kernel).
     const bool active = warp == 1 || cnt == 2;
-    const uint32_t acc_col = warp == 1 ? 0u : 256u;
-    uint32_t s = 0, ph = 0;
-    const uint32_t smem_base = smem_u32(smem);
-    const int ksteps = p.rows_pad >> 4;
-    const uint32_t a_kstep = (uint32_t)(16 * p.sca * 2) >> 4, b_kstep = (uint32_t)(16 * p.scb * 2) >> 4;
+    if (elect_one()) {
+      const uint32_t d = tmem_base + (warp == 1 ? 0u : 256u);
+      uint32_t s = 0, ph = 0, accum = 0;
+      const uint32_t base16 = smem_u32(smem) >> 4, stage16 = p.stage_bytes >> 4;
+      const uint32_t a_hi = (uint32_t)(p.adesc_hi >> 32), b_hi = (uint32_t)(p.bdesc_hi >> 32);
+      const uint32_t a_lo0 = (uint32_t)p.adesc_hi + base16 + (warp == 1 ? 0u : (uint32_t)(p.rpt * p.a_sub_bytes) >> 4);
+      const uint32_t b_lo0 = (uint32_t)p.bdesc_hi + base16 + (p.a_region >> 4);
+      const int ksteps = p.rows_pad >> 4;
+      const uint32_t ak = (uint32_t)(16 * p.sca * 2) >> 4, bk = (uint32_t)(16 * p.scb * 2) >> 4;
 #pragma unroll 1
-    for (int it = 0; it < n_iter; ++it) {
-      if (!mbar_wait_warp(&tail->full[s], ph, abort_flag)) { failed = true; break; }
-      tc_fence_after();
-      const uint32_t a_addr = smem_base + s * p.stage_bytes;
-      const uint64_t bd = smem_desc(p.bdesc_hi, a_addr + p.a_region);
-      const uint64_t ad = smem_desc(p.adesc_hi, a_addr + (warp == 1 ? 0u : (uint32_t)(p.rpt * p.a_sub_bytes)));
-      if (elect_one()) {
+      for (int it = 0; it < n_iter; ++it) {
+        if (!mbar_wait_hot(&tail->full[s], ph, abort_flag)) { failed = true; break; }
+        tc_fence_after();
         if (active) {
+          uint32_t at = a_lo0 + s * stage16, bt = b_lo0 + s * stage16;
+          int k = ksteps;
+          if ((k & 3) == 0) {
 #pragma unroll 1
-          for (int j = 0; j < ksteps; ++j)
-            mma_bf16(tmem_base + acc_col, ad + (uint64_t)(j * a_kstep), bd + (uint64_t)(j * b_kstep), p.idesc, (it | j) ? 1u : 0u);
+            do {
+              mma_bf16_lh(d, at, a_hi, bt, b_hi, p.idesc, accum);
+              accum = 1;
+              mma_bf16_lh(d, at + ak, a_hi, bt + bk, b_hi, p.idesc, 1u);
+              mma_bf16_lh(d, at + 2 * ak, a_hi, bt + 2 * bk, b_hi, p.idesc, 1u);
+              mma_bf16_lh(d, at + 3 * ak, a_hi, bt + 3 * bk, b_hi, p.idesc, 1u);
+              at += 4 * ak; bt += 4 * bk;
+            } while ((k -= 4) > 0);
+          } else {
+#pragma unroll 1
+            do {
+              mma_bf16_lh(d, at, a_hi, bt, b_hi, p.idesc, accum);
+              accum = 1;
+              at += ak; bt += bk;
+            } while (--k > 0);
+          }
           mma_commit(&tail->empty[s]);
         } else {
           mbar_arrive(&tail->empty[s]);
         }
+        if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
       }
-      __syncwarp();
-      if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
-    }
-    if (!failed && n_iter > 0) {
-      if (elect_one()) {
+      if (!failed && n_iter > 0) {
         if (active) mma_commit(&tail->acc_full);
         else mbar_arrive(&tail->acc_full);
       }
-      __syncwarp();
     }
+    __syncwarp();
+    failed = __any_sync(0xffffffffu, failed);
   } else {
     const int q = warp & 3;
     const int row = q * 32 + lane;
@@ -412,39 +428,48 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     // it, so one thread cannot keep the pipe full.  Warp 1 owns accumulators 0 and 1, warp 7 accumulator 2;
     // both wait for every stage and both commit on its "empty" barrier.
     const bool first = warp == 1;
-    uint32_t s = 0, ph = 0;
-    const uint32_t smem_base = smem_u32(smem);
-    const uint32_t a_kstep = p.a_kstep_bytes >> 4, b_kstep = (uint32_t)(16 * p.scb * 2) >> 4;
-    const int ksteps = p.rows >> 4;   // K = 16 pixels per MMA
+    if (elect_one()) {
+      uint32_t s = 0, ph = 0, accum = 0;
+      const uint32_t base16 = smem_u32(smem) >> 4, stage16 = p.stage_bytes >> 4;
+      const uint32_t ak = p.a_kstep_bytes >> 4, bk = (uint32_t)(16 * p.scb * 2) >> 4;
+      const int i0 = first ? 0 : 2;
+      const uint32_t b_lo0 = (uint32_t)p.bdesc_hi + base16 + (p.a_region >> 4), b_hi = (uint32_t)(p.bdesc_hi >> 32);
+      const uint32_t a_lo0 = (uint32_t)p.adesc_hi3[i0] + base16 + (p.a_start3[i0] >> 4), a_hi0 = (uint32_t)(p.adesc_hi3[i0] >> 32);
+      const uint32_t a_lo1 = (uint32_t)p.adesc_hi3[1] + base16 + (p.a_start3[1] >> 4), a_hi1 = (uint32_t)(p.adesc_hi3[1] >> 32);
+      const uint32_t d0 = tmem_base + i0 * p.acc_stride, d1 = tmem_base + p.acc_stride;
+      const int ksteps = p.rows >> 4;   // K = 16 pixels per MMA, an even number of steps
 #pragma unroll 1
-    for (int it = 0; it < n_iter; ++it) {
-      if (!mbar_wait_warp(&tail->full[s], ph, abort_flag)) { failed = true; break; }
-      tc_fence_after();
-      const uint32_t a_addr = smem_base + s * p.stage_bytes;
-      const uint64_t bd = smem_desc(p.bdesc_hi, a_addr + p.a_region);
-      const uint64_t ad0 = smem_desc(p.adesc_hi3[0], a_addr + p.a_start3[0]);
-      const uint64_t ad1 = smem_desc(p.adesc_hi3[1], a_addr + p.a_start3[1]);
-      const uint64_t ad2 = smem_desc(p.adesc_hi3[2], a_addr + p.a_start3[2]);
-      if (elect_one()) {
+      for (int it = 0; it < n_iter; ++it) {
+        if (!mbar_wait_hot(&tail->full[s], ph, abort_flag)) { failed = true; break; }
+        tc_fence_after();
+        uint32_t a0 = a_lo0 + s * stage16, a1 = a_lo1 + s * stage16, bt = b_lo0 + s * stage16;
+        int k = ksteps;
+        if (first) {
 #pragma unroll 1
-        for (int j = 0; j < ksteps; ++j) {
-          const uint32_t acc = (it | j) ? 1u : 0u;
-          if (first) {
-            mma_bf16(tmem_base, ad0 + (uint64_t)(j * a_kstep), bd + (uint64_t)(j * b_kstep), p.idesc, acc);
-            mma_bf16(tmem_base + p.acc_stride, ad1 + (uint64_t)(j * a_kstep), bd + (uint64_t)(j * b_kstep), p.idesc, acc);
-          } else {
-            mma_bf16(tmem_base + 2 * p.acc_stride, ad2 + (uint64_t)(j * a_kstep), bd + (uint64_t)(j * b_kstep), p.idesc, acc);
-          }
+          do {
+            mma_bf16_lh(d0, a0, a_hi0, bt, b_hi, p.idesc, accum);
+            mma_bf16_lh(d1, a1, a_hi1, bt, b_hi, p.idesc, accum);
+            accum = 1;
+            mma_bf16_lh(d0, a0 + ak, a_hi0, bt + bk, b_hi, p.idesc, 1u);
+            mma_bf16_lh(d1, a1 + ak, a_hi1, bt + bk, b_hi, p.idesc, 1u);
+            a0 += 2 * ak; a1 += 2 * ak; bt += 2 * bk;
+          } while ((k -= 2) > 0);
+        } else {
+#pragma unroll 1
+          do {
+            mma_bf16_lh(d0, a0, a_hi0, bt, b_hi, p.idesc, accum);
+            accum = 1;
+            mma_bf16_lh(d0, a0 + ak, a_hi0, bt + bk, b_hi, p.idesc, 1u);
+            a0 += 2 * ak; bt += 2 * bk;
+          } while ((k -= 2) > 0);
         }
         mma_commit(&tail->empty[s]);
+        if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
       }
-      __syncwarp();
-      if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
+      if (!failed && n_iter > 0) mma_commit(&tail->acc_full);
     }
-    if (!failed && n_iter > 0) {
-      if (elect_one()) mma_commit(&tail->acc_full);
-      __syncwarp();
-    }
+    __syncwarp();
+    failed = __any_sync(0xffffffffu, failed);
   } else {
     const int q = warp & 3;
     const int row = q * 32 + lane;
