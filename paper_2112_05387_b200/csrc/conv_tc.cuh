@@ -46,9 +46,6 @@ constexpr int kMaxStages = 12;
 constexpr int kTmemCols = 512;
 constexpr int kMaxSlots = 4;     // accumulator slots in tensor memory
 
-#ifndef LP_EPI_WARPS
-#define LP_EPI_WARPS 4
-#endif
 #ifndef LP_CONV_MIN_BLOCKS
 #define LP_CONV_MIN_BLOCKS 1
 #endif
@@ -166,15 +163,19 @@ struct TcSmemTail {
   int abort_flag;
   int epi_ok[2];                   // outcome of the epilogue's wait, alternating by accumulator (see the epilogue)
 };
+constexpr int kMaxEpiWarps = 8;
 // Scratch of the direct (register -> global) epilogue's statistics, placed right after the tail.
 struct TcStatScratch {
-  float ssum[LP_EPI_WARPS][256];   // per epilogue warp: plain read-modify-write, no shared-memory atomics
-  float ssq[LP_EPI_WARPS][256];
-  uint32_t tr[LP_EPI_WARPS][16 * 33];   // per epilogue warp: transposition scratch of the statistics
+  float ssum[4][256];              // per row quarter (the warps of a quarter own different columns): plain read-modify-write,
+  float ssq[4][256];               // no shared-memory atomics
+  uint32_t tr[kMaxEpiWarps][16 * 33];   // per epilogue warp: transposition scratch of the statistics (as many as there are)
 };
-// Additional scratch of the fused batch-norm-backward sums, placed right after TcStatScratch.
+__host__ __device__ constexpr size_t stat_scratch_bytes(int epi_warps) {
+  return sizeof(TcStatScratch) - (size_t)(kMaxEpiWarps - epi_warps) * 16 * 33 * 4;
+}
+// Additional scratch of the fused batch-norm-backward sums, placed right after that of the statistics.
 struct TcBnBwdScratch {
-  uint32_t tr2[LP_EPI_WARPS][16 * 33];  // transposition scratch of the normalised tensor's tile
+  uint32_t tr2[4][16 * 33];  // transposition scratch of the normalised tensor's tile
   float4 consts[256];                   // per channel of the current channel tile: scale, shift, mean, rstd
 };
 constexpr uint32_t kTailBytes = (uint32_t)((sizeof(TcSmemTail) + 127) / 128 * 128);
@@ -201,10 +202,8 @@ __device__ __forceinline__ void tile_first_pixel(const ConvTcParams& p, int m, i
   w0 = r1 * p.BW; h0 = r2 * p.BH; n0 = q2 * p.BNI;
 }
 
-constexpr int kEpiThreads = 32 * LP_EPI_WARPS;
-constexpr int kConvThreads = 96 + kEpiThreads;
 constexpr int kFirstEpiWarp = 3;
-constexpr int kEpiGroups = LP_EPI_WARPS / 4;
+constexpr int conv_threads(int epi_warps) { return 96 + 32 * epi_warps; }
 
 // kAddend: a residual operand is added in the epilogue (its loads run one channel group ahead);
 // kLoss: the epilogue also takes the local loss of an interior module (implies kAddend);
@@ -220,18 +219,21 @@ constexpr int kEpiGroups = LP_EPI_WARPS / 4;
 //   64 columns) are launched as the two-per-SM instantiation -- registers capped accordingly (the epilogue
 //   drains 64 accumulator columns per pass instead of 160), tensor memory and shared memory sized to need --
 //   so that the kernels of several modules, each bound by latency rather than by any unit, share the SMs.
-template <bool kLoss, bool kAddend, bool kStaged, bool kBnBwd = false, int kMinBlocks = LP_CONV_MIN_BLOCKS>
-__global__ void __launch_bounds__(kConvThreads, kMinBlocks)
+// kEpiWarps: 4, or 8 where a tile's epilogue takes longer than its MMAs (few input channels, many output channels): two
+//   warps per row quarter, which take the 32-column groups of a tile in turn.
+template <bool kLoss, bool kAddend, bool kStaged, bool kBnBwd = false, int kMinBlocks = LP_CONV_MIN_BLOCKS, int kEpiWarps = 4>
+__global__ void __launch_bounds__(conv_threads(kEpiWarps), kMinBlocks)
 conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ CUtensorMap tmAdd,
                const __grid_constant__ ConvTcParams p) {
   static_assert(!(kStaged && kLoss), "the fused local loss uses the direct epilogue");
   static_assert(!(kBnBwd && (kStaged || kLoss)), "the fused batch-norm sums use the plain direct epilogue");
+  constexpr int kEpiThreads = 32 * kEpiWarps, kEpiGroups = kEpiWarps / 4;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   TcSmemTail* tail = reinterpret_cast<TcSmemTail*>(smem + p.tail_offset);
   TcStatScratch* scratch = reinterpret_cast<TcStatScratch*>(smem + p.tail_offset + kTailBytes);
-  TcBnBwdScratch* bscratch = reinterpret_cast<TcBnBwdScratch*>(smem + p.tail_offset + kTailBytes + sizeof(TcStatScratch));
+  TcBnBwdScratch* bscratch = reinterpret_cast<TcBnBwdScratch*>(smem + p.tail_offset + kTailBytes + stat_scratch_bytes(kEpiWarps));
   volatile int* abort_flag = &tail->abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -265,7 +267,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   }
   if (!kStaged && (p.stats || kBnBwd)) {   // (without statistics the scratch is not part of the allocation)
-    for (int i = threadIdx.x; i < LP_EPI_WARPS * 256; i += blockDim.x) {
+    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) {
       (&scratch->ssum[0][0])[i] = 0.f;
       (&scratch->ssq[0][0])[i] = 0.f;
     }
@@ -545,8 +547,9 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if constexpr (kStaged) {
     // ------------------------------- epilogue, staged through shared memory -------------
     // Requires (checked by the launcher): output grid = logical grid (os = 1), channel tile a multiple
-    // of 32, kEpiThreads = 128.  Thread `row` owns tile row `row` (one pixel) as in the direct epilogue.
+    // of 32.  Thread `row` owns tile row `row` (one pixel) as in the direct epilogue.
     const int q = warp & 3;
+    const int grp = (warp - kFirstEpiWarp) >> 2;
     const int row = q * 32 + lane;
     const int et = threadIdx.x - 32 * kFirstEpiWarp;
     const int rows_used = p.BW * p.BH * p.BNI;
@@ -562,7 +565,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint32_t slot = 0, slot_phase = 0, add_phase = 0;
     int epi_turn = 0;
     // per-channel statistics: thread (group sg, word sw) owns two channels and sums them over the rows
-    const int sg = et >> 4, sw = et & 15;
+    const int sg = (et & 127) >> 4, sw = et & 15;
     const bool stat_owner = p.stats != nullptr && sg < ngroups;
     float st_s0 = 0.f, st_s1 = 0.f, st_q0 = 0.f, st_q1 = 0.f;
     auto tile_origin = [&](int tile, int& col0, int& c1, int& c2, int& c3) {
@@ -629,14 +632,19 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (!wait_ok) { failed = true; break; }
         tc_fence_after();
         const uint32_t taddr = tmem_base + buf * p.acc_stride + ((uint32_t)(q * 32) << 16);
+        if (kEpiGroups > 1 && grp >= ngroups) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&tail->tmem_empty[buf]);
+        }
         // one 32-column group at a time, not unrolled: see the direct epilogue
 #pragma unroll 1
-        for (int g = 0; g < ngroups; ++g) {
+        for (int g = grp; g < ngroups; g += kEpiGroups) {
           uint32_t raw[32];
           tmem_ld32_issue(taddr + g * 32, raw);
           tmem_ld_wait();
           tmem_ld_fence(raw);
-          if (g + 1 == ngroups) {            // the accumulator is in registers: hand the slot back
+          if (g + kEpiGroups >= ngroups) {   // the accumulator is in registers: hand the slot back
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tail->tmem_empty[buf]);
@@ -675,7 +683,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           const uint8_t* gbase = stg + sg * kStageGroupBytes;
           const int flip = sg & 1;
 #pragma unroll 4
-          for (int r = 0; r < rows_used; ++r) {
+          for (int r = (et >> 7) * (rows_used >> 1); r < ((et >> 7) + 1 == kEpiGroups ? rows_used : rows_used >> 1); ++r) {
             int rr = r ^ flip;
             if (rr >= rows_used) rr = r;
             const uint32_t w2 = *reinterpret_cast<const uint32_t*>(
@@ -821,6 +829,11 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             a[u] = (g < ngroups && u < nv && valid && col0 + c_in_tile + 8 * u < p.Cout)
                        ? ld_raw(p.addend + obase + col0 + c_in_tile + 8 * u) : make_uint4(0u, 0u, 0u, 0u);
         };
+        if (kEpiGroups > 1 && grp >= ngroups) {   // no column group for this warp: nothing to read from the accumulator
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&tail->tmem_empty[buf]);
+        }
         uint4 add_cur[4], add_next[4];
         if constexpr (kAddend) load_addend(grp, add_cur);
 #pragma unroll 1
@@ -964,7 +977,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               s1 += __shfl_xor_sync(0xffffffffu, s1, 16);
               q0 += __shfl_xor_sync(0xffffffffu, q0, 16);
               q1 += __shfl_xor_sync(0xffffffffu, q1, 16);
-              float* dst = hh ? scratch->ssq[warp - kFirstEpiWarp] : scratch->ssum[warp - kFirstEpiWarp];
+              float* dst = hh ? scratch->ssq[q] : scratch->ssum[q];
               dst[c_in_tile + 2 * jc] += hh ? q0 : s0;
               dst[c_in_tile + 2 * jc + 1] += hh ? q1 : s1;
             }
@@ -980,7 +993,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
           for (int c = et; c < p.n_tile_cols; c += kEpiThreads) {
             float a_s = 0.f, a_q = 0.f;
-            for (int wi = 0; wi < kEpiThreads / 32; ++wi) {
+#pragma unroll
+            for (int wi = 0; wi < 4; ++wi) {
               a_s += scratch->ssum[wi][c];
               a_q += scratch->ssq[wi][c];
               scratch->ssum[wi][c] = 0.f;

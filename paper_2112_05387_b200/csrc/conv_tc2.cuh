@@ -101,8 +101,11 @@ __device__ __forceinline__ Unit2 unit2_at(int t, int t_end, int m_tiles, uint32_
   return u;
 }
 
+constexpr int kEpiThreads = 128;                   // four epilogue warps, one per quarter of the accumulator's rows
+constexpr int kConv2Threads = 96 + kEpiThreads;
+
 template <bool kAddend>
-__global__ void __launch_bounds__(kConvThreads, 1)
+__global__ void __launch_bounds__(kConv2Threads, 1)
 conv_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ ConvTcParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -138,7 +141,7 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     prefetch_tmap(&tmB);
   }
   if (p.stats) {   // (without statistics the scratch is not part of the allocation)
-    for (int i = threadIdx.x; i < LP_EPI_WARPS * 256; i += blockDim.x) {
+    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) {
       (&scratch->ssum[0][0])[i] = 0.f;
       (&scratch->ssq[0][0])[i] = 0.f;
     }

@@ -537,7 +537,7 @@ static int launch_conv_tc2(lp_handle* h, const TcGemmSpec& s, int* dev_err, cuda
   const int row_bytes = 128;
   const int n_half = p.n_tile_cols / 2;
   const uint32_t b_half = (uint32_t)align_up((size_t)n_half * row_bytes, 1024);
-  const size_t tail = tc::kTailBytes + (s.stats ? sizeof(tc::TcStatScratch) : 0) + 1024;
+  const size_t tail = tc::kTailBytes + (s.stats ? tc::stat_scratch_bytes(4) : 0) + 1024;
   p.tx_b = (uint32_t)(n_half * row_bytes);
   p.acc_stride = (p.n_tile_cols + 31) / 32 * 32;
   p.nslots = std::min(tc::kMaxSlots, tc::kTmemCols / p.acc_stride);
@@ -584,7 +584,7 @@ static int launch_conv_tc2(lp_handle* h, const TcGemmSpec& s, int* dev_err, cuda
     // how many CTA pairs fit the device at once (persistent kernel: never more pairs than that)
     cudaLaunchConfig_t q = {};
     q.gridDim = dim3(2 * D.sm_count);
-    q.blockDim = dim3(tc::kConvThreads);
+    q.blockDim = dim3(tc::kConv2Threads);
     q.dynamicSmemBytes = kTcMaxSmem;
     cudaLaunchAttribute qa[1];
     qa[0].id = cudaLaunchAttributeClusterDimension;
@@ -609,7 +609,7 @@ static int launch_conv_tc2(lp_handle* h, const TcGemmSpec& s, int* dev_err, cuda
     pairs = (p.total_tiles + per - 1) / per;
   }
   cudaError_t le;
-  const dim3 g3(2 * pairs), b3(tc::kConvThreads);
+  const dim3 g3(2 * pairs), b3(tc::kConv2Threads);
   if (s.addend) le = launch_pdl_pair(tc::conv_tc2_kernel<true>, g3, b3, smem, st, tmA, tmB, p);
   else le = launch_pdl_pair(tc::conv_tc2_kernel<false>, g3, b3, smem, st, tmA, tmB, p);
   LP_CUDA_OK(le);
@@ -670,7 +670,7 @@ static int launch_conv_tc(lp_handle* h, const TcGemmSpec& s, int* dev_err, cudaS
   // Staged epilogue (output tile through shared memory, TMA stores, TMA-loaded residual): where the output
   // grid is the logical grid, the channel tile is a multiple of 32 and the tensors start on 16-byte boundaries.
   const bool staged0 = !bnbwd && (s.epilogue == 2 || (s.epilogue == 0 && s.addend != nullptr)) && !s.x_next && s.os == 1 && s.oo_h == 0 && s.oo_w == 0 &&
-                      p.n_tile_cols % 32 == 0 && s.out_C % 8 == 0 && tc::kEpiThreads == 128 &&
+                      p.n_tile_cols % 32 == 0 && s.out_C % 8 == 0 &&
                       (reinterpret_cast<uintptr_t>(s.out) & 15) == 0 &&
                       (!s.addend || (reinterpret_cast<uintptr_t>(s.addend) & 15) == 0);
   // Layers of few channels, while the modules are enqueued side by side: the two-per-SM instantiation with
@@ -679,10 +679,16 @@ static int launch_conv_tc(lp_handle* h, const TcGemmSpec& s, int* dev_err, cudaS
   const bool thin = allow_thin && h && h->concurrent && !bnbwd && !s.x_next && p.n_tile_cols <= 64 &&
                     2.0 * s.aN * s.OHl * s.OWl * (double)s.w_rows * s.ntaps * s.aC < kSmallConvFlops;
   const bool staged = staged0 && !thin;
+  // Eight epilogue warps where a tile's epilogue (about 31 cycles a column with four) is longer than its MMAs (N / 2 cycles
+  // each) and the tile is a full 256 columns: the 1x1 convolutions of bottleneck blocks (ResNet-50 3.53 -> 3.50 ms per
+  // step).  Elsewhere the second four warps only cost registers and shared memory (WRN-28-10 4.63 -> 4.65 ms).
+  const bool wide_epi = !thin && !bnbwd && !s.x_next && (staged ? s.addend != nullptr : s.addend == nullptr) &&
+                        p.n_tile_cols == 256 && s.n_cls <= 1 && s.ntaps * s.aC <= 1024;
+  const int epi_warps = wide_epi ? 8 : 4;
   const size_t max_smem = thin ? kTcThinSmem : kTcMaxSmem;
   const size_t stage_bytes = staged ? (size_t)(p.n_tile_cols / 32) * tc::kStageGroupBytes : 0;
   // the direct epilogue's statistics scratch is only there when statistics are asked for
-  const size_t tail = tc::kTailBytes + ((staged || !(s.stats || bnbwd)) ? 0 : sizeof(tc::TcStatScratch)) +
+  const size_t tail = tc::kTailBytes + ((staged || !(s.stats || bnbwd)) ? 0 : tc::stat_scratch_bytes(epi_warps)) +
                       (bnbwd ? sizeof(tc::TcBnBwdScratch) : 0) + stage_bytes + 1024;
   p.tx_b = (uint32_t)(p.n_tile_cols * row_bytes);
   p.acc_stride = (p.n_tile_cols + 31) / 32 * 32;
@@ -810,6 +816,10 @@ static int launch_conv_tc(lp_handle* h, const TcGemmSpec& s, int* dev_err, cudaS
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcThinSmem));
     LP_CUDA_OK(cudaFuncSetAttribute(tc::conv_tc_kernel<false, true, false, false, 2>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcThinSmem));
+    LP_CUDA_OK(cudaFuncSetAttribute(tc::conv_tc_kernel<false, false, false, false, 1, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kTcMaxSmem));
+    LP_CUDA_OK(cudaFuncSetAttribute(tc::conv_tc_kernel<false, true, true, false, 1, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kTcMaxSmem));
     LP_CUDA_OK(cudaFuncSetAttribute(tc::conv_tc_kernel<false, false, false, true>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcMaxSmem));
     LP_CUDA_OK(cudaFuncSetAttribute(tc::conv_tc_kernel<false, true, false, true>,
@@ -830,12 +840,14 @@ static int launch_conv_tc(lp_handle* h, const TcGemmSpec& s, int* dev_err, cudaS
   }
   if (s.x_next && !s.addend) return LP_ERR_UNSUPPORTED;   // the fused loss belongs to a convolution with a shortcut
   cudaError_t le;
-  const dim3 g3(grid), b3(tc::kConvThreads);
+  const dim3 g3(grid), b3(tc::conv_threads(epi_warps));
   if (thin && s.addend) le = launch_pdl(tc::conv_tc_kernel<false, true, false, false, 2>, g3, b3, smem, st, tmA, tmB, tmOut, tmAdd, p);
   else if (thin) le = launch_pdl(tc::conv_tc_kernel<false, false, false, false, 2>, g3, b3, smem, st, tmA, tmB, tmOut, tmAdd, p);
   else if (bnbwd && s.addend) le = launch_pdl(tc::conv_tc_kernel<false, true, false, true>, g3, b3, smem, st, tmA, tmB, tmOut, tmAdd, p);
   else if (bnbwd) le = launch_pdl(tc::conv_tc_kernel<false, false, false, true>, g3, b3, smem, st, tmA, tmB, tmOut, tmAdd, p);
   else if (s.x_next) le = launch_pdl(tc::conv_tc_kernel<true, true, false>, g3, b3, smem, st, tmA, tmB, tmOut, tmAdd, p);
+  else if (wide_epi && staged) le = launch_pdl(tc::conv_tc_kernel<false, true, true, false, 1, 8>, g3, b3, smem, st, tmA, tmB, tmOut, tmAdd, p);
+  else if (wide_epi) le = launch_pdl(tc::conv_tc_kernel<false, false, false, false, 1, 8>, g3, b3, smem, st, tmA, tmB, tmOut, tmAdd, p);
   else if (staged && s.addend) le = launch_pdl(tc::conv_tc_kernel<false, true, true>, g3, b3, smem, st, tmA, tmB, tmOut, tmAdd, p);
   else if (staged) le = launch_pdl(tc::conv_tc_kernel<false, false, true>, g3, b3, smem, st, tmA, tmB, tmOut, tmAdd, p);
   else if (s.addend) le = launch_pdl(tc::conv_tc_kernel<false, true, false>, g3, b3, smem, st, tmA, tmB, tmOut, tmAdd, p);
