@@ -437,7 +437,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
       const uint32_t a_lo0 = (uint32_t)p.adesc_hi3[i0] + base16 + (p.a_start3[i0] >> 4), a_hi0 = (uint32_t)(p.adesc_hi3[i0] >> 32);
       const uint32_t a_lo1 = (uint32_t)p.adesc_hi3[1] + base16 + (p.a_start3[1] >> 4), a_hi1 = (uint32_t)(p.adesc_hi3[1] >> 32);
       const uint32_t d0 = tmem_base + i0 * p.acc_stride, d1 = tmem_base + p.acc_stride;
-      const int ksteps = p.rows >> 4;   // K = 16 pixels per MMA, an even number of steps
+      const int ksteps = p.rows >> 4;   // K = 16 pixels per MMA
 #pragma unroll 1
       for (int it = 0; it < n_iter; ++it) {
         if (!mbar_wait_hot(&tail->full[s], ph, abort_flag)) { failed = true; break; }
@@ -445,23 +445,34 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         uint32_t a0 = a_lo0 + s * stage16, a1 = a_lo1 + s * stage16, bt = b_lo0 + s * stage16;
         int k = ksteps;
         if (first) {
+          if (k & 1) {
+            mma_bf16_lh(d0, a0, a_hi0, bt, b_hi, p.idesc, accum);
+            mma_bf16_lh(d1, a1, a_hi1, bt, b_hi, p.idesc, accum);
+            accum = 1;
+            a0 += ak; a1 += ak; bt += bk; --k;
+          }
 #pragma unroll 1
-          do {
+          for (; k > 0; k -= 2) {
             mma_bf16_lh(d0, a0, a_hi0, bt, b_hi, p.idesc, accum);
             mma_bf16_lh(d1, a1, a_hi1, bt, b_hi, p.idesc, accum);
             accum = 1;
             mma_bf16_lh(d0, a0 + ak, a_hi0, bt + bk, b_hi, p.idesc, 1u);
             mma_bf16_lh(d1, a1 + ak, a_hi1, bt + bk, b_hi, p.idesc, 1u);
             a0 += 2 * ak; a1 += 2 * ak; bt += 2 * bk;
-          } while ((k -= 2) > 0);
+          }
         } else {
+          if (k & 1) {
+            mma_bf16_lh(d0, a0, a_hi0, bt, b_hi, p.idesc, accum);
+            accum = 1;
+            a0 += ak; bt += bk; --k;
+          }
 #pragma unroll 1
-          do {
+          for (; k > 0; k -= 2) {
             mma_bf16_lh(d0, a0, a_hi0, bt, b_hi, p.idesc, accum);
             accum = 1;
             mma_bf16_lh(d0, a0 + ak, a_hi0, bt + bk, b_hi, p.idesc, 1u);
             a0 += 2 * ak; bt += 2 * bk;
-          } while ((k -= 2) > 0);
+          }
         }
         mma_commit(&tail->empty[s]);
         if (++s == (uint32_t)p.stages) { s = 0; ph ^= 1; }
@@ -612,7 +623,9 @@ static int wg_encode_wnh(WgEncodeFn enc, CUtensorMap* m, const void* base, int N
 static const size_t kWgSharedSmem = 100 * 1024;
 static int launch_wgrad_halo(WgEncodeFn enc, int sm_count, bool* attr_done, const bf16* x, const bf16* dy, float* dw, int N, int H, int W,
                              int Cin, int Cout, int* dev_err, cudaStream_t st, bool shared_sm) {
-  if (W % 8 || Cin < 64) return 1;
+  // tiles are 8 pixels wide; where the width is not a multiple of 8 the last tile column reads zero fill: taken where at
+  // most an eighth of the columns is wasted (7, 14, 28, ...), as in the forward kernel
+  if (W * 8 < 7 * 8 * ((W + 7) / 8) || Cin < 64) return 1;
   tc::WgradParams p;
   memset(&p, 0, sizeof(p));
   p.Nimg = N; p.OH = H; p.OW = W; p.stride = 1; p.pad = 1; p.R = 3;
@@ -621,15 +634,24 @@ static int launch_wgrad_halo(WgEncodeFn enc, int sm_count, bool* attr_done, cons
   // instead of 80 KB for a 160-channel tile (five stages in flight instead of two); measured, that is
   // no faster (0.079 against 0.078 ms at 160 channels), so the copy latency is not what limits it.
   constexpr int per_col = LP_WGRAD_HALO_KBLOCK / 8;
-  if (H >= per_col) { p.BH = per_col; p.BNI = 1; }
-  else if (H == 8 || H == 4 || H == 2) { p.BH = H; p.BNI = per_col / H; }
-  else return 1;
+  if (H >= per_col) {                       // rows spread evenly over the tiles of a column (14: 14, 28: 2 x 14, 56: 4 x 14)
+    const int th = (H + per_col - 1) / per_col;
+    p.BH = (H + th - 1) / th;
+    p.BH += p.BH & 1;                       // (a K step of 16 pixels is two of them)
+    if (p.BH * 8 < 96) return 1;
+    p.BNI = 1;
+  } else {
+    p.BH = H;
+    p.BNI = per_col / H;
+    if ((p.BH * p.BNI) & 1) --p.BNI;
+    if (p.BNI < 1 || p.BH * p.BNI * 8 < 96) return 1;
+  }
   if (p.BNI > N) return 1;
   p.BW = 8;
-  p.tiles_w = W / 8;
+  p.tiles_w = (W + 7) / 8;
   p.tiles_h = (H + p.BH - 1) / p.BH;
   p.pix_tiles = p.tiles_w * p.tiles_h * ((N + p.BNI - 1) / p.BNI);
-  p.rows = p.rows_pad = LP_WGRAD_HALO_KBLOCK;
+  p.rows = p.rows_pad = 8 * p.BH * p.BNI;
   // dy sub-boxes as in the plain kernel, one channel tile of at most 160 so that three accumulators fit
   int best_tile = 0;
   for (int sc : {64, 32, 16}) {
@@ -655,11 +677,11 @@ static int launch_wgrad_halo(WgEncodeFn enc, int sm_count, bool* attr_done, cons
   p.groups = 3 * p.cin_chunks;
   p.m_tiles = (p.groups + 1) / 2;
   const int box_rows = 10 * p.BNI * p.BH;
-  p.a_box_bytes = (uint32_t)(box_rows * 128);
+  p.a_box_bytes = (uint32_t)((box_rows * 128 + 1023) / 1024 * 1024);
   p.a_region = 2 * p.a_box_bytes;
   p.b_sub_bytes = (uint32_t)((p.rows * p.scb * 2 + 1023) / 1024 * 1024);
   p.stage_bytes = p.a_region + p.b_sub_bytes * p.nb;
-  p.tx_a = p.a_box_bytes;
+  p.tx_a = (uint32_t)(box_rows * 128);
   p.tx_b = (uint32_t)(p.rows * p.nb * p.scb * 2);
   const size_t tail = sizeof(tc::WgSmemTail) + 1024;
   int stages = (int)((max_smem - tail) / p.stage_bytes);

@@ -140,6 +140,33 @@ def test_tensor_conv_wgrad_matches_oracle(case):
     assert rel_err(dw, O.conv_wgrad(x, dy, w.shape, stride, pad)) < 2e-3
 
 
+# weight gradients on boxes with a halo whose last tile column or row is ragged: 28x28 in rows of 14, 30 columns, pairs of
+# 7-row images with an odd batch, 18 rows as 2 x 10 (too few a tile: plain kernel), 112 pixels a block (7 MMA steps)
+@pytest.mark.parametrize("case", [(3, 28, 28, 64, 64, 3, 1, 1), (2, 14, 30, 64, 160, 3, 1, 1), (5, 7, 14, 128, 64, 3, 1, 1),
+                                  (3, 18, 16, 64, 64, 3, 1, 1), (2, 14, 14, 64, 256, 3, 1, 1)])
+def test_tensor_conv_wgrad_ragged_halo_boxes(case):
+    import paper_2112_05387_b200 as lp
+    N, H, W, Cin, Cout, R, stride, pad = case
+    x, w, dy = make_case(*case, "bf16")
+    st, dw, _ = run_conv(lp.LP_CONV_WGRAD, "bf16", lp.LP_CONV_IMPL_TENSOR, *case, x, dy)
+    assert st == 0, lp.lp_status_string(st)
+    assert rel_err(dw, O.conv_wgrad(x, dy, w.shape, stride, pad)) < 2e-3
+
+
+# 1x1 convolutions of few input channels into 256-column tiles: eight epilogue warps
+@pytest.mark.parametrize("case", [(3, 9, 11, 64, 256, 1, 1, 0), (2, 6, 7, 256, 512, 1, 1, 0), (2, 8, 8, 40, 256, 1, 2, 0)])
+def test_tensor_conv_forward_wide_epilogue(case):
+    import paper_2112_05387_b200 as lp
+    N, H, W, Cin, Cout, R, stride, pad = case
+    x, w, dy = make_case(*case, "bf16")
+    st, y, stats = run_conv(lp.LP_CONV_FWD, "bf16", lp.LP_CONV_IMPL_TENSOR, *case, x, w, want_stats=True)
+    assert st == 0, lp.lp_status_string(st)
+    ref = O.conv_fwd(x, w, stride, pad)
+    assert rel_err(y, ref) < 6e-3
+    np.testing.assert_allclose(stats[:Cout], ref.reshape(-1, Cout).sum(0), rtol=1e-3, atol=2e-2 * np.sqrt(ref.size / Cout))
+    np.testing.assert_allclose(stats[Cout:], (ref ** 2).reshape(-1, Cout).sum(0), rtol=5e-3)
+
+
 def test_unsupported_shapes_are_refused_not_faulted():
     import paper_2112_05387_b200 as lp
     case = (2, 8, 8, 3, 8, 3, 1, 1)
