@@ -56,8 +56,6 @@ template <int KS, bool kDgrad>
 __global__ void __launch_bounds__(32 * KS)
 conv_f32_tile_kernel(const __grid_constant__ ConvF32Params p) {
   extern __shared__ __align__(16) float smf[];
-  pdl_wait();
-  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cls = blockIdx.z;
   const int co0 = blockIdx.y * 16;
@@ -71,14 +69,16 @@ conv_f32_tile_kernel(const __grid_constant__ ConvF32Params p) {
   const int dh0 = p.cls_dh0[cls], dw0 = p.cls_dw0[cls];
   const int nchunks = ntaps ? (p.aC + 15) >> 4 : 0;
 
-  auto load_chunk = [&](int c) {
+  // (the loops of the block's set-up are kept rolled: they run a few times, and unrolled code would first have to be fetched)
+  auto load_patch = [&](int c) {
     float* a = smf + (c & 1) * p.stage_floats;
-    float* wb = a + p.w_off;
     const int c0 = c * 16;
     const int ih0 = h0 * p.in_step + dh0, iw0 = w0 * p.in_step + dw0;
+#pragma unroll 1
     for (int r = warp; r < p.PH; r += KS) {
       const int ih = ih0 + r;
       const bool row_ok = ih >= 0 && ih < p.aH;
+#pragma unroll 1
       for (int l = lane; l < p.PW * 4; l += 32) {
         const int iw = iw0 + (l >> 2), ci = c0 + 4 * (l & 3);
         const bool ok = row_ok && iw >= 0 && iw < p.aW && ci < p.aC;
@@ -86,9 +86,15 @@ conv_f32_tile_kernel(const __grid_constant__ ConvF32Params p) {
         cp_async16(a + r * p.row_pitch + 4 * l, src, ok);
       }
     }
-    // weights in their own order: rows of 16 input channels per (output channel, tap), or (input gradient) rows of
-    // 16 output channels per (input channel, tap)
+  };
+  // weights in their own order: rows of 16 input channels per (output channel, tap), or (input gradient) rows of
+  // 16 output channels per (input channel, tap)
+  auto load_weights = [&](int c) {
+    float* wb = smf + (c & 1) * p.stage_floats + p.w_off;
+    const int c0 = c * 16;
+#pragma unroll 1
     for (int r = warp; r < 16; r += KS) {
+#pragma unroll 1
       for (int l = lane; l < ntaps * 4; l += 32) {
         const int tap = p.tap_w[tap0 + (l >> 2)], v = 4 * (l & 3);
         bool ok;
@@ -103,8 +109,11 @@ conv_f32_tile_kernel(const __grid_constant__ ConvF32Params p) {
         cp_async16(wb + r * p.w_pitch + 4 * l, src, ok);
       }
     }
-    cp_async_commit();
   };
+  // the first weights were written at least one kernel before the preceding one: on their way before its end
+  if (nchunks) load_weights(0);
+  pdl_wait();
+  pdl_launch_dependents();
 
   const int row = lane >> 2, cg = lane & 3;
   float acc[8][4];
@@ -113,10 +122,14 @@ conv_f32_tile_kernel(const __grid_constant__ ConvF32Params p) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc[j][k] = 0.f;
 
-  if (nchunks) load_chunk(0);
+  if (nchunks) load_patch(0);
+  cp_async_commit();
+#pragma unroll 1
   for (int c = 0; c < nchunks; ++c) {
     if (c + 1 < nchunks) {
-      load_chunk(c + 1);
+      load_patch(c + 1);
+      load_weights(c + 1);
+      cp_async_commit();
       cp_async_wait<1>();
     } else {
       cp_async_wait<0>();
@@ -126,6 +139,7 @@ conv_f32_tile_kernel(const __grid_constant__ ConvF32Params p) {
     const float* wb = smf + (c & 1) * p.stage_floats + p.w_off;
     const int nq = min(4, (p.aC - c * 16) >> 2);   // quads of real input channels
     const int items = ntaps * nq;
+#pragma unroll 1
     for (int it = warp; it < items; it += KS) {
       const int tp = nq == 4 ? it >> 2 : it / nq;
       const int q = it - tp * nq;
@@ -186,6 +200,7 @@ conv_f32_tile_kernel(const __grid_constant__ ConvF32Params p) {
   float s[4] = {0.f, 0.f, 0.f, 0.f}, q2[4] = {0.f, 0.f, 0.f, 0.f};
   const int v = threadIdx.x & 3;
   const int c = co0 + 4 * v;
+#pragma unroll 1
   for (int px = threadIdx.x >> 2; px < 64; px += 8 * KS) {
     const int oh = h0 + (px >> 3), ow = w0 + (px & 7);
     const int ph = oh * p.os + p.cls_oh[cls], pw = ow * p.os + p.cls_ow[cls];
