@@ -240,6 +240,14 @@ struct ConvProfile {
 
 using namespace lp;
 
+// Executable graph of one entry point of a handle (see run_as_graph).
+enum { CALL_AUX_FORWARD = 0, CALL_MODULES, CALL_STEP, CALL_LAYER_PARALLEL, CALL_DISTILL, CALL_FORWARD_SERIAL, CALL_SERIAL, CALL_KINDS };
+struct CallGraph {
+  cudaGraphExec_t exec = nullptr;
+  int calls = 0, rebuilt = 0;
+  bool off = false;
+};
+
 struct lp_handle {
   NetDef net;
   int dtype = LP_F32;
@@ -259,6 +267,8 @@ struct lp_handle {
   uint8_t* ws = nullptr;
   size_t ws_bytes = 0;
   int32_t* zero_labels = nullptr;  // N zeros, for forward passes that only want logits
+  CallGraph call_graph[CALL_KINDS];
+  cudaStream_t capture_stream = nullptr;
   std::vector<cudaGraphExec_t> graphs;
   int64_t launches_at_capture = 0;
   std::vector<int64_t> graph_launches;  // kernels recorded in each graph
@@ -2433,6 +2443,55 @@ static int module_fwd_bwd(lp_handle* h, int k, const void* x_k, const void* x_ne
   return LP_OK;
 }
 
+// Runs `enqueue(stream)` as ONE graph launch on `st`.  A call is some hundred launches of a few microseconds each; made one
+// by one, each costs the host 3 to 5 us, so that small networks wait for the host (ResNet-56 on 20 images in three calls:
+// 1136 us of host time for 362 us of work) and large ones lose the overlap of launches across streams.  The call is
+// recorded anew every time, with this call's pointers and arguments, on a stream of the handle's own (recording a launch
+// costs a fraction of making it), the executable graph of the previous call is updated to the recording, and launched;
+// only its topology and memory are kept.  The first two calls of a kind (which also set kernel attributes), calls inside a
+// caller's capture, and profiled calls launch directly.
+template <typename F>
+static int run_as_graph(lp_handle* h, int kind, cudaStream_t st, F enqueue) {
+  CallGraph& g = h->call_graph[kind];
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) { cudaGetLastError(); return enqueue(st); }
+  if (cs != cudaStreamCaptureStatusNone || h->prof.enabled || h->tl.enabled || g.off || !h->capture_stream || ++g.calls <= 2)
+    return enqueue(st);
+  if (cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+    cudaGetLastError();
+    g.off = true;
+    return enqueue(st);
+  }
+  const int64_t launches = h->launches;
+  const int rc = enqueue(h->capture_stream);
+  cudaGraph_t graph = nullptr;
+  cudaError_t e = cudaStreamEndCapture(h->capture_stream, &graph);
+  if (rc != LP_OK) {               // (an argument or launch error: nothing has run)
+    if (graph) cudaGraphDestroy(graph);
+    cudaGetLastError();
+    return rc;
+  }
+  if (e == cudaSuccess && g.exec) {
+    cudaGraphExecUpdateResultInfo info;
+    if (cudaGraphExecUpdate(g.exec, graph, &info) != cudaSuccess) {   // other options than last time: other nodes
+      cudaGetLastError();
+      cudaGraphExecDestroy(g.exec);
+      g.exec = nullptr;
+      g.off = ++g.rebuilt >= 4;        // a caller that keeps changing them is better off without
+    }
+  }
+  if (e == cudaSuccess && !g.exec) e = cudaGraphInstantiate(&g.exec, graph, 0);
+  if (e == cudaSuccess) e = cudaGraphLaunch(g.exec, st);
+  if (graph) cudaGraphDestroy(graph);
+  if (e != cudaSuccess) {          // recording does not work here: launch directly from now on
+    cudaGetLastError();
+    g.off = true;
+    h->launches = launches;
+    return enqueue(st);
+  }
+  return LP_OK;
+}
+
 }  // namespace lp
 
 // =============================================================================================
@@ -2568,6 +2627,7 @@ int lp_create(const lp_net_desc* desc, void* dev_workspace, size_t bytes, lp_han
     }
   }
   if (cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
+  if (cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
   if (cudaStreamCreateWithFlags(&h->aux_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->aux_end, cudaEventDisableTiming) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
   h->aux_done.resize(net.K > 1 ? net.K - 1 : 0);
@@ -2583,6 +2643,8 @@ int lp_destroy(lp_handle* h) {
   for (auto s : h->streams) if (s) cudaStreamDestroy(s);
   for (auto e : h->done) if (e) cudaEventDestroy(e);
   if (h->fork) cudaEventDestroy(h->fork);
+  for (auto& g : h->call_graph) if (g.exec) cudaGraphExecDestroy(g.exec);
+  if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
   if (h->aux_stream) cudaStreamDestroy(h->aux_stream);
   if (h->aux_end) cudaEventDestroy(h->aux_end);
   for (auto e : h->aux_done) if (e) cudaEventDestroy(e);
@@ -2672,13 +2734,15 @@ int lp_auxnet_forward(lp_handle* h, const void* images, void* const* x_out, void
     if (!x_out[k]) return LP_ERR_NULL;
     if (!aligned16(x_out[k])) return LP_ERR_ALIGN;
   }
-  RunCtx c;
-  c.st = (cudaStream_t)stream; c.images = images; c.xout = x_out;
-  for (size_t i = 0; i < h->auxs.size(); ++i) {   // chain order, or stack by stack (units in order)
-    int rc = aux_plan_forward(h, (int)i, c);
-    if (rc != LP_OK) return rc;
-  }
-  return LP_OK;
+  return run_as_graph(h, CALL_AUX_FORWARD, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
+    RunCtx c;
+    c.st = st; c.images = images; c.xout = x_out;
+    for (size_t i = 0; i < h->auxs.size(); ++i) {   // chain order, or stack by stack (units in order)
+      int rc = aux_plan_forward(h, (int)i, c);
+      if (rc != LP_OK) return rc;
+    }
+    return LP_OK;
+  });
 }
 
 static int check_module_args(lp_handle* h, int k, const void* x_k, const void* x_next_or_labels, const void* lambda_k,
@@ -2716,7 +2780,7 @@ int lp_modules_fwd_bwd_all(lp_handle* h, const void* const* x, const int32_t* la
                                dx ? dx[k] : nullptr);
     if (rc != LP_OK) return rc;
   }
-  cudaStream_t st = (cudaStream_t)stream;
+  return run_as_graph(h, CALL_MODULES, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   ConcurrentScope concurrent(h);
   LP_CUDA_OK(cudaEventRecord(h->fork, st));
   // heaviest modules first is not needed: all K are enqueued before any can finish
@@ -2736,6 +2800,7 @@ int lp_modules_fwd_bwd_all(lp_handle* h, const void* const* x, const int32_t* la
       if (first_err == LP_OK) first_err = LP_ERR_CUDA;
   }
   return first_err;
+  });
 }
 
 static int update_module(lp_handle* h, int k, float lr, float momentum, float weight_decay, float kappa_step,
@@ -2763,7 +2828,6 @@ static int update_module(lp_handle* h, int k, float lr, float momentum, float we
 int lp_step(lp_handle* h, float lr, float momentum, float weight_decay, float kappa_step, void* const* lambdas_inout,
             void* stream) {
   if (!h) return LP_ERR_NULL;
-  cudaStream_t st = (cudaStream_t)stream;
   bool any = false;
   for (auto& P : h->modules) any = any || P.ps.grads_fresh;
   if (!any) return LP_ERR_ORDER;
@@ -2771,13 +2835,17 @@ int lp_step(lp_handle* h, float lr, float momentum, float weight_decay, float ka
   if (lambdas_inout)
     for (int k = 0; k + 1 < K; ++k)
       if (lambdas_inout[k] && !aligned16(lambdas_inout[k])) return LP_ERR_ALIGN;
+  std::vector<bool> fresh(K);            // (the flags go down with the first enqueue: a second one needs them as they were)
+  for (int k = 0; k < K; ++k) fresh[k] = h->modules[k].ps.grads_fresh;
+  return run_as_graph(h, CALL_STEP, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   for (int k = 0; k < K; ++k) {
-    if (!h->modules[k].ps.grads_fresh) continue;
+    if (!fresh[k]) continue;
     int rc = update_module(h, k, lr, momentum, weight_decay, kappa_step,
                            (lambdas_inout && k + 1 < K) ? lambdas_inout[k] : nullptr, st);
     if (rc != LP_OK) return rc;
   }
   return LP_OK;
+  });
 }
 
 int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out, const int32_t* labels,
@@ -2793,7 +2861,7 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
         (dx && dx[k + 1] && !aligned16(dx[k + 1])))
       return LP_ERR_ALIGN;
   }
-  cudaStream_t st = (cudaStream_t)stream;
+  return run_as_graph(h, CALL_LAYER_PARALLEL, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   ConcurrentScope concurrent(h);
   LP_CUDA_OK(cudaEventRecord(h->fork, st));
   // Streams forked from the caller's so far; whatever happens below, each is joined back before the
@@ -2865,6 +2933,7 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
       if (first_err == LP_OK) first_err = LP_ERR_CUDA;
   }
   return first_err;
+  });
 }
 
 int lp_auxnet_distill(lp_handle* h, const void* images, void* const* x, const void* const* dx, float lr_lambda,
@@ -2877,7 +2946,7 @@ int lp_auxnet_distill(lp_handle* h, const void* images, void* const* x, const vo
     if (!aligned16(x[k - 1]) || !aligned16(dx[k]) || (x_new && x_new[k - 1] && !aligned16(x_new[k - 1]))) return LP_ERR_ALIGN;
     if (!h->modules[k - 1].ran_fwd_bwd) return LP_ERR_ORDER;  // its terminal adjoint is the other half of g_k
   }
-  cudaStream_t st = (cudaStream_t)stream;
+  return run_as_graph(h, CALL_DISTILL, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   RunCtx c;
   c.st = st; c.images = images; c.xout = x;
   const bool rec = h->net.d.aux_recursive != 0;
@@ -2915,6 +2984,7 @@ int lp_auxnet_distill(lp_handle* h, const void* images, void* const* x, const vo
     }
   }
   return LP_OK;
+  });
 }
 
 int lp_aux_correct(lp_handle* h, void* const* x_inout, const void* const* dx, float lr_lambda, float* norm_out,
@@ -2970,19 +3040,20 @@ static int serial_forward(lp_handle* h, const void* images, const int32_t* label
 int lp_forward_serial(lp_handle* h, const void* images, float* logits, void* stream) {
   if (!h || !images || !logits) return LP_ERR_NULL;
   if (!aligned16(images)) return LP_ERR_ALIGN;
-  cudaStream_t st = (cudaStream_t)stream;
   Plan& L = h->modules[h->net.K - 1];
-  int rc = serial_forward(h, images, nullptr, nullptr, st);
-  if (rc != LP_OK) return rc;
-  LP_CUDA_OK(cudaMemcpyAsync(logits, L.head.logits, (size_t)h->net.d.N * h->net.d.num_classes * 4,
-                             cudaMemcpyDeviceToDevice, st));
-  return LP_OK;
+  return run_as_graph(h, CALL_FORWARD_SERIAL, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
+    int rc = serial_forward(h, images, nullptr, nullptr, st);
+    if (rc != LP_OK) return rc;
+    LP_CUDA_OK(cudaMemcpyAsync(logits, L.head.logits, (size_t)h->net.d.N * h->net.d.num_classes * 4,
+                               cudaMemcpyDeviceToDevice, st));
+    return LP_OK;
+  });
 }
 
 int lp_serial_fwd_bwd(lp_handle* h, const void* images, const int32_t* labels, float* loss_out, void* stream) {
   if (!h || !images || !labels || !loss_out) return LP_ERR_NULL;
   if (!aligned16(images)) return LP_ERR_ALIGN;
-  cudaStream_t st = (cudaStream_t)stream;
+  return run_as_graph(h, CALL_SERIAL, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   const int K = h->net.K;
   for (int k = 0; k < K; ++k) LP_CUDA_OK(cudaMemsetAsync(h->modules[k].ps.g, 0, h->modules[k].ps.n * 4, st));
   int rc = serial_forward(h, images, labels, loss_out, st);
@@ -2999,6 +3070,7 @@ int lp_serial_fwd_bwd(lp_handle* h, const void* images, const int32_t* labels, f
     P.ps.grads_fresh = true;
   }
   return LP_OK;
+  });
 }
 
 int lp_get_residual(lp_handle* h, int k, void* r_dst, void* seed_dst, void* stream) {

@@ -512,6 +512,42 @@ def test_timeline_records_every_operation_of_a_step():
     lp.lp_timeline(h, False, read=False)
 
 
+@pytest.mark.parametrize("which", ["step", "three_calls", "serial"])
+def test_repeated_calls_equal_directly_launched_ones(which):
+    """From the third call of a kind on, a call is recorded and launched as one graph, updated to the call's own pointers
+    and arguments.  Seven calls with new buffers, another learning rate each, and multipliers given or not (other launches)
+    against a handle whose time line is enabled, which always launches directly: the same kernels on the same values, the
+    order of the fp32 atomics aside (1e-6 an update; the fp32 network magnifies no rounding)."""
+    cfg = get_config("tiny")
+    runs = [GpuRun(cfg), GpuRun(cfg)]
+    torch, lp, K = runs[0].torch, runs[0].lp, runs[0].net.K
+    for call in range(7):
+        for i, run in enumerate(runs):
+            if i:
+                lp.lp_timeline(run.h, True, read=False)
+            h = run.h
+            images = (run.d_images * (1.0 + 0.1 * call)).contiguous()
+            x = [torch.zeros_like(t) for t in run.d_x[1:]]
+            dx = [None] + [torch.zeros_like(t) for t in run.d_x[1:]]
+            lam = run.d_kappa if call % 3 else None
+            loss = torch.zeros_like(run.d_loss)
+            lr = 1e-3 * (call + 1)
+            if which == "step":
+                lp.lp_layer_parallel_step(h, images, x, run.d_labels, lam, cfg["rho"], loss, dx, lr, 0.0, 0.0, cfg["rho"])
+            elif which == "three_calls":
+                lp.lp_auxnet_forward(h, images, x)
+                lp.lp_modules_fwd_bwd_all(h, [images] + x, run.d_labels, lam, cfg["rho"], loss, dx)
+                lp.lp_step(h, lr, 0.9, 1e-4, cfg["rho"], lam)
+            else:
+                lp.lp_serial_fwd_bwd(h, images, run.d_labels, loss[K - 1])
+                lp.lp_step(h, lr, 0.0, 0.0, 0.0, None)
+            assert lp.lp_last_device_status(h) == 0
+            run.seen = [to_host(loss)] + [to_host(t) for t in x] + [to_host(t) for t in dx[1:]]
+            run.seen += [lp.lp_get_params(h, k) for k in range(K)]
+        for a, b in zip(runs[0].seen, runs[1].seen):
+            assert np.linalg.norm(a - b) <= 1e-5 * max(np.linalg.norm(b), 1e-30), call
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_update_with_momentum_and_weight_decay(dtype):
     """lp_step with heavy-ball momentum and weight decay, two steps from the same gradients, against
