@@ -330,7 +330,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // One thread runs the whole loop.  What it does between the last MMA of a stage and the first of the next (poll,
     // descriptors, commit) has to be shorter than the MMAs still queued, about four, or the tensor pipe runs dry: with a
     // warp-uniform loop that elected a lane per stage a stage of four MMAs cost 800 to 850 cycles whatever their width
-    // (324 cycles of work at N = 160, 492 at N = 256).
+    // (324 cycles of work at N = 160, 492 at N = 256); now 350 at N = 160 (ResNet-34 3200 -> 3087 us per step, layer-serial
+    // WRN-28-10 on 64 images 2910 -> 2816).
     const int me = warp - 1;
     if (me < p.mpair && elect_one()) {
       uint32_t sa = 0, pha = 0, sb = 0, phb = 0, slot = 0, slot_phase = 0;

@@ -19,7 +19,8 @@
 //  * the epilogue takes the statistics of the next batch norm (forward) or the reduction pass of the next batch-norm
 //    backward (input gradient) as column sums over the staged output tile, which leaves by a TMA store.
 //
-// A residual block is four launches in a row instead of ten.  A CTA runs most of its code once or twice, so fetching
+// A residual block is four launches in a row instead of ten (ResNet-56 on 128 images 1202 -> 785 us per step, ResNet-110
+// 2127 -> 1455; with the rolled loops of the other kernels 738 and 1343).  A CTA runs most of its code once or twice, so fetching
 // instructions costs as much as executing them: loops are kept rolled and whole tiles are moved by single copies (an
 // unrolled version with the loads in registers, 2.5 times the code, took 1.5 times as long per launch).  For the same
 // reason nothing is pipelined inside a CTA; two CTAs share an SM instead (one of the 64-channel layers).

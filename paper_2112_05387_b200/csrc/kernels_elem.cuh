@@ -451,21 +451,6 @@ bn_bwd_apply_kernel(const T* __restrict__ dy, const T* __restrict__ x, int relu_
   }
 }
 
-// out = a + b
-template <typename T>
-__global__ void add_kernel(const T* __restrict__ a, const T* __restrict__ b, T* __restrict__ out, long long total_vecs) {
-  constexpr int V = VecT<T>::N;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total_vecs; i += stride) {
-    float f[V], g[V];
-    ldv(a + i * V, f);
-    ldv(b + i * V, g);
-#pragma unroll
-    for (int j = 0; j < V; ++j) f[j] += g[j];
-    stv(out + i * V, f);
-  }
-}
-
 // ---------------------------------------------------------------------------------------
 // 3x3 / stride 2 / pad 1 max-pool; the first maximum in (r,s) scan order wins (stored as 0..8).
 // ---------------------------------------------------------------------------------------
