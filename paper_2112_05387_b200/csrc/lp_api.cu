@@ -1377,7 +1377,7 @@ static int conv_wgrad(lp_handle* h, int dtype, int impl, const ConvDef& c, int N
     {
       ProfScope ps(h, st, 2.0 * N * c.OH * c.OW * (double)c.cout * c.R * c.R * c.cin);
       int rc = launch_wgrad_tc(D.encode, D.sm_count, &D.wgrad_attr, &D.wgrad_halo_attr, c.xs, (const bf16*)dy, c.dws, N, c.H / 2,
-                               c.W / 2, 16, c.OH, c.OW, c.cout, 4, 1, 2, dev_err, st);
+                               c.W / 2, 16, c.OH, c.OW, c.cout, 4, 1, 2, dev_err, st, false, h && h->concurrent);
       if (h) h->launches++;
       if (rc != LP_OK) return rc;
     }
@@ -1398,9 +1398,9 @@ static int conv_wgrad(lp_handle* h, int dtype, int impl, const ConvDef& c, int N
     // (thin layers: the gradient of the 64 x 64 group blocks, folded back after the pass -- rows of 128 bytes instead
     // of 32 or 64, and a quarter or half of the pixels to sum over)
     int rc = c.g > 1 ? launch_wgrad_tc(D.encode, D.sm_count, &D.wgrad_attr, &D.wgrad_halo_attr, (const bf16*)x, (const bf16*)dy,
-                                       c.dwg, N, c.H, c.W / c.g, 64, c.H, c.W / c.g, 64, 3, 1, 1, dev_err, st, shared_sm)
+                                       c.dwg, N, c.H, c.W / c.g, 64, c.H, c.W / c.g, 64, 3, 1, 1, dev_err, st, shared_sm, h && h->concurrent)
                      : launch_wgrad_tc(D.encode, D.sm_count, &D.wgrad_attr, &D.wgrad_halo_attr, (const bf16*)x, (const bf16*)dy, dw, N,
-                                       c.H, c.W, c.cin, c.OH, c.OW, c.cout, c.R, c.stride, c.pad, dev_err, st, shared_sm);
+                                       c.H, c.W, c.cin, c.OH, c.OW, c.cout, c.R, c.stride, c.pad, dev_err, st, shared_sm, h && h->concurrent);
     if (h) h->launches++;
     return rc;
   }

@@ -623,8 +623,32 @@ static int wg_encode_wnh(WgEncodeFn enc, CUtensorMap* m, const void* base, int N
 // kWgSharedSmem of shared memory) instead of taking the SM for itself; for small layers that several
 // modules run at the same time.
 static const size_t kWgSharedSmem = 100 * 1024;
+
+// Into how many parts the pixel range is split.  A CTA takes its K blocks plus a fixed prologue / epilogue worth about
+// four of them; a launch that has the machine to itself is as long as its waves of SMs.  side_by_side: the launch runs
+// beside other modules' kernels, on a stream nothing waits for until the update.  Then the SM time that it takes from them
+// (CTAs x their duration) counts for more than its own length: every further part repeats the fixed share and adds its
+// partial sums to dw once more.  Six times as much: ResNet-56 744 -> 705 us per step, ResNet-110 1343 -> 1242, ResNet-50
+// 3449 -> 3320, ResNet-50 on 12 images of 176x176 1615 -> 1398, ResNet-34 2920 -> 2875, WRN-28-10 unchanged (its launches
+// have enough blocks for every SM either way).  Three times: 718, 1284, 3353, 1420, 2906; half of the SMs or a third of
+// them whatever the size: ResNet-56 702 and 745, ResNet-110 1240 and 1210, but WRN-28-10 on half 4690 -> 4756 and in
+// layer-serial training (one module at a time, the first rule) 2670 -> 2749.
+static int wgrad_splits(int tiles, int pix_tiles, double block_cost, int sm_count, bool side_by_side) {
+  const double sm_time_weight = side_by_side ? 6.0 : 0.0;
+  int best_s = 1;
+  double best_t = 1e30;
+  const int max_s = std::min(pix_tiles, 64);
+  for (int sp = 1; sp <= max_s; ++sp) {
+    const int waves = (tiles * sp + sm_count - 1) / sm_count;
+    const double cta = (double)((pix_tiles + sp - 1) / sp) * block_cost + 4.0;
+    const double t = (waves + sm_time_weight * tiles * sp / sm_count) * cta;
+    if (t < best_t - 1e-9) { best_t = t; best_s = sp; }
+  }
+  return best_s;
+}
+
 static int launch_wgrad_halo(WgEncodeFn enc, int sm_count, bool* attr_done, const bf16* x, const bf16* dy, float* dw, int N, int H, int W,
-                             int Cin, int Cout, int* dev_err, cudaStream_t st, bool shared_sm) {
+                             int Cin, int Cout, int* dev_err, cudaStream_t st, bool shared_sm, bool side_by_side) {
   // tiles are 8 pixels wide; where the width is not a multiple of 8 the last tile column reads zero fill: taken where at
   // most an eighth of the columns is wasted (7, 14, 28, ...), as in the forward kernel
   if (W * 8 < 7 * 8 * ((W + 7) / 8) || Cin < 64) return 1;
@@ -700,17 +724,7 @@ static int launch_wgrad_halo(WgEncodeFn enc, int sm_count, bool* attr_done, cons
   p.bdesc_hi = tc::smem_desc_hi(p.b_sub_bytes, 8 * p.scb * 2, tc::swizzle_code_for_row_bytes(p.scb * 2));
   p.idesc = tc::instr_desc_bf16(128, p.n_tile, 1, 1);
   const int tiles = p.m_tiles * p.n_tiles;
-  {
-    int best_s = 1;
-    double best_t = 1e30;
-    const int max_s = std::min(p.pix_tiles, 64);
-    for (int sp = 1; sp <= max_s; ++sp) {
-      const int waves = (tiles * sp + sm_count - 1) / sm_count;
-      const double t = waves * ((double)((p.pix_tiles + sp - 1) / sp) * 1.5 * (p.rows / 128.0) + 4.0);
-      if (t < best_t - 1e-9) { best_t = t; best_s = sp; }
-    }
-    p.splits = best_s;
-  }
+  p.splits = wgrad_splits(tiles, p.pix_tiles, 1.5 * (p.rows / 128.0), sm_count, side_by_side);
   p.dw = dw; p.err = dev_err;
   CUtensorMap tmX, tmDY;
   if (wg_encode_wnh(enc, &tmX, x, N, H, W, Cin, 64, 10, p.BNI, p.BH)) return -8;
@@ -745,9 +759,9 @@ static int launch_wgrad_halo(WgEncodeFn enc, int sm_count, bool* attr_done, cons
 
 static int launch_wgrad_tc(WgEncodeFn enc, int sm_count, bool* attr_done, bool* halo_attr_done, const bf16* x,
                            const bf16* dy, float* dw, int N, int H, int W, int Cin, int OH, int OW, int Cout, int R,
-                           int stride, int pad, int* dev_err, cudaStream_t st, bool shared_sm = false) {
+                           int stride, int pad, int* dev_err, cudaStream_t st, bool shared_sm, bool side_by_side) {
   if (R == 3 && stride == 1 && pad == 1) {
-    const int rc = launch_wgrad_halo(enc, sm_count, halo_attr_done, x, dy, dw, N, H, W, Cin, Cout, dev_err, st, shared_sm);
+    const int rc = launch_wgrad_halo(enc, sm_count, halo_attr_done, x, dy, dw, N, H, W, Cin, Cout, dev_err, st, shared_sm, side_by_side);
     if (rc != 1) return rc;
   }
   const size_t max_smem = shared_sm ? kWgSharedSmem : (size_t)220 * 1024;
@@ -798,19 +812,7 @@ static int launch_wgrad_tc(WgEncodeFn enc, int sm_count, bool* attr_done, bool* 
   p.rows = p.BW * p.BH * p.BNI;
   p.rows_pad = (p.rows + 15) / 16 * 16;
   const int tiles = p.pair_tiles * p.n_tiles;
-  // split the pixel range so that the CTAs fill whole waves of SMs: time ~ waves x (K blocks per
-  // CTA + fixed prologue/epilogue worth about 4 K blocks)
-  {
-    int best_s = 1;
-    double best_t = 1e30;
-    const int max_s = std::min(p.pix_tiles, 64);
-    for (int sp = 1; sp <= max_s; ++sp) {
-      const int waves = (tiles * sp + sm_count - 1) / sm_count;
-      const double t = waves * ((double)((p.pix_tiles + sp - 1) / sp) + 4.0);
-      if (t < best_t - 1e-9) { best_t = t; best_s = sp; }
-    }
-    p.splits = best_s;
-  }
+  p.splits = wgrad_splits(tiles, p.pix_tiles, 1.0, sm_count, side_by_side);
   p.a_sub_bytes = (uint32_t)(p.rows_pad * p.sca * 2);
   p.b_sub_bytes = (uint32_t)(p.rows_pad * p.scb * 2);
   p.a_sub_bytes = (p.a_sub_bytes + 1023) / 1024 * 1024;
@@ -822,7 +824,7 @@ static int launch_wgrad_tc(WgEncodeFn enc, int sm_count, bool* attr_done, bool* 
   int stages = (int)((max_smem - tail) / p.stage_bytes);
   stages = std::min(stages, tc::kWgMaxStages);
   if (stages < 2) return shared_sm ? launch_wgrad_tc(enc, sm_count, attr_done, halo_attr_done, x, dy, dw, N, H, W, Cin, OH, OW, Cout,
-                                                     R, stride, pad, dev_err, st, false)
+                                                     R, stride, pad, dev_err, st, false, side_by_side)
                                    : -10;
   p.stages = stages;
   p.idesc = tc::instr_desc_bf16(128, p.n_tile, 1, 1);

@@ -300,6 +300,17 @@ def test_thin_layers_with_their_batch_norms_taken_along(ch, H, W, N):
     full_step_parity(cfg, steps=1)
 
 
+# (channels of the two stages, H, N): pixel ranges of 1, 3, 25 and 128 blocks, split into one part, into unequal parts, and
+# into fewer parts than the same launch would take alone
+@pytest.mark.parametrize("chs,H,N", [((16, 64), 8, 2), ((16, 32), 16, 6), ((64, 128), 14, 16), ((32, 128), 32, 16)])
+def test_weight_gradients_of_modules_side_by_side_over_split_pixel_ranges(chs, H, N):
+    """Weight gradients beside other modules' kernels take fewer, longer parts of the pixel range; one block per module,
+    bf16, one flat tolerance."""
+    cfg = small_cfg("postbn", N=N, H=H, W=H, dtype="bf16", stage_channels=chs, stage_blocks=(1, 1), module_block_end=(1, 2),
+                    stem_channels=chs[0], classes=10)
+    flat_module_parity(cfg, 0, 2e-2)
+
+
 def test_resnet56_reduced_batch_bf16():
     full_step_parity(scaled("resnet56", N=16), steps=1)
 
