@@ -1,0 +1,62 @@
+// Channel tile of the tensor-core convolutions (host code only, no CUDA: the rules are tested without a GPU).
+#pragma once
+#include <algorithm>
+
+namespace lp {
+
+// Fewest tiles of at most 256 channels with the least padding.
+inline void pick_n_tile(int Cout, int& n_tile, int& n_tiles) {
+  int best_nt = 0, best_tile = 0, best_waste = 1 << 30;
+  const int lo = (Cout + 255) / 256;
+  for (int nt = lo; nt <= lo + 3; ++nt) {
+    int tile = (Cout + nt - 1) / nt;
+    tile = (tile + 15) / 16 * 16;
+    if (tile > 256) continue;
+    const int waste = nt * tile - Cout;
+    if (waste < best_waste) { best_waste = waste; best_nt = nt; best_tile = tile; }
+  }
+  n_tile = best_tile;
+  n_tiles = best_nt;
+}
+
+struct ConvTileQuery {
+  int Cout, m_tiles, sm_count;
+  int k_mmas;        // K = 16 slices of a tile
+  int epilogue;      // 0 plain, 1 with statistics, 2 with a shortcut
+  bool wide_epi;     // eight epilogue warps at 256 channels
+};
+
+// Cycles of the busiest CTA.  A tile costs its MMAs (0.46 a column each, at least 82, or 75 where two accumulators
+// alternate: a pipeline stage of narrow MMAs takes that long with its waits and operand reads) and its epilogue, which runs
+// beside the next tile's MMAs; the first tile's MMAs, the last epilogue and 3800 cycles of start and end are not hidden.
+// The constants are fitted to 2334 timings of launches alone on the machine (3x3 and 1x1 layers of 64 to 2048 channels, 5 to
+// 56 pixels wide, 1 to 128 images, plain, with statistics and with a shortcut, every tile of 64 to 256 columns): of the 531
+// choices among them the fastest tile takes 0.828 of the time of pick_n_tile's in the geometric mean, the estimate's choice
+// 0.831, and it is at most 3 % slower than pick_n_tile's anywhere.  (The first form of this estimate, 33 cycles for a narrow
+// MMA and 20 a column for every epilogue, took 64 columns where 160 or 256 are faster: 320 -> 320 channels, 128 images of
+// 16x16 with statistics, 63.7 us instead of 50.6; 64 -> 256, 32 images of 56x56 with a shortcut, 51.0 instead of 29.2.)
+inline double conv_tile_cycles(const ConvTileQuery& q, int tile) {
+  static const double column[2][3] = {{29.0, 33.0, 25.0}, {28.0, 32.0, 18.0}};   // [eight warps][epilogue]
+  const long long tiles = (long long)q.m_tiles * ((q.Cout + tile - 1) / tile);
+  const double per = (double)((tiles + q.sm_count - 1) / q.sm_count);
+  const bool pair = q.m_tiles >= 2 && 2 * tiles >= 3 * std::min<long long>(tiles, q.sm_count);
+  const double mma = q.k_mmas * std::max(pair ? 75.0 : 82.0, tile * 0.46);
+  const double epi = 1250.0 + tile * column[q.wide_epi && tile == 256 ? 1 : 0][q.epilogue];
+  return 3800.0 + mma + epi + (per - 1.0) * std::max(mma, epi);
+}
+
+// Channel tile of a launch that has the machine to itself: the widest tiles leave SMs idle where there are few pixel tiles
+// (74 CTAs of 256 channels on 37 images of 12x16).  A narrower tile has to be estimated 2 % faster.
+inline void pick_n_tile_alone(const ConvTileQuery& q, int& n_tile, int& n_tiles) {
+  pick_n_tile(q.Cout, n_tile, n_tiles);
+  const int widest = n_tile, lo = (q.Cout + 255) / 256;
+  double best = conv_tile_cycles(q, widest);
+  for (int nt = lo; nt <= 8 * lo; ++nt) {
+    const int tile = ((q.Cout + nt - 1) / nt + 31) / 32 * 32;
+    if (tile > 256 || tile < 64 || tile == widest) continue;
+    const double t = conv_tile_cycles(q, tile);
+    if (t < best * 0.98) { best = t; n_tile = tile; n_tiles = (q.Cout + tile - 1) / tile; }
+  }
+}
+
+}  // namespace lp

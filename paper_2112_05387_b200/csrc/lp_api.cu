@@ -16,6 +16,7 @@
 #include "conv_simt.cuh"
 #include "conv_tc.cuh"
 #include "conv_tc2.cuh"
+#include "conv_tiles.h"
 #include "kernels_elem.cuh"
 #include "conv_thin.cuh"
 #include "net.h"
@@ -344,37 +345,6 @@ static int pick_kc(int Cin) {
   return best;
 }
 
-static void pick_n_tile(int Cout, int& n_tile, int& n_tiles) {
-  int best_nt = 0, best_tile = 0, best_waste = 1 << 30;
-  const int lo = (Cout + 255) / 256;
-  for (int nt = lo; nt <= lo + 3; ++nt) {
-    int tile = (Cout + nt - 1) / nt;
-    tile = (tile + 15) / 16 * 16;
-    if (tile > 256) continue;
-    const int waste = nt * tile - Cout;
-    if (waste < best_waste) { best_waste = waste; best_nt = nt; best_tile = tile; }
-  }
-  n_tile = best_tile;
-  n_tiles = best_nt;
-}
-
-// Channel tile of a launch that has the machine to itself: the widest tiles leave SMs idle where there are few pixel
-// tiles (74 CTAs of 256 channels on 37 images of 12x16).  Estimated cycles of the busiest CTA: an MMA takes N / 2 cycles,
-// and no less than 65 (33 where two accumulators alternate); about 4000 for start and end, 20 a column for the epilogue.
-static void pick_n_tile_alone(int Cout, int m_tiles, int k_mmas, int sm_count, int& n_tile, int& n_tiles) {
-  double best = 1e30;
-  const int lo = (Cout + 255) / 256;
-  for (int nt = lo; nt <= 8 * lo; ++nt) {
-    int tile = (Cout + nt - 1) / nt;
-    tile = (tile + 31) / 32 * 32;
-    if (tile > 256 || (nt > lo && tile < 64)) continue;
-    const int real = (Cout + tile - 1) / tile;
-    const int per = (m_tiles * real + sm_count - 1) / sm_count;
-    const double t = per * (k_mmas * std::max(per > 1 ? 33.0 : 65.0, tile * 0.5) + tile * 20.0) + 4000.0;
-    if (t < best * 0.98) { best = t; n_tile = tile; n_tiles = real; }
-  }
-}
-
 static int encode_act_map(CUtensorMap* m, const void* base, int N, int H, int W, int C, int boxC, int BW, int BH,
                           int BNI, int step, int row_bytes) {
   cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
@@ -649,8 +619,14 @@ static int launch_conv_tc(lp_handle* h, const TcGemmSpec& s, int* dev_err, cudaS
   const int tiles_n = (s.aN + p.BNI - 1) / p.BNI;
   p.m_tiles = p.tiles_w * p.tiles_h * tiles_n;
   pick_n_tile(s.w_rows, p.n_tile_cols, p.n_tiles);
-  if (!(h && h->concurrent) && s.n_cls <= 1 && s.w_rows % 32 == 0 && s.w_rows > 64)
-    pick_n_tile_alone(s.w_rows, p.m_tiles, s.ntaps * ((s.aC + 15) / 16), cur_dev().sm_count, p.n_tile_cols, p.n_tiles);
+  // Eight epilogue warps (below) may be taken: not by the epilogues that have four-warp scratch, and only where few MMAs
+  // hide a tile's epilogue.
+  const bool wide_ok = !bnbwd && !s.x_next && s.n_cls <= 1 && s.ntaps * s.aC <= 1024;
+  if (!(h && h->concurrent) && s.n_cls <= 1 && s.w_rows % 32 == 0 && s.w_rows > 64) {
+    const ConvTileQuery q{s.w_rows, p.m_tiles, cur_dev().sm_count, s.ntaps * ((s.aC + 15) / 16),
+                          s.addend || bnbwd ? 2 : (s.stats ? 1 : 0), wide_ok};
+    pick_n_tile_alone(q, p.n_tile_cols, p.n_tiles);
+  }
   p.n_cls = std::max(1, s.n_cls);
   int max_cls_taps = s.ntaps;
   if (s.n_cls > 1) {
@@ -692,8 +668,7 @@ static int launch_conv_tc(lp_handle* h, const TcGemmSpec& s, int* dev_err, cudaS
   // Eight epilogue warps where a tile's epilogue (about 31 cycles a column with four) is longer than its MMAs (N / 2 cycles
   // each) and the tile is a full 256 columns: the 1x1 convolutions of bottleneck blocks (ResNet-50 3.53 -> 3.50 ms per
   // step).  Elsewhere the second four warps only cost registers and shared memory (WRN-28-10 4.63 -> 4.65 ms).
-  const bool wide_epi = !thin && !bnbwd && !s.x_next && (staged ? s.addend != nullptr : s.addend == nullptr) &&
-                        p.n_tile_cols == 256 && s.n_cls <= 1 && s.ntaps * s.aC <= 1024;
+  const bool wide_epi = wide_ok && !thin && (staged ? s.addend != nullptr : s.addend == nullptr) && p.n_tile_cols == 256;
   const int epi_warps = wide_epi ? 8 : 4;
   const size_t max_smem = thin ? kTcThinSmem : kTcMaxSmem;
   const size_t stage_bytes = staged ? (size_t)(p.n_tile_cols / 32) * tc::kStageGroupBytes : 0;
