@@ -13,6 +13,7 @@
 
 #include "../../include/lp.h"
 #include "conv_f32.cuh"
+#include "conv_f32_rules.h"
 #include "conv_simt.cuh"
 #include "conv_tc.cuh"
 #include "conv_tc2.cuh"
@@ -914,6 +915,14 @@ static bool f32_tile_ok(const ConvDef& c) {
   return c.cin % 4 == 0 && c.cout % 4 == 0 && (c.R == 1 || c.R == 3) && c.pad == c.R / 2 && (c.stride == 1 || c.stride == 2) &&
          (reinterpret_cast<uintptr_t>(c.w) & 15) == 0;   // 16-byte copies of the weights (always, in a valid network's blob)
 }
+static F32Conv f32_shape(const ConvDef& c, int N) { return F32Conv{N, c.H, c.W, c.cin, c.OH, c.OW, c.cout, c.R, c.stride}; }
+// stems and first AuxNet convolutions: the direct kernel with the filter bank in shared memory
+static bool fewch_ok(const ConvDef& c, int dtype) {
+  return c.cin <= 4 && fewch_cpt(c.cout, dtype) && (size_t)c.R * c.R * c.cin * c.cout * 4 <= 48 * 1024;
+}
+static bool f32_forward_tiled(const ConvDef& c, int N) {
+  return f32_tile_ok(c) && f32_forward_on_tiles(f32_shape(c, N), fewch_ok(c, LP_F32));
+}
 static const size_t kF32MaxSmem = 100 * 1024;
 static int f32_set_attributes() {
   bool& done = cur_dev().f32_attr;
@@ -1196,15 +1205,14 @@ static int conv_forward(lp_handle* h, int dtype, int impl, const ConvDef& c, int
     return launch_conv_tc(h, s, dev_err, st);
   }
   if (c.cout % 4) return LP_ERR_UNSUPPORTED;
-  if (dtype == LP_F32 && f32_tile_ok(c)) {
+  if (dtype == LP_F32 && f32_forward_tiled(c, N)) {
     if (stats_done) *stats_done = stats != nullptr;
     return conv_forward_f32(h, c, N, (const float*)x, (float*)y, (const float*)addend, stats, st);
   }
   ConvGeom g{N, c.H, c.W, c.cin, c.OH, c.OW, c.cout, c.R, c.R, c.stride, c.pad};
   const size_t few_smem = (size_t)c.R * c.R * c.cin * c.cout * 4;
   const int few_cpt = fewch_cpt(c.cout, dtype);
-  if (c.cin <= 4 && !addend && few_cpt && few_smem <= 48 * 1024) {
-    // stems and the first AuxNet convolution: filter bank in shared memory
+  if (!addend && fewch_ok(c, dtype)) {
     const long long items = (long long)N * c.OH * c.OW * (c.cout / few_cpt);
     const int fgrid = grid_for(items, 256, cur_dev().sm_count, 8);
 #define LP_FEWCH_FWD(CPT)                                                                                      \
@@ -1327,7 +1335,7 @@ static int conv_dgrad(lp_handle* h, int dtype, int impl, const ConvDef& c, int N
     return LP_OK;
   }
   if (c.cin % 4) return LP_ERR_UNSUPPORTED;
-  if (dtype == LP_F32 && f32_tile_ok(c))
+  if (dtype == LP_F32 && f32_tile_ok(c) && f32_dgrad_on_tiles(f32_shape(c, N), cur_dev().sm_count))
     return conv_dgrad_f32(h, c, N, (const float*)dy, (float*)dx, (const float*)addend, st);
   ConvGeom g{N, c.H, c.W, c.cin, c.OH, c.OW, c.cout, c.R, c.R, c.stride, c.pad};
   const long long work = (long long)N * c.H * c.W * (c.cin / 4);
@@ -1557,7 +1565,7 @@ struct Planner {
   }
 
   bool conv_fuses_stats(const ConvDef& c) const {
-    if (dtype == LP_F32) return f32_tile_ok(c);
+    if (dtype == LP_F32) return f32_forward_tiled(c, net.d.N);
     return dtype == LP_BF16 && impl != LP_CONV_IMPL_SIMT && !(net.d.conv_impl & 16) && (tc_fwd_ok(c) || c.s2d) && c.wf;
   }
   Tensor emit_conv(Plan& P, std::vector<Op>& ops, const Tensor& in, int conv, const Tensor* addend, int stats_bn) {

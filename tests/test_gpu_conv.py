@@ -243,3 +243,13 @@ def test_tensor_conv_dgrad_stride_2_of_odd_sizes_matches_oracle(case):
     st, dx, _ = run_conv(lp.LP_CONV_DGRAD, "bf16", lp.LP_CONV_IMPL_TENSOR, *case, dy, w)
     assert st == 0, lp.lp_status_string(st)
     assert rel_err(dx, O.conv_dgrad(dy, w, stride, pad, x.shape)) < 6e-3
+
+
+# fp32 shapes on both sides of the lines between the tiled and the direct kernels: 4 channels into 16 at 496 and 512 tiles,
+# 8 into 8 (1x1) at 396, 4 into 4 at 1024, and two 1x1 input gradients that the direct kernel takes
+@pytest.mark.parametrize("case", [(31, 32, 32, 4, 16, 3, 1, 1), (32, 32, 32, 4, 16, 3, 1, 1), (33, 24, 32, 8, 8, 1, 1, 0),
+                                  (64, 32, 32, 4, 4, 3, 1, 1), (130, 9, 9, 20, 12, 1, 1, 0), (24, 11, 11, 128, 128, 1, 1, 0)])
+def test_fp32_convolutions_on_either_side_of_the_dispatch_match_oracle(case):
+    """K is at most 65536 here (weight gradients): sqrt(K) x 2^-24 = 1.6e-5 in the worst case, 1e-5 measured for sums in
+    tiles; the bound of the tiled kernels holds."""
+    test_fp32_tile_kernels_match_oracle(case)

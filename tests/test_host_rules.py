@@ -72,3 +72,41 @@ def test_channel_tiles_cover_the_channels(tile_rules):
                     tile, n_tiles = tile_rules(cout, m_tiles, k, epilogue, k < 60)
                     assert 16 <= tile <= 256 and tile % 16 == 0
                     assert (n_tiles - 1) * tile < cout <= n_tiles * tile
+
+
+@pytest.fixture(scope="module")
+def f32_rules(tmp_path_factory):
+    return build_host(tmp_path_factory.mktemp("f32"), "f32", """
+#include "conv_f32_rules.h"
+extern "C" int forward(int N, int H, int cin, int cout, int R, int s, int few) {
+  const int o = (H - 1) / s + 1;
+  return lp::f32_forward_on_tiles(lp::F32Conv{N, H, H, cin, o, o, cout, R, s}, few != 0);
+}
+extern "C" int dgrad(int N, int H, int cin, int cout, int R, int s) {
+  const int o = (H - 1) / s + 1;
+  return lp::f32_dgrad_on_tiles(lp::F32Conv{N, H, H, cin, o, o, cout, R, s}, 148);
+}
+""")
+
+
+# (N, H = W, C_in, C_out, R, stride): microseconds on the tiled and on the direct kernel, measured alone on a B200
+@pytest.mark.parametrize("c,tiled,direct", [
+    ((64, 32, 4, 64, 3, 1), 48.4, 22.6), ((128, 32, 4, 16, 3, 1), 28.1, 14.6), ((64, 32, 4, 64, 1, 1), 29.1, 10.3),
+    ((128, 32, 4, 4, 3, 1), 20.6, 11.4), ((128, 32, 8, 8, 1, 1), 15.1, 8.3), ((128, 32, 4, 64, 3, 2), 34.0, 15.4),
+    ((4, 32, 4, 64, 3, 1), 7.3, 14.4), ((1, 32, 4, 64, 1, 1), 3.2, 6.2), ((32, 32, 16, 16, 3, 1), 14.0, 60.0),
+    ((64, 14, 64, 256, 1, 1), 59.1, 733.0), ((64, 32, 16, 32, 1, 2), 7.8, 12.4),
+])
+def test_fp32_forward_takes_the_faster_kernel(f32_rules, c, tiled, direct):
+    few = c[2] <= 4 and c[3] % 8 == 0
+    assert bool(f32_rules.forward(*c, int(few))) == (tiled < direct)
+
+
+@pytest.mark.parametrize("c,tiled,direct", [
+    ((64, 28, 128, 128, 1, 1), 205.3, 133.3), ((24, 28, 128, 128, 1, 1), 80.7, 59.5), ((64, 14, 256, 64, 1, 1), 55.9, 41.0),
+    ((16, 56, 256, 64, 1, 1), 165.7, 135.9), ((64, 11, 128, 128, 1, 1), 53.6, 36.2), ((128, 32, 4, 4, 1, 1), 9.1, 5.2),
+    ((128, 32, 4, 4, 3, 1), 18.1, 12.4),
+    ((4, 28, 128, 128, 1, 1), 19.6, 23.8), ((64, 7, 512, 512, 1, 1), 204.7, 233.7), ((16, 7, 512, 512, 1, 1), 74.3, 82.0),
+    ((128, 32, 8, 64, 1, 1), 31.3, 49.2), ((64, 16, 32, 64, 1, 2), 8.9, 14.4), ((64, 32, 16, 16, 3, 1), 24.4, 53.3),
+])
+def test_fp32_input_gradient_takes_the_faster_kernel(f32_rules, c, tiled, direct):
+    assert bool(f32_rules.dgrad(*c)) == (tiled < direct)
