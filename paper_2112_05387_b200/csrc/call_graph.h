@@ -1,0 +1,65 @@
+// A call of the C ABI as one graph launch (host code; the CUDA runtime calls are the only dependency, so that the paths taken
+// when one of them fails are tested with fakes, without a GPU).
+#pragma once
+#include <cuda_runtime_api.h>
+
+#include "../../include/lp.h"
+
+namespace lp {
+
+// Executable graph of one entry point of a handle.
+struct CallGraph {
+  cudaGraphExec_t exec = nullptr;
+  int calls = 0, rebuilt = 0;
+  bool off = false;
+};
+
+// Runs `enqueue(stream)` as ONE graph launch on `st`.  A call is some hundred launches of a few microseconds each; made one
+// by one, each costs the host 3 to 5 us, so that small networks wait for the host (ResNet-56 on 20 images in three calls:
+// 915 us, 362 as graph launches) and large ones lose the overlap of launches across streams.  The call is recorded anew every
+// time, with this call's pointers and arguments, on a stream of the handle's own (recording a launch costs a fraction of
+// making it), the executable graph of the previous call is updated to the recording, and launched; only its topology and
+// memory are kept.  The first two calls of a kind, calls inside a caller's capture, and profiled calls (`direct`) launch
+// directly.  `enqueue` changes host state (which gradients are fresh, launch counts) as if its work had been launched:
+// `restore` puts that back wherever a recording does not become a launch.
+template <typename Enqueue, typename Restore>
+int run_as_graph(CallGraph& g, cudaStream_t capture, cudaStream_t st, bool direct, Enqueue enqueue, Restore restore) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) { cudaGetLastError(); return enqueue(st); }
+  if (cs != cudaStreamCaptureStatusNone || direct || g.off || !capture || ++g.calls <= 2) return enqueue(st);
+  if (cudaStreamBeginCapture(capture, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+    cudaGetLastError();
+    g.off = true;
+    return enqueue(st);
+  }
+  const int rc = enqueue(capture);
+  cudaGraph_t graph = nullptr;
+  cudaError_t e = cudaStreamEndCapture(capture, &graph);
+  if (rc != LP_OK) {               // (an argument or launch error: nothing has run)
+    if (graph) cudaGraphDestroy(graph);
+    cudaGetLastError();
+    restore();
+    return rc;
+  }
+  if (e == cudaSuccess && g.exec) {
+    cudaGraphExecUpdateResultInfo info;
+    if (cudaGraphExecUpdate(g.exec, graph, &info) != cudaSuccess) {   // other options than last time: other nodes
+      cudaGetLastError();
+      cudaGraphExecDestroy(g.exec);
+      g.exec = nullptr;
+      g.off = ++g.rebuilt >= 4;        // a caller that keeps changing them is better off without
+    }
+  }
+  if (e == cudaSuccess && !g.exec) e = cudaGraphInstantiate(&g.exec, graph, 0);
+  if (e == cudaSuccess) e = cudaGraphLaunch(g.exec, st);
+  if (graph) cudaGraphDestroy(graph);
+  if (e != cudaSuccess) {          // recording does not work here: launch directly from now on
+    cudaGetLastError();
+    g.off = true;
+    restore();
+    return enqueue(st);
+  }
+  return LP_OK;
+}
+
+}  // namespace lp

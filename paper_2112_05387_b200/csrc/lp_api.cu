@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "../../include/lp.h"
+#include "call_graph.h"
 #include "conv_f32.cuh"
 #include "conv_f32_rules.h"
 #include "conv_simt.cuh"
@@ -242,13 +243,8 @@ struct ConvProfile {
 
 using namespace lp;
 
-// Executable graph of one entry point of a handle (see run_as_graph).
+// Entry points that run as one graph launch (call_graph.h).
 enum { CALL_AUX_FORWARD = 0, CALL_MODULES, CALL_STEP, CALL_LAYER_PARALLEL, CALL_DISTILL, CALL_FORWARD_SERIAL, CALL_SERIAL, CALL_KINDS };
-struct CallGraph {
-  cudaGraphExec_t exec = nullptr;
-  int calls = 0, rebuilt = 0;
-  bool off = false;
-};
 
 struct lp_handle {
   NetDef net;
@@ -2426,53 +2422,34 @@ static int module_fwd_bwd(lp_handle* h, int k, const void* x_k, const void* x_ne
   return LP_OK;
 }
 
-// Runs `enqueue(stream)` as ONE graph launch on `st`.  A call is some hundred launches of a few microseconds each; made one
-// by one, each costs the host 3 to 5 us, so that small networks wait for the host (ResNet-56 on 20 images in three calls:
-// 1136 us of host time for 362 us of work) and large ones lose the overlap of launches across streams.  The call is
-// recorded anew every time, with this call's pointers and arguments, on a stream of the handle's own (recording a launch
-// costs a fraction of making it), the executable graph of the previous call is updated to the recording, and launched;
-// only its topology and memory are kept.  The first two calls of a kind (which also set kernel attributes), calls inside a
-// caller's capture, and profiled calls launch directly.
+// What an enqueued call has changed on the host: the state of the parameter sets and the launch count.
+struct HostState {
+  uint32_t fresh = 0, ran = 0;      // bit k: module k
+  int64_t launches = 0;
+};
+static_assert(LP_MAX_MODULES <= 32, "one bit per module");
+static HostState host_state(const lp_handle* h) {
+  HostState s;
+  for (size_t k = 0; k < h->modules.size(); ++k) {
+    s.fresh |= (uint32_t)h->modules[k].ps.grads_fresh << k;
+    s.ran |= (uint32_t)h->modules[k].ran_fwd_bwd << k;
+  }
+  s.launches = h->launches;
+  return s;
+}
+static void set_host_state(lp_handle* h, const HostState& s) {
+  for (size_t k = 0; k < h->modules.size(); ++k) {
+    h->modules[k].ps.grads_fresh = (s.fresh >> k) & 1;
+    h->modules[k].ran_fwd_bwd = (s.ran >> k) & 1;
+  }
+  h->launches = s.launches;
+}
+
 template <typename F>
 static int run_as_graph(lp_handle* h, int kind, cudaStream_t st, F enqueue) {
-  CallGraph& g = h->call_graph[kind];
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) { cudaGetLastError(); return enqueue(st); }
-  if (cs != cudaStreamCaptureStatusNone || h->prof.enabled || h->tl.enabled || g.off || !h->capture_stream || ++g.calls <= 2)
-    return enqueue(st);
-  if (cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-    cudaGetLastError();
-    g.off = true;
-    return enqueue(st);
-  }
-  const int64_t launches = h->launches;
-  const int rc = enqueue(h->capture_stream);
-  cudaGraph_t graph = nullptr;
-  cudaError_t e = cudaStreamEndCapture(h->capture_stream, &graph);
-  if (rc != LP_OK) {               // (an argument or launch error: nothing has run)
-    if (graph) cudaGraphDestroy(graph);
-    cudaGetLastError();
-    return rc;
-  }
-  if (e == cudaSuccess && g.exec) {
-    cudaGraphExecUpdateResultInfo info;
-    if (cudaGraphExecUpdate(g.exec, graph, &info) != cudaSuccess) {   // other options than last time: other nodes
-      cudaGetLastError();
-      cudaGraphExecDestroy(g.exec);
-      g.exec = nullptr;
-      g.off = ++g.rebuilt >= 4;        // a caller that keeps changing them is better off without
-    }
-  }
-  if (e == cudaSuccess && !g.exec) e = cudaGraphInstantiate(&g.exec, graph, 0);
-  if (e == cudaSuccess) e = cudaGraphLaunch(g.exec, st);
-  if (graph) cudaGraphDestroy(graph);
-  if (e != cudaSuccess) {          // recording does not work here: launch directly from now on
-    cudaGetLastError();
-    g.off = true;
-    h->launches = launches;
-    return enqueue(st);
-  }
-  return LP_OK;
+  const HostState before = host_state(h);
+  return run_as_graph(h->call_graph[kind], h->capture_stream, st, h->prof.enabled || h->tl.enabled, enqueue,
+                      [&] { set_host_state(h, before); });
 }
 
 }  // namespace lp
@@ -2818,11 +2795,9 @@ int lp_step(lp_handle* h, float lr, float momentum, float weight_decay, float ka
   if (lambdas_inout)
     for (int k = 0; k + 1 < K; ++k)
       if (lambdas_inout[k] && !aligned16(lambdas_inout[k])) return LP_ERR_ALIGN;
-  std::vector<bool> fresh(K);            // (the flags go down with the first enqueue: a second one needs them as they were)
-  for (int k = 0; k < K; ++k) fresh[k] = h->modules[k].ps.grads_fresh;
   return run_as_graph(h, CALL_STEP, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   for (int k = 0; k < K; ++k) {
-    if (!fresh[k]) continue;
+    if (!h->modules[k].ps.grads_fresh) continue;
     int rc = update_module(h, k, lr, momentum, weight_decay, kappa_step,
                            (lambdas_inout && k + 1 < K) ? lambdas_inout[k] : nullptr, st);
     if (rc != LP_OK) return rc;
