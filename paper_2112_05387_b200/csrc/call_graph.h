@@ -27,7 +27,8 @@ int run_as_graph(CallGraph& g, cudaStream_t capture, cudaStream_t st, bool direc
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) { cudaGetLastError(); return enqueue(st); }
   if (cs != cudaStreamCaptureStatusNone || direct || g.off || !capture || ++g.calls <= 2) return enqueue(st);
-  if (cudaStreamBeginCapture(capture, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+  // (relaxed, as lp_graph_begin: a kernel that is launched for the first time may be loaded then)
+  if (cudaStreamBeginCapture(capture, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
     cudaGetLastError();
     g.off = true;
     return enqueue(st);
@@ -35,12 +36,13 @@ int run_as_graph(CallGraph& g, cudaStream_t capture, cudaStream_t st, bool direc
   const int rc = enqueue(capture);
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamEndCapture(capture, &graph);
-  if (rc != LP_OK) {               // (an argument or launch error: nothing has run)
+  if (rc != LP_OK && rc != LP_ERR_CUDA) {   // refused (nothing has run): a direct call would be too
     if (graph) cudaGraphDestroy(graph);
     cudaGetLastError();
     restore();
     return rc;
   }
+  if (rc == LP_ERR_CUDA) e = cudaErrorUnknown;   // something that a recording does not take, or a real error: direct, below
   if (e == cudaSuccess && g.exec) {
     cudaGraphExecUpdateResultInfo info;
     if (cudaGraphExecUpdate(g.exec, graph, &info) != cudaSuccess) {   // other options than last time: other nodes

@@ -11,7 +11,7 @@ CSRC = os.path.join(ROOT, "paper_2112_05387_b200", "csrc")
 FAKE_RUNTIME = """
 #pragma once
 typedef int cudaError_t;
-enum { cudaSuccess = 0, cudaErrorFake = 1 };
+enum { cudaSuccess = 0, cudaErrorFake = 1, cudaErrorUnknown = 999 };
 typedef struct FakeStream* cudaStream_t;
 typedef struct FakeGraph* cudaGraph_t;
 typedef struct FakeExec* cudaGraphExec_t;
@@ -129,6 +129,27 @@ SCENARIOS = {
       h.call(); h.call();
       fake.fail_begin = true;
       CHECK(h.call() == LP_OK && h.done == 15 && h.launches == 15);
+    """,
+    "what only a recording refuses is made directly, now and from then on": """
+      h.call(); h.call(); h.call();
+      h.rc_recording = LP_ERR_CUDA;
+      CHECK(h.call() == LP_OK && h.done == 15 && h.launches == 20 && h.fresh);
+      CHECK(h.call() == LP_OK && h.done == 20 && fake.begin == 2);
+      CHECK(fake.live_graphs == 0);
+    """,
+    "an error of the direct call too is returned": """
+      h.call(); h.call();
+      h.rc = LP_ERR_CUDA;
+      CHECK(h.call() == LP_ERR_CUDA && fake.launch == 0);
+    """,
+    "a recording that cannot be ended is made directly": """
+      h.call(); h.call();
+      fake.fail_end = true;
+      CHECK(h.call() == LP_OK && h.done == 15 && h.launches == 15);
+    """,
+    "the mode of lp_graph_begin": """
+      h.call(); h.call(); h.call();
+      CHECK(fake.mode == cudaStreamCaptureModeRelaxed);
     """,
     "profiled calls and calls inside a caller's capture are enqueued as they are": """
       h.call(); h.call();
