@@ -10,9 +10,14 @@ namespace lp {
 // Executable graph of one entry point of a handle.
 struct CallGraph {
   cudaGraphExec_t exec = nullptr;
-  int calls = 0, rebuilt = 0;
+  int calls = 0;
+  int rebuilt = 0, kept = 0;       // executable graphs given up; launches since the last one
   bool off = false;
 };
+// A caller that changes the launches of a call (multipliers given or not, another loss) pays for a new executable graph:
+// once in a while it is worth it, at every other call it is not.  After kMaxRebuilt of them without kForgiveAfter launches
+// of one graph in a row the calls are launched directly.
+constexpr int kMaxRebuilt = 4, kForgiveAfter = 16;
 
 // Runs `enqueue(stream)` as ONE graph launch on `st`.  A call is some hundred launches of a few microseconds each; made one
 // by one, each costs the host 3 to 5 us, so that small networks wait for the host (ResNet-56 on 20 images in three calls:
@@ -49,7 +54,10 @@ int run_as_graph(CallGraph& g, cudaStream_t capture, cudaStream_t st, bool direc
       cudaGetLastError();
       cudaGraphExecDestroy(g.exec);
       g.exec = nullptr;
-      g.off = ++g.rebuilt >= 4;        // a caller that keeps changing them is better off without
+      g.kept = 0;
+      g.off = ++g.rebuilt >= kMaxRebuilt;
+    } else if (++g.kept >= kForgiveAfter) {
+      g.rebuilt = g.kept = 0;
     }
   }
   if (e == cudaSuccess && !g.exec) e = cudaGraphInstantiate(&g.exec, graph, 0);

@@ -151,6 +151,19 @@ SCENARIOS = {
       h.call(); h.call(); h.call();
       CHECK(fake.mode == cudaStreamCaptureModeRelaxed);
     """,
+    "launches that change now and then stay graph launches": """
+      h.call(); h.call();
+      for (int epoch = 0; epoch < 12; ++epoch) {
+        h.topology = epoch & 1;
+        for (int i = 0; i < 20; ++i) h.call();
+      }
+      CHECK(fake.instantiate == 12 && h.done == 10 && fake.launch == 240 && fake.live_execs == 1);
+    """,
+    "launches that change all the time are made directly": """
+      h.call(); h.call();
+      for (int i = 0; i < 40; ++i) { h.topology = i & 1; CHECK(h.call() == LP_OK); }
+      CHECK(fake.instantiate == 5 && h.ran() == 5 * 42 && h.done == 5 * (2 + 35));
+    """,
     "profiled calls and calls inside a caller's capture are enqueued as they are": """
       h.call(); h.call();
       h.profiled = true;
