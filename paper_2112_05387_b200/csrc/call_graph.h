@@ -10,10 +10,12 @@ namespace lp {
 // Executable graph of one entry point of a handle.
 struct CallGraph {
   cudaGraphExec_t exec = nullptr;
-  int calls = 0;
+  int direct_calls = 0;            // of the first kDirectCalls
   int rebuilt = 0, kept = 0;       // executable graphs given up; launches since the last one
   bool off = false;
 };
+// The first calls of a kind are launched directly: a program that makes one or two does not pay for a graph.
+constexpr int kDirectCalls = 2;
 // A caller that changes the launches of a call (multipliers given or not, another loss) pays for a new executable graph:
 // once in a while it is worth it, at every other call it is not.  After kMaxRebuilt of them without kForgiveAfter launches
 // of one graph in a row the calls are launched directly.
@@ -31,7 +33,8 @@ template <typename Enqueue, typename Restore>
 int run_as_graph(CallGraph& g, cudaStream_t capture, cudaStream_t st, bool direct, Enqueue enqueue, Restore restore) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) { cudaGetLastError(); return enqueue(st); }
-  if (cs != cudaStreamCaptureStatusNone || direct || g.off || !capture || ++g.calls <= 2) return enqueue(st);
+  if (cs != cudaStreamCaptureStatusNone || direct || g.off || !capture) return enqueue(st);
+  if (g.direct_calls < kDirectCalls) { ++g.direct_calls; return enqueue(st); }
   // (relaxed, as lp_graph_begin: a kernel that is launched for the first time may be loaded then)
   if (cudaStreamBeginCapture(capture, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
     cudaGetLastError();

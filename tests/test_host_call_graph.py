@@ -164,6 +164,10 @@ SCENARIOS = {
       for (int i = 0; i < 40; ++i) { h.topology = i & 1; CHECK(h.call() == LP_OK); }
       CHECK(fake.instantiate == 5 && h.ran() == 5 * 42 && h.done == 5 * (2 + 35));
     """,
+    "no count runs over": """
+      for (int i = 0; i < 100; ++i) h.call();
+      CHECK(h.g.direct_calls == 2 && h.g.rebuilt == 0 && h.g.kept < kForgiveAfter);   // the only counts that a call keeps
+    """,
     "profiled calls and calls inside a caller's capture are enqueued as they are": """
       h.call(); h.call();
       h.profiled = true;
