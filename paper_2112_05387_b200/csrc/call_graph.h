@@ -21,6 +21,29 @@ constexpr int kDirectCalls = 2;
 // of one graph in a row the calls are launched directly.
 constexpr int kMaxRebuilt = 4, kForgiveAfter = 16;
 
+// Stream that a handle's calls are recorded on.  A kernel of a graph runs at the priority of the stream it was recorded on, so
+// it has the priority of the caller's stream (of the first one that a call is recorded for; calls on streams of another
+// priority are launched directly).
+struct CaptureStream {
+  cudaStream_t stream = nullptr;
+  int priority = 0;
+  bool failed = false;
+};
+inline cudaStream_t capture_stream_for(CaptureStream& c, cudaStream_t st) {
+  int priority = 0;
+  if (c.failed || cudaStreamGetPriority(st, &priority) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+  if (!c.stream) {
+    if (cudaStreamCreateWithPriority(&c.stream, cudaStreamNonBlocking, priority) != cudaSuccess) {
+      cudaGetLastError();
+      c.stream = nullptr;
+      c.failed = true;
+      return nullptr;
+    }
+    c.priority = priority;
+  }
+  return c.priority == priority ? c.stream : nullptr;
+}
+
 // Runs `enqueue(stream)` as ONE graph launch on `st`.  A call is some hundred launches of a few microseconds each; made one
 // by one, each costs the host 3 to 5 us, so that small networks wait for the host (ResNet-56 on 20 images in three calls:
 // 915 us, 362 as graph launches) and large ones lose the overlap of launches across streams.  The call is recorded anew every
@@ -30,11 +53,13 @@ constexpr int kMaxRebuilt = 4, kForgiveAfter = 16;
 // directly.  `enqueue` changes host state (which gradients are fresh, launch counts) as if its work had been launched:
 // `restore` puts that back wherever a recording does not become a launch.
 template <typename Enqueue, typename Restore>
-int run_as_graph(CallGraph& g, cudaStream_t capture, cudaStream_t st, bool direct, Enqueue enqueue, Restore restore) {
+int run_as_graph(CallGraph& g, CaptureStream& capture_stream, cudaStream_t st, bool direct, Enqueue enqueue, Restore restore) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) { cudaGetLastError(); return enqueue(st); }
-  if (cs != cudaStreamCaptureStatusNone || direct || g.off || !capture) return enqueue(st);
+  if (cs != cudaStreamCaptureStatusNone || direct || g.off) return enqueue(st);
   if (g.direct_calls < kDirectCalls) { ++g.direct_calls; return enqueue(st); }
+  const cudaStream_t capture = capture_stream_for(capture_stream, st);
+  if (!capture) return enqueue(st);
   // (relaxed, as lp_graph_begin: a kernel that is launched for the first time may be loaded then)
   if (cudaStreamBeginCapture(capture, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
     cudaGetLastError();

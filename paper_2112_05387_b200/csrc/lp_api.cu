@@ -266,7 +266,7 @@ struct lp_handle {
   size_t ws_bytes = 0;
   int32_t* zero_labels = nullptr;  // N zeros, for forward passes that only want logits
   CallGraph call_graph[CALL_KINDS];
-  cudaStream_t capture_stream = nullptr;
+  CaptureStream capture_stream;
   std::vector<cudaGraphExec_t> graphs;
   int64_t launches_at_capture = 0;
   std::vector<int64_t> graph_launches;  // kernels recorded in each graph
@@ -2587,7 +2587,6 @@ int lp_create(const lp_net_desc* desc, void* dev_workspace, size_t bytes, lp_han
     }
   }
   if (cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
-  if (cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
   if (cudaStreamCreateWithFlags(&h->aux_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->aux_end, cudaEventDisableTiming) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
   h->aux_done.resize(net.K > 1 ? net.K - 1 : 0);
@@ -2604,7 +2603,7 @@ int lp_destroy(lp_handle* h) {
   for (auto e : h->done) if (e) cudaEventDestroy(e);
   if (h->fork) cudaEventDestroy(h->fork);
   for (auto& g : h->call_graph) if (g.exec) cudaGraphExecDestroy(g.exec);
-  if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
+  if (h->capture_stream.stream) cudaStreamDestroy(h->capture_stream.stream);
   if (h->aux_stream) cudaStreamDestroy(h->aux_stream);
   if (h->aux_end) cudaEventDestroy(h->aux_end);
   for (auto e : h->aux_done) if (e) cudaEventDestroy(e);

@@ -24,10 +24,18 @@ struct FakeExec { int nodes, topology; };
 // how often each call has been made, and which of them fail from now on
 struct Fake { int begin, end, update, instantiate, launch, live_graphs, live_execs, live_streams, launched_nodes; bool fail_begin, fail_end, fail_instantiate, fail_launch, fail_stream; cudaStreamCaptureMode mode; };
 extern Fake fake;
-extern FakeStream* capturing_stream;
+
 inline cudaError_t cudaGetLastError() { return cudaSuccess; }
 inline cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* c) {
   *c = s->capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+  return cudaSuccess;
+}
+enum { cudaStreamNonBlocking = 1 };
+inline cudaError_t cudaStreamGetPriority(cudaStream_t s, int* p) { *p = s->priority; return cudaSuccess; }
+inline cudaError_t cudaStreamCreateWithPriority(cudaStream_t* s, unsigned, int p) {
+  if (fake.fail_stream) return cudaErrorFake;
+  *s = new FakeStream; (*s)->priority = p;
+  ++fake.live_streams;
   return cudaSuccess;
 }
 inline cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode m) {
@@ -77,17 +85,19 @@ using namespace lp;
 // A handle's host state and a call that changes it: five launches and a flag.
 struct Handle {
   CallGraph g;
-  FakeStream capture, user;
+  CaptureStream capture;
+  FakeStream user;
   bool fresh = false;
   int launches = 0, done = 0;      // launches counted; launched directly
   int topology = 0, rc = LP_OK, rc_recording = LP_OK;
   bool profiled = false;
+  int recorded_priority = 99;
   int call() {
     const bool f = fresh; const int l = launches;
-    return run_as_graph(g, &capture, &user, profiled, [&](cudaStream_t s) -> int {
+    return run_as_graph(g, capture, &user, profiled, [&](cudaStream_t s) -> int {
       fresh = true;
       launches += 5;
-      if (s->capturing) { s->recorded = 5; s->topology = topology; if (rc_recording != LP_OK) return rc_recording; }
+      if (s->capturing) { s->recorded = 5; recorded_priority = s->priority; s->topology = topology; if (rc_recording != LP_OK) return rc_recording; }
       else done += 5;
       return rc;
     }, [&] { fresh = f; launches = l; });
@@ -167,6 +177,20 @@ SCENARIOS = {
     "no count runs over": """
       for (int i = 0; i < 100; ++i) h.call();
       CHECK(h.g.direct_calls == 2 && h.g.rebuilt == 0 && h.g.kept < kForgiveAfter);   // the only counts that a call keeps
+    """,
+    "recorded at the priority of the caller's stream": """
+      h.user.priority = -5;
+      for (int i = 0; i < 4; ++i) h.call();
+      CHECK(h.recorded_priority == -5 && fake.launch == 2 && fake.live_streams == 1);
+      h.user.priority = 0;                       // another stream: neither recorded at -5 nor a graph of its own
+      CHECK(h.call() == LP_OK && h.done == 15 && fake.launch == 2 && fake.live_streams == 1);
+      h.user.priority = -5;
+      CHECK(h.call() == LP_OK && fake.launch == 3);
+    """,
+    "no stream to record on": """
+      fake.fail_stream = true;
+      for (int i = 1; i <= 5; ++i) CHECK(h.call() == LP_OK && h.done == 5 * i);
+      CHECK(fake.begin == 0);
     """,
     "profiled calls and calls inside a caller's capture are enqueued as they are": """
       h.call(); h.call();
