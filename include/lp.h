@@ -312,7 +312,7 @@ int lp_graph_launch(lp_handle* h, int graph_id, void* stream);
  * op = LP_CONV_WGRAD: a = x,               b = dy (activation dtype),  out = dw fp32 [Cout,R,R,Cin]
  * scratch: device buffer of lp_conv2d_scratch_bytes() (packed bf16 weights, statistics).
  * stats (nullable, FWD only): device double[2*Cout] receives per-channel sum and sum of squares
- * of y.  Returns LP_ERR_UNSUPPORTED if `impl` cannot run this shape. */
+ * of y (Cout a multiple of 8 in LP_BF16).  Returns LP_ERR_UNSUPPORTED if `impl` cannot run this shape. */
 size_t lp_conv2d_scratch_bytes(int Cin, int Cout, int R);
 int lp_conv2d(int op, int dtype, int impl, int N, int H, int W, int Cin, int Cout, int R,
               int stride, int pad, const void* a, const void* b, void* out, double* stats,

@@ -292,6 +292,7 @@ static inline int grid_for(long long work_items, int threads, int sm_count, int 
 static inline int threads_for_channels(int C, int dtype) {
   const int V = dtype == LP_F32 ? 4 : 8;
   const int CV = C / V;
+  if (C % V || CV < 1) return 0;
   if (CV >= 256) return CV <= 1024 ? CV : 0;
   return CV * (256 / CV);
 }
@@ -3176,6 +3177,7 @@ int lp_conv2d(int op, int dtype, int impl, int N, int H, int W, int Cin, int Cou
   if (!a || !b || !out || !scratch) return LP_ERR_NULL;
   if (N < 1 || H < 1 || W < 1 || Cin < 1 || Cout < 1 || R < 1 || stride < 1 || pad < 0) return LP_ERR_SIZE;
   if (scratch_bytes < lp_conv2d_scratch_bytes(Cin, Cout, R)) return LP_ERR_WORKSPACE;
+  if (op == LP_CONV_FWD && stats && Cout % (dtype == LP_F32 ? 4 : 8)) return LP_ERR_UNSUPPORTED;   // (statistics read 16 bytes at a time)
   if (!aligned16(a) || !aligned16(b) || !aligned16(out) || (reinterpret_cast<uintptr_t>(scratch) & 255)) return LP_ERR_ALIGN;
   int rc = init_cur_dev();
   if (rc != LP_OK) return rc;

@@ -127,3 +127,11 @@ def test_recursive_auxnet_layouts_match_the_oracle():
         lp.lp_param_layout(desc, lp.LP_REAUX(net.K, 0))
     desc.aux_recursive = 2
     assert lp.lp_validate_desc(desc) != 0
+
+
+@pytest.mark.parametrize("dtype,cout", [(lp.LP_BF16, 4), (lp.LP_BF16, 12), (lp.LP_F32, 6)])
+def test_statistics_of_channel_counts_off_the_vector_width_are_refused(dtype, cout):
+    """Host check, made before anything is launched (the pointers are never followed)."""
+    p = ctypes.c_void_p(1 << 20)
+    rc = lp.library().lp_conv2d(lp.LP_CONV_FWD, dtype, lp.LP_CONV_IMPL_AUTO, 2, 8, 8, 8, cout, 3, 1, 1, p, p, p, p, p, 1 << 20, None, None)
+    assert lp.lp_status_string(rc) == "unsupported"
