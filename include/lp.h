@@ -156,7 +156,10 @@ int lp_boundary_shape_desc(const lp_net_desc* desc, int k, int shape_nhwc[4]);
 /* Create a handle over the caller's device workspace.  The call zero-fills the workspace with a
  * synchronous cudaMemset (it returns after the fill; work of the caller still running on other
  * streams must not touch the workspace meanwhile); parameters start at zero until lp_set_params.
- * The handle owns host memory, streams and events only. */
+ * The handle owns host memory, streams, events and -- from the third call of a kind on -- one executable graph for each
+ * of lp_auxnet_forward, lp_modules_fwd_bwd_all, lp_step, lp_layer_parallel_step, lp_auxnet_distill, lp_forward_serial and
+ * lp_serial_fwd_bwd, as which the call is then launched (recorded anew each time with its own arguments).  The driver
+ * keeps the nodes of such a graph in device memory of its own; lp_destroy gives it back. */
 int lp_create(const lp_net_desc* desc, void* dev_workspace, size_t bytes, lp_handle** out);
 int lp_destroy(lp_handle* h);
 
@@ -253,6 +256,10 @@ int lp_last_device_status(lp_handle* h, void* stream);
 int lp_selftest_bounded_wait(lp_handle* h, double limit_ms, double* waited_ms, void* stream);
 /* Number of kernels the library launched since the counter was last reset. */
 int64_t lp_launch_count(lp_handle* h, int reset);
+/* How the calls that may become graph launches (see lp_create) were made since lp_create: as graph launches, with how many
+ * executable graphs built, and launch by launch (the first two of a kind, calls while a profile or the time line is
+ * enabled or inside a caller's capture, and calls whose launches change too often).  Any pointer may be NULL. */
+int lp_call_graphs(lp_handle* h, int64_t* launched, int64_t* built, int64_t* direct);
 /* Time (ms, CUDA events on the launching stream) spent in tensor-core convolution kernels and
  * their count since the last reset; only collected while profiling is enabled (serialises). */
 int lp_conv_profile(lp_handle* h, int enable, double* ms, double* flops, int64_t* launches);

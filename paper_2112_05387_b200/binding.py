@@ -13,7 +13,7 @@ __all__ = [
     "lp_modules_fwd_bwd_all", "lp_step", "lp_forward_serial", "lp_serial_fwd_bwd", "lp_get_residual",
     "lp_last_device_status", "lp_launch_count", "lp_conv_profile", "lp_conv2d", "lp_conv2d_scratch_bytes", "lp_graph_begin", "lp_graph_end",
     "lp_graph_launch", "lp_conv2d_fwd_noalloc", "LP_NOALLOC_SCRATCH_BYTES", "lp_layer_parallel_step", "lp_auxnet_distill", "lp_aux_correct", "lp_timeline", "lp_timeline_record",
-    "LP_PHASE_NAMES", "LP_OP_NAMES", "EXPORTED_SYMBOLS", "lp_selftest_bounded_wait",
+    "LP_PHASE_NAMES", "LP_OP_NAMES", "EXPORTED_SYMBOLS", "lp_selftest_bounded_wait", "lp_call_graphs",
 ]
 
 LP_OK = 0
@@ -39,7 +39,7 @@ EXPORTED_SYMBOLS = [
     "lp_forward_serial", "lp_serial_fwd_bwd", "lp_get_residual", "lp_last_device_status", "lp_launch_count",
     "lp_conv_profile", "lp_conv2d_scratch_bytes", "lp_conv2d", "lp_graph_begin", "lp_graph_end", "lp_graph_launch",
     "lp_conv2d_fwd_noalloc", "lp_layer_parallel_step", "lp_auxnet_distill", "lp_timeline", "lp_aux_correct",
-    "lp_selftest_bounded_wait",
+    "lp_selftest_bounded_wait", "lp_call_graphs",
 ]
 
 
@@ -131,6 +131,7 @@ def library():
     lib.lp_selftest_bounded_wait.argtypes = [vp, ctypes.c_double, ctypes.POINTER(ctypes.c_double), vp]
     lib.lp_launch_count.restype = ctypes.c_int64
     lib.lp_launch_count.argtypes = [vp, i32]
+    lib.lp_call_graphs.argtypes = [vp] + [ctypes.POINTER(ctypes.c_int64)] * 3
     lib.lp_timeline.argtypes = [vp, i32, i32, ctypes.POINTER(lp_timeline_record), ctypes.POINTER(ctypes.c_int)]
     lib.lp_timeline.restype = i32
     lib.lp_conv_profile.argtypes = [vp, i32, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double),
@@ -357,6 +358,13 @@ def lp_selftest_bounded_wait(h, limit_ms, stream=None):
 
 def lp_launch_count(h, reset=False):
     return int(library().lp_launch_count(h.ptr, 1 if reset else 0))
+
+
+def lp_call_graphs(h):
+    """(graph launches, executable graphs built, calls launched directly) since lp_create."""
+    n = [ctypes.c_int64(0) for _ in range(3)]
+    _check(library().lp_call_graphs(h.ptr, *[ctypes.byref(v) for v in n]), "lp_call_graphs")
+    return tuple(v.value for v in n)
 
 
 def lp_conv_profile(h, enable, read=True):

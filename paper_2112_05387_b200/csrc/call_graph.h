@@ -21,15 +21,16 @@ constexpr int kDirectCalls = 2;
 // of one graph in a row the calls are launched directly.
 constexpr int kMaxRebuilt = 4, kForgiveAfter = 16;
 
-// Stream that a handle's calls are recorded on.  A kernel of a graph runs at the priority of the stream it was recorded on, so
+// What a handle's calls are recorded with, and how they were made.  A kernel of a graph runs at the priority of the stream it was recorded on, so
 // it has the priority of the caller's stream (of the first one that a call is recorded for; calls on streams of another
 // priority are launched directly).
-struct CaptureStream {
+struct CallRecorder {
   cudaStream_t stream = nullptr;
   int priority = 0;
   bool failed = false;
+  long long launched = 0, built = 0, direct = 0;   // graph launches; executable graphs; calls launched directly
 };
-inline cudaStream_t capture_stream_for(CaptureStream& c, cudaStream_t st) {
+inline cudaStream_t capture_stream_for(CallRecorder& c, cudaStream_t st) {
   int priority = 0;
   if (c.failed || cudaStreamGetPriority(st, &priority) != cudaSuccess) { cudaGetLastError(); return nullptr; }
   if (!c.stream) {
@@ -49,22 +50,23 @@ inline cudaStream_t capture_stream_for(CaptureStream& c, cudaStream_t st) {
 // 915 us, 362 as graph launches) and large ones lose the overlap of launches across streams.  The call is recorded anew every
 // time, with this call's pointers and arguments, on a stream of the handle's own (recording a launch costs a fraction of
 // making it), the executable graph of the previous call is updated to the recording, and launched; only its topology and
-// memory are kept.  The first two calls of a kind, calls inside a caller's capture, and profiled calls (`direct`) launch
+// memory are kept.  The first two calls of a kind, calls inside a caller's capture, and profiled calls launch
 // directly.  `enqueue` changes host state (which gradients are fresh, launch counts) as if its work had been launched:
 // `restore` puts that back wherever a recording does not become a launch.
 template <typename Enqueue, typename Restore>
-int run_as_graph(CallGraph& g, CaptureStream& capture_stream, cudaStream_t st, bool direct, Enqueue enqueue, Restore restore) {
+int run_as_graph(CallGraph& g, CallRecorder& rec, cudaStream_t st, bool profiled, Enqueue enqueue, Restore restore) {
+  const auto direct = [&]() -> int { ++rec.direct; return enqueue(st); };
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) { cudaGetLastError(); return enqueue(st); }
-  if (cs != cudaStreamCaptureStatusNone || direct || g.off) return enqueue(st);
-  if (g.direct_calls < kDirectCalls) { ++g.direct_calls; return enqueue(st); }
-  const cudaStream_t capture = capture_stream_for(capture_stream, st);
-  if (!capture) return enqueue(st);
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) { cudaGetLastError(); return direct(); }
+  if (cs != cudaStreamCaptureStatusNone || profiled || g.off) return direct();
+  if (g.direct_calls < kDirectCalls) { ++g.direct_calls; return direct(); }
+  const cudaStream_t capture = capture_stream_for(rec, st);
+  if (!capture) return direct();
   // (relaxed, as lp_graph_begin: a kernel that is launched for the first time may be loaded then)
   if (cudaStreamBeginCapture(capture, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
     cudaGetLastError();
     g.off = true;
-    return enqueue(st);
+    return direct();
   }
   const int rc = enqueue(capture);
   cudaGraph_t graph = nullptr;
@@ -88,15 +90,19 @@ int run_as_graph(CallGraph& g, CaptureStream& capture_stream, cudaStream_t st, b
       g.rebuilt = g.kept = 0;
     }
   }
-  if (e == cudaSuccess && !g.exec) e = cudaGraphInstantiate(&g.exec, graph, 0);
+  if (e == cudaSuccess && !g.exec) {
+    e = cudaGraphInstantiate(&g.exec, graph, 0);
+    if (e == cudaSuccess) ++rec.built;
+  }
   if (e == cudaSuccess) e = cudaGraphLaunch(g.exec, st);
   if (graph) cudaGraphDestroy(graph);
   if (e != cudaSuccess) {          // recording does not work here: launch directly from now on
     cudaGetLastError();
     g.off = true;
     restore();
-    return enqueue(st);
+    return direct();
   }
+  ++rec.launched;
   return LP_OK;
 }
 

@@ -266,7 +266,7 @@ struct lp_handle {
   size_t ws_bytes = 0;
   int32_t* zero_labels = nullptr;  // N zeros, for forward passes that only want logits
   CallGraph call_graph[CALL_KINDS];
-  CaptureStream capture_stream;
+  CallRecorder recorder;
   std::vector<cudaGraphExec_t> graphs;
   int64_t launches_at_capture = 0;
   std::vector<int64_t> graph_launches;  // kernels recorded in each graph
@@ -2449,7 +2449,7 @@ static void set_host_state(lp_handle* h, const HostState& s) {
 template <typename F>
 static int run_as_graph(lp_handle* h, int kind, cudaStream_t st, F enqueue) {
   const HostState before = host_state(h);
-  return run_as_graph(h->call_graph[kind], h->capture_stream, st, h->prof.enabled || h->tl.enabled, enqueue,
+  return run_as_graph(h->call_graph[kind], h->recorder, st, h->prof.enabled || h->tl.enabled, enqueue,
                       [&] { set_host_state(h, before); });
 }
 
@@ -2604,7 +2604,7 @@ int lp_destroy(lp_handle* h) {
   for (auto e : h->done) if (e) cudaEventDestroy(e);
   if (h->fork) cudaEventDestroy(h->fork);
   for (auto& g : h->call_graph) if (g.exec) cudaGraphExecDestroy(g.exec);
-  if (h->capture_stream.stream) cudaStreamDestroy(h->capture_stream.stream);
+  if (h->recorder.stream) cudaStreamDestroy(h->recorder.stream);
   if (h->aux_stream) cudaStreamDestroy(h->aux_stream);
   if (h->aux_end) cudaEventDestroy(h->aux_end);
   for (auto e : h->aux_done) if (e) cudaEventDestroy(e);
@@ -3082,6 +3082,14 @@ int64_t lp_launch_count(lp_handle* h, int reset) {
   const int64_t v = h->launches;
   if (reset) h->launches = 0;
   return v;
+}
+
+int lp_call_graphs(lp_handle* h, int64_t* launched, int64_t* built, int64_t* direct) {
+  if (!h) return LP_ERR_NULL;
+  if (launched) *launched = h->recorder.launched;
+  if (built) *built = h->recorder.built;
+  if (direct) *direct = h->recorder.direct;
+  return LP_OK;
 }
 
 int lp_conv_profile(lp_handle* h, int enable, double* ms, double* flops, int64_t* launches) {

@@ -85,7 +85,7 @@ using namespace lp;
 // A handle's host state and a call that changes it: five launches and a flag.
 struct Handle {
   CallGraph g;
-  CaptureStream capture;
+  CallRecorder capture;
   FakeStream user;
   bool fresh = false;
   int launches = 0, done = 0;      // launches counted; launched directly
@@ -112,6 +112,7 @@ SCENARIOS = {
       for (int i = 1; i <= 10; ++i) { CHECK(h.call() == LP_OK); CHECK(h.ran() == 5 * i && h.launches == 5 * i); }
       CHECK(h.done == 10 && fake.launch == 8 && fake.instantiate == 1 && fake.update == 7);
       CHECK(fake.live_graphs == 0 && fake.live_execs == 1);
+      CHECK(h.capture.launched == 8 && h.capture.built == 1 && h.capture.direct == 2);
     """,
     "an argument error while recording leaves the state of before": """
       h.call(); h.call(); h.call();
