@@ -253,3 +253,12 @@ def test_fp32_convolutions_on_either_side_of_the_dispatch_match_oracle(case):
     """K is at most 65536 here (weight gradients): sqrt(K) x 2^-24 = 1.6e-5 in the worst case, 1e-5 measured for sums in
     tiles; the bound of the tiled kernels holds."""
     test_fp32_tile_kernels_match_oracle(case)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("case", [(3, 9, 7, 6, 8, 3, 1, 1), (2, 10, 12, 5, 16, 3, 2, 1), (2, 13, 16, 8, 16, 7, 2, 3),
+                                  (2, 9, 8, 12, 8, 5, 1, 2)])
+def test_convolutions_that_only_the_generic_kernels_take(case, dtype):
+    """Channel counts and filter sizes outside the tiled, the tensor-core and the few-channel kernels; bounds of the other
+    CUDA-core cases."""
+    test_simt_conv_matches_oracle(case, dtype)

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 from conftest import small_cfg
-from harness import GpuRun, allowance, log_parity, noise_floors, oracle_modules, per_tensor_errors, rel_err, to_host
+from harness import GpuRun, allowance, log_parity, noise_floors, oracle_modules, per_tensor_errors, rel_err, to_dev, to_host
 from oracle import lp_oracle as O
 from workloads import gen, get_config, scaled
 
@@ -557,6 +557,98 @@ def test_repeated_calls_equal_directly_launched_ones(which):
             run.seen += [lp.lp_get_params(h, k) for k in range(K)]
         for a, b in zip(runs[0].seen, runs[1].seen):
             assert np.linalg.norm(a - b) <= 1e-5 * max(np.linalg.norm(b), 1e-30), call
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_every_kind_of_call_repeated_as_graph_launches(dtype):
+    """The whole of Algorithm 1 with distillation, evaluation and layer-serial training, nine rounds on new images and new
+    buffers, against a handle that always launches directly.  bf16: the kernels with tensor maps among their parameters, the
+    weight-gradient streams, the grouped weight gradients and their fold.  Multipliers are given for the first time in round
+    3, momentum in round 5, so that kernels and launches are met first by a recording.  One handle runs on a stream of high
+    priority.  Parameters and multipliers are set anew before each update, so that forward passes before it run on the same
+    values and agree to the last bit; what follows an update differs by the order of its fp32 atomics, which bf16 storage
+    turns into flips of the last bit (2 % of the logits of a whole network): 3e-2 in the norm, 1e-5 for the fp32 network; a
+    stale pointer or argument is off by 1."""
+    cfg = get_config("tiny") if dtype == "f32" else \
+        small_cfg("postbn", N=6, H=16, W=16, dtype="bf16", stage_channels=(16, 32, 64), stage_blocks=(2, 2, 2),
+                  stage_stride=(1, 2, 2), module_block_end=(2, 4, 6), stem_channels=16, classes=10)
+    runs = [GpuRun(cfg), GpuRun(cfg)]
+    torch, lp, K = runs[0].torch, runs[0].lp, runs[0].net.K
+    high = torch.cuda.Stream(priority=-1)
+    tol = 1e-5 if dtype == "f32" else 3e-2
+    rounds = 9
+
+    def reset(run):
+        for k in range(K):
+            lp.lp_set_params(run.h, k, run.mods[k])
+        for k in range(K - 1):
+            lp.lp_set_params(run.h, lp.LP_AUX(k), run.auxs[k])
+            run.d_kappa[k].copy_(to_dev(run.kappa[k], cfg))
+
+    for call in range(rounds):
+        g = torch.Generator(device="cuda:0").manual_seed(call)
+        new_images = torch.randn(runs[0].d_images.shape, generator=g, device="cuda:0").to(runs[0].d_images.dtype)
+        for i, run in enumerate(runs):
+            if i:
+                lp.lp_timeline(run.h, True, read=False)
+            h = run.h
+            reset(run)
+            images = new_images.clone()
+            x = [torch.zeros_like(t) for t in run.d_x[1:]]
+            dx = [None] + [torch.zeros_like(t) for t in run.d_x[1:]]
+            lam = run.d_kappa if call >= 3 else None
+            mom = 0.9 if call >= 5 else 0.0
+            loss, dloss = torch.zeros_like(run.d_loss), torch.zeros(K - 1, device="cuda:0")
+            logits = torch.zeros(cfg["N"], cfg["num_classes"], device="cuda:0")
+            high.wait_stream(torch.cuda.current_stream())
+            st = high.cuda_stream if i == 0 else torch.cuda.current_stream().cuda_stream
+            lp.lp_layer_parallel_step(h, images, x, run.d_labels, lam, cfg["rho"], loss, dx, 1e-3, mom, 1e-4, cfg["rho"], st)
+            lp.lp_auxnet_distill(h, images, x, dx, 0.1, 1e-3, None, dloss, st)
+            lp.lp_forward_serial(h, images, logits, st)
+            assert lp.lp_last_device_status(h, st) == 0
+            run.seen = [to_host(loss), to_host(dloss), to_host(logits)] + [to_host(t) for t in x] + [to_host(t) for t in dx[1:]]
+            reset(run)
+            loss2, x2 = torch.zeros_like(run.d_loss), [torch.zeros_like(t) for t in x]
+            high.wait_stream(torch.cuda.current_stream())
+            lp.lp_auxnet_forward(h, images, x2, st)
+            lp.lp_modules_fwd_bwd_all(h, [images] + x2, run.d_labels, lam, cfg["rho"], loss2, dx, st)
+            lp.lp_step(h, 1e-3 * (call + 1), mom, 1e-4, cfg["rho"], lam, st)
+            lp.lp_serial_fwd_bwd(h, images, run.d_labels, loss[K - 1], st)
+            lp.lp_step(h, 1e-3, mom, 0.0, 0.0, None, st)
+            assert lp.lp_last_device_status(h, st) == 0
+            run.seen += [to_host(loss2), to_host(loss[K - 1])] + [to_host(t) for t in run.d_kappa] + [to_host(t) for t in x2] + [to_host(t) for t in dx[1:]]
+            run.seen += [lp.lp_get_params(h, k) for k in range(K)] + [lp.lp_get_params(h, lp.LP_AUX(k)) for k in range(K - 1)]
+        for j, (a, b) in enumerate(zip(runs[0].seen, runs[1].seen)):
+            assert np.linalg.norm(a - b) <= tol * max(np.linalg.norm(b), 1e-30), (call, j, rel_err(a, b))
+    launched, built, direct = lp.lp_call_graphs(runs[0].h)
+    assert lp.lp_call_graphs(runs[1].h) == (0, 0, 8 * rounds)
+    # seven kinds, two direct calls each.  lp_step comes twice a round, from round 3 on by turns with and without multipliers:
+    # four new graphs, each launched once, then directly.  lp_layer_parallel_step builds a second graph in round 3, the other
+    # kinds (and momentum) change no launches.
+    assert (launched, built, direct) == (6 * (rounds - 2) + 8, 6 + 1 + 5, 12 + 2 + 8)
+
+
+@pytest.mark.parametrize("ch,H,W,N", [(16, 33, 32, 2), (16, 7, 36, 3), (32, 5, 20, 5), (64, 9, 17, 2), (64, 8, 8, 5),
+                                      (64, 2, 3, 9), (32, 1, 16, 20), (16, 12, 4, 7), (16, 9, 36, 150), (16, 7, 72, 101),
+                                      (64, 7, 9, 150)])
+def test_thin_layers_with_the_reduction_pass_of_the_next_batch_norm(ch, H, W, N):
+    """The same shapes with the reduction pass of the batch-norm backward in the epilogue whatever the tensor's size (the
+    default takes it from 32768 elements on), whole-row tiles of 9 and 10 groups among them; then 150, 153 and 150
+    tiles on 148 SMs, so that a CTA runs two, whole-row ones and ones ragged in columns and images."""
+    import paper_2112_05387_b200 as lp
+    cfg = small_cfg("postbn", N=N, H=H, W=W, dtype="bf16", stage_channels=(ch, ch), stage_blocks=(2, 2), stage_stride=(1, 1),
+                    module_block_end=(2, 4), stem_channels=ch, classes=10, aux_width_div=1)
+    full_step_parity(cfg, conv_impl=lp.LP_CONV_BN_REDUCE_IN_EPILOGUE, steps=1)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("classes,N", [(131, 5), (1030, 11), (2049, 9)])
+def test_heads_of_many_classes(classes, N, dtype):
+    """More than 128 classes (the head's kernels of their own): numbers of classes that are no multiple of 4, above one chunk
+    of 1024 and of two, batches that are no multiple of 8; one block per module, one flat tolerance."""
+    cfg = small_cfg("postbn", N=N, H=8, W=8, dtype=dtype, stage_channels=(16, 32), stage_blocks=(1, 1), module_block_end=(1, 2),
+                    stem_channels=16, classes=classes)
+    flat_module_parity(cfg, 0, 1e-4 if dtype == "f32" else 2e-2)
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
