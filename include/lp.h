@@ -85,8 +85,9 @@ enum { LP_CONV_TWO_CTA = 1024 };
  * takes the reduction pass of that batch norm's backward (sum dy_m, sum dy_m * xhat) in its epilogue, and only the
  * apply pass is left to run (Eq. Parallel-ResNet-Backpropagation: a module's backward pass is the chain
  * conv^T -> BN' -> conv^T ...; the sums are taken where dy is produced).  Same gradients up to the order of fp32
- * additions.  Not the default: the epilogue's extra shared-memory traffic costs the convolution more than the
- * separate kernel takes. */
+ * additions.  Not the default, except where a 3x3 stride-1 layer of 16, 32 or 64 channels of a post-BN network produces more
+ * than 32768 elements (its kernel sums over a tile that is staged anyway): elsewhere the epilogue's extra shared-memory
+ * traffic costs the convolution more than the separate kernel takes. */
 enum { LP_CONV_BN_REDUCE_IN_EPILOGUE = 2048 };
 /* May be OR-ed into conv_impl: the weight gradients of a module stay in its stream, in the order of the
  * backward pass.  By default each module has a second stream for them (they feed nothing but the update), so

@@ -81,7 +81,7 @@ struct ConvTcParams {
   int Nimg, OHl, OWl;            // logical output grid
   int BW, BH, BNI;               // tile box (logical pixels), BW*BH*BNI <= 128
   int tiles_w, tiles_h, m_tiles, n_tiles, total_tiles;
-  FastDiv fd_tiles_w, fd_tiles_h, fd_m_tiles, fd_n_tiles, fd_chunks;   // the same numbers as divisors
+  FastDiv fd_tiles_w, fd_tiles_h, fd_m_tiles, fd_n_tiles;   // the same numbers as divisors
   int in_step;                   // input coordinate = logical * in_step + tap offset
   int out_H, out_W, out_C;       // physical output tensor
   int os, oo_h, oo_w;            // physical pixel = logical * os + oo
@@ -216,9 +216,9 @@ constexpr int conv_threads(int epi_warps) { return 96 + 32 * epi_warps; }
 // kBnBwd: the direct epilogue also takes the reduction pass of the batch-norm backward that consumes
 //   this convolution's output (see ConvTcParams::bwd_x).
 // kMinBlocks: CTAs of this kernel that must fit on one SM.  Layers of few channels (a channel tile of at most
-//   64 columns) are launched as the two-per-SM instantiation -- registers capped accordingly (the epilogue
-//   drains 64 accumulator columns per pass instead of 160), tensor memory and shared memory sized to need --
-//   so that the kernels of several modules, each bound by latency rather than by any unit, share the SMs.
+//   64 columns) are launched as the two-per-SM instantiation -- registers capped accordingly, tensor memory and
+//   shared memory sized to need -- so that the kernels of several modules, each bound by latency rather than by
+//   any unit, share the SMs.
 // kEpiWarps: 4, or 8 where a tile's epilogue takes longer than its MMAs (few input channels, many output channels): two
 //   warps per row quarter, which take the 32-column groups of a tile in turn.
 template <bool kLoss, bool kAddend, bool kStaged, bool kBnBwd = false, int kMinBlocks = LP_CONV_MIN_BLOCKS, int kEpiWarps = 4>

@@ -246,7 +246,7 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           const uint32_t b_addr = smem_base + p.b_ring_offset + sb * p.b_stage_bytes;
           if (elect_one()) {
             for (int i = 0; i < n_taps; ++i) {
-              const uint64_t ad = smem_desc(p.desc_hi_a, a_addr + p.tap_off9[ti0 + i]);
+              const uint64_t ad = smem_desc(p.desc_hi_a, a_addr + (p.tap_off9[ti0 + i] << 4));
               const uint64_t bd = smem_desc(p.desc_hi, b_addr + i * p.b_tile_bytes);
               for (int j = 0; j < nkc; ++j)
                 mma2_bf16(d, ad + (uint64_t)(2 * j), bd + (uint64_t)(2 * j), p.idesc, (accum | i | j) ? 1u : 0u);
@@ -305,7 +305,6 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         tc_fence_after();
         const uint32_t taddr = tmem_base + buf * p.acc_stride + ((uint32_t)(q * 32) << 16);
         const uint32_t release_addr = mapa_u32(smem_u32(&tail->tmem_empty[buf]), 0);   // the leader's barrier
-        constexpr int kBatch = 1;   // (see conv_tc_kernel)
         auto load_addend = [&](int g, uint4 (&ad)[4]) {
           const int c_in_tile = g * 32;
           const int nv = c_in_tile + 32 <= p.n_tile_cols ? 4 : 2;
@@ -320,46 +319,34 @@ conv_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           if (lane == 0) mbar_arrive_cluster(release_addr);
         }
 #pragma unroll 1
-        for (int g0 = 0; have && g0 < ngroups; g0 += kBatch) {
-          uint32_t raw[kBatch][32];
-          uint4 add_cur[4], add_next[4];
-          if constexpr (kAddend) load_addend(g0, add_cur);
-#pragma unroll
-          for (int i = 0; i < kBatch; ++i) {
-            const int g = g0 + i;
-            if (g < ngroups) {
-              if (g * 32 + 32 <= p.n_tile_cols) tmem_ld32_issue(taddr + g * 32, raw[i]);
-              else tmem_ld16_issue(taddr + g * 32, raw[i]);
-            }
-          }
+        for (int g = 0; have && g < ngroups; ++g) {   // (one 32-column group at a time: see conv_tc_kernel)
+          uint32_t raw[32];
+          uint4 add[4];
+          if constexpr (kAddend) load_addend(g, add);
+          if (g * 32 + 32 <= p.n_tile_cols) tmem_ld32_issue(taddr + g * 32, raw);
+          else tmem_ld16_issue(taddr + g * 32, raw);
           tmem_ld_wait();
-#pragma unroll
-          for (int i = 0; i < kBatch; ++i) tmem_ld_fence(raw[i]);
-          if (g0 + kBatch >= ngroups) {
+          tmem_ld_fence(raw);
+          if (g + 1 >= ngroups) {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(release_addr);
           }
-#pragma unroll
-          for (int i = 0; i < kBatch; ++i) {
-            const int g = g0 + i;
-            if (g >= ngroups) continue;
+          {
             const int c_in_tile = g * 32;
             const int col = col0 + c_in_tile;
             const bool wide = c_in_tile + 32 <= p.n_tile_cols;
             const int nv = wide ? 4 : 2;
             float v[32];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = (wide || j < 16) ? __uint_as_float(raw[i][j]) : 0.f;
+            for (int j = 0; j < 32; ++j) v[j] = (wide || j < 16) ? __uint_as_float(raw[j]) : 0.f;
             if constexpr (kAddend) {
-              if (i + 1 < kBatch) load_addend(g + 1, add_next);
 #pragma unroll
               for (int v4 = 0; v4 < 4; ++v4) {
                 float f[8];
-                cvt_raw(add_cur[v4], f);
+                cvt_raw(add[v4], f);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) v[8 * v4 + j] += f[j];
-                add_cur[v4] = add_next[v4];
               }
             }
             uint32_t pk[16];

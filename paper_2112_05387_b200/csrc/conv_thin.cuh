@@ -23,7 +23,8 @@
 // 2127 -> 1455; with the rolled loops of the other kernels 738 and 1343).  A CTA runs most of its code once or twice, so fetching
 // instructions costs as much as executing them: loops are kept rolled and whole tiles are moved by single copies (an
 // unrolled version with the loads in registers, 2.5 times the code, took 1.5 times as long per launch).  For the same
-// reason nothing is pipelined inside a CTA; two CTAs share an SM instead (one of the 64-channel layers).
+// reason nothing is pipelined inside a CTA: beside it run the kernels of the other modules' streams (a launch takes one CTA
+// per SM at most; registers and, up to 32 channels, shared memory leave room for a CTA of another launch).
 //
 // Tile geometry: M row r of a tile sits at box position (r / 8) * S + r % 8 (rows of 128 bytes; box dimensions W, image,
 // H with P = BW + 2 columns).  S = P and BW = 8: eight columns per row group; S = 8: the box rows are taken as one run,

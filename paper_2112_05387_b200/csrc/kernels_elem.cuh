@@ -811,10 +811,8 @@ head_bwd_w_kernel(const float* __restrict__ dlogits, const float* __restrict__ p
   // (consecutive threads write consecutive channels: 4 of an item, then those of the next)
   for (int t = threadIdx.x; t < 32 * 20; t += 256) {
     const int q = t / 128, r = t % 128;
-    const int k = q < 4 ? r >> 2 : r;                       // item
-    if (q == 4 && r >= 128) break;
+    const int kk = q < 4 ? r >> 2 : r & 31;                 // item
     const int e = q < 4 ? q * 4 + (r & 3) : 16 + (r >> 5);  // element of the item; the last 128: sums of dlogits
-    const int kk = q < 4 ? k : (r & 31);
     float a = 0.f;
 #pragma unroll
     for (int g = 0; g < 8; ++g) a += part[g][kk][e];

@@ -525,7 +525,7 @@ static int launch_conv_tc2(lp_handle* h, const TcGemmSpec& s, int* dev_err, cuda
   for (int dy = 0; dy < 3; ++dy)
     for (int dx = 0; dx < 3; ++dx) {
       p.tap_widx9[dy * 3 + dx] = tapw3[dx][dy];
-      p.tap_off9[dy * 3 + dx] = (uint32_t)((dy * kHaloBoxW * p.BNI + dx) * row_bytes);
+      p.tap_off9[dy * 3 + dx] = (uint32_t)((dy * kHaloBoxW * p.BNI + dx) * row_bytes) >> 4;
     }
   p.desc_hi_a = tc::smem_desc_hi(16, kHaloBoxW * row_bytes, tc::swizzle_code_for_row_bytes(row_bytes));
   p.desc_hi = tc::smem_desc_hi(16, 8 * row_bytes, tc::swizzle_code_for_row_bytes(row_bytes));
@@ -663,9 +663,12 @@ static int launch_conv_tc(lp_handle* h, const TcGemmSpec& s, int* dev_err, cudaS
   const bool thin = allow_thin && h && h->concurrent && !bnbwd && !s.x_next && p.n_tile_cols <= 64 &&
                     2.0 * s.aN * s.OHl * s.OWl * (double)s.w_rows * s.ntaps * s.aC < kSmallConvFlops;
   const bool staged = staged0 && !thin;
-  // Eight epilogue warps where a tile's epilogue (about 31 cycles a column with four) is longer than its MMAs (N / 2 cycles
-  // each) and the tile is a full 256 columns: the 1x1 convolutions of bottleneck blocks (ResNet-50 3.53 -> 3.50 ms per
-  // step).  Elsewhere the second four warps only cost registers and shared memory (WRN-28-10 4.63 -> 4.65 ms).
+  // Eight epilogue warps where a tile's epilogue (about 33 cycles a column with four) is longer than its MMAs and the tile is
+  // a full 256 columns: K of at most 1024, that is the 1x1 convolutions of bottleneck blocks and 3x3 layers of up to 113
+  // channels (ResNet-50 3.53 -> 3.50 ms per step).  Alone, four against eight warps: 64 -> 256, 1x1, 32 images of 56x56
+  // 37.7 -> 34.4 us with statistics and 34.5 -> 28.9 with a shortcut; 112 -> 512, 3x3, 32 of 28x28 40.2 -> 37.6 and
+  // 36.5 -> 35.7; plain epilogues equal within 2 %.  At larger K the second four warps only cost registers and shared memory
+  // (WRN-28-10 4.63 -> 4.65 ms).
   const bool wide_epi = wide_ok && !thin && (staged ? s.addend != nullptr : s.addend == nullptr) && p.n_tile_cols == 256;
   const int epi_warps = wide_epi ? 8 : 4;
   const size_t max_smem = thin ? kTcThinSmem : kTcMaxSmem;
@@ -752,7 +755,6 @@ static int launch_conv_tc(lp_handle* h, const TcGemmSpec& s, int* dev_err, cudaS
   }
   p.fd_tiles_w = tc::make_fastdiv(p.tiles_w); p.fd_tiles_h = tc::make_fastdiv(p.tiles_h);
   p.fd_m_tiles = tc::make_fastdiv(p.m_tiles); p.fd_n_tiles = tc::make_fastdiv(p.n_tiles);
-  p.fd_chunks = tc::make_fastdiv(p.chunks);
   p.idesc = tc::instr_desc_bf16(128, p.n_tile_cols, 0, 0);
   p.desc_hi = tc::smem_desc_hi(16, 8 * row_bytes, tc::swizzle_code_for_row_bytes(row_bytes));
   p.out = s.out; p.addend = s.addend; p.stats = s.stats; p.err = dev_err;
@@ -1466,7 +1468,10 @@ struct Planner {
       if (name == e.name) return &e;
     return nullptr;
   }
-  // Layers that take the thin kernel with its fusions (post-activation networks; none of the variant flags).
+  // Layers that take the thin kernel with its fusions (post-activation networks; none of the variant flags).  The limit is that
+  // of layers which cannot fill the machine; it holds for a module alone too (thin against general kernels: evaluation of
+  // ResNet-34 on 16 images of 224x224, its 64-channel layers just below the limit, 595 against 602 us, layer-serial training
+  // 1531 against 1570; of ResNet-56 on 128 images 411 against 594, 1149 against 1849).
   bool thin_ok(const ConvDef& c) const {
     return dtype == LP_BF16 && net.d.block_kind != LP_PREACT && impl != LP_CONV_IMPL_SIMT &&
            !(net.d.conv_impl & ~(15 | LP_CONV_WGRAD_IN_CHAIN | LP_CONV_BN_REDUCE_IN_EPILOGUE)) && c.R == 3 && c.stride == 1 && c.pad == 1 && c.cin == c.cout &&
@@ -1598,7 +1603,10 @@ struct Planner {
            !(net.d.conv_impl & 32) && tc_dgrad_ok(c) && c.wt && !dgrad_has_empty_class(c);
   }
   // The input gradient of a thin layer takes the reduction pass of the batch-norm backward that follows it; on tensors of
-  // up to 32768 elements, where the pass is a block or two, only on request as for every other convolution.
+  // up to 32768 elements only on request (LP_CONV_BN_REDUCE_IN_EPILOGUE), as for every other convolution: the pass as its own
+  // kernel is the documented default that the fused form is compared with, and small tensors keep it.  It costs them a launch
+  // in the chain: ResNet-56 takes 298 us per step at 1 image, 352 at 8, on request 261 and 295; from 16 images on the
+  // two are equal (313).
   bool thin_fuses_bn_bwd(const ConvDef& c, const Tensor& dy) const {
     return c.g > 0 && ((net.d.conv_impl & LP_CONV_BN_REDUCE_IN_EPILOGUE) || dy.elems() > 32768);
   }

@@ -57,7 +57,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 }
 
 // The same for one thread in a loop that issues MMAs: no call, because keeping the loop's values across one costs some
-// fifty cycles a trip.
+// fifty cycles a trip.  The clock is read and the flag looked at after every 1024th failed poll only, and the first reading
+// starts the time: it gives up after kWaitLimitCycles and at most 2048 polls more.
 __device__ __forceinline__ bool mbar_wait_hot(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   uint32_t polls = 0;
   long long t0 = 0;
