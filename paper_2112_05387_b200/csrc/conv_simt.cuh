@@ -3,6 +3,9 @@
 // the tensor-core path does not take (3-channel stems).  fp32 accumulation throughout;
 // weights are the fp32 masters w[co][r][s][ci], rounded to the activation type as they are read
 // so that both convolution paths of a bf16 network contract the same operands.
+// fp32 results are added up in partial sums (per filter position, four channels at a time or in four chains), as the tiled
+// kernels do: one chain over all terms was up to twice as far from the exact sum (input gradient of 128 -> 128, 1x1: 2.0e-7
+// against 1.1e-7).
 #pragma once
 #include "common.cuh"
 
@@ -18,6 +21,7 @@ struct ConvGeom {
 template <typename T>
 __global__ void conv_fwd_simt_kernel(const T* __restrict__ x, const float* __restrict__ w, const T* __restrict__ addend,
                                      T* __restrict__ y, ConvGeom g) {
+  constexpr bool kPartial = sizeof(T) == 4;
   const int CG = g.Cout >> 2;
   const long long total = (long long)g.N * g.OH * g.OW * CG;
   const long long tap_stride = (long long)g.R * g.S * g.Cin;
@@ -38,11 +42,20 @@ __global__ void conv_fwd_simt_kernel(const T* __restrict__ x, const float* __res
         if (iw < 0 || iw >= g.W) continue;
         const T* xp = x + (((long long)n * g.H + ih) * g.W + iw) * g.Cin;
         const float* wp = w + ((long long)co * g.R * g.S + (r * g.S + s)) * g.Cin;
+        float part[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) part[j] = kPartial ? 0.f : acc[j];
         for (int ci = 0; ci < g.Cin; ++ci) {
           const float xv = to_f(xp[ci]);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[j] += xv * round_storage<T>(__ldg(wp + j * tap_stride + ci));
+          for (int j = 0; j < 4; ++j) part[j] += xv * round_storage<T>(__ldg(wp + j * tap_stride + ci));
+          if (kPartial && (ci & 3) == 3) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) { acc[j] += part[j]; part[j] = 0.f; }
+          }
         }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j] = kPartial ? acc[j] + part[j] : part[j];
       }
     }
     const long long o = p * g.Cout + co;
@@ -82,7 +95,21 @@ __global__ void conv_dgrad_simt_kernel(const T* __restrict__ dy, const float* __
         if (ow >= g.OW) continue;
         const T* dp = dy + (((long long)n * g.OH + oh) * g.OW + ow) * g.Cout;
         const float* wp = w + (long long)(r * g.S + s) * g.Cin + ci;
-        for (int co = 0; co < g.Cout; ++co) {
+        int co = 0;
+        if constexpr (sizeof(T) == 4) {
+          float part[4][4] = {};
+          for (; co + 4 <= g.Cout; co += 4) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const float d = to_f(dp[co + u]);
+              const float4 wv = __ldg(reinterpret_cast<const float4*>(wp + (long long)(co + u) * g.R * g.S * g.Cin));
+              part[u][0] += d * wv.x; part[u][1] += d * wv.y; part[u][2] += d * wv.z; part[u][3] += d * wv.w;
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[j] += (part[0][j] + part[1][j]) + (part[2][j] + part[3][j]);
+        }
+        for (; co < g.Cout; ++co) {
           const float d = to_f(dp[co]);
           const float4 wv = __ldg(reinterpret_cast<const float4*>(wp + (long long)co * g.R * g.S * g.Cin));
           acc[0] += d * round_storage<T>(wv.x);
@@ -146,7 +173,9 @@ __global__ void conv_wgrad_simt_kernel(const T* __restrict__ x, const T* __restr
 // pixel: one activation load and CPT/4 broadcast reads of the filter bank feed CPT multiply-adds.
 // Same operands as the generic kernels (weights rounded to the activation type, fp32 accumulation).
 // ---------------------------------------------------------------------------------------------
-template <typename T, int CPT>
+// kPartial: a filter position at a time is added up by itself (fp32 layers that the tiled kernel would take too, at a CPT of 32 at
+// most: 127 registers, two blocks an SM).
+template <typename T, int CPT, bool kPartial = false>
 __global__ void __launch_bounds__(256)
 conv_fwd_fewch_kernel(const T* __restrict__ x, const float* __restrict__ w, T* __restrict__ y, ConvGeom g) {
   constexpr int V = VecT<T>::N;
@@ -167,7 +196,7 @@ conv_fwd_fewch_kernel(const T* __restrict__ x, const float* __restrict__ w, T* _
     const long long q = p / g.OW;
     const int oh = (int)(q % g.OH);
     const int n = (int)(q / g.OH);
-    float acc[CPT];
+    float sum[kPartial ? CPT : 1], acc[CPT];
 #pragma unroll
     for (int j = 0; j < CPT; ++j) acc[j] = 0.f;
     for (int r = 0; r < g.R; ++r) {
@@ -176,6 +205,10 @@ conv_fwd_fewch_kernel(const T* __restrict__ x, const float* __restrict__ w, T* _
       for (int s = 0; s < g.S; ++s) {
         const int iw = ow * g.stride + s - g.pad;
         if (iw < 0 || iw >= g.W) continue;
+        if constexpr (kPartial) {
+#pragma unroll
+          for (int j = 0; j < CPT; ++j) { sum[j] = acc[j]; acc[j] = 0.f; }
+        }
         const T* xp = x + (((long long)n * g.H + ih) * g.W + iw) * g.Cin;
         const float* wr = ws + (r * g.S + s) * g.Cin * g.Cout + cg * CPT;
         for (int ci = 0; ci < g.Cin; ++ci) {
@@ -185,6 +218,10 @@ conv_fwd_fewch_kernel(const T* __restrict__ x, const float* __restrict__ w, T* _
             const float4 wv = *reinterpret_cast<const float4*>(wr + ci * g.Cout + j4);
             acc[j4] += xv * wv.x; acc[j4 + 1] += xv * wv.y; acc[j4 + 2] += xv * wv.z; acc[j4 + 3] += xv * wv.w;
           }
+        }
+        if constexpr (kPartial) {
+#pragma unroll
+          for (int j = 0; j < CPT; ++j) acc[j] += sum[j];
         }
       }
     }

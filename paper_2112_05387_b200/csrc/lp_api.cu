@@ -1212,19 +1212,30 @@ static int conv_forward(lp_handle* h, int dtype, int impl, const ConvDef& c, int
   const size_t few_smem = (size_t)c.R * c.R * c.cin * c.cout * 4;
   const int few_cpt = fewch_cpt(c.cout, dtype);
   if (!addend && fewch_ok(c, dtype)) {
-    const long long items = (long long)N * c.OH * c.OW * (c.cout / few_cpt);
+    const bool partial = dtype == LP_F32 && f32_tile_ok(c) && c.R > 1;   // (sums no longer than the tiled kernel's)
+    const int cpt = partial ? std::min(few_cpt, 32) : few_cpt;
+    const long long items = (long long)N * c.OH * c.OW * (c.cout / cpt);
     const int fgrid = grid_for(items, 256, cur_dev().sm_count, 8);
+#define LP_FEWCH_PARTIAL(CPT) \
+    conv_fwd_fewch_kernel<float, CPT, true><<<fgrid, 256, few_smem, st>>>((const float*)x, c.w, (float*)y, g)
 #define LP_FEWCH_FWD(CPT)                                                                                      \
     if (dtype == LP_F32)                                                                                       \
       conv_fwd_fewch_kernel<float, CPT><<<fgrid, 256, few_smem, st>>>((const float*)x, c.w, (float*)y, g);       \
     else                                                                                                       \
       conv_fwd_fewch_kernel<bf16, CPT><<<fgrid, 256, few_smem, st>>>((const bf16*)x, c.w, (bf16*)y, g)
-    switch (few_cpt) {
-      case 64: LP_FEWCH_FWD(64); break;
-      case 32: LP_FEWCH_FWD(32); break;
-      case 16: LP_FEWCH_FWD(16); break;
-      default: LP_FEWCH_FWD(8); break;
+    if (partial) {
+      if (cpt == 32) LP_FEWCH_PARTIAL(32);
+      else if (cpt == 16) LP_FEWCH_PARTIAL(16);
+      else LP_FEWCH_PARTIAL(8);
+    } else {
+      switch (cpt) {
+        case 64: LP_FEWCH_FWD(64); break;
+        case 32: LP_FEWCH_FWD(32); break;
+        case 16: LP_FEWCH_FWD(16); break;
+        default: LP_FEWCH_FWD(8); break;
+      }
     }
+#undef LP_FEWCH_PARTIAL
 #undef LP_FEWCH_FWD
     if (h) h->launches++;
     LP_CUDA_OK(cudaGetLastError());
