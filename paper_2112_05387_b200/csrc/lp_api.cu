@@ -1397,7 +1397,9 @@ static int conv_wgrad(lp_handle* h, int dtype, int impl, const ConvDef& c, int N
     if (h) h->launches++;
     return rc;
   }
-  if (dtype == LP_F32 && f32_tile_ok(c)) return conv_wgrad_f32(h, c, N, (const float*)x, (const float*)dy, dw, st);
+  // (one block row per pair of 16-channel tiles: 4096 channels on both sides are more than a grid's 65535)
+  if (dtype == LP_F32 && f32_tile_ok(c) && (long long)((c.cin + 15) / 16) * ((c.cout + 15) / 16) <= 65535)
+    return conv_wgrad_f32(h, c, N, (const float*)x, (const float*)dy, dw, st);
   ConvGeom g{N, c.H, c.W, c.cin, c.OH, c.OW, c.cout, c.R, c.R, c.stride, c.pad};
   const int n_out = c.cout * c.R * c.R * c.cin;
   const long long npix = (long long)N * c.OH * c.OW;

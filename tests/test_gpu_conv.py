@@ -262,3 +262,13 @@ def test_convolutions_that_only_the_generic_kernels_take(case, dtype):
     """Channel counts and filter sizes outside the tiled, the tensor-core and the few-channel kernels; bounds of the other
     CUDA-core cases."""
     test_simt_conv_matches_oracle(case, dtype)
+
+
+def test_fp32_weight_gradient_of_4096_channels_on_both_sides():
+    """256 x 256 pairs of 16-channel tiles: one more than the largest grid has rows.  Four pixels: a sum of four terms."""
+    import paper_2112_05387_b200 as lp
+    case = (1, 2, 2, 4096, 4096, 1, 1, 0)
+    x, w, dy = make_case(*case, "f32")
+    st, dw, _ = run_conv(lp.LP_CONV_WGRAD, "f32", 0, *case, x, dy)
+    assert st == 0, lp.lp_status_string(st)
+    assert rel_err(dw, np.einsum("nhwo,nhwi->oi", dy, x)) < 1e-6
