@@ -879,8 +879,15 @@ head_bwd_x_kernel(const float* __restrict__ dlogits, const float* __restrict__ W
 }
 
 // ---------------------------------------------------------------------------------------
-// updates
+// clearing, updates
 // ---------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) zero_kernel(uint4* __restrict__ p, long long n) {
+  pdl_wait();
+  pdl_launch_dependents();
+  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256)
+    p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 __global__ void sgd_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ mom, long long n,
                            float lr, float momentum, float wd) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {

@@ -118,6 +118,12 @@ struct HeadDef {
   float *pooled = nullptr, *logits = nullptr, *dlogits = nullptr;
 };
 
+// Part of the workspace that starts a pass at zero (both ends on 256-byte boundaries).
+struct ZeroRange {
+  uint8_t* p = nullptr;
+  size_t bytes = 0;
+};
+
 struct Plan {  // one module or one AuxNet
   std::vector<Op> fwd, bwd;
   std::vector<ConvDef> convs;
@@ -128,12 +134,11 @@ struct Plan {  // one module or one AuxNet
   Tensor out;    // module output (interior modules; serial mode) / AuxNet output
   Tensor r, seed;
   double* loss_acc = nullptr;  // [2]
-  void* stats_region = nullptr;
-  size_t stats_bytes = 0;
+  // what a pass accumulates into: batch-norm statistics (and a module's loss sums) of the forward pass; gradients, those of
+  // regrouped layers, and an AuxNet's loss sum, of the backward pass
+  ZeroRange state, grads;
   void* dx_fallback = nullptr;
-  // weight gradients of the grouped layers: one region, cleared before the first of them, folded back after the last
-  void* dwg_region = nullptr;
-  size_t dwg_bytes = 0;
+  // weight gradients of the grouped layers are folded back after the last of them
   std::vector<tc::FoldEntry> host_fold;
   tc::FoldEntry* dev_fold = nullptr;
   bool interior = false;
@@ -155,6 +160,25 @@ struct Arena {
     off += bytes;
     return p;
   }
+  ZeroRange range_from(size_t begin) {   // everything allocated since `off` was `begin`
+    begin = align_up(begin, 256);
+    off = align_up(off, 256);
+    return ZeroRange{base + begin, off - begin};
+  }
+};
+// Parts of the workspace.  What a pass starts at zero is kept together, modules first, then AuxNets, so that a call clears it
+// with one launch for the statistics and one for the gradients.
+struct Arenas {
+  Arena main, state, grads;
+  size_t bytes() const { return align_up(main.off, 256) + align_up(state.off, 256) + align_up(grads.off, 256); }
+  void place(uint8_t* base, const Arenas& sized) {
+    main.base = base;
+    state.base = main.base + align_up(sized.main.off, 256);
+    grads.base = state.base + align_up(sized.state.off, 256);
+  }
+};
+struct ZeroRanges {
+  ZeroRange module_state, aux_state, all_state, module_grads, aux_grads;
 };
 
 struct RunCtx {
@@ -255,6 +279,9 @@ struct lp_handle {
   std::vector<cudaEvent_t> done;
   cudaEvent_t fork = nullptr;
   cudaStream_t aux_stream = nullptr;
+  cudaStream_t zero_stream = nullptr; // clears the gradients beside the forward passes
+  cudaEvent_t grads_zeroed = nullptr;
+  ZeroRanges zero;
   std::vector<cudaEvent_t> aux_done;  // aux_done[k]: x_{k+1} has been produced
   cudaEvent_t aux_end = nullptr;
   int64_t launches = 0;
@@ -1359,13 +1386,12 @@ static int conv_dgrad(lp_handle* h, int dtype, int impl, const ConvDef& c, int N
   return LP_OK;
 }
 
-// dw += x (*) dy     (dw zeroed by the caller beforehand)
+// dw += x (*) dy     (dw, or its regrouped form in c, zeroed by the caller beforehand)
 static int conv_wgrad(lp_handle* h, int dtype, int impl, const ConvDef& c, int N, const void* x, const void* dy,
                       float* dw, int* dev_err, cudaStream_t st) {
   if (c.s2d) {
     // weight gradient of the regrouped 4x4 convolution (x is the image: its regrouped copy was kept by the
     // forward pass), then the real filter positions are picked out of it
-    LP_CUDA_OK(cudaMemsetAsync(c.dws, 0, (size_t)c.cout * 256 * 4, st));
     Device& D = cur_dev();
     {
       ProfScope ps(h, st, 2.0 * N * c.OH * c.OW * (double)c.cout * c.R * c.R * c.cin);
@@ -1451,10 +1477,12 @@ static int conv_wgrad(lp_handle* h, int dtype, int impl, const ConvDef& c, int N
 // ---------------------------------------------------------------------------------------------
 struct Planner {
   const NetDef& net;
-  Arena& A;
+  Arena &A, &Z, &G;      // everything; cleared before a forward pass; cleared before a backward pass
+  size_t z_begin = 0, g_begin = 0;
   int dtype;
   int impl;
-  Planner(const NetDef& n, Arena& a) : net(n), A(a), dtype(n.d.dtype), impl(n.d.conv_impl & 15) {}
+  Planner(const NetDef& n, Arenas& a)
+      : net(n), A(a.main), Z(a.state), G(a.grads), dtype(n.d.dtype), impl(n.d.conv_impl & 15) {}
 
   Tensor new_tensor(int n, int h, int w, int c) {
     Tensor t;
@@ -1471,9 +1499,10 @@ struct Planner {
   void alloc_params(Plan& P, int which) {
     uint64_t total = 0;
     net.layout(which, P.ps.layout, &total);
+    z_begin = Z.off; g_begin = G.off;
     P.ps.n = (size_t)total;
     P.ps.p = (float*)A.alloc(total * 4);
-    P.ps.g = (float*)A.alloc(total * 4);
+    P.ps.g = (float*)G.alloc(total * 4);
     P.ps.m = (float*)A.alloc(total * 4);
   }
   const lp_param_entry* find(const Plan& P, const std::string& name) const {
@@ -1528,7 +1557,7 @@ struct Planner {
                !need_dgrad && s2d_stem_ok(c)) {
       c.s2d = true;
       c.wf = (bf16*)A.alloc((size_t)cout * 256 * 2);
-      c.dws = (float*)A.alloc((size_t)cout * 256 * 4);
+      c.dws = (float*)G.alloc((size_t)cout * 256 * 4);
       c.xs = (bf16*)A.alloc((size_t)net.d.N * (H / 2) * (W / 2) * 16 * 2);
     }
     P.convs.push_back(c);
@@ -1544,23 +1573,21 @@ struct Planner {
     P.bns.push_back(b);
     return (int)P.bns.size() - 1;
   }
-  void finish_stats(Plan& P) {
+  void finish_stats(Plan& P, bool aux) {
     size_t total = 0;
     for (auto& b : P.bns) total += (size_t)2 * b.C;
-    P.stats_bytes = total * sizeof(double);
-    double* base = (double*)A.alloc(std::max<size_t>(P.stats_bytes, 16));
-    P.stats_region = base;
+    double* base = (double*)Z.alloc(std::max<size_t>(total * sizeof(double), 16));
     size_t off = 0;
     for (auto& b : P.bns) { b.stats = base + off; off += (size_t)2 * b.C; }
-    P.loss_acc = (double*)A.alloc(2 * sizeof(double));
+    // (an AuxNet's loss belongs to its backward pass, which needs the statistics of the forward pass)
+    P.loss_acc = (double*)(aux ? G : Z).alloc(2 * sizeof(double));
     for (auto& c : P.convs) {
       if (c.g <= 1) continue;
-      const size_t bytes = (size_t)64 * 9 * 64 * 4;      // (a multiple of the arena's alignment: the region is contiguous)
-      c.dwg = (float*)A.alloc(bytes);
-      if (!P.dwg_bytes) P.dwg_region = c.dwg;
-      P.dwg_bytes += bytes;
+      c.dwg = (float*)G.alloc((size_t)64 * 9 * 64 * 4);
       P.host_fold.push_back({c.dwg, c.gw, c.cin});
     }
+    P.state = Z.range_from(z_begin);
+    P.grads = G.range_from(g_begin);
     if (!P.host_fold.empty()) P.dev_fold = (tc::FoldEntry*)A.alloc(P.host_fold.size() * sizeof(tc::FoldEntry));
     if (!P.ps.host_pack.empty()) {
       P.ps.dev_pack = (PackEntry*)A.alloc(P.ps.host_pack.size() * sizeof(PackEntry));
@@ -1767,7 +1794,7 @@ struct Planner {
       hd.logits = (float*)A.alloc((size_t)d.N * hd.classes * 4);
       hd.dlogits = (float*)A.alloc((size_t)d.N * hd.classes * 4);
     }
-    finish_stats(P);
+    finish_stats(P, false);
 
     // ---- forward ----
     std::vector<Op>& F = P.fwd;
@@ -1981,7 +2008,7 @@ struct Planner {
                             i > 0 || dx_out != nullptr));
       bi.push_back(add_bn(P, "bn" + id, cv[i].cout, (long long)s.n * cv[i].hout * cv[i].wout));
     }
-    finish_stats(P);
+    finish_stats(P, true);
     Tensor cur = x;
     std::vector<Tensor> ins, ys, acts;
     for (size_t i = 0; i < cv.size(); ++i) {
@@ -2321,11 +2348,9 @@ static int run_ops(lp_handle* h, Plan& P, const std::vector<Op>& ops, const RunC
       ++nside;
       RunCtx c2 = c;
       c2.st = P.side;
-      if (grouped && !folds && cudaMemsetAsync(P.dwg_region, 0, P.dwg_bytes, P.side) != cudaSuccess) { rc = LP_ERR_CUDA; break; }
       folds = folds || grouped;
       rc = h->dtype == LP_F32 ? run_op_t<float>(h, P, op, c2) : run_op_t<bf16>(h, P, op, c2);
     } else {
-      if (grouped && !folds && cudaMemsetAsync(P.dwg_region, 0, P.dwg_bytes, c.st) != cudaSuccess) { rc = LP_ERR_CUDA; break; }
       folds = folds || grouped;
       TimelineScope ts(h, c.st, c.plan_id, (int)op.type, c.phase, h->tl.enabled ? op_bytes(h, P, op) : 0.0);
       rc = h->dtype == LP_F32 ? run_op_t<float>(h, P, op, c) : run_op_t<bf16>(h, P, op, c);
@@ -2343,10 +2368,23 @@ static int run_ops(lp_handle* h, Plan& P, const std::vector<Op>& ops, const RunC
   return rc;
 }
 
-static int zero_forward_state(Plan& P, cudaStream_t st) {
-  if (P.stats_bytes) LP_CUDA_OK(cudaMemsetAsync(P.stats_region, 0, P.stats_bytes, st));
-  LP_CUDA_OK(cudaMemsetAsync(P.loss_acc, 0, 2 * sizeof(double), st));
+// Clears what a pass accumulates into.  A kernel and not a memset: a memset between two kernels of a graph costs the chain
+// 10 to 25 us (a module began with three of them, 25 us for ResNet-110's and up to 55 for ResNet-50's on 12 images).
+static int zero_range(lp_handle* h, const ZeroRange& r, cudaStream_t st) {
+  if (!r.bytes) return LP_OK;
+  const long long n = (long long)(r.bytes / 16);
+  // (two blocks per SM: the gradients are cleared beside the first kernels of the forward passes)
+  LP_CUDA_OK(launch_pdl(zero_kernel, dim3(grid_for(n, 256 * 4, cur_dev().sm_count, 2)), dim3(256), 0, st, (uint4*)r.p, n));
+  h->launches++;
   return LP_OK;
+}
+// The gradients of all modules, on a stream of their own forked from `fork`: nothing needs them before the backward passes.
+static int zero_grads_beside(lp_handle* h) {
+  LP_CUDA_OK(cudaStreamWaitEvent(h->zero_stream, h->fork, 0));
+  const int rc = zero_range(h, h->zero.module_grads, h->zero_stream);
+  // (recorded whatever happened: the caller joins the stream through this event)
+  LP_CUDA_OK(cudaEventRecord(h->grads_zeroed, h->zero_stream));
+  return rc;
 }
 
 // bf16 copies of the regrouped stem weights (space-to-depth stems), after every change of the master weights
@@ -2421,21 +2459,21 @@ static int sgd_update_inner(lp_handle* h, Plan& P, float lr, float momentum, flo
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
+// `grads_wait`: the gradients are cleared once this event has been reached (the statistics are clear already).
 static int module_fwd_bwd(lp_handle* h, int k, const void* x_k, const void* x_next_or_labels, const void* lambda_k,
-                          float rho, float* loss_out, void* dx_k, cudaStream_t st, cudaEvent_t loss_wait = nullptr) {
+                          float rho, float* loss_out, void* dx_k, cudaStream_t st, cudaEvent_t grads_wait,
+                          cudaEvent_t loss_wait = nullptr) {
   Plan& P = h->modules[k];
   const bool last = k == h->net.K - 1;
   RunCtx c;
   c.st = st; c.x = x_k; c.rho = rho; c.loss_out = loss_out; c.dx = dx_k; c.loss_wait = loss_wait;
   if (last) c.labels = (const int32_t*)x_next_or_labels;
   else { c.xnext = x_next_or_labels; c.kappa = lambda_k; }
-  int rc = zero_forward_state(P, st);
-  if (rc != LP_OK) return rc;
-  LP_CUDA_OK(cudaMemsetAsync(P.ps.g, 0, P.ps.n * 4, st));
   c.plan_id = k;
   c.phase = LP_PHASE_FORWARD;
-  rc = run_ops(h, P, P.fwd, c);
+  int rc = run_ops(h, P, P.fwd, c);
   if (rc != LP_OK) return rc;
+  if (grads_wait) LP_CUDA_OK(cudaStreamWaitEvent(st, grads_wait, 0));
   c.phase = LP_PHASE_BACKWARD;
   rc = run_ops(h, P, P.bwd, c);
   if (rc != LP_OK) return rc;
@@ -2503,31 +2541,38 @@ int lp_validate_desc(const lp_net_desc* desc) {
   return n.build(desc);
 }
 
-static int plan_all(const NetDef& net, Arena& A, std::vector<Plan>* modules, std::vector<Plan>* auxs, int** dev_err,
-                    int32_t** zero_labels) {
+static int plan_all(const NetDef& net, Arenas& A, std::vector<Plan>* modules, std::vector<Plan>* auxs, int** dev_err,
+                    int32_t** zero_labels, ZeroRanges* zero) {
   Planner pl(net, A);
-  *dev_err = (int*)A.alloc(256);
-  *zero_labels = (int32_t*)A.alloc((size_t)net.d.N * 4);
+  *dev_err = (int*)A.main.alloc(256);
+  *zero_labels = (int32_t*)A.main.alloc((size_t)net.d.N * 4);
   modules->resize(net.K);
   for (int k = 0; k < net.K; ++k) pl.build_module((*modules)[k], k);
+  zero->module_state = A.state.range_from(0);
+  zero->module_grads = A.grads.range_from(0);
+  const size_t z_aux = A.state.off, g_aux = A.grads.off;
   auxs->resize(net.n_aux_plans());
   if (net.d.aux_recursive) {
     for (int k = 1; k < net.K; ++k) pl.build_reaux_stack(*auxs, k);
   } else {
     for (int k = 0; k + 1 < net.K; ++k) pl.build_aux((*auxs)[k], k);
   }
+  zero->aux_state = A.state.range_from(z_aux);
+  zero->aux_grads = A.grads.range_from(g_aux);
+  zero->all_state = A.state.range_from(0);
   return LP_OK;
 }
 
 size_t lp_workspace_bytes(const lp_net_desc* desc) {
   NetDef net;
   if (net.build(desc) != LP_OK) return 0;
-  Arena A;
+  Arenas A;
   std::vector<Plan> m, a;
   int* e = nullptr;
   int32_t* z = nullptr;
-  plan_all(net, A, &m, &a, &e, &z);
-  return align_up(A.off, 256) + 256;
+  ZeroRanges r;
+  plan_all(net, A, &m, &a, &e, &z, &r);
+  return A.bytes() + 256;
 }
 
 int lp_param_layout(const lp_net_desc* desc, int which, lp_param_entry* entries, int max_entries, int* n_entries) {
@@ -2570,9 +2615,12 @@ int lp_create(const lp_net_desc* desc, void* dev_workspace, size_t bytes, lp_han
   h->conv_impl = net.d.conv_impl;
   h->ws = (uint8_t*)dev_workspace;
   h->ws_bytes = bytes;
-  Arena A;
-  A.base = h->ws;
-  plan_all(h->net, A, &h->modules, &h->auxs, &h->dev_err, &h->zero_labels);
+  Arenas A, sized;
+  plan_all(h->net, sized, &h->modules, &h->auxs, &h->dev_err, &h->zero_labels, &h->zero);
+  h->modules.clear();
+  h->auxs.clear();
+  A.place(h->ws, sized);
+  plan_all(h->net, A, &h->modules, &h->auxs, &h->dev_err, &h->zero_labels, &h->zero);
   if (cudaMemset(dev_workspace, 0, need) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
   auto upload = [&](Plan& P) -> int {
     if (!P.host_fold.empty())
@@ -2611,6 +2659,8 @@ int lp_create(const lp_net_desc* desc, void* dev_workspace, size_t bytes, lp_han
   if (cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
   if (cudaStreamCreateWithFlags(&h->aux_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->aux_end, cudaEventDisableTiming) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
+  if (cudaStreamCreateWithFlags(&h->zero_stream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->grads_zeroed, cudaEventDisableTiming) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
   h->aux_done.resize(net.K > 1 ? net.K - 1 : 0);
   for (auto& e : h->aux_done)
     if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
@@ -2628,6 +2678,8 @@ int lp_destroy(lp_handle* h) {
   if (h->recorder.stream) cudaStreamDestroy(h->recorder.stream);
   if (h->aux_stream) cudaStreamDestroy(h->aux_stream);
   if (h->aux_end) cudaEventDestroy(h->aux_end);
+  if (h->zero_stream) cudaStreamDestroy(h->zero_stream);
+  if (h->grads_zeroed) cudaEventDestroy(h->grads_zeroed);
   for (auto e : h->aux_done) if (e) cudaEventDestroy(e);
   for (auto& pr : h->prof.events) { cudaEventDestroy(pr.first); cudaEventDestroy(pr.second); }
   for (auto& r : h->tl.recs) { if (r.a) cudaEventDestroy(r.a); if (r.b) cudaEventDestroy(r.b); }
@@ -2699,9 +2751,7 @@ int lp_boundary_shape(lp_handle* h, int k, int shape[4]) {
   return LP_OK;
 }
 
-static int aux_plan_forward(lp_handle* h, int idx, RunCtx& c) {
-  int rc = zero_forward_state(h->auxs[idx], c.st);
-  if (rc != LP_OK) return rc;
+static int aux_plan_forward(lp_handle* h, int idx, RunCtx& c) {   // (statistics clear)
   c.plan_id = LP_AUX(idx); c.phase = LP_PHASE_AUX_FORWARD;
   return run_ops(h, h->auxs[idx], h->auxs[idx].fwd, c);
 }
@@ -2718,8 +2768,10 @@ int lp_auxnet_forward(lp_handle* h, const void* images, void* const* x_out, void
   return run_as_graph(h, CALL_AUX_FORWARD, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
     RunCtx c;
     c.st = st; c.images = images; c.xout = x_out;
+    int rc = zero_range(h, h->zero.aux_state, st);
+    if (rc != LP_OK) return rc;
     for (size_t i = 0; i < h->auxs.size(); ++i) {   // chain order, or stack by stack (units in order)
-      int rc = aux_plan_forward(h, (int)i, c);
+      rc = aux_plan_forward(h, (int)i, c);
       if (rc != LP_OK) return rc;
     }
     return LP_OK;
@@ -2740,7 +2792,10 @@ int lp_module_fwd_bwd(lp_handle* h, int k, const void* x_k, const void* x_next_o
                       float rho, float* loss_out, void* dx_k, void* stream) {
   int rc = check_module_args(h, k, x_k, x_next_or_labels, lambda_k, loss_out, dx_k);
   if (rc != LP_OK) return rc;
-  return module_fwd_bwd(h, k, x_k, x_next_or_labels, lambda_k, rho, loss_out, dx_k, (cudaStream_t)stream);
+  rc = zero_range(h, h->modules[k].state, (cudaStream_t)stream);
+  if (rc == LP_OK) rc = zero_range(h, h->modules[k].grads, (cudaStream_t)stream);
+  if (rc != LP_OK) return rc;
+  return module_fwd_bwd(h, k, x_k, x_next_or_labels, lambda_k, rho, loss_out, dx_k, (cudaStream_t)stream, nullptr);
 }
 
 // Marks the handle while the modules are being enqueued side by side (convolution grids then leave SMs
@@ -2763,19 +2818,22 @@ int lp_modules_fwd_bwd_all(lp_handle* h, const void* const* x, const int32_t* la
   }
   return run_as_graph(h, CALL_MODULES, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   ConcurrentScope concurrent(h);
+  const int rc0 = zero_range(h, h->zero.module_state, st);
+  if (rc0 != LP_OK) return rc0;
   LP_CUDA_OK(cudaEventRecord(h->fork, st));
   // heaviest modules first is not needed: all K are enqueued before any can finish
   // A failure part-way still joins every stream that was forked back into the caller's (a stream left
   // unjoined would invalidate a capture in progress); the first error is what the call returns.
-  int first_err = LP_OK;
+  int first_err = zero_grads_beside(h);
   int forked = 0;
   for (int k = 0; k < K && first_err == LP_OK; ++k) {
     if (cudaStreamWaitEvent(h->streams[k], h->fork, 0) != cudaSuccess) { first_err = LP_ERR_CUDA; break; }
     forked = k + 1;
     const void* tgt = k == K - 1 ? (const void*)labels : x[k + 1];
     first_err = module_fwd_bwd(h, k, x[k], tgt, (lambdas && k < K - 1) ? lambdas[k] : nullptr, rho, loss_out + 2 * k,
-                               dx ? dx[k] : nullptr, h->streams[k]);
+                               dx ? dx[k] : nullptr, h->streams[k], h->grads_zeroed);
   }
+  if (cudaStreamWaitEvent(st, h->grads_zeroed, 0) != cudaSuccess && first_err == LP_OK) first_err = LP_ERR_CUDA;
   for (int k = 0; k < forked; ++k) {
     if (cudaEventRecord(h->done[k], h->streams[k]) != cudaSuccess || cudaStreamWaitEvent(st, h->done[k], 0) != cudaSuccess)
       if (first_err == LP_OK) first_err = LP_ERR_CUDA;
@@ -2842,7 +2900,10 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
   }
   return run_as_graph(h, CALL_LAYER_PARALLEL, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   ConcurrentScope concurrent(h);
+  const int rc0 = zero_range(h, h->zero.all_state, st);
+  if (rc0 != LP_OK) return rc0;
   LP_CUDA_OK(cudaEventRecord(h->fork, st));
+  const int rc1 = zero_grads_beside(h);
   // Streams forked from the caller's so far; whatever happens below, each is joined back before the
   // call returns (a stream left unjoined would invalidate a capture in progress).
   bool aux_forked = false;
@@ -2860,6 +2921,7 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
     return rc;
   };
   auto enqueue = [&]() -> int {
+    if (rc1 != LP_OK) return rc1;
     int rc = fork(h->aux_stream, &aux_forked);
     if (rc != LP_OK) return rc;
     if (h->net.d.aux_recursive) {
@@ -2894,7 +2956,7 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
       const void* tgt = last ? (const void*)labels : (const void*)x_out[k];
       void* lam = (lambdas_inout && !last) ? lambdas_inout[k] : nullptr;
       rc = module_fwd_bwd(h, k, xk, tgt, lam, rho, loss_out + 2 * k, dx ? dx[k] : nullptr, sk,
-                          last ? nullptr : h->aux_done[k]);
+                          h->grads_zeroed, last ? nullptr : h->aux_done[k]);
       if (rc != LP_OK) return rc;
       rc = update_module(h, k, lr, momentum, weight_decay, kappa_step, lam, sk);
       if (rc != LP_OK) return rc;
@@ -2902,6 +2964,7 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
     return LP_OK;
   };
   int first_err = enqueue();
+  if (cudaStreamWaitEvent(st, h->grads_zeroed, 0) != cudaSuccess && first_err == LP_OK) first_err = LP_ERR_CUDA;
   if (aux_forked) {
     if (cudaEventRecord(h->aux_end, h->aux_stream) != cudaSuccess || cudaStreamWaitEvent(st, h->aux_end, 0) != cudaSuccess)
       if (first_err == LP_OK) first_err = LP_ERR_CUDA;
@@ -2928,6 +2991,8 @@ int lp_auxnet_distill(lp_handle* h, const void* images, void* const* x, const vo
   return run_as_graph(h, CALL_DISTILL, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   RunCtx c;
   c.st = st; c.images = images; c.xout = x;
+  const int rc0 = zero_range(h, h->zero.aux_grads, st);
+  if (rc0 != LP_OK) return rc0;
   const bool rec = h->net.d.aux_recursive != 0;
   for (int k = 1; k < K; ++k) {
     // the network that produced x_k: AuxNet_{k-1}, or the last unit of stack k
@@ -2935,8 +3000,6 @@ int lp_auxnet_distill(lp_handle* h, const void* images, void* const* x, const vo
     const int first_idx = rec ? NetDef::reaux_index(k, 0) : k - 1;
     Plan& A = h->auxs[last_idx];
     const long long n = A.seed.elems();
-    LP_CUDA_OK(cudaMemsetAsync(A.loss_acc, 0, 2 * sizeof(double), st));
-    for (int i = first_idx; i <= last_idx; ++i) LP_CUDA_OK(cudaMemsetAsync(h->auxs[i].ps.g, 0, h->auxs[i].ps.n * 4, st));
     void* xn = x_new ? x_new[k - 1] : nullptr;
     if (h->dtype == LP_F32)
       distill_seed_kernel<float><<<grid_for(n / 4, 256, cur_dev().sm_count, 8), 256, 0, st>>>(
@@ -3002,12 +3065,12 @@ int lp_aux_correct(lp_handle* h, void* const* x_inout, const void* const* dx, fl
 static int serial_forward(lp_handle* h, const void* images, const int32_t* labels, float* loss_out, cudaStream_t st) {
   const int K = h->net.K;
   const void* x = images;
+  int rc = zero_range(h, h->zero.module_state, st);
+  if (rc != LP_OK) return rc;
   for (int k = 0; k < K; ++k) {
     Plan& P = h->modules[k];
     RunCtx c;
     c.st = st; c.x = x; c.serial = true; c.labels = labels; c.loss_out = loss_out;
-    int rc = zero_forward_state(P, st);
-    if (rc != LP_OK) return rc;
     c.plan_id = k; c.phase = LP_PHASE_FORWARD;
     rc = run_ops(h, P, P.fwd, c);
     if (rc != LP_OK) return rc;
@@ -3034,8 +3097,10 @@ int lp_serial_fwd_bwd(lp_handle* h, const void* images, const int32_t* labels, f
   if (!aligned16(images)) return LP_ERR_ALIGN;
   return run_as_graph(h, CALL_SERIAL, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   const int K = h->net.K;
-  for (int k = 0; k < K; ++k) LP_CUDA_OK(cudaMemsetAsync(h->modules[k].ps.g, 0, h->modules[k].ps.n * 4, st));
-  int rc = serial_forward(h, images, labels, loss_out, st);
+  LP_CUDA_OK(cudaEventRecord(h->fork, st));
+  int rc = zero_grads_beside(h);
+  if (rc == LP_OK) rc = serial_forward(h, images, labels, loss_out, st);
+  if (cudaStreamWaitEvent(st, h->grads_zeroed, 0) != cudaSuccess && rc == LP_OK) rc = LP_ERR_CUDA;
   if (rc != LP_OK) return rc;
   for (int k = K - 1; k >= 0; --k) {
     Plan& P = h->modules[k];
