@@ -212,15 +212,26 @@ void launch_bn_apply(int grid, int threads, cudaStream_t st, const T* x, const B
 // ---------------------------------------------------------------------------------------
 // Interior local loss, fused into the kernel that produces the module output:
 //   out = bnA(x) [+ bnB(x2)] [+ addend];  r = out - x_next;  seed = rho*r + kappa
-// writes r and seed, accumulates sum r^2 and sum kappa*r (double atomics, one pair per block).
-// With x == nullptr the output is taken from `addend` alone (already final).
+// writes r and seed, accumulates sum r^2 and sum kappa*r (double atomics, one pair per block); the last block turns the
+// sums into the two results.  With x == nullptr the output is taken from `addend` alone (already final).
 // ---------------------------------------------------------------------------------------
+// Sums of a loss over the blocks of a launch: [0], [1] the sums, [2] the number of blocks that have added theirs.  Returns
+// true in the last one, which then reads them.
+__device__ __forceinline__ bool loss_block_done(double* acc) {
+  __threadfence();
+  unsigned int* count = reinterpret_cast<unsigned int*>(acc + 2);
+  const bool last = atomicAdd(count, 1u) == gridDim.x - 1;
+  if (last) __threadfence();
+  return last;
+}
 template <typename T>
 __global__ void module_out_loss_kernel(const T* __restrict__ x, BnArgs A, const T* __restrict__ x2, BnArgs B,
                                        const T* __restrict__ addend, const T* __restrict__ x_next,
                                        const T* __restrict__ kappa, float rho, T* __restrict__ r_out,
-                                       T* __restrict__ seed_out, double* __restrict__ acc,
+                                       T* __restrict__ seed_out, double* acc, float* __restrict__ loss_out,
                                        long long total_vecs, int C) {
+  pdl_wait();
+  pdl_launch_dependents();
   constexpr int V = VecT<T>::N;
   const int CV = C / V;
   const int c0 = (threadIdx.x % CV) * V;
@@ -304,10 +315,16 @@ __global__ void module_out_loss_kernel(const T* __restrict__ x, BnArgs A, const 
     if (threadIdx.x == 0) {
       atomicAdd(&acc[0], (double)a);
       atomicAdd(&acc[1], (double)b);
+      if (loss_block_done(acc)) {
+        const double rr = __ldcg(&acc[0]), kr = __ldcg(&acc[1]);
+        loss_out[0] = (float)(0.5 * (double)rho * rr + kr);
+        loss_out[1] = (float)rr;
+      }
     }
   }
 }
 
+// (where the sums came from the epilogue of the module's last convolution)
 __global__ void loss_finalize_kernel(const double* __restrict__ acc, float rho, float* __restrict__ loss_out) {
   loss_out[0] = (float)(0.5 * (double)rho * acc[0] + acc[1]);
   loss_out[1] = (float)acc[0];
@@ -528,6 +545,8 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 maxpool_bwd_kernel(const T* __restrict__ dy, const uint8_t* __restrict__ arg, T* __restrict__ dx,
                    int N, int H, int W, int C, int OH, int OW) {
+  pdl_wait();
+  pdl_launch_dependents();
   constexpr int V = VecT<T>::N;
   const int CV = C / V;
   const int cg = threadIdx.x % CV, per_block = blockDim.x / CV;
@@ -584,6 +603,8 @@ maxpool_bwd_kernel(const T* __restrict__ dy, const uint8_t* __restrict__ arg, T*
 template <typename T>
 __global__ void __launch_bounds__(256)
 avgpool_kernel(const T* __restrict__ x, float* __restrict__ pooled, int HW, int C) {
+  pdl_wait();
+  pdl_launch_dependents();
   constexpr int V = VecT<T>::N;
   __shared__ float part[8][32][V + 1];
   const int n = blockIdx.x, lane = threadIdx.x & 31, pl = threadIdx.x >> 5;
@@ -625,6 +646,8 @@ __device__ __forceinline__ float4 ld4(const float* p) {
 __global__ void __launch_bounds__(128)
 head_logits_kernel(const float* __restrict__ pooled, const float* __restrict__ Wt, const float* __restrict__ bias,
                    float* __restrict__ logits, int N, int C, int classes) {
+  pdl_wait();
+  pdl_launch_dependents();
   const int lane = threadIdx.x & 31;
   const int j0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * 4, n0 = blockIdx.y * 8;
   if (j0 >= classes) return;
@@ -658,9 +681,21 @@ head_logits_kernel(const float* __restrict__ pooled, const float* __restrict__ W
   if (j < classes && n < N) logits[(long long)n * classes + j] = acc[0] + bias[j];
 }
 
+// Loss of a sample into the mean over the batch; the last block of the launch (one per sample) writes the result.
+__device__ __forceinline__ void head_add_loss(double* acc, double loss, float* loss_out) {
+  atomicAdd(acc, loss);
+  if (loss_out && loss_block_done(acc)) {
+    loss_out[0] = (float)__ldcg(acc);
+    loss_out[1] = 0.f;
+  }
+}
+
 // one block per sample; softmax of the logits, loss (atomic mean), dlogits = (softmax - onehot)/N
 __global__ void head_fwd_kernel(const int32_t* __restrict__ labels, const float* __restrict__ logits,
-                                float* __restrict__ dlogits, double* __restrict__ loss_acc, int N, int classes) {
+                                float* __restrict__ dlogits, double* loss_acc, float* __restrict__ loss_out, int N,
+                                int classes) {
+  pdl_wait();
+  pdl_launch_dependents();
   extern __shared__ float sh[];  // [classes] logits, then reduction scratch [32]
   float* lg = sh;
   float* red = sh + classes;
@@ -688,7 +723,7 @@ __global__ void head_fwd_kernel(const int32_t* __restrict__ labels, const float*
     const float p = __expf(lg[j] - lse);
     dlogits[(long long)n * classes + j] = (p - (j == lab ? 1.f : 0.f)) / (float)N;
   }
-  if (threadIdx.x == 0) atomicAdd(loss_acc, (double)(lse - lg[lab]) / (double)N);
+  if (threadIdx.x == 0) head_add_loss(loss_acc, (double)(lse - lg[lab]) / (double)N, loss_out);
 }
 
 // Heads of few classes (at most 128: the CIFAR-shaped networks) in one launch, one block of 256 threads per
@@ -699,7 +734,10 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 head_fused_kernel(const T* __restrict__ x, const float* __restrict__ Wt, const float* __restrict__ bias,
                   const int32_t* __restrict__ labels, float* __restrict__ pooled, float* __restrict__ logits,
-                  float* __restrict__ dlogits, double* __restrict__ loss_acc, int N, int HW, int C, int classes) {
+                  float* __restrict__ dlogits, double* loss_acc, float* __restrict__ loss_out, int N, int HW, int C,
+                  int classes) {
+  pdl_wait();
+  pdl_launch_dependents();
   extern __shared__ float sh[];  // [C] pooled, then [classes] logits
   float* sp = sh;
   float* lg = sh + C;
@@ -768,12 +806,7 @@ head_fused_kernel(const T* __restrict__ x, const float* __restrict__ Wt, const f
     const float pj = __expf(lg[j] - lse);
     dlogits[(long long)n * classes + j] = (pj - (j == lab ? 1.f : 0.f)) / (float)N;
   }
-  if (lane == 0) atomicAdd(loss_acc, (double)(lse - lg[lab]) / (double)N);
-}
-
-__global__ void ce_finalize_kernel(const double* __restrict__ acc, float* __restrict__ loss_out) {
-  loss_out[0] = (float)acc[0];
-  loss_out[1] = 0.f;
+  if (lane == 0) head_add_loss(loss_acc, (double)(lse - lg[lab]) / (double)N, loss_out);
 }
 
 // dW[j][c] = sum_n dlogits[n][j]*pooled[n][c]; db[j] = sum_n dlogits[n][j].  Block: 32 items of 4 classes x 4 channels,
@@ -782,6 +815,8 @@ __global__ void ce_finalize_kernel(const double* __restrict__ acc, float* __rest
 __global__ void __launch_bounds__(256)
 head_bwd_w_kernel(const float* __restrict__ dlogits, const float* __restrict__ pooled,
                   float* __restrict__ dW, float* __restrict__ db, int N, int C, int classes) {
+  pdl_wait();
+  pdl_launch_dependents();
   __shared__ float part[8][32][21];     // 16 products, 4 sums of dlogits
   const int it = threadIdx.x & 31, ng = threadIdx.x >> 5;
   const int c4n = C >> 2;
@@ -834,6 +869,8 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 head_bwd_x_kernel(const float* __restrict__ dlogits, const float* __restrict__ Wt, T* __restrict__ d, int N, int HW, int C,
                   int classes) {
+  pdl_wait();
+  pdl_launch_dependents();
   extern __shared__ float sh[];          // [min(classes, chunk)][8] dlogits; afterwards [8 warps][8 samples][32] partial sums
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + lane, n0 = blockIdx.y * 8;
@@ -1054,6 +1091,26 @@ __global__ void pack_weights_tiled_kernel(const PackEntry* __restrict__ tab, int
   }
 }
 
+// Parameters that have no packed copy (normalisation, head, convolutions on the CUDA-core path): ranges of the blob.
+struct SgdRange {
+  long long begin;
+  int count;
+};
+__device__ __forceinline__ void sgd_range(const SgdRange& r, float* __restrict__ p, const float* __restrict__ g,
+                                          float* __restrict__ mom, float lr, float momentum, float wd) {
+  // (ranges are at most 4096 elements; their start need not be a multiple of 4)
+#pragma unroll 4
+  for (int i = threadIdx.x; i < r.count; i += 256) {
+    const long long j = r.begin + i;
+    float gi = g[j] + wd * p[j];
+    if (momentum != 0.f) {
+      gi = momentum * mom[j] + gi;
+      mom[j] = gi;
+    }
+    p[j] -= lr * gi;
+  }
+}
+
 // The update and the weight copies in one pass over the packed convolution weights:
 //   w <- w - lr*(g + wd*w [momentum])   then the two bf16 copies of the new w, as above,
 // on 64 (c_out) x 64 (c_in) tiles of one tap with 16-byte accesses: a thread holds four float4 pieces of the
@@ -1062,12 +1119,20 @@ __global__ void pack_weights_tiled_kernel(const PackEntry* __restrict__ tab, int
 // `m_base` are the parameter, gradient and momentum blobs the entries point into (m_base may be null when
 // momentum is 0).  Requires c_in % 4 == 0, c_out % 2 == 0 and 16-byte aligned weight tensors inside the blobs
 // (checked when the table is built; otherwise the plain update and pack_weights_tiled_kernel run instead).
-// blockDim = 256.
+// blockDim = 256.  The first n_ranges blocks update the parameters without a packed copy: a launch of their own took another
+// 3 to 7 us at the end of every module's chain.
 __global__ void __launch_bounds__(256)
-sgd_pack_tiled64_kernel(const PackEntry* __restrict__ tab, int n_entries, float* __restrict__ p_base,
-                        const float* __restrict__ g_base, float* __restrict__ m_base, float lr, float momentum, float wd) {
+sgd_pack_tiled64_kernel(const SgdRange* __restrict__ ranges, int n_ranges, const PackEntry* __restrict__ tab, int n_entries,
+                        float* __restrict__ p_base, const float* __restrict__ g_base, float* __restrict__ m_base, float lr,
+                        float momentum, float wd) {
+  pdl_wait();
+  pdl_launch_dependents();
+  if ((int)blockIdx.x < n_ranges) {
+    sgd_range(ranges[blockIdx.x], p_base, g_base, m_base, lr, momentum, wd);
+    return;
+  }
   __shared__ float tile[64][65];
-  const long long b = blockIdx.x;
+  const long long b = blockIdx.x - n_ranges;
   int lo = 0, hi = n_entries - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -1208,29 +1273,6 @@ __global__ void s2d_unpack_wgrad_kernel(const float* __restrict__ dws, float* __
     const int ah = (r - 3 - by) / 2, aw = (q - 3 - bx) / 2;   // exact: the numerators are even
     const int tap = (ah + 2) * 4 + (aw + 2);
     gw[i] = dws[((long long)co * 16 + tap) * 16 + (by * 2 + bx) * C + c];
-  }
-}
-
-// Plain update of the parameters that have no packed copy (normalisation, head, convolutions on
-// the CUDA-core path): one block per range of the blob.
-struct SgdRange {
-  long long begin;
-  int count;
-};
-__global__ void sgd_ranges_kernel(const SgdRange* __restrict__ ranges, float* __restrict__ p,
-                                  const float* __restrict__ g, float* __restrict__ mom, float lr, float momentum,
-                                  float wd) {
-  const SgdRange r = ranges[blockIdx.x];
-  // (ranges are at most 4096 elements; their start need not be a multiple of 4)
-#pragma unroll 4
-  for (int i = threadIdx.x; i < r.count; i += 256) {
-    const long long j = r.begin + i;
-    float gi = g[j] + wd * p[j];
-    if (momentum != 0.f) {
-      gi = momentum * mom[j] + gi;
-      mom[j] = gi;
-    }
-    p[j] -= lr * gi;
   }
 }
 
