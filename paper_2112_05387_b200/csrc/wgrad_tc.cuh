@@ -57,6 +57,7 @@ struct WgradParams {
   // halo kernel (3x3, stride 1)
   int groups, acc_stride;        // (ci chunk, kernel row) groups; TMEM column stride of an accumulator
   uint32_t a_box_bytes;          // one x box: (8+2) x BNI x BH pixels x 64 channels
+  int one_box;                   // 1: one box of BH + 1 image rows serves both groups of a CTA (see wgrad_halo_kernel)
   uint32_t a_start3[3];          // first row of the three accumulators' A operands (bytes into the A region)
   uint64_t adesc_hi3[3];         // their descriptors (the leading byte offset differs)
   uint32_t a_kstep_bytes;        // 16 pixels further along K
@@ -351,6 +352,9 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 // box, (box size - 256) across the two boxes.  Per 128 pixels of K a CTA fetches x boxes of 40 KB and
 // the dy tile (128 x n_tile) for 24 MMAs, against 6 sub-boxes (96 KB) without the reuse.
 // Roles as in wgrad_tc_kernel, plus a second MMA-issuing warp (warp 7; 256 threads).
+// Where C_in is a single chunk of 64 the two groups of a CTA are kernel rows r and r + 1 of the same channels: ONE box of
+// BH + 1 image rows serves both (the second group starts one image row into it), and the last CTA of the three kernel rows
+// has one group and leaves out its third accumulator.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256, 1)
 wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmDY,
@@ -362,6 +366,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m_tile = blockIdx.x % p.m_tiles, n_tile = blockIdx.x / p.m_tiles;
   const int g0 = 2 * m_tile;                       // groups g0 and g0 + 1 (the second may not exist)
+  const bool second = g0 + 1 < p.groups;
   const int split = blockIdx.y;
   const int pt_begin = (int)(((long long)p.pix_tiles * split) / p.splits);
   const int pt_end = (int)(((long long)p.pix_tiles * (split + 1)) / p.splits);
@@ -409,8 +414,10 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
       uint8_t* sa = smem + s * p.stage_bytes;
       const bool leader = elect_one();
       if (leader && do_a) {
-        mbar_expect_tx(&tail->full[s], 2 * p.tx_a);
-        for (int j = 0; j < 2; ++j) {
+        const int boxes = p.one_box ? 1 : 2;
+        mbar_expect_tx(&tail->full[s], boxes * p.tx_a);
+#pragma unroll 1
+        for (int j = 0; j < boxes; ++j) {
           const int g = min(g0 + j, p.groups - 1);   // a missing second group: any finite data
           const int c0 = (g / 3) * 64, r = g % 3;
           tma_load_4d(sa + j * p.a_box_bytes, &tmX, &tail->full[s], c0, w0 - 1, n0, h0 + r - 1);
@@ -462,7 +469,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
             mma_bf16_lh(d1, a1 + ak, a_hi1, bt + bk, b_hi, p.idesc, 1u);
             a0 += 2 * ak; a1 += 2 * ak; bt += 2 * bk;
           }
-        } else {
+        } else if (second) {
           if (k & 1) {
             mma_bf16_lh(d0, a0, a_hi0, bt, b_hi, p.idesc, accum);
             accum = 1;
@@ -501,7 +508,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
       const int rounds_in_flight = p.epi_bufs >> 1;
       const int co0 = n_tile * p.n_tile;
 #pragma unroll 1
-      for (int a = 0; a < 3; ++a) {
+      for (int a = 0; a < (second ? 3 : 2); ++a) {
         if (a >= rounds_in_flight) {
           if (et == 0) bulk_wait_read(rounds_in_flight - 1);
           asm volatile("bar.sync 1, 128;" ::: "memory");
@@ -533,7 +540,7 @@ wgrad_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     } else if (*(volatile int*)&tail->epi_ok) {
       tc_fence_after();
 #pragma unroll 1
-      for (int a = 0; a < 3; ++a) {
+      for (int a = 0; a < (second ? 3 : 2); ++a) {
         const int chunk = 2 * a + (row >> 6);          // 0..5: group chunk/3, kernel column chunk%3
         const int g = g0 + chunk / 3, sx = chunk % 3;
         const int ci_raw = (g / 3) * 64 + (row & 63);
@@ -659,18 +666,19 @@ static int launch_wgrad_halo(WgEncodeFn enc, int sm_count, bool* attr_done, cons
   // pixel box (K block): 8 x BH x BNI = LP_WGRAD_HALO_KBLOCK pixels.  Blocks of 64 make a stage 40 KB
   // instead of 80 KB for a 160-channel tile (five stages in flight instead of two); measured, that is
   // no faster (0.079 against 0.078 ms at 160 channels), so the copy latency is not what limits it.
-  constexpr int per_col = LP_WGRAD_HALO_KBLOCK / 8;
+  // (A launch that shares its SM has 100 KB: three stages of 64 pixels.)
+  const int per_col = (shared_sm ? 64 : LP_WGRAD_HALO_KBLOCK) / 8;
   if (H >= per_col) {                       // rows spread evenly over the tiles of a column (14: 14, 28: 2 x 14, 56: 4 x 14)
     const int th = (H + per_col - 1) / per_col;
     p.BH = (H + th - 1) / th;
     p.BH += p.BH & 1;                       // (a K step of 16 pixels is two of them)
-    if (p.BH * 8 < 96) return 1;
+    if (4 * p.BH < 3 * per_col) return 1;
     p.BNI = 1;
   } else {
     p.BH = H;
     p.BNI = per_col / H;
     if ((p.BH * p.BNI) & 1) --p.BNI;
-    if (p.BNI < 1 || p.BH * p.BNI * 8 < 96) return 1;
+    if (p.BNI < 1 || 4 * p.BH * p.BNI < 3 * per_col) return 1;
   }
   if (p.BNI > N) return 1;
   p.BW = 8;
@@ -702,9 +710,10 @@ static int launch_wgrad_halo(WgEncodeFn enc, int sm_count, bool* attr_done, cons
   p.cin_chunks = (Cin + 63) / 64;
   p.groups = 3 * p.cin_chunks;
   p.m_tiles = (p.groups + 1) / 2;
-  const int box_rows = 10 * p.BNI * p.BH;
+  p.one_box = p.cin_chunks == 1 ? 1 : 0;
+  const int box_rows = 10 * p.BNI * (p.BH + p.one_box);
   p.a_box_bytes = (uint32_t)((box_rows * 128 + 1023) / 1024 * 1024);
-  p.a_region = 2 * p.a_box_bytes;
+  p.a_region = (p.one_box ? 1 : 2) * p.a_box_bytes;
   p.b_sub_bytes = (uint32_t)((p.rows * p.scb * 2 + 1023) / 1024 * 1024);
   p.stage_bytes = p.a_region + p.b_sub_bytes * p.nb;
   p.tx_a = (uint32_t)(box_rows * 128);
@@ -716,18 +725,21 @@ static int launch_wgrad_halo(WgEncodeFn enc, int sm_count, bool* attr_done, cons
   p.stages = stages;
   // A operands: rows of 128 bytes; an 8-pixel K group is 8 rows, the next group 10 rows further
   const uint32_t sbo = 10 * 128;
-  const uint32_t lbo_in = 128, lbo_across = p.a_box_bytes - 2 * 128;
+  const uint32_t g1_start = p.one_box ? (uint32_t)(10 * p.BNI * 128) : p.a_box_bytes;   // first row of the second group
+  const uint32_t lbo_in = 128, lbo_across = g1_start - 2 * 128;
   p.a_start3[0] = 0;                p.adesc_hi3[0] = tc::smem_desc_hi(lbo_in, sbo, 2);
   p.a_start3[1] = 2 * 128;          p.adesc_hi3[1] = tc::smem_desc_hi(lbo_across, sbo, 2);
-  p.a_start3[2] = p.a_box_bytes + 128; p.adesc_hi3[2] = tc::smem_desc_hi(lbo_in, sbo, 2);
+  p.a_start3[2] = g1_start + 128;   p.adesc_hi3[2] = tc::smem_desc_hi(lbo_in, sbo, 2);
   p.a_kstep_bytes = 2 * sbo;                             // 16 pixels = two groups
   p.bdesc_hi = tc::smem_desc_hi(p.b_sub_bytes, 8 * p.scb * 2, tc::swizzle_code_for_row_bytes(p.scb * 2));
   p.idesc = tc::instr_desc_bf16(128, p.n_tile, 1, 1);
   const int tiles = p.m_tiles * p.n_tiles;
-  p.splits = wgrad_splits(tiles, p.pix_tiles, 1.5 * (p.rows / 128.0), sm_count, side_by_side);
+  // (three accumulators: 1.5 blocks' time.  64 channels with one box: 760 cycles for 64 pixels against 8 to 9 thousand of start,
+  // first fill and epilogue)
+  p.splits = wgrad_splits(tiles, p.pix_tiles, (p.one_box && p.n_tile == 64 ? 0.75 : 1.5) * (p.rows / 128.0), sm_count, side_by_side);
   p.dw = dw; p.err = dev_err;
   CUtensorMap tmX, tmDY;
-  if (wg_encode_wnh(enc, &tmX, x, N, H, W, Cin, 64, 10, p.BNI, p.BH)) return -8;
+  if (wg_encode_wnh(enc, &tmX, x, N, H, W, Cin, 64, 10, p.BNI, p.BH + p.one_box)) return -8;
   if (wg_encode_wnh(enc, &tmDY, dy, N, H, W, Cout, p.scb, 8, p.BNI, p.BH)) return -8;
   // dw as a (C_in, tap, C_out) fp32 tensor for the bulk-reduction epilogue: boxes of 64 input channels
   // of one tap and the CTA's output channels; staged in the operand ring after the main loop
