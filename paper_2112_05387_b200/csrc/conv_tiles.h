@@ -45,18 +45,37 @@ inline double conv_tile_cycles(const ConvTileQuery& q, int tile) {
   return 3800.0 + mma + epi + (per - 1.0) * std::max(mma, epi);
 }
 
-// Channel tile of a launch that has the machine to itself: the widest tiles leave SMs idle where there are few pixel tiles
-// (74 CTAs of 256 channels on 37 images of 12x16).  A narrower tile has to be estimated 2 % faster.
-inline void pick_n_tile_alone(const ConvTileQuery& q, int& n_tile, int& n_tiles) {
+// What SM time is worth beside the length of a launch, where modules run side by side: a launch of length t on a share s of the
+// SMs costs t (1 + w s).  `step_flops`: convolutions of one training step.  Steps of little work are as long as their chains of
+// launches, and narrower tiles shorten a launch of few CTAs (8 CTAs of 256 channels took 40 to 46 us of ResNet-50's last module
+// on 12 images of 176x176); steps of much work are bound by the SM time that narrow tiles waste.  us per step for w = none, 1,
+// 2, 4, 8, 16: ResNet-34 on 3 images of 256x176 (0.06 TFLOP) 781, 683, 640, 638, 642, 674, on 25 of 128x160 with recursive
+// AuxNets and distillation (0.22) 1234, 1159, 1158, 1196, 1232, 1232; ResNet-50 on 12 of 176x176 (0.18) 1405, 1369, 1360, 1361,
+// 1370, 1410, on 19 with distillation (0.29) 2130, 2091, 2086, 2090, 2106, 2134, on 32 of 224x224 (0.79) 3303, 3358, 3332, 3325,
+// 3306, 3308.
+inline double sm_time_worth(double step_flops) {
+  const double x = step_flops / 0.25e12;
+  return 2.5 * std::max(1.0, x * x * x);
+}
+
+// Channel tile of least cost: `worth` = 0 for a launch that has the machine to itself, sm_time_worth() beside other modules.  The
+// widest tiles leave SMs idle where there are few pixel tiles (74 CTAs of 256 channels on 37 images of 12x16).  A narrower tile
+// has to be estimated 2 % cheaper.
+inline void pick_n_tile_by_cost(const ConvTileQuery& q, double worth, int& n_tile, int& n_tiles) {
+  const auto cost = [&](int tile) {
+    const long long tiles = (long long)q.m_tiles * ((q.Cout + tile - 1) / tile);
+    return conv_tile_cycles(q, tile) * (1.0 + worth * (double)std::min<long long>(tiles, q.sm_count) / q.sm_count);
+  };
   pick_n_tile(q.Cout, n_tile, n_tiles);
   const int widest = n_tile, lo = (q.Cout + 255) / 256;
-  double best = conv_tile_cycles(q, widest);
+  double best = cost(widest);
   for (int nt = lo; nt <= 8 * lo; ++nt) {
     const int tile = ((q.Cout + nt - 1) / nt + 31) / 32 * 32;
     if (tile > 256 || tile < 64 || tile == widest) continue;
-    const double t = conv_tile_cycles(q, tile);
+    const double t = cost(tile);
     if (t < best * 0.98) { best = t; n_tile = tile; n_tiles = (q.Cout + tile - 1) / tile; }
   }
 }
+inline void pick_n_tile_alone(const ConvTileQuery& q, int& n_tile, int& n_tiles) { pick_n_tile_by_cost(q, 0.0, n_tile, n_tiles); }
 
 }  // namespace lp

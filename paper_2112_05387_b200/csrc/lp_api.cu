@@ -292,6 +292,7 @@ struct lp_handle {
   ConvProfile prof;
   Timeline tl;
   int conv_impl = LP_CONV_IMPL_AUTO;
+  double step_flops = 0.0;   // convolutions of the modules, forward and backward
   bool concurrent = false;   // set while a call enqueues the K modules on their own streams
   uint8_t* ws = nullptr;
   size_t ws_bytes = 0;
@@ -651,10 +652,10 @@ static int launch_conv_tc(lp_handle* h, const TcGemmSpec& s, int* dev_err, cudaS
   // Eight epilogue warps (below) may be taken: not by the epilogues that have four-warp scratch, and only where few MMAs
   // hide a tile's epilogue.
   const bool wide_ok = !bnbwd && !s.x_next && s.n_cls <= 1 && s.ntaps * s.aC <= 1024;
-  if (!(h && h->concurrent) && s.n_cls <= 1 && s.w_rows % 32 == 0 && s.w_rows > 64) {
+  if (s.n_cls <= 1 && s.w_rows % 32 == 0 && s.w_rows > 64) {
     const ConvTileQuery q{s.w_rows, p.m_tiles, cur_dev().sm_count, s.ntaps * ((s.aC + 15) / 16),
                           s.addend || bnbwd ? 2 : (s.stats ? 1 : 0), wide_ok};
-    pick_n_tile_alone(q, p.n_tile_cols, p.n_tiles);
+    pick_n_tile_by_cost(q, h && h->concurrent ? sm_time_worth(h->step_flops) : 0.0, p.n_tile_cols, p.n_tiles);
   }
   p.n_cls = std::max(1, s.n_cls);
   int max_cls_taps = s.ntaps;
@@ -2655,6 +2656,8 @@ int lp_create(const lp_net_desc* desc, void* dev_workspace, size_t bytes, lp_han
   };
   for (auto& P : h->modules) if ((rc = upload(P)) != LP_OK) { delete h; return rc; }
   for (auto& P : h->auxs) if ((rc = upload(P)) != LP_OK) { delete h; return rc; }
+  for (const Plan& P : h->modules)
+    for (const ConvDef& c : P.convs) h->step_flops += 6.0 * net.d.N * c.OH * c.OW * (double)c.cout * c.R * c.R * c.cin;
   h->streams.resize(net.K);
   h->done.resize(net.K);
   for (int k = 0; k < net.K; ++k) {

@@ -27,16 +27,34 @@ extern "C" int alone(int cout, int m_tiles, int k_mmas, int epilogue, int wide, 
   lp::pick_n_tile_alone(lp::ConvTileQuery{cout, m_tiles, 148, k_mmas, epilogue, wide != 0}, tile, *n_tiles);
   return tile;
 }
+extern "C" int beside(int cout, int m_tiles, int k_mmas, int epilogue, int wide, double step_flops) {
+  int tile = 0, n = 0;
+  lp::pick_n_tile_by_cost(lp::ConvTileQuery{cout, m_tiles, 148, k_mmas, epilogue, wide != 0}, lp::sm_time_worth(step_flops), tile, n);
+  return n * tile >= cout ? tile : -1;
+}
 """)
+    lib.beside.argtypes = [ctypes.c_int] * 5 + [ctypes.c_double]
 
     def alone(cout, m_tiles, k_mmas, epilogue, wide):
         n = ctypes.c_int(0)
         tile = lib.alone(cout, m_tiles, k_mmas, epilogue, int(wide), ctypes.byref(n))
         return tile, n.value
+    alone.beside = lib.beside
     return alone
 
 
 PLAIN, STATS, SHORTCUT = 0, 1, 2
+
+
+@pytest.mark.parametrize("q,tflop,tiles", [
+    ((512, 4, 288, STATS, False), 0.18, (64, 128)),       # 12 images of 6x6, a step of little work: more than 8 CTAs
+    ((256, 12, 144, STATS, False), 0.18, (64, 128)),
+    ((256, 896, 4, STATS, True), 0.18, (256,)),           # a launch that fills the machine as it is
+    ((512, 4, 288, STATS, False), 30.0, (256,)),          # a step bound by SM time
+    ((64, 4, 36, STATS, False), 0.01, (64,)),
+])
+def test_channel_tile_beside_other_modules(tile_rules, q, tflop, tiles):
+    assert tile_rules.beside(*[int(v) for v in q], tflop * 1e12) in tiles
 
 
 # Measured microseconds of a launch alone on a B200, by channel tile: (C_out, pixel tiles, K slices, epilogue, 1x1-like)
