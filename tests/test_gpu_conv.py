@@ -71,6 +71,24 @@ def test_simt_conv_matches_oracle(case, dtype):
     assert rel_err(dw, O.conv_wgrad(x, dy, w.shape, stride, pad)) < tol
 
 
+# images of three channels: ragged tiles of 32 columns x 4 to 16 rows, both strides, one to sixteen groups of 8 output channels
+# (32 and 2 tiles; 8 and 16: fewer and more items than warps), more tiles than blocks.  Bounds: one bf16 rounding of the output
+# (2^-9 at most, 1.7e-3 in the norm), fp32 sums of 27 or of some thousand products.
+@pytest.mark.parametrize("case", [(3, 9, 37, 3, 8, 3, 2, 1), (1, 5, 3, 3, 24, 3, 1, 1), (2, 33, 70, 3, 128, 3, 2, 1),
+                                  (2, 11, 32, 3, 8, 3, 1, 1), (1, 17, 33, 3, 40, 3, 1, 1), (1, 1, 1, 3, 16, 3, 2, 1),
+                                  (40, 40, 40, 3, 16, 3, 1, 1), (2, 6, 64, 3, 136, 3, 1, 1)])
+def test_image_convolutions_match_oracle(case):
+    import paper_2112_05387_b200 as lp
+    N, H, W, Cin, Cout, R, stride, pad = case
+    x, w, dy = make_case(*case, "bf16")
+    st, y, stats = run_conv(lp.LP_CONV_FWD, "bf16", lp.LP_CONV_IMPL_AUTO, *case, x, w, want_stats=True)
+    assert st == 0 and rel_err(y, O.conv_fwd(x, w, stride, pad)) < 2.5e-3
+    np.testing.assert_allclose(stats[:Cout], y.reshape(-1, Cout).sum(0), rtol=1e-5, atol=1e-3)
+    np.testing.assert_allclose(stats[Cout:], (y ** 2).reshape(-1, Cout).sum(0), rtol=1e-5, atol=1e-3)
+    st, dw, _ = run_conv(lp.LP_CONV_WGRAD, "bf16", lp.LP_CONV_IMPL_AUTO, *case, x, dy)
+    assert st == 0 and rel_err(dw, O.conv_wgrad(x, dy, w.shape, stride, pad)) < 5e-6
+
+
 # tensor-core shapes: several tiles, ragged tails, every swizzle width, strides 1 and 2, 1x1 and 3x3
 TC_CASES = [
     (2, 8, 8, 64, 64, 3, 1, 1),       # one tile, 128-byte rows
