@@ -3,6 +3,8 @@
 // All tensors are NHWC; every thread moves 16 bytes per access and keeps a fixed channel group,
 // so per-channel scale/shift live in registers (block size is a multiple of C / VEC).
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace lp {
@@ -130,7 +132,7 @@ __global__ void bn_stats_kernel(const T* __restrict__ x, long long total_vecs, i
 // ---------------------------------------------------------------------------------------
 // X2 / ADD select at compile time whether a second normalised input and a plain addend exist, so
 // that the common one-input form keeps few enough registers for four 256-thread blocks per SM.
-template <typename T, bool X2, bool ADD>
+template <typename T, bool X2, bool ADD, bool kLast>
 __global__ void __launch_bounds__(256, X2 ? 2 : (ADD ? 3 : 4))
 bn_apply_kernel(const T* __restrict__ x, BnArgs A, const T* __restrict__ x2, BnArgs B,
                 const T* __restrict__ addend, T* __restrict__ out, long long total_vecs, int C, int relu) {
@@ -168,9 +170,9 @@ bn_apply_kernel(const T* __restrict__ x, BnArgs A, const T* __restrict__ x2, BnA
     for (int u = 0; u < U; ++u) {
       const long long i = i0 + u * stride;
       if (i < total_vecs) {
-        rf[u] = ld_raw(x + i * V);
-        if (X2) rg[X2 ? u : 0] = ld_raw(x2 + i * V);
-        if (ADD) ra[ADD ? u : 0] = ld_raw(addend + i * V);
+        rf[u] = ld_raw_last<kLast>(x + i * V);
+        if (X2) rg[X2 ? u : 0] = ld_raw_last<kLast>(x2 + i * V);
+        if (ADD) ra[ADD ? u : 0] = ld_raw_last<kLast>(addend + i * V);
       }
     }
 #pragma unroll
@@ -203,10 +205,17 @@ bn_apply_kernel(const T* __restrict__ x, BnArgs A, const T* __restrict__ x2, BnA
 template <typename T>
 void launch_bn_apply(int grid, int threads, cudaStream_t st, const T* x, const BnArgs& A, const T* x2, const BnArgs& B,
                      const T* addend, T* out, long long total_vecs, int C, int relu) {
-  if (x2 && addend) launch_pdl(bn_apply_kernel<T, true, true>, dim3(grid), dim3(threads), 0, st, x, A, x2, B, addend, out, total_vecs, C, relu);
-  else if (x2) launch_pdl(bn_apply_kernel<T, true, false>, dim3(grid), dim3(threads), 0, st, x, A, x2, B, addend, out, total_vecs, C, relu);
-  else if (addend) launch_pdl(bn_apply_kernel<T, false, true>, dim3(grid), dim3(threads), 0, st, x, A, x2, B, addend, out, total_vecs, C, relu);
-  else launch_pdl(bn_apply_kernel<T, false, false>, dim3(grid), dim3(threads), 0, st, x, A, x2, B, addend, out, total_vecs, C, relu);
+  const auto launch = [&](auto with_x2, auto with_addend) {
+    constexpr bool X2 = decltype(with_x2)::value, ADD = decltype(with_addend)::value;
+    const auto kernel = total_vecs * 16 >= kLastBytes ? bn_apply_kernel<T, X2, ADD, true> : bn_apply_kernel<T, X2, ADD, false>;
+    launch_pdl(kernel, dim3(grid), dim3(threads), 0, st, x, A, x2, B, addend, out, total_vecs, C, relu);
+  };
+  const std::true_type yes;
+  const std::false_type no;
+  if (x2 && addend) launch(yes, yes);
+  else if (x2) launch(yes, no);
+  else if (addend) launch(no, yes);
+  else launch(no, no);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -394,7 +403,7 @@ bn_bwd_reduce_kernel(const T* __restrict__ dy, const T* __restrict__ x, int relu
   }
 }
 
-template <typename T>
+template <typename T, bool kLast>
 __global__ void __launch_bounds__(256, 2)
 bn_bwd_apply_kernel(const T* __restrict__ dy, const T* __restrict__ x, int relu_mask, BnArgs A,
                     const float* __restrict__ dgamma, const float* __restrict__ dbeta,
@@ -440,9 +449,9 @@ bn_bwd_apply_kernel(const T* __restrict__ dy, const T* __restrict__ x, int relu_
     for (int u = 0; u < U; ++u) {
       const long long i = i0 + u * stride;
       if (i < total_vecs) {
-        rd[u] = ld_raw(dy + i * V);
-        rx[u] = ld_raw(x + i * V);
-        if (addend) ra[u] = ld_raw(addend + i * V);
+        rd[u] = ld_raw_last<kLast>(dy + i * V);
+        rx[u] = ld_raw_last<kLast>(x + i * V);
+        if (addend) ra[u] = ld_raw_last<kLast>(addend + i * V);
       }
     }
 #pragma unroll
@@ -918,11 +927,13 @@ head_bwd_x_kernel(const float* __restrict__ dlogits, const float* __restrict__ W
 // ---------------------------------------------------------------------------------------
 // clearing, updates
 // ---------------------------------------------------------------------------------------
+template <bool kLast>
 __global__ void __launch_bounds__(256) zero_kernel(uint4* __restrict__ p, long long n) {
   pdl_wait();
   pdl_launch_dependents();
   for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256)
-    p[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (kLast) __stcs(p + i, make_uint4(0u, 0u, 0u, 0u));
+    else p[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 __global__ void sgd_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ mom, long long n,

@@ -2265,7 +2265,8 @@ static int run_op_t(lp_handle* h, Plan& P, const Op& op, const RunCtx& c) {
       }
       if (op.apply_fused) break;   // the input gradient that follows takes the rest
       const int grid_a = grid_for(vecs, threads * 4, cur_dev().sm_count, 2);
-      LP_CUDA_OK(launch_pdl(bn_bwd_apply_kernel<T>, dim3(grid_a), dim3(threads), 0, st, (const T*)resolve(op.in, c),
+      const auto kernel = vecs * 16 >= kLastBytes ? bn_bwd_apply_kernel<T, true> : bn_bwd_apply_kernel<T, false>;
+      LP_CUDA_OK(launch_pdl(kernel, dim3(grid_a), dim3(threads), 0, st, (const T*)resolve(op.in, c),
                             (const T*)resolve(op.in2, c), mask, A, (const float*)b.dgamma, (const float*)b.dbeta, addend,
                             (T*)resolve(op.out, c), vecs, b.C));
       h->launches++;
@@ -2435,7 +2436,8 @@ static int zero_range(lp_handle* h, const ZeroRange& r, cudaStream_t st) {
   if (!r.bytes) return LP_OK;
   const long long n = (long long)(r.bytes / 16);
   // (two blocks per SM: the gradients are cleared beside the first kernels of the forward passes)
-  LP_CUDA_OK(launch_pdl(zero_kernel, dim3(grid_for(n, 256 * 4, cur_dev().sm_count, 2)), dim3(256), 0, st, (uint4*)r.p, n));
+  const auto kernel = r.bytes >= (size_t)kLastBytes ? zero_kernel<true> : zero_kernel<false>;
+  LP_CUDA_OK(launch_pdl(kernel, dim3(grid_for(n, 256 * 4, cur_dev().sm_count, 2)), dim3(256), 0, st, (uint4*)r.p, n));
   h->launches++;
   return LP_OK;
 }
