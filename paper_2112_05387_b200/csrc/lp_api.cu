@@ -1232,7 +1232,11 @@ static int conv_forward(lp_handle* h, int dtype, int impl, const ConvDef& c, int
     // 7x7 / stride-2 stem: regroup the image, then a 4x4 stride-1 tensor-core convolution over 16 channels
     const int H2 = c.H / 2, W2 = c.W / 2;
     const long long pix = (long long)N * H2 * W2;
-    s2d_input_kernel<bf16><<<grid_for(pix, 256, cur_dev().sm_count, 8), 256, 0, st>>>((const bf16*)x, c.xs, N, c.H, c.W, c.cin);
+    if (c.cin == 3 && pix < (1LL << 30))
+      LP_CUDA_OK(launch_pdl(s2d_image3_kernel, dim3(grid_for(pix, 256, cur_dev().sm_count, 8)), dim3(256), 0, st, (const uint32_t*)x,
+                            (uint4*)c.xs, H2, W2, (int)pix));
+    else
+      s2d_input_kernel<bf16><<<grid_for(pix, 256, cur_dev().sm_count, 8), 256, 0, st>>>((const bf16*)x, c.xs, N, c.H, c.W, c.cin);
     if (h) h->launches++;
     LP_CUDA_OK(cudaGetLastError());
     TcGemmSpec s;
