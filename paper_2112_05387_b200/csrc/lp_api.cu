@@ -2680,7 +2680,15 @@ int lp_create(const lp_net_desc* desc, void* dev_workspace, size_t bytes, lp_han
   int rc = net.build(desc);
   if (rc != LP_OK) return rc;
   if (reinterpret_cast<uintptr_t>(dev_workspace) & 255) return LP_ERR_WORKSPACE;
-  const size_t need = lp_workspace_bytes(desc);
+  Arenas A, sized;
+  {
+    std::vector<Plan> m, a;
+    int* e = nullptr;
+    int32_t* z = nullptr;
+    ZeroRanges r;
+    plan_all(net, sized, &m, &a, &e, &z, &r);
+  }
+  const size_t need = sized.bytes() + 256;     // (as lp_workspace_bytes)
   if (bytes < need) return LP_ERR_WORKSPACE;
   rc = init_cur_dev();
   if (rc != LP_OK) return rc;
@@ -2690,10 +2698,6 @@ int lp_create(const lp_net_desc* desc, void* dev_workspace, size_t bytes, lp_han
   h->conv_impl = net.d.conv_impl;
   h->ws = (uint8_t*)dev_workspace;
   h->ws_bytes = bytes;
-  Arenas A, sized;
-  plan_all(h->net, sized, &h->modules, &h->auxs, &h->dev_err, &h->zero_labels, &h->zero);
-  h->modules.clear();
-  h->auxs.clear();
   A.place(h->ws, sized);
   plan_all(h->net, A, &h->modules, &h->auxs, &h->dev_err, &h->zero_labels, &h->zero);
   if (cudaMemset(dev_workspace, 0, need) != cudaSuccess) { delete h; return LP_ERR_CUDA; }
@@ -2726,7 +2730,10 @@ int lp_create(const lp_net_desc* desc, void* dev_workspace, size_t bytes, lp_han
       size_t n_wgrad = 0;
       for (const Op& op : P.bwd) n_wgrad += op.side() ? 1 : 0;
       if (!n_wgrad) continue;
-      const int lanes = 2;   // (ResNet-56 in three calls on 20 images 342 -> 333 us, three are no faster)
+      // Two where thin layers make the weight gradients many and short (ResNet-56 622 -> 602 us, in three calls on 20 images 342 ->
+      // 333; three are no faster).  Elsewhere a second one changes nothing but the number of branches of a recorded call, which
+      // its first launch pays for.
+      const int lanes = std::any_of(P.convs.begin(), P.convs.end(), [](const ConvDef& c) { return c.g > 1; }) ? 2 : 1;
       P.side.assign(lanes, nullptr);
       P.side_done.assign(lanes, nullptr);
       for (int l = 0; l < lanes; ++l)
