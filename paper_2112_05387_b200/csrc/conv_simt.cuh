@@ -408,13 +408,12 @@ image_wgrad_kernel(const bf16* __restrict__ x, const bf16* __restrict__ dy, floa
     __syncthreads();
     image_stage<kStride>(g, x, patch, n, oh0, ow0);
     __syncthreads();
-    if (item >= items) continue;
-    const int rows = min(g.TH, g.OH - oh0);
+    // (a lane past the last column adds nothing: not a product with a zero, since the patch may hold an infinity of the image)
+    const int rows = item < items && ow < g.OW ? min(g.TH, g.OH - oh0) : 0;
     const bf16* dp = dy + ((long long)(n * g.OH + oh0) * g.OW + ow) * g.Cout + co0;
 #pragma unroll 2
     for (int h = 0; h < rows; ++h) {
-      uint2 d = make_uint2(0u, 0u);
-      if (ow < g.OW) d = *reinterpret_cast<const uint2*>(dp + (long long)h * g.OW * g.Cout);
+      const uint2 d = *reinterpret_cast<const uint2*>(dp + (long long)h * g.OW * g.Cout);
       const uint64_t d2[2] = {pair_of(__uint_as_float(d.x << 16), __uint_as_float(d.x & 0xFFFF0000u)),
                               pair_of(__uint_as_float(d.y << 16), __uint_as_float(d.y & 0xFFFF0000u))};
 #pragma unroll

@@ -89,6 +89,27 @@ def test_image_convolutions_match_oracle(case):
     assert st == 0 and rel_err(dw, O.conv_wgrad(x, dy, w.shape, stride, pad)) < 5e-6
 
 
+@pytest.mark.parametrize("W,stride", [(37, 1), (32, 1), (6, 2), (70, 2)])
+def test_image_weight_gradient_with_an_infinite_pixel(W, stride):
+    """An infinity in the last column of an image reaches the filter positions that see that column and no others: columns of a
+    tile past the end of the output add nothing, not a product with zero."""
+    import paper_2112_05387_b200 as lp
+    case = (2, 6, W, 3, 16, 3, stride, 1)
+    x, w, dy = make_case(*case, "bf16")
+    x[1, 2, W - 1, 1] = 0.0
+    ref = O.conv_wgrad(x, dy, w.shape, stride, 1)
+    touched = np.zeros(ref.shape, bool)           # filter rows and columns through which the pixel enters a sum
+    for r in range(3):
+        for s in range(3):
+            oh, ow = 2 + 1 - r, W - 1 + 1 - s
+            touched[:, r, s, 1] = oh % stride == 0 and ow % stride == 0 and 0 <= oh // stride < dy.shape[1] and 0 <= ow // stride < dy.shape[2]
+    x[1, 2, W - 1, 1] = np.inf
+    st, dw, _ = run_conv(lp.LP_CONV_WGRAD, "bf16", lp.LP_CONV_IMPL_AUTO, *case, x, dy)
+    assert st == 0 and touched.any() and not touched.all()
+    assert not np.isfinite(dw[touched]).any()
+    assert rel_err(dw[~touched], ref[~touched]) < 5e-6
+
+
 # tensor-core shapes: several tiles, ragged tails, every swizzle width, strides 1 and 2, 1x1 and 3x3
 TC_CASES = [
     (2, 8, 8, 64, 64, 3, 1, 1),       # one tile, 128-byte rows
