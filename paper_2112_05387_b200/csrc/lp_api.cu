@@ -2448,6 +2448,8 @@ static int zero_range(lp_handle* h, const ZeroRange& r, cudaStream_t st) {
 // The gradients of all modules, on a stream of their own forked from `fork`: nothing needs them before the backward passes.
 static int zero_grads_beside(lp_handle* h) {
   LP_CUDA_OK(cudaStreamWaitEvent(h->zero_stream, h->fork, 0));
+  // (a module whose pass is not enqueued after this has no gradients any more: lp_step passes it by)
+  for (auto& P : h->modules) P.ps.grads_fresh = false;
   const int rc = zero_range(h, h->zero.module_grads, h->zero_stream);
   // (recorded whatever happened: the caller joins the stream through this event)
   LP_CUDA_OK(cudaEventRecord(h->grads_zeroed, h->zero_stream));

@@ -685,6 +685,40 @@ def test_update_with_momentum_and_weight_decay(dtype):
         np.testing.assert_allclose(lp.lp_get_params(h, k), want, rtol=2e-6, atol=1e-7)
 
 
+def test_gradients_of_a_call_that_fails_part_way_are_not_applied():
+    """lp_modules_fwd_bwd_all clears the gradients of all modules, then fails on the host before module 0 (whose stream is in
+    another recording): the gradients that module K-1 had from before are gone, and lp_step has nothing to apply."""
+    cfg = small_cfg("preact", N=4, H=8, W=8, stage_channels=(8, 16), stage_blocks=(1, 1), module_block_end=(1, 2))
+    run = GpuRun(cfg)
+    lp, h, torch, K = run.lp, run.h, run.torch, run.net.K
+    run.auxnet()
+    run.fwd_bwd_all()
+    recording, stream = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    lp.lp_graph_begin(h, recording.cuda_stream)
+    lp.lp_step(h, 0.0, 0.0, 0.0, 0.0, None, recording.cuda_stream)     # (the modules' streams are in the recording now)
+    lp.lp_module_fwd_bwd(h, K - 1, run.d_x[K - 1], run.d_labels, None, cfg["rho"], run.d_loss[K - 1], run.d_dx[K - 1],
+                         stream.cuda_stream)
+    with pytest.raises(lp.LpError) as e:
+        lp.lp_modules_fwd_bwd_all(h, run.d_x, run.d_labels, None, cfg["rho"], run.d_loss, run.d_dx, stream.cuda_stream)
+    assert e.value.status == -8
+    with pytest.raises(lp.LpError) as e:
+        lp.lp_step(h, 0.0, 0.0, 0.1, 0.0, None, stream.cuda_stream)
+    assert e.value.status == -6
+    for _ in range(2):                # the recording may have become invalid; the runtime's last error belongs to this test
+        try:
+            lp.lp_graph_end(h, recording.cuda_stream)
+        except lp.LpError:
+            pass
+        try:
+            lp.lp_set_params(h, 0, run.mods[0])
+        except lp.LpError:
+            pass
+    run.fwd_bwd_all()
+    lp.lp_step(h, 0.0, 0.0, 0.0, 0.0, None)
+    assert lp.lp_last_device_status(h) == 0
+
+
 def test_speedup_accounting_on_the_tiny_workload():
     """The speed-up accounting (Section 4.3) runs end to end: K = 1 has no auxiliary phases and the
     model ratio 1; K = 2 has all five phases and a model ratio between 1 and K."""
