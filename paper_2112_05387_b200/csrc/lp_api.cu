@@ -2389,9 +2389,11 @@ static double op_bytes(const lp_handle* h, const Plan& P, const Op& op) {
   }
 }
 
+// Per-operation timing: what the records of a phase add up to is the time of its work, so a module's weight gradients stay in
+// its chain, and the modules' updates and the AuxNets' distillation follow one another.
+static bool timed(const lp_handle* h) { return h->tl.enabled || h->prof.enabled; }
 static int run_ops(lp_handle* h, Plan& P, const std::vector<Op>& ops, const RunCtx& c) {
-  // (per-operation timing wants one stream: the time line and the convolution profile keep everything in order)
-  const size_t lanes = h->tl.enabled || h->prof.enabled ? 0 : P.side.size();
+  const size_t lanes = timed(h) ? 0 : P.side.size();
   size_t nside = 0;
   bool folds = false, fold_last = false;   // there are gradients to fold back; so is that of the chain's last operation
   int rc = LP_OK;
@@ -2952,12 +2954,15 @@ static int update_kappa(lp_handle* h, int k, float kappa_step, void* lambda_inou
 static int update_module(lp_handle* h, int k, float lr, float momentum, float weight_decay, float kappa_step,
                          void* lambda_inout, cudaStream_t st) {
   Plan& P = h->modules[k];
-  // parameters read and written, gradients read, both bf16 copies of the packed weights written
-  TimelineScope ts(h, st, k, LP_OP_UPDATE, LP_PHASE_UPDATE, 12.0 * (double)P.ps.n + 4.0 * (double)P.ps.pack_total);
+  const bool kappa = lambda_inout && k + 1 < h->net.K;
+  // parameters (and momentum) read and written, gradients read, both bf16 copies of the packed weights written; multipliers
+  // read and written, residual read
+  TimelineScope ts(h, st, k, LP_OP_UPDATE, LP_PHASE_UPDATE, (momentum != 0.f ? 20.0 : 12.0) * (double)P.ps.n +
+                   4.0 * (double)P.ps.pack_total + (kappa ? 3.0 * (double)boundary_bytes(h, k + 1) : 0.0));
   int rc = sgd_update(h, P, lr, momentum, weight_decay, st);
   if (rc != LP_OK) return rc;
   P.ps.grads_fresh = false;
-  return lambda_inout && k + 1 < h->net.K ? update_kappa(h, k, kappa_step, lambda_inout, st) : LP_OK;
+  return kappa ? update_kappa(h, k, kappa_step, lambda_inout, st) : LP_OK;
 }
 
 int lp_step(lp_handle* h, float lr, float momentum, float weight_decay, float kappa_step, void* const* lambdas_inout,
@@ -2972,7 +2977,7 @@ int lp_step(lp_handle* h, float lr, float momentum, float weight_decay, float ka
       if (lambdas_inout[k] && !aligned16(lambdas_inout[k])) return LP_ERR_ALIGN;
   return run_as_graph(h, CALL_STEP, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   // the modules' updates side by side (one after another where a buffer of multipliers serves two modules)
-  bool apart = true;
+  bool apart = !timed(h);
   for (int k = 0; lambdas_inout && k + 1 < K; ++k)
     for (int j = 0; j < k; ++j)
       apart = apart && !overlap(lambdas_inout[k], boundary_bytes(h, k + 1), lambdas_inout[j], boundary_bytes(h, j + 1));
@@ -3064,14 +3069,15 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
       const void* xk = k == 0 ? images : x_out[k - 1];
       const void* tgt = last ? (const void*)labels : (const void*)x_out[k];
       void* lam = (lambdas_inout && !last) ? lambdas_inout[k] : nullptr;
+      const bool beside = lam && !timed(h);
       rc = module_fwd_bwd(h, k, xk, tgt, lam, rho, loss_out + 2 * k, dx ? dx[k] : nullptr, sk,
-                          h->grads_zeroed, last ? nullptr : h->aux_done[k], lam ? h->loss_done[k] : nullptr);
+                          h->grads_zeroed, last ? nullptr : h->aux_done[k], beside ? h->loss_done[k] : nullptr);
       if (rc != LP_OK) return rc;
-      if (lam) {   // beside the backward pass, on the stream that the AuxNet chain has left
+      if (beside) {   // beside the backward pass, on the stream that the AuxNet chain has left
         LP_CUDA_OK(cudaStreamWaitEvent(h->aux_stream, h->loss_done[k], 0));
         if ((rc = update_kappa(h, k, kappa_step, lam, h->aux_stream)) != LP_OK) return rc;
       }
-      rc = update_module(h, k, lr, momentum, weight_decay, kappa_step, nullptr, sk);
+      rc = update_module(h, k, lr, momentum, weight_decay, kappa_step, beside ? nullptr : lam, sk);
       if (rc != LP_OK) return rc;
     }
     return LP_OK;
@@ -3108,7 +3114,7 @@ int lp_auxnet_distill(lp_handle* h, const void* images, void* const* x, const vo
   ConcurrentScope concurrent(h);
   // One AuxNet (or stack) does not depend on another, unless a corrected variable is written over what another one reads
   // (x_new = x: then one after another, and AuxNet_k sees the corrected x_k).
-  bool apart = true;
+  bool apart = !timed(h);
   for (int k = 1; x_new && k < K; ++k) {
     const size_t nk = boundary_bytes(h, k);
     apart = apart && !overlap(x_new[k - 1], nk, images, boundary_bytes(h, 0));

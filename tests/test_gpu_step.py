@@ -719,6 +719,46 @@ def test_gradients_of_a_call_that_fails_part_way_are_not_applied():
     assert lp.lp_last_device_status(h) == 0
 
 
+@pytest.mark.parametrize("one_call", [False, True])
+def test_timeline_of_updates_and_distillation(one_call):
+    """Records of the distillation, and of the update where it is a call of its own, do not overlap and can be added up; every
+    module's update has one, whose bytes count the multipliers."""
+    cfg = small_cfg("preact", N=64, H=16, W=16, dtype="bf16", stage_channels=(32, 64), stage_blocks=(2, 2),
+                    module_block_end=(1, 2, 3, 4), stem_channels=32, classes=10)
+    run = GpuRun(cfg)
+    lp, h, K = run.lp, run.h, run.net.K
+    lam = [run.torch.zeros_like(t) for t in run.d_x[1:]]
+    dloss = run.torch.zeros(K - 1, device="cuda:0")
+
+    def step(multipliers):
+        if one_call:
+            lp.lp_layer_parallel_step(h, run.d_images, run.d_x[1:], run.d_labels, multipliers, 0.1, run.d_loss, run.d_dx, 1e-3,
+                                      0.0, 0.0, 0.1)
+        else:
+            lp.lp_auxnet_forward(h, run.d_images, run.d_x[1:])
+            lp.lp_modules_fwd_bwd_all(h, run.d_x, run.d_labels, multipliers, 0.1, run.d_loss, run.d_dx)
+            lp.lp_step(h, 1e-3, 0.0, 0.0, 0.1, multipliers)
+        lp.lp_auxnet_distill(h, run.d_images, run.d_x[1:], run.d_dx, 0.1, 1e-3, None, dloss)
+
+    updates = []
+    for multipliers in (None, lam):
+        step(multipliers)                        # (kernels are loaded at their first launch)
+        run.torch.cuda.synchronize()
+        lp.lp_timeline(h, True, read=False)
+        step(multipliers)
+        recs = lp.lp_timeline(h, False)
+        for phase in ["distill"] if one_call else ["distill", "update"]:
+            rs = sorted((r for r in recs if r["phase"] == phase), key=lambda r: r["start_ms"])
+            assert len(rs) >= K - 1
+            for a, b in zip(rs, rs[1:]):         # (event times are rounded to about half a microsecond)
+                assert b["start_ms"] >= a["end_ms"] - 1e-3, (a, b)
+        updates.append({r["plan"]: r["bytes"] for r in recs if r["phase"] == "update"})
+        assert sorted(updates[-1]) == list(range(K))
+    for k in range(K):
+        want = 3 * 2 * int(np.prod(run.net.boundary[k + 1])) if k + 1 < K else 0
+        assert updates[1][k] - updates[0][k] == want
+
+
 def test_speedup_accounting_on_the_tiny_workload():
     """The speed-up accounting (Section 4.3) runs end to end: K = 1 has no auxiliary phases and the
     model ratio 1; K = 2 has all five phases and a model ratio between 1 and K."""
