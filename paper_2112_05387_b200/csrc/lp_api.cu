@@ -22,6 +22,7 @@
 #include "kernels_elem.cuh"
 #include "conv_thin.cuh"
 #include "net.h"
+#include "order_rules.h"
 #include "wgrad_tc.cuh"
 
 namespace lp {
@@ -2525,10 +2526,6 @@ static int sgd_update_inner(lp_handle* h, Plan& P, float lr, float momentum, flo
   return LP_OK;
 }
 
-static bool overlap(const void* a, size_t na, const void* b, size_t nb) {
-  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
-  return a && b && x < y + nb && y < x + na;
-}
 static size_t boundary_bytes(const lp_handle* h, int k) {   // of x_k
   const Shape4& s = h->net.boundary[k];
   return (size_t)s.n * s.h * s.w * s.c * esize(h->dtype);
@@ -2978,9 +2975,11 @@ int lp_step(lp_handle* h, float lr, float momentum, float weight_decay, float ka
   return run_as_graph(h, CALL_STEP, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   // the modules' updates side by side (one after another where a buffer of multipliers serves two modules)
   bool apart = !timed(h);
-  for (int k = 0; lambdas_inout && k + 1 < K; ++k)
-    for (int j = 0; j < k; ++j)
-      apart = apart && !overlap(lambdas_inout[k], boundary_bytes(h, k + 1), lambdas_inout[j], boundary_bytes(h, j + 1));
+  if (lambdas_inout) {
+    Span lambda[LP_MAX_MODULES];
+    for (int k = 0; k + 1 < K; ++k) lambda[k] = Span{lambdas_inout[k], boundary_bytes(h, k + 1)};
+    apart = apart && multipliers_apart(lambda, K - 1);
+  }
   LP_CUDA_OK(cudaEventRecord(h->fork, st));
   int first_err = LP_OK, forked = 0;
   for (int k = 0; k < K && first_err == LP_OK; ++k) {
@@ -3112,17 +3111,17 @@ int lp_auxnet_distill(lp_handle* h, const void* images, void* const* x, const vo
   if (rc0 != LP_OK) return rc0;
   const bool rec = h->net.d.aux_recursive != 0;
   ConcurrentScope concurrent(h);
-  // One AuxNet (or stack) does not depend on another, unless a corrected variable is written over what another one reads
-  // (x_new = x: then one after another, and AuxNet_k sees the corrected x_k).
+  // the AuxNets (or stacks) side by side, or one after another where one is given what another one corrects
   bool apart = !timed(h);
-  for (int k = 1; x_new && k < K; ++k) {
-    const size_t nk = boundary_bytes(h, k);
-    apart = apart && !overlap(x_new[k - 1], nk, images, boundary_bytes(h, 0));
-    for (int j = 1; j < K; ++j) {
-      const size_t nj = boundary_bytes(h, j);
-      apart = apart && !overlap(x_new[k - 1], nk, x[j - 1], nj);
-      if (j != k) apart = apart && !overlap(x_new[k - 1], nk, dx[j], nj) && !overlap(x_new[k - 1], nk, x_new[j - 1], nj);
+  if (x_new) {
+    Span xs[LP_MAX_MODULES], dxs[LP_MAX_MODULES], corrected[LP_MAX_MODULES];
+    for (int k = 1; k < K; ++k) {
+      const size_t n = boundary_bytes(h, k);
+      xs[k - 1] = Span{x[k - 1], n};
+      dxs[k - 1] = Span{dx[k], n};
+      corrected[k - 1] = Span{x_new[k - 1], n};
     }
+    apart = apart && corrections_apart(Span{images, boundary_bytes(h, 0)}, xs, dxs, corrected, K - 1);
   }
   const auto distill = [&](int k, cudaStream_t sk) -> int {
     RunCtx c;

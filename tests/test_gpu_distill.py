@@ -93,6 +93,45 @@ def test_distill_small_bf16(split):
     run_case(cfg, 2e-2)
 
 
+@pytest.mark.parametrize("recursive", [False, True])
+def test_corrected_variables_over_the_given_ones(recursive):
+    """x_new = x, four modules: AuxNet_k's weight gradient is taken with the x_k that AuxNet_{k-1}'s distillation has corrected
+    (its kept activations are those of the forward pass).  Against calls with buffers of their own: the corrections and the first
+    AuxNet come from one call; AuxNet_k, whose input is x_k, from one that is given the corrected x_k but the x_{k+1} of before.
+    fp32: sums of up to 1024 products in another order, 1e-5 with margin.  A recursive stack reads the images only."""
+    cfg = small_cfg("preact", N=4, H=8, W=8, stage_channels=(8, 16), stage_blocks=(2, 2), module_block_end=(1, 2, 3, 4))
+    run = GpuRun(cfg, aux_recursive=recursive)
+    run.auxnet()
+    run.fwd_bwd_all()
+    lp, torch, K, lr = run.lp, run.torch, run.net.K, 0.3
+    auxs = ([lp.LP_REAUX(k, j) for k in range(1, K) for j in range(k)] if recursive else [lp.LP_AUX(k) for k in range(K - 1)])
+    before = [t.clone() for t in run.d_x[1:]]
+    loss = torch.zeros(K - 1, device="cuda:0")
+
+    def distill(x, x_new):
+        lp.lp_auxnet_distill(run.h, run.d_images, x, run.d_dx, lr, 0.0, x_new, loss)     # (no update: the calls can be repeated)
+        assert lp.lp_last_device_status(run.h) == 0
+        return [lp.lp_get_grads(run.h, w) for w in auxs], loss.cpu().numpy().copy()
+
+    new = [torch.zeros_like(t) for t in before]
+    want, want_loss = distill([t.clone() for t in before], new)
+    stale = want[-1]
+    if not recursive:
+        for k in range(1, K - 1):
+            x = [t.clone() for t in before]
+            x[k - 1] = new[k - 1]
+            want[k] = distill(x, [torch.zeros_like(t) for t in before])[0][k]
+        assert rel_err(stale, want[-1]) > 1e-3        # (the order is seen)
+    for _ in range(3):                                # launched directly, then as a graph
+        x = [t.clone() for t in before]
+        got, got_loss = distill(x, x)
+        for a, b in zip(x, new):
+            assert torch.equal(a, b)
+        np.testing.assert_allclose(got_loss, want_loss, rtol=1e-5)
+        for a, b in zip(got, want):
+            assert rel_err(a, b) < 1e-5
+
+
 def test_distill_needs_module_passes_first():
     cfg = get_config("tiny")
     run = GpuRun(cfg)

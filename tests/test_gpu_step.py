@@ -759,6 +759,28 @@ def test_timeline_of_updates_and_distillation(one_call):
         assert updates[1][k] - updates[0][k] == want
 
 
+def test_one_multiplier_buffer_for_two_modules():
+    """lp_step with one buffer given to two modules whose boundaries have one shape: both residuals arrive.  fp32: two roundings
+    of a sum, 2^-24 of it each."""
+    cfg = small_cfg("preact", N=16, H=16, W=16, stage_channels=(16,), stage_blocks=(4,), stage_stride=(1,), stem_channels=16,
+                    module_block_end=(1, 2, 4))
+    run = GpuRun(cfg)
+    lp, torch, K = run.lp, run.torch, run.net.K
+    run.auxnet()
+    assert tuple(run.net.boundary[1]) == tuple(run.net.boundary[2])
+    for _ in range(4):                                   # launched directly, then as a graph
+        run.fwd_bwd_all()
+        r = [torch.zeros_like(t) for t in run.d_x[1:]]
+        for k in range(K - 1):
+            lp.lp_get_residual(run.h, k, r[k], None, None)
+        lam = torch.randn_like(r[0])
+        want = (lam.double() + 0.5 * r[0].double()) + 0.5 * r[1].double()
+        largest = float((lam.abs() + 0.5 * r[0].abs() + 0.5 * r[1].abs()).max())
+        lp.lp_step(run.h, 0.0, 0.0, 0.0, 0.5, [lam, lam])
+        assert lp.lp_last_device_status(run.h) == 0
+        assert float((lam.double() - want).abs().max()) < 2.0 ** -23 * largest
+
+
 def test_speedup_accounting_on_the_tiny_workload():
     """The speed-up accounting (Section 4.3) runs end to end: K = 1 has no auxiliary phases and the
     model ratio 1; K = 2 has all five phases and a model ratio between 1 and K."""

@@ -93,6 +93,68 @@ def test_channel_tiles_cover_the_channels(tile_rules):
 
 
 @pytest.fixture(scope="module")
+def order_rules(tmp_path_factory):
+    return build_host(tmp_path_factory.mktemp("order"), "order", """
+#include "order_rules.h"
+#include <vector>
+static std::vector<lp::Span> spans(const long long* at, int n) {   // pairs (address, bytes); address 0: not given
+  std::vector<lp::Span> v;
+  for (int i = 0; i < n; ++i) v.push_back(lp::Span{reinterpret_cast<const void*>(at[2 * i]), (size_t)at[2 * i + 1]});
+  return v;
+}
+extern "C" int multipliers(const long long* lambda, int n) { return lp::multipliers_apart(spans(lambda, n).data(), n); }
+extern "C" int corrections(const long long* images, const long long* x, const long long* dx, const long long* x_new, int n) {
+  return lp::corrections_apart(spans(images, 1)[0], spans(x, n).data(), spans(dx, n).data(), spans(x_new, n).data(), n);
+}
+""")
+
+
+def _spans(pairs):
+    flat = [v for p in pairs for v in p]
+    return (ctypes.c_longlong * max(1, len(flat)))(*flat)
+
+
+@pytest.mark.parametrize("spans,apart", [
+    ([(64, 16), (80, 16), (96, 16)], True),       # neighbours
+    ([(64, 16), (96, 16), (64, 16)], False),      # one buffer for two modules
+    ([(64, 16), (79, 16)], False), ([(79, 16), (64, 16)], False), ([(64, 32), (70, 2)], False),
+    ([(0, 16), (0, 16), (64, 16)], True), ([], True), ([(64, 16)], True),
+])
+def test_multipliers_apart(order_rules, spans, apart):
+    assert bool(order_rules.multipliers(_spans(spans), len(spans))) == apart
+
+
+def test_corrections_apart(order_rules):
+    """Buffers drawn over one another, partially too: two AuxNets are apart if neither writes what the other one touches and no
+    correction goes over the images or an x_k (one AuxNet's output is another one's input); sets of bytes, not intervals."""
+    import random
+    rng = random.Random(7)
+    seen = set()
+
+    def given():
+        return rng.randint(1, 400), rng.choice([4, 8, 24])
+
+    def meet(a, b):
+        return bool(a[0] and b[0] and set(range(a[0], a[0] + a[1])) & set(range(b[0], b[0] + b[1])))
+    for _ in range(4000):
+        n = rng.randint(1, 4)
+        images, x, dx = given(), [given() for _ in range(n)], [given() for _ in range(n)]
+        new = [given() if rng.random() < 0.4 else (0, 8) for _ in range(n)]
+        want = not any(meet(new[i], other) for i in range(n)
+                       for other in [images] + x + [dx[j] for j in range(n) if j != i] + [new[j] for j in range(n) if j != i])
+        seen.add((want, n))
+        assert bool(order_rules.corrections(_spans([images]), _spans(x), _spans(dx), _spans(new), n)) == want
+    assert len(seen) == 8
+    for k in range(3):
+        x, dx = [(100 * (i + 1), 96) for i in range(3)], [(2000 + 100 * i, 96) for i in range(3)]
+        new = [(1000 + 100 * i, 96) for i in range(3)]
+        new[k] = x[k]                             # in place
+        assert not order_rules.corrections(_spans([(900, 50)]), _spans(x), _spans(dx), _spans(new), 3)
+        new[k] = dx[k]                            # over its own dx: its own business
+        assert order_rules.corrections(_spans([(900, 50)]), _spans(x), _spans(dx), _spans(new), 3)
+
+
+@pytest.fixture(scope="module")
 def f32_rules(tmp_path_factory):
     return build_host(tmp_path_factory.mktemp("f32"), "f32", """
 #include "conv_f32_rules.h"
