@@ -2895,7 +2895,7 @@ int lp_module_fwd_bwd(lp_handle* h, int k, const void* x_k, const void* x_next_o
 // to the other streams, see launch_conv_tc).
 struct ConcurrentScope {
   lp_handle* h;
-  explicit ConcurrentScope(lp_handle* h_) : h(h_) { h->concurrent = true; }
+  explicit ConcurrentScope(lp_handle* h_, bool beside = true) : h(h_) { h->concurrent = beside; }
   ~ConcurrentScope() { h->concurrent = false; }
 };
 
@@ -3110,7 +3110,6 @@ int lp_auxnet_distill(lp_handle* h, const void* images, void* const* x, const vo
   const int rc0 = zero_range(h, h->zero.aux_grads, st);
   if (rc0 != LP_OK) return rc0;
   const bool rec = h->net.d.aux_recursive != 0;
-  ConcurrentScope concurrent(h);
   // the AuxNets (or stacks) side by side, or one after another where one is given what another one corrects
   bool apart = !timed(h);
   if (x_new) {
@@ -3157,6 +3156,7 @@ int lp_auxnet_distill(lp_handle* h, const void* images, void* const* x, const vo
     }
     return LP_OK;
   };
+  const ConcurrentScope concurrent(h, apart && K > 2);     // (one after another, each has the machine to itself)
   LP_CUDA_OK(cudaEventRecord(h->fork, st));
   int first_err = LP_OK, forked = 1;
   for (int k = 1; k < K && first_err == LP_OK; ++k) {
