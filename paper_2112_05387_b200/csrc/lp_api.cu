@@ -2526,6 +2526,20 @@ static int sgd_update_inner(lp_handle* h, Plan& P, float lr, float momentum, flo
   return LP_OK;
 }
 
+// Whether work can be forked from `st` onto another stream: not while that one is in a recording that `st` is not in.  (A
+// handle's streams stay in a caller's recording until it ends; meanwhile the caller may make other calls, recorded or not.)
+static bool can_fork(cudaStream_t st, cudaStream_t onto) {
+  cudaStreamCaptureStatus a = cudaStreamCaptureStatusNone, b = cudaStreamCaptureStatusNone;
+  unsigned long long ia = 0, ib = 0;
+  if (cudaStreamGetCaptureInfo(onto, &b, &ib) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (b == cudaStreamCaptureStatusNone) return true;
+  if (cudaStreamGetCaptureInfo(st, &a, &ia) != cudaSuccess) { cudaGetLastError(); return false; }
+  return a != cudaStreamCaptureStatusNone && ia == ib;
+}
+static bool can_fork(cudaStream_t st, const std::vector<cudaStream_t>& onto) {
+  return std::all_of(onto.begin(), onto.end(), [&](cudaStream_t s) { return can_fork(st, s); });
+}
+
 static size_t boundary_bytes(const lp_handle* h, int k) {   // of x_k
   const Shape4& s = h->net.boundary[k];
   return (size_t)s.n * s.h * s.w * s.c * esize(h->dtype);
@@ -2974,7 +2988,7 @@ int lp_step(lp_handle* h, float lr, float momentum, float weight_decay, float ka
       if (lambdas_inout[k] && !aligned16(lambdas_inout[k])) return LP_ERR_ALIGN;
   return run_as_graph(h, CALL_STEP, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   // the modules' updates side by side (one after another where a buffer of multipliers serves two modules)
-  bool apart = !timed(h);
+  bool apart = !timed(h) && can_fork(st, h->streams);
   if (lambdas_inout) {
     Span lambda[LP_MAX_MODULES];
     for (int k = 0; k + 1 < K; ++k) lambda[k] = Span{lambdas_inout[k], boundary_bytes(h, k + 1)};
@@ -3111,7 +3125,7 @@ int lp_auxnet_distill(lp_handle* h, const void* images, void* const* x, const vo
   if (rc0 != LP_OK) return rc0;
   const bool rec = h->net.d.aux_recursive != 0;
   // the AuxNets (or stacks) side by side, or one after another where one is given what another one corrects
-  bool apart = !timed(h);
+  bool apart = !timed(h) && can_fork(st, h->streams);
   if (x_new) {
     Span xs[LP_MAX_MODULES], dxs[LP_MAX_MODULES], corrected[LP_MAX_MODULES];
     for (int k = 1; k < K; ++k) {

@@ -759,6 +759,50 @@ def test_timeline_of_updates_and_distillation(one_call):
         assert updates[1][k] - updates[0][k] == want
 
 
+def test_update_and_distillation_in_two_recordings_at_once():
+    """A caller may have two recordings open, lp_step in one, lp_auxnet_distill in the other, and make a call beside them; the
+    replays give what the calls themselves give."""
+    cfg = small_cfg("preact", N=4, H=8, W=8, stage_channels=(8, 16), stage_blocks=(2, 2), module_block_end=(1, 3, 4))
+    runs = [GpuRun(cfg), GpuRun(cfg)]
+    torch = runs[0].torch
+    s1, s2, s3 = (torch.cuda.Stream() for _ in range(3))
+    for i, run in enumerate(runs):
+        lp, h, K = run.lp, run.h, run.net.K
+        loss = torch.zeros(K - 1, device="cuda:0")
+        run.auxnet()
+        run.fwd_bwd_all()
+        torch.cuda.synchronize()
+
+        def step(s):
+            lp.lp_step(h, 0.01, 0.0, 0.0, 0.5, run.d_kappa, s.cuda_stream)
+
+        def distill(s):
+            lp.lp_auxnet_distill(h, run.d_images, run.d_x[1:], run.d_dx, 0.1, 0.01, None, loss, s.cuda_stream)
+        if i == 0:
+            lp.lp_graph_begin(h, s1.cuda_stream)
+            step(s1)
+            lp.lp_graph_begin(h, s2.cuda_stream)
+            distill(s2)
+            distill(s3)                               # launched, while the handle's streams are in a recording
+            g2 = lp.lp_graph_end(h, s2.cuda_stream)
+            g1 = lp.lp_graph_end(h, s1.cuda_stream)
+            s3.synchronize()
+            lp.lp_graph_launch(h, g1, s1.cuda_stream)
+            s1.synchronize()
+            lp.lp_graph_launch(h, g2, s2.cuda_stream)
+        else:
+            distill(s3)
+            s3.synchronize()
+            step(s1)
+            s1.synchronize()
+            distill(s2)
+        assert lp.lp_last_device_status(h) == 0
+        run.seen = ([to_host(loss)] + [to_host(t) for t in run.d_kappa] + [lp.lp_get_params(h, k) for k in range(K)] +
+                    [lp.lp_get_params(h, lp.LP_AUX(k)) for k in range(K - 1)])
+    for a, b in zip(runs[0].seen, runs[1].seen):
+        assert rel_err(a, b) < 1e-5                   # (fp32 sums in another order)
+
+
 def test_one_multiplier_buffer_for_two_modules():
     """lp_step with one buffer given to two modules whose boundaries have one shape: both residuals arrive.  fp32: two roundings
     of a sum, 2^-24 of it each."""
