@@ -90,8 +90,8 @@ enum { LP_CONV_TWO_CTA = 1024 };
  * traffic costs the convolution more than the separate kernel takes. */
 enum { LP_CONV_BN_REDUCE_IN_EPILOGUE = 2048 };
 /* May be OR-ed into conv_impl: the weight gradients of a module stay in its stream, in the order of the
- * backward pass.  By default each module has a second stream for them (they feed nothing but the update), so
- * that the chain of input gradients and batch-norm backward passes does not wait for them. */
+ * backward pass.  By default each module has a stream of its own for them, or two where it has thin layers (they feed
+ * nothing but the update), so that the chain of input gradients and batch-norm backward passes does not wait for them. */
 enum { LP_CONV_WGRAD_IN_CHAIN = 4096 };
 enum { LP_CONV_FWD = 0, LP_CONV_DGRAD = 1, LP_CONV_WGRAD = 2 };
 
@@ -157,6 +157,12 @@ int lp_boundary_shape_desc(const lp_net_desc* desc, int k, int shape_nhwc[4]);
 /* Create a handle over the caller's device workspace.  The call zero-fills the workspace with a
  * synchronous cudaMemset (it returns after the fill; work of the caller still running on other
  * streams must not touch the workspace meanwhile); parameters start at zero until lp_set_params.
+ * Calls on one handle are made by one thread at a time.  The handle has streams and events of its own: lp_modules_fwd_bwd_all,
+ * lp_step, lp_layer_parallel_step, lp_auxnet_distill and lp_serial_fwd_bwd fork work onto them and join it before what follows
+ * the call on its `stream`; lp_module_fwd_bwd uses those of its module only.  Calls on different streams are therefore ordered
+ * where they share one.  During a caller's recording of one such call the handle's streams belong to the recording: until it
+ * ends, lp_step and lp_auxnet_distill stay on the stream they are given (recorded elsewhere or not), the other three return
+ * LP_ERR_CUDA outside that recording.
  * The handle owns host memory, streams, events and -- from the third call of a kind on -- one executable graph for each
  * of lp_auxnet_forward, lp_modules_fwd_bwd_all, lp_step, lp_layer_parallel_step, lp_auxnet_distill, lp_forward_serial and
  * lp_serial_fwd_bwd, as which the call is then launched (recorded anew each time with its own arguments).  The driver

@@ -76,6 +76,5 @@ inline void pick_n_tile_by_cost(const ConvTileQuery& q, double worth, int& n_til
     if (t < best * 0.98) { best = t; n_tile = tile; n_tiles = (q.Cout + tile - 1) / tile; }
   }
 }
-inline void pick_n_tile_alone(const ConvTileQuery& q, int& n_tile, int& n_tiles) { pick_n_tile_by_cost(q, 0.0, n_tile, n_tiles); }
 
 }  // namespace lp

@@ -666,7 +666,7 @@ static int launch_wgrad_halo(WgEncodeFn enc, int sm_count, bool* attr_done, cons
   // pixel box (K block): 8 x BH x BNI = LP_WGRAD_HALO_KBLOCK pixels.  Blocks of 64 make a stage 40 KB
   // instead of 80 KB for a 160-channel tile (five stages in flight instead of two); measured, that is
   // no faster (0.079 against 0.078 ms at 160 channels), so the copy latency is not what limits it.
-  // (A launch that shares its SM has 100 KB: three stages of 64 pixels.)
+  // (A launch that shares its SM has 100 KB: four stages of 64 pixels, 12 + 8 KB each.)
   const int per_col = (shared_sm ? 64 : LP_WGRAD_HALO_KBLOCK) / 8;
   if (H >= per_col) {                       // rows spread evenly over the tiles of a column (14: 14, 28: 2 x 14, 56: 4 x 14)
     const int th = (H + per_col - 1) / per_col;

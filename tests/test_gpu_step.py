@@ -196,9 +196,9 @@ def test_bn_backward_sums_in_the_conv_epilogue_equal_the_separate_kernel(kind):
 
 
 def test_weight_gradients_on_their_own_stream_equal_those_in_the_chain():
-    """A module's weight gradients run on a second stream by default and inside the module's stream with
+    """A module's weight gradients run on streams of their own by default and inside the module's stream with
     LP_CONV_WGRAD_IN_CHAIN: the same kernels on the same operands, so losses are identical and gradients agree
-    to the order of the fp32 reductions; run twice to show that nothing races between the two streams."""
+    to the order of the fp32 reductions; run twice to show that nothing races between the streams."""
     import paper_2112_05387_b200 as lp
     cfg = small_cfg("postbn", N=8, H=16, W=16, dtype="bf16", stage_channels=(16, 32), stage_blocks=(2, 2),
                     module_block_end=(1, 3, 4), stem_channels=16, classes=10)

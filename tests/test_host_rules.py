@@ -24,7 +24,7 @@ def tile_rules(tmp_path_factory):
 #include "conv_tiles.h"
 extern "C" int alone(int cout, int m_tiles, int k_mmas, int epilogue, int wide, int* n_tiles) {
   int tile = 0;
-  lp::pick_n_tile_alone(lp::ConvTileQuery{cout, m_tiles, 148, k_mmas, epilogue, wide != 0}, tile, *n_tiles);
+  lp::pick_n_tile_by_cost(lp::ConvTileQuery{cout, m_tiles, 148, k_mmas, epilogue, wide != 0}, 0.0, tile, *n_tiles);
   return tile;
 }
 extern "C" int beside(int cout, int m_tiles, int k_mmas, int epilogue, int wide, double step_flops) {
@@ -51,7 +51,6 @@ PLAIN, STATS, SHORTCUT = 0, 1, 2
     ((256, 12, 144, STATS, False), 0.18, (64, 128)),
     ((256, 896, 4, STATS, True), 0.18, (256,)),           # a launch that fills the machine as it is
     ((512, 4, 288, STATS, False), 30.0, (256,)),          # a step bound by SM time
-    ((64, 4, 36, STATS, False), 0.01, (64,)),
 ])
 def test_channel_tile_beside_other_modules(tile_rules, q, tflop, tiles):
     assert tile_rules.beside(*[int(v) for v in q], tflop * 1e12) in tiles
