@@ -64,9 +64,11 @@ __device__ __forceinline__ void stv(bf16* p, const float (&f)[8]) {
   *reinterpret_cast<uint4*>(p) = v;
 }
 // Reads of what nothing reads again for a long time: those lines leave L2 first, and what the next kernel reads stays
-// (batch-norm apply passes and clearing: ResNet-50 on 32 images 3300 -> 3260 us per step, ResNet-34 2803 -> 2761).  For tensors of kLastBytes on, in kernels of their own: where the tensors of a step fit in L2 the backward pass
-// still finds them there, and a choice at run time costs as much as it gains (ResNet-50 on 12 images of 176x176, tensors of up
-// to 12 MB: 1346 us, 1351 with such reads, 1358 with the choice in the kernel).
+// (batch-norm apply passes and clearing).  For tensors of kLastBytes on, in kernels of their own: where the tensors are smaller
+// the backward pass still finds them in L2, and a choice at run time costs as much as it gains.  us per step without and with
+// such reads, ResNet-50 by its largest tensor: 11.9 MB (12 images of 176x176) 1346 and 1351 (1358 with the choice in the
+// kernel), 12.9 MB (13) 1285 and 1283, 15.9 MB (16) 1464 and 1462, 19.8 MB (20) 1697 and 1692, 28 MB (24 of 192x192) 2163 and
+// 2137, 51 MB (32 of 224x224) 3274 and 3240; ResNet-34 on 32 of 176x176 1250 and 1246, on 64 of 224x224 2907 and 2872.
 constexpr long long kLastBytes = 12LL << 20;
 template <bool kLast, typename T>
 __device__ __forceinline__ uint4 ld_raw_last(const T* p) {

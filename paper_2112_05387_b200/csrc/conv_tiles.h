@@ -46,13 +46,17 @@ inline double conv_tile_cycles(const ConvTileQuery& q, int tile) {
 }
 
 // What SM time is worth beside the length of a launch, where modules run side by side: a launch of length t on a share s of the
-// SMs costs t (1 + w s).  `step_flops`: convolutions of one training step.  Steps of little work are as long as their chains of
+// SMs costs t (1 + w s).  `step_flops`: convolutions of the modules in one training step (not those of the AuxNets).  Steps of little work are as long as their chains of
 // launches, and narrower tiles shorten a launch of few CTAs (8 CTAs of 256 channels took 40 to 46 us of ResNet-50's last module
 // on 12 images of 176x176); steps of much work are bound by the SM time that narrow tiles waste.  us per step for w = none, 1,
 // 2, 4, 8, 16: ResNet-34 on 3 images of 256x176 (0.06 TFLOP) 781, 683, 640, 638, 642, 674, on 25 of 128x160 with recursive
 // AuxNets and distillation (0.22) 1234, 1159, 1158, 1196, 1232, 1232; ResNet-50 on 12 of 176x176 (0.18) 1405, 1369, 1360, 1361,
 // 1370, 1410, on 19 with distillation (0.29) 2130, 2091, 2086, 2090, 2106, 2134, on 32 of 224x224 (0.79) 3303, 3358, 3332, 3325,
-// 3306, 3308.
+// 3306, 3308.  Where the cubic goes beyond 16 it is as good as infinite: against a limit of 16, ResNet-50 on 32 of 224x224 (w = 79)
+// 3240 and 3239, ResNet-34 on 64 of them (w in the hundreds) 2875 and 2872, WRN-28-10 on 128 of 32x32 (w = 10 000) 4690 and 4682.
+// The rule does not know the number of modules: with one module, which only its own weight gradients run beside, w = 0 would be
+// right for some networks (WRN-28-10 on 16 images 1530 -> 1435) and wrong for others (ResNet-34 on 8 of 160x160 1295 -> 1408).
+// Tiles of 64 columns also select the two-per-SM instantiation for small layers, which conv_tile_cycles() takes for the other one.
 inline double sm_time_worth(double step_flops) {
   const double x = step_flops / 0.25e12;
   return 2.5 * std::max(1.0, x * x * x);
