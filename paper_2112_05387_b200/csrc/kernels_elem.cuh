@@ -928,14 +928,12 @@ head_bwd_x_kernel(const float* __restrict__ dlogits, const float* __restrict__ W
 // clearing, updates
 // ---------------------------------------------------------------------------------------
 template <bool kLast>
-__global__ void __launch_bounds__(256) zero_kernel(uint4* __restrict__ p, long long n, uint4* __restrict__ p2, long long n2) {
+__global__ void __launch_bounds__(256) zero_kernel(uint4* __restrict__ p, long long n) {
   pdl_wait();
   pdl_launch_dependents();
-  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n + n2; i += (long long)gridDim.x * 256) {
-    uint4* at = i < n ? p + i : p2 + (i - n);
-    if (kLast) __stcs(at, make_uint4(0u, 0u, 0u, 0u));
-    else *at = make_uint4(0u, 0u, 0u, 0u);
-  }
+  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256)
+    if (kLast) __stcs(p + i, make_uint4(0u, 0u, 0u, 0u));
+    else p[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 __global__ void sgd_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ mom, long long n,

@@ -422,8 +422,8 @@ static int encode_tile32_map(CUtensorMap* m, const void* base, int N, int H, int
 
 static const size_t kTcMinSmem = 120 * 1024;   // more than half an SM: one CTA (and one TMEM owner) per SM
 static const size_t kTcMaxSmem = 220 * 1024;
-// A convolution of fewer FLOPs than this (and a tile of at most 64 channels: a layer of 64, or of more where the tile rule
-// divides it so) cannot fill the machine whatever its launch shape: a few microseconds of fixed cost dominate.  While several modules are enqueued side by side such
+// A convolution of fewer FLOPs than this (and at most 64 channels) cannot fill the machine whatever its launch
+// shape: a few microseconds of fixed cost dominate.  While several modules are enqueued side by side such
 // launches are sized to share the SMs with the other modules' kernels instead of taking them whole.
 static const double kSmallConvFlops = 4e9;
 static const size_t kTcThinSmem = 100 * 1024;  // two CTAs of the few-channel instantiation (or other kernels) per SM
@@ -2439,25 +2439,14 @@ static int run_ops(lp_handle* h, Plan& P, const std::vector<Op>& ops, const RunC
 
 // Clears what a pass accumulates into.  A kernel and not a memset: a memset between two kernels of a graph costs the chain
 // 10 to 25 us (a module began with three of them, 25 us for ResNet-110's and up to 55 for ResNet-50's on 12 images).
-static int zero_range(lp_handle* h, const ZeroRange& r, cudaStream_t st, const ZeroRange& r2 = ZeroRange()) {
-  if (!r.bytes && !r2.bytes) return LP_OK;
-  const long long n = (long long)(r.bytes / 16), n2 = (long long)(r2.bytes / 16);
+static int zero_range(lp_handle* h, const ZeroRange& r, cudaStream_t st) {
+  if (!r.bytes) return LP_OK;
+  const long long n = (long long)(r.bytes / 16);
   // (two blocks per SM: the gradients are cleared beside the first kernels of the forward passes)
   const auto kernel = r.bytes >= (size_t)kLastBytes ? zero_kernel<true> : zero_kernel<false>;
-  LP_CUDA_OK(launch_pdl(kernel, dim3(grid_for(n + n2, 256 * 4, cur_dev().sm_count, 2)), dim3(256), 0, st, (uint4*)r.p, n,
-                        (uint4*)r2.p, n2));
+  LP_CUDA_OK(launch_pdl(kernel, dim3(grid_for(n, 256 * 4, cur_dev().sm_count, 2)), dim3(256), 0, st, (uint4*)r.p, n));
   h->launches++;
   return LP_OK;
-}
-static bool recording(cudaStream_t st) {
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) { cudaGetLastError(); return false; }
-  return cs != cudaStreamCaptureStatusNone;
-}
-// Statistics of the AuxNets of stack k: its units were planned one after another.
-static ZeroRange stack_state(const lp_handle* h, int k) {
-  const ZeroRange &a = h->auxs[NetDef::reaux_index(k, 0)].state, &b = h->auxs[NetDef::reaux_index(k, k - 1)].state;
-  return ZeroRange{a.p, (size_t)(b.p + b.bytes - a.p)};
 }
 // The gradients of all modules, on a stream of their own forked from `fork`: nothing needs them before the backward passes.
 static int zero_grads_beside(lp_handle* h) {
@@ -3038,15 +3027,8 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
   }
   return run_as_graph(h, CALL_LAYER_PARALLEL, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   ConcurrentScope concurrent(h);
-  // Statistics: one launch clears all of them, which is the cheapest to make launch by launch.  In a graph every branch clears
-  // its own: a graph with one root starts when its last node has reached the device, one with a root for every branch meanwhile
-  // (first launch of a graph, us, one and several roots: ResNet-110 on 128 images 1480 and 1234, ResNet-56 816 and 782, WRN-28-10
-  // 4340 and 4175, ResNet-50 on 32 images 3592 and 3351, on 12 of 176x176 with recursive AuxNets 1677 and 1465).
-  const bool own_roots = recording(st) && K > 1;
-  if (!own_roots) {
-    const int rc0 = zero_range(h, h->zero.all_state, st);
-    if (rc0 != LP_OK) return rc0;
-  }
+  const int rc0 = zero_range(h, h->zero.all_state, st);
+  if (rc0 != LP_OK) return rc0;
   LP_CUDA_OK(cudaEventRecord(h->fork, st));
   const int rc1 = zero_grads_beside(h);
   // Streams forked from the caller's so far; whatever happens below, each is joined back before the
@@ -3077,7 +3059,6 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
         if ((rc = fork_module(k)) != LP_OK) return rc;
         RunCtx c;
         c.st = sk; c.images = images; c.xout = x_out;
-        if (own_roots && (rc = zero_range(h, h->modules[k].state, sk, stack_state(h, k))) != LP_OK) return rc;
         for (int j = 0; j < k; ++j)
           if ((rc = aux_plan_forward(h, NetDef::reaux_index(k, j), c)) != LP_OK) return rc;
         LP_CUDA_OK(cudaEventRecord(h->aux_done[k - 1], sk));
@@ -3086,7 +3067,6 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
       // AuxNet chain on its own stream; aux_done[k] marks x_{k+1}
       RunCtx c;
       c.st = h->aux_stream; c.images = images; c.xout = x_out;
-      if (own_roots && (rc = zero_range(h, h->zero.aux_state, h->aux_stream)) != LP_OK) return rc;
       for (int k = 0; k + 1 < K; ++k) {
         if ((rc = aux_plan_forward(h, k, c)) != LP_OK) return rc;
         LP_CUDA_OK(cudaEventRecord(h->aux_done[k], h->aux_stream));
@@ -3097,7 +3077,6 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
     for (int k = 0; k < K; ++k) {
       cudaStream_t sk = h->streams[k];
       if ((rc = fork_module(k)) != LP_OK) return rc;
-      if (own_roots && (k == 0 || !h->net.d.aux_recursive) && (rc = zero_range(h, h->modules[k].state, sk)) != LP_OK) return rc;
       if (k > 0) LP_CUDA_OK(cudaStreamWaitEvent(sk, h->aux_done[k - 1], 0));
       const bool last = k == K - 1;
       const void* xk = k == 0 ? images : x_out[k - 1];

@@ -803,45 +803,6 @@ def test_update_and_distillation_in_two_recordings_at_once():
         assert rel_err(a, b) < 1e-5                   # (fp32 sums in another order)
 
 
-@pytest.mark.parametrize("recursive", [False, True])
-@pytest.mark.parametrize("dtype,ends", [("f32", (1, 2)), ("bf16", (1, 3, 4)), ("bf16", (1, 2, 3, 4))])
-def test_replays_of_a_recorded_step_start_from_cleared_statistics(dtype, ends, recursive):
-    """In a recorded step every branch (AuxNet chain or stack, module) clears its own statistics and loss sums, launch by launch
-    one launch clears all: three replays against direct calls.  Rates of zero, so that every pass is the same; what is left over
-    from the pass before would double a variance.  Sums in another order: 1e-5 in fp32, 2e-2 once bf16 values flip."""
-    cfg = small_cfg("preact", N=4, H=8, W=8, dtype=dtype, stage_channels=(16, 32), stage_blocks=(2, 2) if len(ends) > 2 else (1, 1),
-                    module_block_end=ends, stem_channels=16, classes=10)
-    runs = [GpuRun(cfg, aux_recursive=recursive), GpuRun(cfg, aux_recursive=recursive)]
-    torch, tol = runs[0].torch, 1e-5 if dtype == "f32" else 2e-2
-    stream = torch.cuda.Stream()
-    for run in runs:
-        lp, h = run.lp, run.h
-
-        def step():
-            lp.lp_layer_parallel_step(h, run.d_images, run.d_x[1:], run.d_labels, run.d_kappa, cfg["rho"], run.d_loss, run.d_dx, 0.0,
-                                      0.0, 0.0, 0.0, stream.cuda_stream)
-        torch.cuda.synchronize()
-        step()
-        if run is runs[0]:
-            lp.lp_graph_begin(h, stream.cuda_stream)
-            step()
-            gid = lp.lp_graph_end(h, stream.cuda_stream)
-        else:
-            lp.lp_timeline(h, True, read=False)          # (keeps its calls direct)
-        run.seen = []
-        for _ in range(3):
-            for t in [run.d_loss] + run.d_x[1:] + run.d_dx[1:]:
-                t.fill_(7.0)
-            torch.cuda.synchronize()
-            lp.lp_graph_launch(h, gid, stream.cuda_stream) if run is runs[0] else step()
-            assert lp.lp_last_device_status(h, stream.cuda_stream) == 0
-            run.seen.append([to_host(run.d_loss)] + [to_host(t) for t in run.d_x[1:] + run.d_dx[1:]] +
-                            [lp.lp_get_grads(h, k) for k in range(run.net.K)])
-    for a, b in zip(*(run.seen for run in runs)):
-        for i, (u, v) in enumerate(zip(a, b)):
-            assert rel_err(u, v) < tol, i
-
-
 def test_one_multiplier_buffer_for_two_modules():
     """lp_step with one buffer given to two modules whose boundaries have one shape: both residuals arrive.  fp32: two roundings
     of a sum, 2^-24 of it each."""
