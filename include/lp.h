@@ -315,7 +315,8 @@ int lp_timeline(lp_handle* h, int enable, int max_records, lp_timeline_record* r
  * (the internal module streams are forked from and joined into it), then replay the recording.
  * Pointer arguments of the recorded calls are baked into the graph.  Up to 8 graphs per handle;
  * *graph_id receives the slot.  The first call of every kind must have run once outside a capture
- * (kernel attributes are set on first use). */
+ * (kernel attributes are set on first use).  lp_graph_end sends the graph to the device (asynchronously on `stream`), so that its
+ * first launch need not; it may be launched at once, on any stream. */
 int lp_graph_begin(lp_handle* h, void* stream);
 int lp_graph_end(lp_handle* h, void* stream, int* graph_id);
 int lp_graph_launch(lp_handle* h, int graph_id, void* stream);

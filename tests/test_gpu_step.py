@@ -803,6 +803,36 @@ def test_update_and_distillation_in_two_recordings_at_once():
         assert rel_err(a, b) < 1e-5                   # (fp32 sums in another order)
 
 
+@pytest.mark.parametrize("recursive", [False, True])
+def test_a_recording_is_launched_at_once_on_another_stream(recursive):
+    """lp_graph_end, then launches on a stream that nothing orders behind the recording's: three steps, each from cleared statistics,
+    against direct calls (rates of zero: every step is the same; fp32 sums in another order)."""
+    cfg = small_cfg("preact", N=4, H=8, W=8, stage_channels=(8, 16), stage_blocks=(2, 2), module_block_end=(1, 3, 4))
+    runs = [GpuRun(cfg, aux_recursive=recursive), GpuRun(cfg, aux_recursive=recursive)]
+    torch = runs[0].torch
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    for run in runs:
+        lp, h = run.lp, run.h
+
+        def step(stream):
+            lp.lp_layer_parallel_step(h, run.d_images, run.d_x[1:], run.d_labels, run.d_kappa, cfg["rho"], run.d_loss, run.d_dx, 0.0,
+                                      0.0, 0.0, 0.0, stream.cuda_stream)
+        torch.cuda.synchronize()
+        step(s1)
+        torch.cuda.synchronize()
+        if run is runs[0]:
+            lp.lp_graph_begin(h, s1.cuda_stream)
+            step(s1)
+            gid = lp.lp_graph_end(h, s1.cuda_stream)
+            for _ in range(3):
+                lp.lp_graph_launch(h, gid, s2.cuda_stream)
+        assert lp.lp_last_device_status(h, s2.cuda_stream) == 0
+        run.seen = ([to_host(run.d_loss)] + [to_host(t) for t in run.d_x[1:] + run.d_dx[1:]] +
+                    [lp.lp_get_grads(h, k) for k in range(run.net.K)])
+    for i, (a, b) in enumerate(zip(runs[0].seen, runs[1].seen)):
+        assert rel_err(a, b) < 1e-5, i
+
+
 def test_one_multiplier_buffer_for_two_modules():
     """lp_step with one buffer given to two modules whose boundaries have one shape: both residuals arrive.  fp32: two roundings
     of a sum, 2^-24 of it each."""
