@@ -160,9 +160,9 @@ int lp_boundary_shape_desc(const lp_net_desc* desc, int k, int shape_nhwc[4]);
  * Calls on one handle are made by one thread at a time.  The handle has streams and events of its own: lp_modules_fwd_bwd_all,
  * lp_step, lp_layer_parallel_step, lp_auxnet_distill and lp_serial_fwd_bwd fork work onto them and join it before what follows
  * the call on its `stream`; lp_module_fwd_bwd uses those of its module only.  Calls on different streams are therefore ordered
- * where they share one.  During a caller's recording of one such call the handle's streams belong to the recording: until it
- * ends, lp_step and lp_auxnet_distill stay on the stream they are given (recorded elsewhere or not), the other three return
- * LP_ERR_CUDA outside that recording.
+ * where they share one.  Streams of the handle that a caller's recording has reached belong to it until it ends: meanwhile
+ * lp_step and lp_auxnet_distill, called outside that recording, stay on the stream they are given; the other calls that need
+ * such a stream return LP_ERR_CUDA.
  * The handle owns host memory, streams, events and -- from the third call of a kind on -- one executable graph for each
  * of lp_auxnet_forward, lp_modules_fwd_bwd_all, lp_step, lp_layer_parallel_step, lp_auxnet_distill, lp_forward_serial and
  * lp_serial_fwd_bwd, as which the call is then launched (recorded anew each time with its own arguments).  The driver
