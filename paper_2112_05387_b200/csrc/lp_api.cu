@@ -2448,14 +2448,29 @@ static int zero_range(lp_handle* h, const ZeroRange& r, cudaStream_t st) {
   h->launches++;
   return LP_OK;
 }
+// Whether work can be forked from `st` onto another stream: not while that one is in a recording that `st` is not in.  (A
+// handle's streams stay in a caller's recording until it ends; meanwhile the caller may make other calls, recorded or not.)
+static bool can_fork(cudaStream_t st, cudaStream_t onto) {
+  cudaStreamCaptureStatus a = cudaStreamCaptureStatusNone, b = cudaStreamCaptureStatusNone;
+  unsigned long long ia = 0, ib = 0;
+  if (cudaStreamGetCaptureInfo(onto, &b, &ib) != cudaSuccess) { cudaGetLastError(); return false; }
+  if (b == cudaStreamCaptureStatusNone) return true;
+  if (cudaStreamGetCaptureInfo(st, &a, &ia) != cudaSuccess) { cudaGetLastError(); return false; }
+  return a != cudaStreamCaptureStatusNone && ia == ib;
+}
+static bool can_fork(cudaStream_t st, const std::vector<cudaStream_t>& onto) {
+  return std::all_of(onto.begin(), onto.end(), [&](cudaStream_t s) { return can_fork(st, s); });
+}
+
 // The gradients of all modules, on a stream of their own forked from `fork`: nothing needs them before the backward passes.
-static int zero_grads_beside(lp_handle* h) {
-  LP_CUDA_OK(cudaStreamWaitEvent(h->zero_stream, h->fork, 0));
+static int zero_grads_beside(lp_handle* h, cudaStream_t st) {
+  const cudaStream_t on = can_fork(st, h->zero_stream) ? h->zero_stream : st;
+  if (on != st) LP_CUDA_OK(cudaStreamWaitEvent(on, h->fork, 0));
   // (a module whose pass is not enqueued after this has no gradients any more: lp_step passes it by)
   for (auto& P : h->modules) P.ps.grads_fresh = false;
-  const int rc = zero_range(h, h->zero.module_grads, h->zero_stream);
+  const int rc = zero_range(h, h->zero.module_grads, on);
   // (recorded whatever happened: the caller joins the stream through this event)
-  LP_CUDA_OK(cudaEventRecord(h->grads_zeroed, h->zero_stream));
+  LP_CUDA_OK(cudaEventRecord(h->grads_zeroed, on));
   return rc;
 }
 
@@ -2524,20 +2539,6 @@ static int sgd_update_inner(lp_handle* h, Plan& P, float lr, float momentum, flo
   h->launches++;
   LP_CUDA_OK(cudaGetLastError());
   return LP_OK;
-}
-
-// Whether work can be forked from `st` onto another stream: not while that one is in a recording that `st` is not in.  (A
-// handle's streams stay in a caller's recording until it ends; meanwhile the caller may make other calls, recorded or not.)
-static bool can_fork(cudaStream_t st, cudaStream_t onto) {
-  cudaStreamCaptureStatus a = cudaStreamCaptureStatusNone, b = cudaStreamCaptureStatusNone;
-  unsigned long long ia = 0, ib = 0;
-  if (cudaStreamGetCaptureInfo(onto, &b, &ib) != cudaSuccess) { cudaGetLastError(); return false; }
-  if (b == cudaStreamCaptureStatusNone) return true;
-  if (cudaStreamGetCaptureInfo(st, &a, &ia) != cudaSuccess) { cudaGetLastError(); return false; }
-  return a != cudaStreamCaptureStatusNone && ia == ib;
-}
-static bool can_fork(cudaStream_t st, const std::vector<cudaStream_t>& onto) {
-  return std::all_of(onto.begin(), onto.end(), [&](cudaStream_t s) { return can_fork(st, s); });
 }
 
 static size_t boundary_bytes(const lp_handle* h, int k) {   // of x_k
@@ -2931,7 +2932,7 @@ int lp_modules_fwd_bwd_all(lp_handle* h, const void* const* x, const int32_t* la
   // heaviest modules first is not needed: all K are enqueued before any can finish
   // A failure part-way still joins every stream that was forked back into the caller's (a stream left
   // unjoined would invalidate a capture in progress); the first error is what the call returns.
-  int first_err = zero_grads_beside(h);
+  int first_err = zero_grads_beside(h, st);
   int forked = 0;
   for (int k = 0; k < K && first_err == LP_OK; ++k) {
     if (cudaStreamWaitEvent(h->streams[k], h->fork, 0) != cudaSuccess) { first_err = LP_ERR_CUDA; break; }
@@ -3030,7 +3031,7 @@ int lp_layer_parallel_step(lp_handle* h, const void* images, void* const* x_out,
   const int rc0 = zero_range(h, h->zero.all_state, st);
   if (rc0 != LP_OK) return rc0;
   LP_CUDA_OK(cudaEventRecord(h->fork, st));
-  const int rc1 = zero_grads_beside(h);
+  const int rc1 = zero_grads_beside(h, st);
   // Streams forked from the caller's so far; whatever happens below, each is joined back before the
   // call returns (a stream left unjoined would invalidate a capture in progress).
   bool aux_forked = false;
@@ -3255,7 +3256,7 @@ int lp_serial_fwd_bwd(lp_handle* h, const void* images, const int32_t* labels, f
   return run_as_graph(h, CALL_SERIAL, (cudaStream_t)stream, [&](cudaStream_t st) -> int {
   const int K = h->net.K;
   LP_CUDA_OK(cudaEventRecord(h->fork, st));
-  int rc = zero_grads_beside(h);
+  int rc = zero_grads_beside(h, st);
   if (rc == LP_OK) rc = serial_forward(h, images, labels, loss_out, st);
   if (cudaStreamWaitEvent(st, h->grads_zeroed, 0) != cudaSuccess && rc == LP_OK) rc = LP_ERR_CUDA;
   if (rc != LP_OK) return rc;

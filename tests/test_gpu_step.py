@@ -833,6 +833,37 @@ def test_a_recording_is_launched_at_once_on_another_stream(recursive):
         assert rel_err(a, b) < 1e-5, i
 
 
+def test_layer_serial_pass_beside_a_recording_of_one():
+    """With its weight gradients in the chain a layer-serial pass needs no stream but the caller's: it runs beside an open recording
+    of the same call, and both give the gradients that a call by itself gives (fp32 sums in another order)."""
+    import paper_2112_05387_b200 as lp
+    cfg = small_cfg("preact", N=4, H=8, W=8, stage_channels=(8, 16), stage_blocks=(2, 2), module_block_end=(1, 3, 4))
+    run = GpuRun(cfg, conv_impl=lp.LP_CONV_WGRAD_IN_CHAIN)
+    h, torch, K = run.h, run.torch, run.net.K
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def serial(stream):
+        lp.lp_serial_fwd_bwd(h, run.d_images, run.d_labels, run.d_loss[K - 1], stream.cuda_stream)
+
+    def grads():
+        assert lp.lp_last_device_status(h) == 0
+        return [lp.lp_get_grads(h, k) for k in range(K)]
+    serial(s2)
+    seen = [grads()]
+    lp.lp_graph_begin(h, s1.cuda_stream)
+    serial(s1)
+    serial(s2)
+    s2.synchronize()
+    gid = lp.lp_graph_end(h, s1.cuda_stream)
+    seen.append(grads())
+    lp.lp_graph_launch(h, gid, s1.cuda_stream)
+    seen.append(grads())
+    for other in seen[1:]:
+        for a, b in zip(other, seen[0]):
+            assert rel_err(a, b) < 1e-5
+
+
 def test_one_multiplier_buffer_for_two_modules():
     """lp_step with one buffer given to two modules whose boundaries have one shape: both residuals arrive.  fp32: two roundings
     of a sum, 2^-24 of it each."""
